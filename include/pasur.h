@@ -59,13 +59,11 @@ typedef struct {
  *                Umax = max |leaf value| in the subtree of the FGT root being solved (so each
  *                root's solve depends on its own subtree only), t = iteration index (1-based)
  *   dcfr_alpha/beta/gamma  DCFR discount exponents (the paper ran 1.5, 0, 2)
- *   slots_per_item  score slots solved together by one thread block: 0 = automatic (the
- *                smallest shared-memory class a root fits with one slot, then as many slots as
- *                that class holds, at most 32); n > 0 = up to n (at most the root's own and 32),
- *                in the smallest class that holds them.  Every block takes a power-of-two number
- *                of slots; results do not depend on the grouping
- *   threads      threads per block of the CFR kernel (0 = choose per subtree size, else a
- *                multiple of 32 up to 1024)
+ *   slots_per_item  score slots solved together by one thread block (or cluster): 0 = automatic (as
+ *                many as its shared memory holds, at most 6; fewer when there are few slots in all);
+ *                n > 0 = up to n (at most the root's own and 6).  Results do not depend on the grouping
+ *   threads      threads per block of the CFR kernels (0 = choose per launch, else a multiple of 32
+ *                up to 1024; more than 512 runs as 512)
  *   split_bytes  a root subtree whose state needs more shared memory than one block has is split
  *                over a thread-block cluster (up to 16 SMs, distributed shared memory); with
  *                split_bytes > 0 every subtree needing more than that many bytes is split too
@@ -275,9 +273,8 @@ typedef struct pasur_batch pasur_batch;
 /* Build rounds first_round..5 of n_deals seeded deals (decks: host, 52 bytes per deal), each from
  * the standalone root of first_round (pool = deck[0:4], score (0,0,0,0)), with every round's
  * unfolding and links, and plan their CFR: the work items of all deals' trees of one round are
- * merged into one persistent launch per shared-memory class (largest subtrees first).  With
- * cfg->threads == 0 an autotuner times candidate block sizes per class on the round with the most
- * work and keeps the fastest.  cfg is fixed for the batch.  The batch owns its trees.
+ * merged into one launch per slot count and shared-memory need (largest subtrees first).  cfg is fixed
+ * for the batch.  The batch owns its trees.
  * The deals are built on up to 8 host threads (at most one per deal and per host core; the
  * environment variable PASUR_BUILD_WORKERS lowers the count), each on its own CUDA stream; the
  * result does not depend on the count.  Their device memory counts against ctx's budget; on any

@@ -223,7 +223,7 @@ int pasur_destroy(pasur_ctx *ctx) {
     dev_free(ctx, ctx->counter, 64);
     dev_free(ctx, ctx->errflag, 64);
     cudaStreamSynchronize(ctx->stream);
-    for (int c = 0; c < 12; c++) {
+    for (int c = 0; c < kAuxStreams; c++) {
         if (ctx->aux[c]) cudaStreamDestroy(ctx->aux[c]);
         if (ctx->join[c]) cudaEventDestroy(ctx->join[c]);
         if (ctx->cls_t0[c]) cudaEventDestroy(ctx->cls_t0[c]);

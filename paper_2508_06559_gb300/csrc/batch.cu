@@ -1,8 +1,7 @@
 // Batched exact solve of many seeded deals: every deal's rounds are built and unfolded up front,
-// the work items of all deals' trees of one round are merged into one plan (one persistent
-// launch per shared-memory class, largest subtrees first across all deals), an autotuner picks
-// the block size of every class on the largest round, and the whole backward sweep (leaf values,
-// CFR, root utilities, round 5 down to the first round) is captured once into a CUDA graph and
+// the work items of all deals' trees of one round are merged into one plan (one launch per slot count
+// and shared-memory need, largest subtrees first across all deals), and the whole backward sweep (leaf
+// values, CFR, root utilities, round 5 down to the first round) is captured once into a CUDA graph and
 // replayed.
 #include <algorithm>
 #include <atomic>
@@ -64,11 +63,10 @@ int batch_alloc(pasur_batch *b, void **p, size_t bytes) {
     return PASUR_OK;
 }
 
-// What one deal leaves for the merged plans: per round its work items by launch class, the
-// shared memory each class needs and its cluster items.
+// What one deal leaves for the merged plans: per round its work items by storage class
+// and its cluster items.
 struct DealPlan {
     std::vector<CfrItem> own[6][8];
-    size_t need[6][8] = {};
     std::vector<ClusterItem> clu[6];
     int64_t edges = 0, solved_edges = 0, swept_edges = 0, swept_pairs = 0;
 };
@@ -110,7 +108,7 @@ int build_deal(pasur_batch *b, pasur_ctx *wc, const uint8_t *deck, int64_t d, De
         PASUR_TRY(plan_solve_slots(t, b->cfg.merge_delta != 0 && !cut, nullptr));
         PASUR_TRY(tree_alloc(t, (void **)&t->leaf_v, sizeof(float) * (size_t)(t->cQ[8] + 1)));
         if (t->M[8] > 0) PASUR_CUDA(wc, cudaMemsetAsync(t->leaf_v, 0, sizeof(float) * (size_t)(t->cQ[8] + 1), wc->stream));
-        PASUR_TRY(cfr_setup_tree(t, &b->cfg, (int)d, o.own[ri], o.need[ri], &o.clu[ri]));
+        PASUR_TRY(cfr_setup_tree(t, &b->cfg, (int)d, o.own[ri], &o.clu[ri]));
         t->cfr_ready = true;
         t->variant = b->cfg.variant;
         // the tree keeps its own items for exporting its average strategy
@@ -232,63 +230,6 @@ int build_deals(pasur_batch *b, const uint8_t *decks, std::vector<DealPlan> &dp,
     return rc;
 }
 
-// Time one class of a plan alone (no other class, no cluster item) for a few iterations at each
-// candidate block size; keep the best.  Class 5 (the level-streaming sweep) and the cluster
-// items have no block size to choose.
-int autotune(pasur_batch *b, CfrPlan &plan) {
-    pasur_ctx *ctx = b->ctx;
-    pasur_config cfg = b->cfg;
-    cfg.iters = 8;
-    cudaEvent_t e0, e1;
-    PASUR_CUDA(ctx, cudaEventCreate(&e0));
-    PASUR_CUDA(ctx, cudaEventCreate(&e1));
-    for (int c = 0; c < 5; c++) {
-        if (plan.cls_end[c] == plan.cls_begin[c]) continue;
-        const int def = plan.cls_threads[c];
-        const int cand_small[3] = {64, 128, 256}, cand_wide[3] = {256, 512, 1024};
-        const int *cand = def > 256 ? cand_wide : cand_small;
-        CfrPlan one = plan;
-        for (int o = 0; o < 8; o++)
-            if (o != c) one.cls_begin[o] = one.cls_end[o] = 0;
-        for (int o = 0; o < kCluGroups; o++) one.clu_begin[o] = one.clu_end[o] = 0;
-        float best_ms = 1e30f;
-        int best = def;
-        for (int i = 0; i < 3; i++) {
-            int blocks = 0;
-            PASUR_TRY(cfr_occupancy(ctx, cand[i], c, one.cls_smem[c], one.cls_end[c] - one.cls_begin[c], &blocks));
-            if (blocks <= 0) continue;
-            one.cls_threads[c] = cand[i];
-            one.cls_blocks[c] = blocks;
-            PASUR_CUDA(ctx, cudaEventRecord(e0, ctx->stream));
-            PASUR_TRY(cfr_launch_plan(ctx, one, &cfg, 0, nullptr));
-            PASUR_CUDA(ctx, cudaEventRecord(e1, ctx->stream));
-            PASUR_CUDA(ctx, cudaEventSynchronize(e1));
-            float ms = 0.f;
-            PASUR_CUDA(ctx, cudaEventElapsedTime(&ms, e0, e1));
-            if (getenv("PASUR_VERBOSE"))
-                fprintf(stderr, "[pasur] autotune class %d alone: %d blocks x %d threads, %d iterations in %.3f ms\n", c, blocks,
-                        cand[i], cfg.iters, ms);
-            if (ms < best_ms) {
-                best_ms = ms;
-                best = cand[i];
-            }
-        }
-        // apply to every round's plan
-        for (CfrPlan &pl : b->plans) {
-            if (pl.cls_end[c] == pl.cls_begin[c]) continue;
-            int blocks = 0;
-            PASUR_TRY(cfr_occupancy(ctx, best, c, pl.cls_smem[c], pl.cls_end[c] - pl.cls_begin[c], &blocks));
-            if (blocks > 0) {
-                pl.cls_threads[c] = best;
-                pl.cls_blocks[c] = blocks;
-            }
-        }
-    }
-    cudaEventDestroy(e0);
-    cudaEventDestroy(e1);
-    return PASUR_OK;
-}
-
 // one backward sweep on ctx->stream without host synchronisation (captured into the graph)
 int record_sweep(pasur_batch *b) {
     pasur_ctx *ctx = b->ctx;
@@ -339,25 +280,7 @@ int print_batch(pasur_batch *b) {
             PASUR_TRY(cfr_export_utilities_n(tree_of(b, d, ri), b->cfg.iters, b->util[(size_t)(d * b->n_rounds + ri)]));
         fprintf(stderr, "[pasur] batch round %d: %lld items, %d iterations in %.3f ms\n", b->first_round + ri,
                 (long long)pl.n_items, b->cfg.iters, ms);
-        for (int bk = 0; bk < kCluGroups; bk++)
-            if (pl.clu_end[bk] != pl.clu_begin[bk])
-                fprintf(stderr, "[pasur]   cluster items: %lld, %d CTAs x %d threads, smem %zu B, %.3f ms\n",
-                        (long long)(pl.clu_end[bk] - pl.clu_begin[bk]), pl.clu_ctas[bk], pl.clu_threads, pl.clu_smem[bk],
-                        pl.cls_ms[6 + bk]);
-        for (int c = 0; c < 8; c++) {
-            const int64_t n = pl.cls_end[c] - pl.cls_begin[c];
-            if (!n) continue;
-            int64_t cost = 0, slots = 0, maxcost = 0;
-            for (int64_t i = pl.cls_begin[c]; i < pl.cls_end[c]; i++) {
-                cost += pl.items_h[(size_t)i].cost;
-                slots += pl.items_h[(size_t)i].ns;
-                maxcost = std::max(maxcost, pl.items_h[(size_t)i].cost);
-            }
-            fprintf(stderr, "[pasur]   class %d: items %lld (slots %lld), smem %zu B, blocks %d x %d threads, "
-                            "active-node-slots %lld (largest item %lld), %.3f ms\n",
-                    c, (long long)n, (long long)slots, pl.cls_smem[c], pl.cls_blocks[c], pl.cls_threads[c], (long long)cost,
-                    (long long)maxcost, pl.cls_ms[c]);
-        }
+        cfr_print_plan(pl);
     }
     PASUR_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
     return PASUR_OK;
@@ -457,7 +380,7 @@ static int batch_create(pasur_ctx *ctx, const uint8_t *decks, int64_t n_deals, i
     int rc = PASUR_OK;
     const bool verbose = getenv("PASUR_VERBOSE") != nullptr;
     using clk = std::chrono::steady_clock;
-    double ph_ms[4] = {0};  // rounds and layouts, surrogate, merged plans, autotune
+    double ph_ms[3] = {0};  // rounds and layouts, surrogate, merged plans
     int n_workers = 1;
     auto lap = [&](clk::time_point &t0, int i) {
         if (!verbose) return;
@@ -488,19 +411,15 @@ static int batch_create(pasur_ctx *ctx, const uint8_t *decks, int64_t n_deals, i
     b->plans.resize((size_t)b->n_rounds);
     for (int ri = 0; ri < b->n_rounds && rc == PASUR_OK; ri++) {
         std::vector<CfrItem> cls_items[8];
-        size_t need[8] = {0};
-        std::vector<TreeView> views;
+        std::vector<pasur_tree *> trees;
         std::vector<ClusterItem> clu;
         for (int64_t d = 0; d < n_deals; d++) {
             DealPlan &o = dp[(size_t)d];
-            for (int c = 0; c < 8; c++) {
-                cls_items[c].insert(cls_items[c].end(), o.own[ri][c].begin(), o.own[ri][c].end());
-                need[c] = std::max(need[c], o.need[ri][c]);
-            }
+            for (int c = 0; c < 8; c++) cls_items[c].insert(cls_items[c].end(), o.own[ri][c].begin(), o.own[ri][c].end());
             clu.insert(clu.end(), o.clu[ri].begin(), o.clu[ri].end());
-            views.push_back(tree_of(b, d, ri)->view);
+            trees.push_back(tree_of(b, d, ri));
         }
-        rc = cfr_finalize_plan(ctx, b->plans[(size_t)ri], cls_items, need, views, cfg, b->owned, clu);
+        rc = cfr_finalize_plan(ctx, b->plans[(size_t)ri], cls_items, trees, cfg, b->owned, clu);
     }
     for (const DealPlan &o : dp) {
         b->edges += o.edges;
@@ -513,22 +432,10 @@ static int batch_create(pasur_ctx *ctx, const uint8_t *decks, int64_t n_deals, i
     if (rc == PASUR_OK && b->dcfr) b->owned.push_back({b->dcfr, b->dcfr_bytes});
     if (rc == PASUR_OK && cudaStreamSynchronize(ctx->stream) != cudaSuccess) rc = set_err(ctx, PASUR_ECUDA, "pasur_batch_create: sync");
     lap(tp, 2);
-    // autotune the block size of every class on the round with the most work
-    if (rc == PASUR_OK && cfg->threads == 0) {
-        int big = 0;
-        int64_t best = -1;
-        for (int ri = 0; ri < b->n_rounds; ri++) {
-            int64_t cost = 0;
-            for (const CfrItem &it : b->plans[(size_t)ri].items_h) cost += it.cost;
-            if (cost > best) best = cost, big = ri;
-        }
-        rc = autotune(b, b->plans[(size_t)big]);
-    }
     if (rc == PASUR_OK) rc = ensure_aux(ctx);
-    lap(tp, 3);
     if (rc == PASUR_OK && verbose) {
         fprintf(stderr, "[pasur] batch create: rounds and layouts %.1f ms (%d build workers), surrogate %.1f, "
-                        "merged plans %.1f, autotune %.1f\n", ph_ms[0], n_workers, ph_ms[1], ph_ms[2], ph_ms[3]);
+                        "merged plans %.1f\n", ph_ms[0], n_workers, ph_ms[1], ph_ms[2]);
         rc = print_batch(b);
     }
     if (rc != PASUR_OK) {

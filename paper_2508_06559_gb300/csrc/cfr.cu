@@ -3,11 +3,10 @@
 //
 // Round roots are independent (open hands: every FGT node is its own information set and root
 // reach is 1), so the round is cut into work items: one GT root and a run of W of its score
-// slots.  A persistent grid takes items from a queue (largest first).  One thread block runs all
-// T iterations of an item: per iteration a top-down pass over levels 0..6 (regret matching and
-// reach) and a bottom-up pass over levels 7..0 (values, regret and strategy-sum updates), with a
-// block barrier between levels; an (active node, slot) pair belongs to one thread in each pass,
-// so the updates of a node's child edges need no atomics.
+// slots.  One thread block runs all T iterations of an item (cfr_sweep.cuh): per iteration a top-down
+// pass over levels 0..6 (regret matching and reach) and a bottom-up pass over levels 7..0 (values,
+// regret and strategy-sum updates), with a block barrier between levels; an (active node, slot) pair
+// belongs to one thread in each pass, so the updates of a node's child edges need no atomics.
 //
 // Forced-move chains are resolved once: a node whose whole subtree is one path of single moves
 // has sigma = 1 and zero regret on every edge below it and the value of its one leaf, so only the
@@ -16,9 +15,9 @@
 // S, values V and reaches live in shared memory for all T iterations (no DRAM traffic per
 // iteration).  A root whose state does not fit one block is split over a thread-block cluster
 // (distributed shared memory) or, beyond a cluster, swept level by level over every SM with its
-// state in device memory.  Item layout: local node index times slots, slot-minor; the local nodes
-// of each level are numbered in the order of their parents' entries, so the children of
-// consecutive entries are consecutive.
+// state in device memory.  Between calls R and S lie in device memory, local node index times slots,
+// slot-minor; the local nodes of each level are numbered in the order of their parents' entries, so
+// the children of consecutive entries are consecutive.
 #include <algorithm>
 #include <atomic>
 #include <cmath>
@@ -28,35 +27,33 @@
 #include <string>
 #include <thread>
 
+#include "cfr_block.cuh"
+#include "cfr_node.cuh"
 #include "pasur_internal.cuh"
 
 namespace pasur {
 namespace {
 
-// shared-memory classes of the resident items: budget per block (several blocks per SM), then
-// the global-memory fallback.  Class 0 is sized for six 128-thread blocks per SM (228 KB per SM,
-// 1 KB reserved per block, under 0.4 KB of static shared memory; six is also the register limit
-// at 80 registers): on the full game it measured 2 % faster than 40 KB at five blocks per SM.
+// classes by which R and S are stored in device memory (slots per stored item): budget of a block's
+// shared memory at 16 bytes per (node, slot), then the streamed items.  A checkpoint holds R and S in
+// this order, so the classes stay as they are whatever the sweep's own layout is.
 constexpr int kNumCls = 6;
+constexpr size_t kStorageReserve = 352;  // part of a block's shared memory the storage classes leave free
 constexpr size_t kClsBudget[kNumCls - 1] = {37536, 54 * 1024, 74 * 1024, 112 * 1024, 0 /* opt-in max */};
 constexpr int kClsGlobal = kNumCls - 1;
 constexpr int kClsCluster = 6;       // plan class of the cluster items' pseudo-items (exports only)
 constexpr int kMaxClusterCtas = 16;  // CTAs of a cluster (16: non-portable size)
-// default block size per class (the batch autotuner measures its own); class 3 at two 256-thread
-// blocks per SM measured faster than one 512-thread block of the 512-thread instantiation; class 4
-// (one block per SM) at 512 threads: more warps to cover the level steps' latency than at 256
-// (seed-47 CFR 1234 -> 1175 ms) and fewer idle at the barriers than at 1024
-constexpr int kClsThreads[kNumCls] = {128, 128, 256, 256, 512, 1024};
+// forked streams: the level-streaming sweep, the cluster groups, the block sweep's groups
+constexpr int kAuxStream = 0, kAuxCluster = 1, kAuxBlock = kAuxCluster + kCluGroups;
+constexpr int64_t kSlotsPerSm = 2;
 
 struct CfrParams {
     const CfrItem *items;
-    int64_t i_begin, i_end;
     const TreeView *views;
     const float *dcfr;  // per iteration: regret factor if R > 0, if R <= 0, strategy-sum factor
     int iters;
     int64_t t0;
     float tau;  // dead zone: a regret counts as positive above tau * t * Umax(root)
-    int32_t *counter;
     int32_t *err;
 };
 
@@ -79,34 +76,6 @@ constexpr int64_t kStreamMinSlots = 16;
 template <bool W1>
 __device__ __forceinline__ int at(int c, int a, int sh, int w) {
     return W1 ? c + a : ((c + a) << sh) + w;
-}
-
-// Pairwise sum of D values (a short dependency chain: about log2(D) additions deep).
-template <int D>
-__device__ __forceinline__ float tree_sum(const float *x) {
-    if (D == 1) return x[0];
-    if (D == 2) return x[0] + x[1];
-    constexpr int H = D / 2;
-    return tree_sum<H>(x) + tree_sum<D - H>(x + H);
-}
-
-// 1 / s for a positive regret sum: the fast reciprocal (at most 2 ulp; the sum is a normal
-// number, since counted regrets exceed the dead zone).
-__device__ __forceinline__ float rcp_pos(float s) { return __fdividef(1.f, s); }
-
-// Regret matching over the regrets r of D > 1 child edges: the children's reaches own * sigma.
-template <int D>
-__device__ __forceinline__ void rm_reach(const float *r, float own, float thr, float *x) {
-    float rp[D];
-#pragma unroll
-    for (int a = 0; a < D; a++) rp[a] = r[a] > thr ? r[a] : 0.f;
-    const float sum = tree_sum<D>(rp);
-    const bool pos = sum > 0.f;
-    // pos: rp * scale (an fma with a zero addend rounds the product alone); otherwise every rp is
-    // zero and the fma gives the uniform share: one instruction per child instead of two
-    const float scale = pos ? own * rcp_pos(sum) : 0.f, u = pos ? 0.f : own * (1.f / (float)D);
-#pragma unroll
-    for (int a = 0; a < D; a++) x[a] = __fmaf_rn(rp[a], scale, u);
 }
 
 // Regret matching at one (active node, slot) with D children and the reach of the children.
@@ -145,39 +114,6 @@ __device__ __forceinline__ void td_node_any(int c, int d, int sh, int w, float o
         const float u = own * (1.f / (float)d);
         for (int a = 0; a < d; a++) X[at<W1>(c, a, sh, w)] = u;
     }
-}
-
-// Value of a node from the regrets r, strategy sums s and values v of its D child edges, then
-// R(h,a) += s_p pi_{-p}(h) (v(h.a) - v(h)) and S(h,a) += pi_p(h) sigma(h,a) in place in r and s.
-// Returns v(h).
-template <int VARIANT, int D>
-__device__ __forceinline__ float bu_vals(float *r, const float *v, float *s, float pp, float spo, float thr, float fpos,
-                                         float fneg, float fs) {
-    float rp[D];
-#pragma unroll
-    for (int a = 0; a < D; a++) rp[a] = r[a] > thr ? r[a] : 0.f;
-    const float sum = tree_sum<D>(rp);
-    const bool pos = sum > 0.f;
-    const float inv = pos ? rcp_pos(sum) : 0.f, u = pos ? 0.f : 1.f / (float)D;
-    float sg[D], dv[D];
-#pragma unroll
-    for (int a = 0; a < D; a++) {
-        sg[a] = __fmaf_rn(rp[a], inv, u);  // rp * inv, or the uniform share (as in td_node)
-        dv[a] = a == 0 ? 0.f : sg[a] * (v[a] - v[0]);
-    }
-    const float vh = D == 1 ? v[0] : v[0] + tree_sum<D>(dv);
-#pragma unroll
-    for (int a = 0; a < D; a++) {
-        const float inst = spo * (v[a] - vh);
-        if (VARIANT == 1) {
-            r[a] = r[a] * (r[a] > 0.f ? fpos : fneg) + inst;
-            s[a] = s[a] * fs + pp * sg[a];
-        } else {
-            r[a] = r[a] + inst;
-            s[a] = s[a] + pp * sg[a];
-        }
-    }
-    return vh;
 }
 
 // Value of one (active node, slot) with D children and the updates of its child edges (bu_vals)
@@ -382,118 +318,6 @@ __device__ __forceinline__ void dcfr_factors(const CfrParams &p, int il, float &
     }
 }
 
-// The T iterations of one item over its level schedule.
-template <int VARIANT, bool W1, bool PACKED>
-__device__ __forceinline__ double iterate(const CfrParams &p, int W, const Entries<PACKED> &A, float *R, float *S,
-                                          float *V, float *X, const int32_t *sb, const int32_t *sn, const int32_t *sf,
-                                          const float *s_tu) {
-    const int tid = threadIdx.x;
-    const int sh = __ffs(W) - 1;  // W is a power of two
-    double acc = 0.0;
-    for (int il = 0; il < p.iters; il++) {
-        const float tf = (float)(p.t0 + il + 1);
-        float fpos, fneg, fs;
-        dcfr_factors<VARIANT>(p, il, fpos, fneg, fs);
-        run_passes<VARIANT, W1, PACKED>(0, 15, W, sh, A, R, S, V, X, sb, sn, sf, s_tu, tf, fpos, fneg, fs);
-        // the root values were written before the last step's block barrier and are next
-        // written by the last step of the next iteration
-        if (tid < W) acc += (double)V[tid];
-    }
-    __syncthreads();
-    return acc;
-}
-
-// All T iterations of one item, its arrays in shared memory (carved from sm): the packed active
-// entries, then R, S, V, X per (local node, slot).
-template <int VARIANT>
-__device__ __forceinline__ void run_item(const CfrParams &p, const TreeView &tv, const CfrItem &it, const CfrRoot &cr,
-                                         const int32_t *s_as, float *s_tu, int32_t *sb, int32_t *sn, int32_t *sf,
-                                         unsigned char *sm) {
-    const int tid = threadIdx.x, nth = blockDim.x;
-    const int W = it.ns;
-    const int L = cr.ls[9], nA = s_as[9];
-    const int32_t *gli = tv.act_li + cr.act_off, *gpl = tv.act_pl + cr.act_off, *gcs = tv.act_cs + cr.act_off;
-    const uint16_t *gd = tv.act_d + cr.act_off;
-    Entries<true> P{};
-    size_t o = 0;
-    uint32_t *scd = (uint32_t *)(sm + o); o += al16((size_t)nA * 4);
-    uint32_t *slp = (uint32_t *)(sm + o); o += al16((size_t)nA * 4);
-    float *R = (float *)(sm + o); o += al16((size_t)L * W * 4);
-    float *S = (float *)(sm + o); o += al16((size_t)L * W * 4);
-    float *V = (float *)(sm + o); o += al16((size_t)L * W * 4);
-    float *X = (float *)(sm + o);
-    for (int i = tid; i < nA; i += nth) {
-        scd[i] = (uint32_t)gcs[i] | ((uint32_t)gd[i] << 16);
-        slp[i] = (uint32_t)gli[i] | ((uint32_t)(gpl[i] < 0 ? 0xFFFF : gpl[i]) << 16);
-    }
-    {
-        const float *gR = tv.R + it.data_base, *gS = tv.S + it.data_base;
-        for (int i = tid; i < L * W; i += nth) {
-            R[i] = gR[i];
-            S[i] = gS[i];
-        }
-    }
-    P.cd = scd;
-    P.lp = slp;
-    // values of the terminals (leaves and chain heads), constant over the iterations; root reach;
-    // per slot the largest |leaf value| of the root's subtree, the scale of the dead zone
-    for (int w = tid; w < W; w += nth) s_tu[w] = 0.f;
-    __syncthreads();
-    {
-        const int64_t *tq = tv.loc_tq + cr.loc_off;
-        for (int x = tid; x < L * W; x += nth) {
-            const int li = x / W, w = x - li * W;
-            const int64_t q = tq[li];
-            if (q >= 0) {
-                const float v = tv.leaf_v[q + it.s0 + w];
-                V[x] = v;
-                atomicMax((unsigned *)&s_tu[w], __float_as_uint(fabsf(v)));
-            }
-        }
-        for (int w = tid; w < W; w += nth) X[w] = 1.f;
-    }
-    // level schedule: a level of at most 32 (node, slot) pairs runs on warp 0 alone, and only a
-    // change between warp-0 and whole-block levels needs a block barrier
-    if (tid == 0) make_schedule(s_as, W, sb, sn, sf);
-    __syncthreads();
-    for (int w = tid; w < W; w += nth) s_tu[w] = p.tau * s_tu[w];
-    __syncthreads();
-    const double acc = W == 1 ? iterate<VARIANT, true, true>(p, W, P, R, S, V, X, sb, sn, sf, s_tu)
-                              : iterate<VARIANT, false, true>(p, W, P, R, S, V, X, sb, sn, sf, s_tu);
-    if (tid < W) {
-        if (!isfinite(acc)) atomicOr(p.err, 1);
-        tv.uacc[tv.fgt_off0[it.root] + it.s0 + tid] += acc;
-    }
-    float *gR = tv.R + it.data_base, *gS = tv.S + it.data_base;
-    for (int i = tid; i < L * W; i += nth) {
-        gR[i] = R[i];
-        gS[i] = S[i];
-    }
-    __syncthreads();
-}
-
-template <int VARIANT, int MAXT, int MINB = (MAXT == 256 ? 3 : 1)>
-__global__ void __launch_bounds__(MAXT, MINB) k_cfr_items(CfrParams p) {
-    extern __shared__ __align__(16) unsigned char sm[];
-    __shared__ int32_t s_item;
-    __shared__ int32_t s_as[10];
-    __shared__ int32_t s_sb[15], s_sn[15], s_sf[15];
-    __shared__ float s_tu[kMaxSlots];
-    const int tid = threadIdx.x;
-    for (;;) {
-        if (tid == 0) s_item = atomicAdd(p.counter, 1);
-        __syncthreads();
-        const int64_t id = p.i_begin + s_item;
-        if (tid < 10) s_as[tid] = id < p.i_end ? p.views[p.items[id].tree].roots[p.items[id].root].as[tid] : 0;
-        __syncthreads();
-        if (id >= p.i_end) break;
-        const CfrItem it = p.items[id];
-        const TreeView tv = p.views[it.tree];
-        const CfrRoot &cr = tv.roots[it.root];
-        run_item<VARIANT>(p, tv, it, cr, s_as, s_tu, s_sb, s_sn, s_sf, sm);
-    }
-}
-
 // ---- class 5: a level-streaming sweep over every SM --------------------------------------------
 //
 // Items whose state lives in device memory are not given one block each: every level step of an
@@ -664,17 +488,6 @@ __global__ void k_stream_finalize(CfrParams p, StreamPlan sp) {
         if (!isfinite(acc)) atomicOr(p.err, 1);
         tv.uacc[tv.fgt_off0[it.root] + it.s0 + w] += acc;
     }
-}
-
-// The instantiation for blocks of `threads` threads of size class c: up to 256 threads at up to 80
-// registers (three 256-thread blocks per SM), class 3 (two blocks per SM by its shared memory) at
-// up to 128 (96 used: seed-47 CFR 1111 -> 1087 ms against 80), up to 512 at up to 128 (no spills),
-// up to 1024 at 64 (the register file of one SM).
-const void *cfr_kernel_for(int variant, int threads, int cls) {
-    if (threads <= 256 && cls == 3) return variant == 1 ? (const void *)k_cfr_items<1, 256, 2> : (const void *)k_cfr_items<0, 256, 2>;
-    if (threads <= 256) return variant == 1 ? (const void *)k_cfr_items<1, 256> : (const void *)k_cfr_items<0, 256>;
-    if (threads <= 512) return variant == 1 ? (const void *)k_cfr_items<1, 512> : (const void *)k_cfr_items<0, 512>;
-    return variant == 1 ? (const void *)k_cfr_items<1, 1024> : (const void *)k_cfr_items<0, 1024>;
 }
 
 // ---- a root subtree split over a thread-block cluster ------------------------------------------
@@ -1088,6 +901,117 @@ __global__ void k_renumber_tq(int64_t n, const int64_t *lmap, const int64_t *tq_
         tq[lmap[x]] = tq_old[x];
 }
 
+// ---- the block sweep's order (BlockRun, BlockRoot) ---------------------------------------------
+
+// 1 for an active entry whose children are all terminals
+__global__ void k_block_bottom(int64_t n, const int32_t *act_rk, const CfrRoot *roots, const int32_t *act_cs, const uint16_t *act_d,
+                               const int64_t *loc_tq, int32_t *bottom) {
+    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t *tq = loc_tq + roots[act_rk[e] >> 3].loc_off + act_cs[e];
+        int b = 1;
+        for (int a = 0; a < act_d[e]; a++) b &= tq[a] >= 0;
+        bottom[e] = b;
+    }
+}
+
+// stable partition of every (root, level) segment: entries with an active child first
+// (brank: exclusive scan of the bottom flags); src = entry at each place, deg its degree
+__global__ void k_block_order(int64_t n, const int32_t *act_rk, const CfrRoot *roots, const int32_t *bottom, const int64_t *brank,
+                              const uint16_t *act_d, int64_t *src, int32_t *deg) {
+    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
+        const CfrRoot &cr = roots[act_rk[e] >> 3];
+        const int k = act_rk[e] & 7;
+        const int64_t a = cr.act_off + cr.as[k], b = cr.act_off + cr.as[k + 1];
+        const int64_t before = brank[e] - brank[a], all = brank[b] - brank[a];
+        const int64_t i = bottom[e] ? a + (b - a - all) + before : e - before;
+        src[i] = e;
+        deg[i] = act_d[e];
+    }
+}
+
+// 1 at the first place of every run of one (root, level), bottom flag and degree
+__global__ void k_block_runs(int64_t n, const int64_t *src, const int32_t *act_rk, const int32_t *bottom, const int32_t *deg,
+                             int32_t *first) {
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+        int f = 1;
+        if (i > 0) {
+            const int64_t e = src[i], p = src[i - 1];
+            f = act_rk[e] != act_rk[p] || bottom[e] != bottom[p] || deg[i] != deg[i - 1];
+        }
+        first[i] = f;
+    }
+}
+
+// run_at[r] = first place of run r (runs numbered by the exclusive scan `run` of `first`); run_at[runs] = n
+__global__ void k_block_run_starts(int64_t n, const int32_t *first, const int64_t *run, int64_t *run_at) {
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i <= n; i += (int64_t)gridDim.x * blockDim.x)
+        if (i == n || first[i]) run_at[run[i]] = i;
+}
+
+// the runs, and the block index of every child (bmap: local -> block index, per root).  dpos:
+// exclusive scan of deg over the places.  Indices of roots with more than 65535 nodes are cut to
+// 16 bits: such roots are not solved in a block.
+__global__ void k_block_children(int64_t n, const int64_t *src, const int32_t *act_rk, const CfrRoot *roots, const int32_t *first,
+                                 const int64_t *run, const int64_t *run_at, const int64_t *dpos, const int32_t *deg,
+                                 const int32_t *act_cs, int32_t *bmap, BlockRun *runs) {
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t e = src[i], r = run[i] + first[i] - 1, a = run_at[r];
+        const int m = (int)(run_at[r + 1] - a), d = deg[i];
+        const CfrRoot &cr = roots[act_rk[e] >> 3];
+        const int k = act_rk[e] & 7;
+        const int c0 = cr.ls[k + 1] + (int)(dpos[a] - dpos[cr.act_off + cr.as[k]]);
+        int32_t *bm = bmap + cr.loc_off + act_cs[e];
+        for (int x = 0; x < d; x++) bm[x] = c0 + x * m + (int)(i - a);
+        if (first[i]) runs[r] = BlockRun{(uint16_t)c0, (uint16_t)(i - cr.act_off), (uint16_t)m, (uint16_t)d};
+        if (k == 0) bmap[cr.loc_off] = 0;
+    }
+}
+
+// entries and masks at their places
+__global__ void k_block_entries(int64_t n, const int64_t *src, const int32_t *act_rk, const CfrRoot *roots, const int32_t *act_li,
+                                const int32_t *act_pl, const int32_t *act_cs, const uint16_t *act_d, const int64_t *loc_tq,
+                                const int32_t *bmap, uint32_t *ent, uint8_t *msk) {
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t e = src[i];
+        const CfrRoot &cr = roots[act_rk[e] >> 3];
+        const int32_t *bm = bmap + cr.loc_off;
+        const uint32_t li = (uint32_t)bm[act_li[e]], pl = act_pl[e] < 0 ? (uint32_t)cr.ls[9] : (uint32_t)bm[act_pl[e]];
+        ent[i] = (li & 0xFFFFu) | (pl << 16);
+        unsigned mk = 0;
+        const int64_t *tq = loc_tq + cr.loc_off + act_cs[e];
+        for (int x = 0; x < act_d[e] && x < 8; x++) mk |= (tq[x] < 0 ? 1u : 0u) << x;
+        msk[i] = (uint8_t)mk;
+    }
+}
+
+// inv: block -> local index; term: terminals by block index; roots without an active node keep their one local node at 0
+__global__ void k_block_inverse(const int32_t *bmap, const CfrRoot *roots, int64_t nr, const int64_t *loc_tq, int32_t *inv,
+                                uint8_t *term) {
+    for (int64_t g = (int64_t)blockIdx.x; g < nr; g += gridDim.x) {
+        const CfrRoot &cr = roots[g];
+        const int L = cr.ls[9];
+        for (int l = threadIdx.x; l < L; l += blockDim.x) {
+            const int64_t b = cr.loc_off + (cr.as[9] == 0 ? l : bmap[cr.loc_off + l]);
+            inv[b] = l;
+            term[b] = loc_tq[cr.loc_off + l] >= 0;
+        }
+    }
+}
+
+__global__ void k_block_roots(int64_t nr, const CfrRoot *roots, const int64_t *run, const int64_t *brank, BlockRoot *out) {
+    for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < nr; g += (int64_t)gridDim.x * blockDim.x) {
+        const CfrRoot &cr = roots[g];
+        BlockRoot br;
+        br.run_off = run[cr.act_off];
+        for (int k = 0; k < 9; k++) br.rs[k] = (int32_t)(run[cr.act_off + cr.as[k]] - br.run_off);
+        for (int k = 0; k < 7; k++) {
+            const int64_t a = cr.act_off + cr.as[k], b = cr.act_off + cr.as[k + 1];
+            br.rt[k] = (int32_t)(run[b - (brank[b] - brank[a])] - br.run_off);
+        }
+        out[g] = br;
+    }
+}
+
 __global__ void k_iota(int64_t *out, int64_t n) {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) out[i] = i;
 }
@@ -1122,6 +1046,81 @@ struct Slab {
         return PASUR_OK;
     }
 };
+
+// The block sweep's order of the tree's entries: runs, entries, masks, index maps and per-root
+// ranges (act_rk: root << 3 | level per entry).
+int build_block_order(pasur_tree *t, const int32_t *act_rk) {
+    pasur_ctx *ctx = t->ctx;
+    const int64_t n = t->n_active, nr = t->n_roots;
+    std::vector<std::pair<void *, size_t>> tmp;
+    struct Guard {
+        pasur_ctx *c;
+        std::vector<std::pair<void *, size_t>> *v;
+        ~Guard() {
+            for (auto &x : *v) dev_free(c, x.first, x.second);
+        }
+    } guard{ctx, &tmp};
+    int32_t *bottom, *deg, *first, *bmap;
+    int64_t *brank, *src, *run, *run_at, *dpos;
+    Slab sl;
+    sl.add(&bottom, n);
+    sl.add(&deg, n);
+    sl.add(&first, n);
+    sl.add(&bmap, t->n_local);
+    sl.add(&brank, n);
+    sl.add(&src, n);
+    sl.add(&run, n);
+    sl.add(&run_at, n + 1);
+    sl.add(&dpos, n);
+    PASUR_TRY(sl.alloc(ctx, tmp));
+    PASUR_TRY(tree_alloc(t, (void **)&t->b_ent, sizeof(uint32_t) * (size_t)(n + 1)));
+    PASUR_TRY(tree_alloc(t, (void **)&t->b_msk, sizeof(uint8_t) * (size_t)(n + 1)));
+    PASUR_TRY(tree_alloc(t, (void **)&t->b_inv, sizeof(int32_t) * (size_t)(t->n_local + 1)));
+    PASUR_TRY(tree_alloc(t, (void **)&t->b_term, sizeof(uint8_t) * (size_t)(t->n_local + 1)));
+    PASUR_TRY(tree_alloc(t, (void **)&t->broots_d, sizeof(BlockRoot) * (size_t)(nr + 1)));
+    const unsigned grid = grid_for(n, 256);
+    auto launched = [&]() -> int {
+        ctx->launches++;
+        PASUR_CUDA(ctx, cudaGetLastError());
+        return PASUR_OK;
+    };
+    if (n > 0) {
+        k_block_bottom<<<grid, 256, 0, ctx->stream>>>(n, act_rk, t->croots_d, t->act_cs, t->act_d, t->loc_tq, bottom);
+        PASUR_TRY(launched());
+    }
+    PASUR_TRY(exclusive_scan_i32(ctx, bottom, brank, n));
+    if (n > 0) {
+        k_block_order<<<grid, 256, 0, ctx->stream>>>(n, act_rk, t->croots_d, bottom, brank, t->act_d, src, deg);
+        PASUR_TRY(launched());
+        k_block_runs<<<grid, 256, 0, ctx->stream>>>(n, src, act_rk, bottom, deg, first);
+        PASUR_TRY(launched());
+    }
+    PASUR_TRY(exclusive_scan_i32(ctx, deg, dpos, n));
+    PASUR_TRY(exclusive_scan_i32(ctx, first, run, n));
+    k_block_run_starts<<<grid_for(n + 1, 256), 256, 0, ctx->stream>>>(n, first, run, run_at);
+    PASUR_TRY(launched());
+    int64_t n_runs = 0;
+    PASUR_TRY(read_i64(ctx, run + n, &n_runs));
+    PASUR_TRY(tree_alloc(t, (void **)&t->b_run, sizeof(BlockRun) * (size_t)(n_runs + 1)));
+    if (n > 0) {
+        k_block_children<<<grid, 256, 0, ctx->stream>>>(n, src, act_rk, t->croots_d, first, run, run_at, dpos, deg, t->act_cs, bmap,
+                                                        t->b_run);
+        PASUR_TRY(launched());
+        k_block_entries<<<grid, 256, 0, ctx->stream>>>(n, src, act_rk, t->croots_d, t->act_li, t->act_pl, t->act_cs, t->act_d,
+                                                       t->loc_tq, bmap, t->b_ent, t->b_msk);
+        PASUR_TRY(launched());
+    }
+    t->broots_h.resize((size_t)nr);
+    if (nr > 0) {
+        k_block_inverse<<<(unsigned)std::min<int64_t>(nr, 65535), 256, 0, ctx->stream>>>(bmap, t->croots_d, nr, t->loc_tq, t->b_inv, t->b_term);
+        PASUR_TRY(launched());
+        k_block_roots<<<grid_for(nr, 256), 256, 0, ctx->stream>>>(nr, t->croots_d, run, brank, t->broots_d);
+        PASUR_TRY(launched());
+        PASUR_CUDA(ctx, cudaMemcpyAsync(t->broots_h.data(), t->broots_d, sizeof(BlockRoot) * (size_t)nr, cudaMemcpyDeviceToHost,
+                                        ctx->stream));
+    }
+    return PASUR_OK;
+}
 
 int build_layout(pasur_tree *t) {
     pasur_ctx *ctx = t->ctx;
@@ -1307,6 +1306,7 @@ int build_layout(pasur_tree *t) {
         ctx->launches++;
         PASUR_CUDA(ctx, cudaGetLastError());
     }
+    PASUR_TRY(build_block_order(t, act_rk));
     PASUR_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
     return PASUR_OK;
 }
@@ -1606,30 +1606,34 @@ int plan_splits(pasur_tree *t, const pasur_config *cfg, size_t dyn_max, size_t p
 
 }  // namespace
 
-// Largest dynamic shared memory a CFR block may request: the per-block opt-in limit minus the
-// kernel's own static shared memory (largest over its instantiations).
+// Largest dynamic shared memory a block of the sweep may request: the per-block opt-in limit minus
+// the kernels' own static shared memory (largest over the variants).
 int cfr_dyn_smem_limit(pasur_ctx *ctx, size_t *limit) {
     size_t st = 0;
     cudaFuncAttributes fa;
-    PASUR_CUDA(ctx, cudaFuncGetAttributes(&fa, k_cfr_items<0, 256>));
-    st = std::max(st, fa.sharedSizeBytes);
-    PASUR_CUDA(ctx, cudaFuncGetAttributes(&fa, k_cfr_items<1, 256>));
-    st = std::max(st, fa.sharedSizeBytes);
-    PASUR_CUDA(ctx, cudaFuncGetAttributes(&fa, k_cfr_items<0, 512>));
-    st = std::max(st, fa.sharedSizeBytes);
-    PASUR_CUDA(ctx, cudaFuncGetAttributes(&fa, k_cfr_items<1, 512>));
-    st = std::max(st, fa.sharedSizeBytes);
-    PASUR_CUDA(ctx, cudaFuncGetAttributes(&fa, k_cfr_items<0, 1024>));
-    st = std::max(st, fa.sharedSizeBytes);
-    PASUR_CUDA(ctx, cudaFuncGetAttributes(&fa, k_cfr_items<1, 1024>));
-    st = std::max(st, fa.sharedSizeBytes);
+    for (int v = 0; v < 2; v++)
+        for (int w = 1; w <= kBlockSlots; w++) {
+            PASUR_CUDA(ctx, cudaFuncGetAttributes(&fa, block_kernel(v, w)));
+            st = std::max(st, fa.sharedSizeBytes);
+        }
     *limit = ctx->smem_optin > st ? ctx->smem_optin - st : 0;
     return PASUR_OK;
 }
 
+const void *block_kernel(int variant, int W) {
+    switch (W) {
+        case 1: return block_kernel_w1(variant);
+        case 2: return block_kernel_w2(variant);
+        case 3: return block_kernel_w3(variant);
+        case 4: return block_kernel_w4(variant);
+        case 5: return block_kernel_w5(variant);
+        default: return block_kernel_w6(variant);
+    }
+}
+
 int cfr_cluster_smem_limit(pasur_ctx *ctx, size_t *limit);
 
-int cfr_setup_tree(pasur_tree *t, const pasur_config *cfg, int tree, std::vector<CfrItem> *cls_items, size_t *need,
+int cfr_setup_tree(pasur_tree *t, const pasur_config *cfg, int tree, std::vector<CfrItem> *cls_items,
                    std::vector<ClusterItem> *clu) {
     pasur_ctx *ctx = t->ctx;
     PhaseTimer pt(ctx->stream, "cfr plan");
@@ -1637,8 +1641,7 @@ int cfr_setup_tree(pasur_tree *t, const pasur_config *cfg, int tree, std::vector
     pt.mark("layout");
     // every root goes to the smallest shared-memory class its subtree fits with one slot; its
     // items then take as many slots as that class holds
-    size_t dyn_max = 0;
-    PASUR_TRY(cfr_dyn_smem_limit(ctx, &dyn_max));
+    const size_t dyn_max = ctx->smem_optin > kStorageReserve ? ctx->smem_optin - kStorageReserve : 0;
     size_t budget[kNumCls - 1];
     for (int c = 0; c < kNumCls - 1; c++) budget[c] = kClsBudget[c] ? std::min<size_t>(kClsBudget[c], dyn_max) : dyn_max;
     const int wcap = cfg->slots_per_item > 0 ? std::min(cfg->slots_per_item, kMaxSlots) : kMaxSlots;
@@ -1668,6 +1671,8 @@ int cfr_setup_tree(pasur_tree *t, const pasur_config *cfg, int tree, std::vector
     PASUR_TRY(plan_splits(t, cfg, dyn_max, std::min(dyn_max, dyn_cl), streamed, splits, split_of, nli, npl, ncs, nd, ngt,
                           ntq));
     pt.mark("cluster splits");
+    std::vector<int64_t> sbase((size_t)t->csoff_h[(size_t)t->n_roots] + 1, 0);
+    std::vector<int32_t> sstr(sbase.size(), 0);
     int64_t data = 0, scratch = 0;
     for (int64_t g = 0; g < t->n_roots; g++) {
         CfrRoot &cr = t->croots_h[(size_t)g];
@@ -1736,18 +1741,17 @@ int cfr_setup_tree(pasur_tree *t, const pasur_config *cfg, int tree, std::vector
             it.ns = (int32_t)ns;
             it.s0 = s0;
             it.data_base = data;
+            for (int64_t w = 0; w < ns; w++) {
+                sbase[(size_t)(t->csoff_h[(size_t)g] + s0 + w)] = data + w;
+                sstr[(size_t)(t->csoff_h[(size_t)g] + s0 + w)] = (int32_t)ns;
+            }
             data += L * it.ns;
+            it.scratch_base = -1;
             if (cls == kClsGlobal) {
                 it.scratch_base = scratch;
                 scratch += L * it.ns;
-            } else {
-                it.scratch_base = -1;
-                need[cls] = std::max(need[cls], resident_bytes(L, nA, it.ns));
             }
             it.cost = std::max<int64_t>(nA, 1) * it.ns;
-            int32_t wmax = 0;
-            for (int k = 0; k < 8; k++) wmax = std::max<int32_t>(wmax, (cr.as[k + 1] - cr.as[k]) * it.ns);
-            it.width = wmax;
             cls_items[cls].push_back(it);
         }
     }
@@ -1813,7 +1817,19 @@ int cfr_setup_tree(pasur_tree *t, const pasur_config *cfg, int tree, std::vector
     }
     PASUR_TRY(tree_alloc(t, (void **)&t->uacc, sizeof(double) * (size_t)(t->cQ[0] + 1)));
     PASUR_CUDA(ctx, cudaMemsetAsync(t->uacc, 0, sizeof(double) * (size_t)(t->cQ[0] + 1), ctx->stream));
+    PASUR_TRY(tree_alloc(t, (void **)&t->slot_base, sizeof(int64_t) * sbase.size()));
+    PASUR_TRY(tree_alloc(t, (void **)&t->slot_str, sizeof(int32_t) * sstr.size()));
+    PASUR_CUDA(ctx, cudaMemcpyAsync(t->slot_base, sbase.data(), sizeof(int64_t) * sbase.size(), cudaMemcpyHostToDevice, ctx->stream));
+    PASUR_CUDA(ctx, cudaMemcpyAsync(t->slot_str, sstr.data(), sizeof(int32_t) * sstr.size(), cudaMemcpyHostToDevice, ctx->stream));
     TreeView &v = t->view;
+    v.broots = t->broots_d;
+    v.b_run = t->b_run;
+    v.b_ent = t->b_ent;
+    v.b_msk = t->b_msk;
+    v.b_inv = t->b_inv;
+    v.b_term = t->b_term;
+    v.slot_base = t->slot_base;
+    v.slot_str = t->slot_str;
     v.roots = t->croots_d;
     v.act_li = t->act_li;
     v.act_pl = t->act_pl;
@@ -1837,22 +1853,123 @@ int cfr_setup_tree(pasur_tree *t, const pasur_config *cfg, int tree, std::vector
 
 int cfr_cluster_check(pasur_ctx *ctx, CfrPlan *plan, const pasur_config *cfg);
 
-int cfr_finalize_plan(pasur_ctx *ctx, CfrPlan &plan, std::vector<CfrItem> *cls_items, const size_t *need,
-                      const std::vector<TreeView> &views, const pasur_config *cfg, std::vector<std::pair<void *, size_t>> &owned,
+// The block sweep's items and launch groups: every root of the storage classes 0..4 of the trees.
+int plan_blocks(pasur_ctx *ctx, CfrPlan &plan, const std::vector<pasur_tree *> &trees, const pasur_config *cfg,
+                std::vector<std::pair<void *, size_t>> &owned) {
+    plan.blk_h.clear();
+    plan.groups.clear();
+    size_t lim = 0;
+    PASUR_TRY(cfr_dyn_smem_limit(ctx, &lim));
+    if (!ctx->cfr_smem_raised) {
+        // the attribute is global per kernel: raise it once to the largest dynamic size any plan
+        // can ask for, so that plans prepared later never lower it under an earlier plan's need
+        for (int v = 0; v < 2; v++)
+            for (int w = 1; w <= kBlockSlots; w++)
+                PASUR_CUDA(ctx, cudaFuncSetAttribute(block_kernel(v, w), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lim));
+        ctx->cfr_smem_raised = true;
+    }
+    auto in_block = [&](const pasur_tree *t, int64_t g) {
+        const int c = t->croots_h[(size_t)g].cls;
+        return c >= 0 && c < kClsGlobal;
+    };
+    int64_t slots = 0;
+    for (const pasur_tree *t : trees)
+        for (int64_t g = 0; g < t->n_roots; g++)
+            if (in_block(t, g)) slots += t->csoff_h[(size_t)g + 1] - t->csoff_h[(size_t)g];
+    if (slots == 0) return PASUR_OK;
+    const int wcap = (int)std::max<int64_t>(1, std::min<int64_t>(kBlockSlots, slots / (kSlotsPerSm * ctx->num_sms)));
+    // blocks per SM by shared memory (228 KB per SM, 1 KB reserved per block, some static)
+    auto per_sm = [&](size_t smem) {
+        for (int n = 6; n > 1; n--)
+            if ((smem + 1024 + (ctx->smem_optin - lim)) * (size_t)n <= 228 * 1024) return n;
+        return 1;
+    };
+    struct Tagged {
+        BlockItem it;
+        int per, chunks;
+        size_t smem;
+    };
+    std::vector<Tagged> all;
+    for (size_t ti = 0; ti < trees.size(); ti++) {
+        const pasur_tree *t = trees[ti];
+        for (int64_t g = 0; g < t->n_roots; g++) {
+            if (!in_block(t, g)) continue;
+            const CfrRoot &cr = t->croots_h[(size_t)g];
+            const BlockRoot &br = t->broots_h[(size_t)g];
+            const int64_t S = t->csoff_h[(size_t)g + 1] - t->csoff_h[(size_t)g], L = cr.ls[9], nA = cr.as[9], nR = br.rs[8];
+            int64_t w = std::min<int64_t>(S, wcap);
+            while (w > 1 && block_offsets(L, nA, nR, (int)w, kBlockMaxThreads / 32).end > lim) w--;
+            const int64_t n = (S + w - 1) / w;
+            for (int64_t i = 0, s0 = 0; i < n; i++) {
+                const int W = (int)(S / n + (i < S % n ? 1 : 0));
+                Tagged x{};
+                x.it.tree = (int32_t)ti;
+                x.it.root = (int32_t)g;
+                x.it.s0 = (int32_t)s0;
+                x.it.ns = W;
+                x.it.cost = std::max<int64_t>(nA, 1) * W;
+                x.chunks = 1;
+                for (int k = 0; k < 8; k++)
+                    x.chunks = std::max(x.chunks, (cr.as[k + 1] - cr.as[k]) / 32 + br.rs[k + 1] - br.rs[k]);
+                x.smem = block_offsets(L, nA, nR, W, kBlockMaxThreads / 32).end;
+                if (x.smem > lim) return set_err(ctx, PASUR_EINVAL, "a block item exceeds a block's shared memory");
+                x.per = per_sm(x.smem);
+                all.push_back(x);
+                s0 += W;
+            }
+        }
+    }
+    std::stable_sort(all.begin(), all.end(), [](const Tagged &a, const Tagged &b) {
+        if (a.per != b.per) return a.per < b.per;
+        if (a.it.ns != b.it.ns) return a.it.ns > b.it.ns;
+        return a.it.cost > b.it.cost;
+    });
+    const bool few = (int64_t)all.size() <= ctx->num_sms;
+    int chunks = 1;
+    for (size_t i = 0; i < all.size(); i++) {
+        const Tagged &x = all[i];
+        if (i == 0 || x.per != all[i - 1].per || x.it.ns != all[i - 1].it.ns) {
+            BlockGroup gr;
+            gr.W = x.it.ns;
+            gr.begin = (int64_t)i;
+            plan.groups.push_back(gr);
+            chunks = 1;
+        }
+        BlockGroup &gr = plan.groups.back();
+        gr.end = (int64_t)i + 1;
+        gr.smem = std::max(gr.smem, x.smem);
+        chunks = std::max(chunks, x.chunks);
+        cudaFuncAttributes fa;
+        PASUR_CUDA(ctx, cudaFuncGetAttributes(&fa, block_kernel(cfg->variant, x.it.ns)));
+        const int regs = (fa.numRegs + 7) & ~7;
+        int th = 65536 / regs / (few ? 1 : x.per) / 32 * 32;
+        gr.threads = std::max(32, std::min({th, kBlockMaxThreads, 32 * chunks}));
+        if (cfg->threads > 0) gr.threads = std::min(cfg->threads, kBlockMaxThreads);
+        plan.blk_h.push_back(x.it);
+    }
+    size_t b = sizeof(BlockItem) * plan.blk_h.size();
+    PASUR_TRY(dev_alloc(ctx, (void **)&plan.blk_d, b));
+    owned.push_back({plan.blk_d, b});
+    PASUR_CUDA(ctx, cudaMemcpyAsync(plan.blk_d, plan.blk_h.data(), b, cudaMemcpyHostToDevice, ctx->stream));
+    return PASUR_OK;
+}
+
+int cfr_finalize_plan(pasur_ctx *ctx, CfrPlan &plan, std::vector<CfrItem> *cls_items, const std::vector<pasur_tree *> &trees,
+                      const pasur_config *cfg, std::vector<std::pair<void *, size_t>> &owned,
                       const std::vector<ClusterItem> &clu) {
     if (cfg->threads < 0 || cfg->threads > 1024 || cfg->threads % 32)
         return set_err(ctx, PASUR_EINVAL, "cfg.threads must be 0 or a multiple of 32 <= 1024");
     if (cfg->split_bytes < 0) return set_err(ctx, PASUR_EINVAL, "cfg.split_bytes must be >= 0");
     if (cfg->stream_bytes < 0) return set_err(ctx, PASUR_EINVAL, "cfg.stream_bytes must be >= 0");
     plan.items_h.clear();
-    // classes 0..5 are launched by k_cfr_items; class 6 holds the cluster items' pseudo-items
+    // classes 0..4: storage of the roots the block sweep solves; 5 the level-streaming sweep's items;
+    // 6 the cluster items' pseudo-items
     for (int c = 0; c <= kClsCluster; c++) {
         std::stable_sort(cls_items[c].begin(), cls_items[c].end(),
                          [](const CfrItem &a, const CfrItem &b) { return a.cost > b.cost; });
         plan.cls_begin[c] = (int64_t)plan.items_h.size();
         plan.items_h.insert(plan.items_h.end(), cls_items[c].begin(), cls_items[c].end());
         plan.cls_end[c] = (int64_t)plan.items_h.size();
-        plan.cls_smem[c] = c < kNumCls ? need[c] : 0;
     }
     plan.n_items = (int64_t)plan.items_h.size();
     plan.clu_h = clu;
@@ -1888,6 +2005,8 @@ int cfr_finalize_plan(pasur_ctx *ctx, CfrPlan &plan, std::vector<CfrItem> *cls_i
         owned.push_back({plan.items_d, b});
         PASUR_CUDA(ctx, cudaMemcpyAsync(plan.items_d, plan.items_h.data(), b, cudaMemcpyHostToDevice, ctx->stream));
     }
+    std::vector<TreeView> views;
+    for (const pasur_tree *t : trees) views.push_back(t->view);
     if (!views.empty()) {
         size_t b = sizeof(TreeView) * views.size();
         PASUR_TRY(dev_alloc(ctx, (void **)&plan.views_d, b));
@@ -1921,49 +2040,9 @@ int cfr_finalize_plan(pasur_ctx *ctx, CfrPlan &plan, std::vector<CfrItem> *cls_i
         PASUR_CUDA(ctx, cudaGetLastError());
         PASUR_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
     }
-    if (!ctx->cfr_smem_raised) {
-        // the attribute is global per kernel: raise it once to the largest dynamic size any plan
-        // can ask for, so that plans prepared later never lower it under an earlier plan's need
-        // (static plus dynamic shared memory above 48 KB needs it)
-        size_t lim = 0;
-        PASUR_TRY(cfr_dyn_smem_limit(ctx, &lim));
-        for (int v = 0; v < 2; v++)
-            for (int t : {256, 512, 1024})
-                for (int c : {0, 3})
-                    PASUR_CUDA(ctx, cudaFuncSetAttribute(cfr_kernel_for(v, t, c), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lim));
-        ctx->cfr_smem_raised = true;
-    }
-    for (int c = 0; c < kNumCls; c++) {
-        plan.cls_blocks[c] = 0;
-        int64_t n = plan.cls_end[c] - plan.cls_begin[c];
-        int threads = cfg->threads > 0 ? cfg->threads : kClsThreads[c];
-        if (cfg->threads == 0 && n > 0 && n < ctx->num_sms) {
-            // fewer items than SMs: every item has an SM to itself, so widen its block towards its
-            // widest level (fewer tasks per thread per level step); beyond 256 threads the block
-            // barriers cost more than the shorter level steps save (measured on GB300)
-            int32_t wmax = 0;
-            for (int64_t i = plan.cls_begin[c]; i < plan.cls_end[c]; i++) wmax = std::max(wmax, plan.items_h[(size_t)i].width);
-            int t = 128;
-            while (t < wmax && t < 256) t *= 2;
-            threads = std::min(std::max(threads, t), std::max(t, 256));
-            // items whose state lives in device memory wait on L2/DRAM latency at every access:
-            // they take a whole SM each, so give them the widest block for latency hiding
-            if (c == kClsGlobal) threads = 1024;
-        }
-        plan.cls_threads[c] = threads;
-        if (n == 0) continue;
-        int per_sm = 0;
-        PASUR_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, cfr_kernel_for(0, threads, c), threads, plan.cls_smem[c]));
-        if (per_sm < 1) return set_err(ctx, PASUR_EINVAL, "CFR kernel cannot be resident with this shared-memory plan");
-        plan.cls_blocks[c] = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)per_sm * ctx->num_sms, n));
-    }
-    return PASUR_OK;
-}
-
-int cfr_occupancy(pasur_ctx *ctx, int threads, int cls, size_t smem, int64_t n_items, int *blocks) {
-    int per_sm = 0;
-    PASUR_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, cfr_kernel_for(0, threads, cls), threads, smem));
-    *blocks = per_sm < 1 ? 0 : (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)per_sm * ctx->num_sms, n_items));
+    PASUR_TRY(plan_blocks(ctx, plan, trees, cfg, owned));
+    // the uploads read host vectors of this call
+    PASUR_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
     return PASUR_OK;
 }
 
@@ -1990,10 +2069,10 @@ int ensure_aux(pasur_ctx *ctx) {
     PASUR_CUDA(ctx, cudaEventCreateWithFlags(&ctx->fork, cudaEventDisableTiming));
     int least = 0, greatest = 0;
     PASUR_CUDA(ctx, cudaDeviceGetStreamPriorityRange(&least, &greatest));
-    for (int c = 0; c < kClsCluster + kCluGroups; c++) {
+    for (int c = 0; c < kAuxStreams; c++) {
         // the level-streaming sweep is a chain of short dependent launches: its blocks go first
-        // whenever an SM frees up, the persistent classes and the clusters fill the rest
-        PASUR_CUDA(ctx, cudaStreamCreateWithPriority(&ctx->aux[c], cudaStreamNonBlocking, c == kClsGlobal ? greatest : least));
+        // whenever an SM frees up, the block sweep and the clusters fill the rest
+        PASUR_CUDA(ctx, cudaStreamCreateWithPriority(&ctx->aux[c], cudaStreamNonBlocking, c == kAuxStream ? greatest : least));
         PASUR_CUDA(ctx, cudaEventCreateWithFlags(&ctx->join[c], cudaEventDisableTiming));
         PASUR_CUDA(ctx, cudaEventCreate(&ctx->cls_t0[c]));
         PASUR_CUDA(ctx, cudaEventCreate(&ctx->cls_t1[c]));
@@ -2042,42 +2121,44 @@ int cfr_launch_plan(pasur_ctx *ctx, CfrPlan &plan, const pasur_config *cfg, int6
     p.t0 = t0;
     p.tau = cfg->rm_deadzone;
     p.err = ctx->errflag;
-    PASUR_CUDA(ctx, cudaMemsetAsync(ctx->counter, 0, sizeof(int32_t) * kNumCls, ctx->stream));
     PASUR_CUDA(ctx, cudaEventRecord(ctx->fork, ctx->stream));
-    // the classes are independent: each runs on its own forked stream, largest subtrees first; the
-    // level-streaming sweep (thousands of short launches) is queued last, after every persistent
-    // class and cluster launch, so that the host never waits on its queue before the others start
-    for (int oi = 0; oi < kNumCls; oi++) {
-        const int c = kNumCls - 1 - oi;
-        if (plan.cls_end[c] == plan.cls_begin[c] || c == kClsGlobal) continue;
-        cudaStream_t st = ctx->aux[c];
-        PASUR_CUDA(ctx, cudaStreamWaitEvent(st, ctx->fork, 0));
-        PASUR_CUDA(ctx, cudaEventRecord(ctx->cls_t0[c], st));
-        p.i_begin = plan.cls_begin[c];
-        p.i_end = plan.cls_end[c];
-        p.counter = ctx->counter + c;
-        void *args[] = {&p};
-        PASUR_CUDA(ctx, cudaLaunchKernel(cfr_kernel_for(cfg->variant, plan.cls_threads[c], c), dim3((unsigned)plan.cls_blocks[c]),
-                                         dim3((unsigned)plan.cls_threads[c]), args, plan.cls_smem[c], st));
-        ctx->launches++;
-        PASUR_CUDA(ctx, cudaEventRecord(ctx->cls_t1[c], st));
-        PASUR_CUDA(ctx, cudaEventRecord(ctx->join[c], st));
+    auto fork = [&](int c) -> int {
+        PASUR_CUDA(ctx, cudaStreamWaitEvent(ctx->aux[c], ctx->fork, 0));
+        PASUR_CUDA(ctx, cudaEventRecord(ctx->cls_t0[c], ctx->aux[c]));
+        return PASUR_OK;
+    };
+    auto join = [&](int c) -> int {
+        PASUR_CUDA(ctx, cudaEventRecord(ctx->cls_t1[c], ctx->aux[c]));
+        PASUR_CUDA(ctx, cudaEventRecord(ctx->join[c], ctx->aux[c]));
         PASUR_CUDA(ctx, cudaStreamWaitEvent(ctx->stream, ctx->join[c], 0));
+        return PASUR_OK;
+    };
+    // the launches are independent: each runs on its own forked stream (beyond their number,
+    // several share one), largest subtrees first; the level-streaming sweep (thousands of short
+    // launches) is queued last, so that the host never waits on its queue before the others start
+    const int nb = (int)std::min<size_t>(plan.groups.size(), kAuxStreams - kAuxBlock);
+    for (int c = 0; c < nb; c++) PASUR_TRY(fork(kAuxBlock + c));
+    for (size_t i = 0; i < plan.groups.size(); i++) {
+        const BlockGroup &gr = plan.groups[i];
+        BlockParams bp{plan.blk_d + gr.begin, plan.views_d, dcfr, cfg->iters, t0, cfg->rm_deadzone, ctx->errflag};
+        void *args[] = {&bp};
+        PASUR_CUDA(ctx, cudaLaunchKernel(block_kernel(cfg->variant, gr.W), dim3((unsigned)(gr.end - gr.begin)),
+                                         dim3((unsigned)gr.threads), args, gr.smem, ctx->aux[kAuxBlock + (int)(i % (size_t)nb)]));
+        ctx->launches++;
     }
+    for (int c = 0; c < nb; c++) PASUR_TRY(join(kAuxBlock + c));
     // roots split over thread-block clusters: one cluster per item, a launch (and a stream) per
     // cluster size
     for (int b = 0; b < kCluGroups; b++) {
         const int64_t n = plan.clu_end[b] - plan.clu_begin[b];
         if (n == 0) continue;
-        const int c = kClsCluster + b;
-        cudaStream_t st = ctx->aux[c];
-        PASUR_CUDA(ctx, cudaStreamWaitEvent(st, ctx->fork, 0));
-        PASUR_CUDA(ctx, cudaEventRecord(ctx->cls_t0[c], st));
+        const int c = kAuxCluster + b;
+        PASUR_TRY(fork(c));
         cudaLaunchConfig_t lc{};
         lc.gridDim = dim3((unsigned)(n * plan.clu_ctas[b]), 1, 1);
         lc.blockDim = dim3((unsigned)plan.clu_threads, 1, 1);
         lc.dynamicSmemBytes = plan.clu_smem[b];
-        lc.stream = st;
+        lc.stream = ctx->aux[c];
         cudaLaunchAttribute at[1];
         at[0].id = cudaLaunchAttributeClusterDimension;
         at[0].val.clusterDim.x = (unsigned)plan.clu_ctas[b];
@@ -2089,18 +2170,12 @@ int cfr_launch_plan(pasur_ctx *ctx, CfrPlan &plan, const pasur_config *cfg, int6
         void *args[] = {&p, &ci};
         PASUR_CUDA(ctx, cudaLaunchKernelExC(&lc, cluster_kernel_for(cfg->variant, plan.clu_threads), args));
         ctx->launches++;
-        PASUR_CUDA(ctx, cudaEventRecord(ctx->cls_t1[c], st));
-        PASUR_CUDA(ctx, cudaEventRecord(ctx->join[c], st));
-        PASUR_CUDA(ctx, cudaStreamWaitEvent(ctx->stream, ctx->join[c], 0));
+        PASUR_TRY(join(c));
     }
     if (plan.cls_end[kClsGlobal] != plan.cls_begin[kClsGlobal]) {
-        cudaStream_t st = ctx->aux[kClsGlobal];
-        PASUR_CUDA(ctx, cudaStreamWaitEvent(st, ctx->fork, 0));
-        PASUR_CUDA(ctx, cudaEventRecord(ctx->cls_t0[kClsGlobal], st));
-        PASUR_TRY(stream_sweep(ctx, plan, p, cfg, st));
-        PASUR_CUDA(ctx, cudaEventRecord(ctx->cls_t1[kClsGlobal], st));
-        PASUR_CUDA(ctx, cudaEventRecord(ctx->join[kClsGlobal], st));
-        PASUR_CUDA(ctx, cudaStreamWaitEvent(ctx->stream, ctx->join[kClsGlobal], 0));
+        PASUR_TRY(fork(kAuxStream));
+        PASUR_TRY(stream_sweep(ctx, plan, p, cfg, ctx->aux[kAuxStream]));
+        PASUR_TRY(join(kAuxStream));
     }
     return PASUR_OK;
 }
@@ -2149,16 +2224,42 @@ int cfr_cluster_check(pasur_ctx *ctx, CfrPlan *plan, const pasur_config *cfg) {
 }
 
 void cfr_plan_times(pasur_ctx *ctx, CfrPlan &plan) {
-    for (int c = 0; c < kNumCls; c++) {
-        float m = 0.f;
-        if (plan.cls_end[c] != plan.cls_begin[c]) cudaEventElapsedTime(&m, ctx->cls_t0[c], ctx->cls_t1[c]);
-        plan.cls_ms[c] = m;
+    const size_t nb = std::min<size_t>(plan.groups.size(), kAuxStreams - kAuxBlock);
+    for (size_t i = 0; i < plan.groups.size(); i++) {
+        plan.groups[i].ms = 0.f;
+        if (i < nb) cudaEventElapsedTime(&plan.groups[i].ms, ctx->cls_t0[kAuxBlock + i], ctx->cls_t1[kAuxBlock + i]);
     }
+    plan.str_ms = 0.f;
+    if (plan.cls_end[kClsGlobal] != plan.cls_begin[kClsGlobal])
+        cudaEventElapsedTime(&plan.str_ms, ctx->cls_t0[kAuxStream], ctx->cls_t1[kAuxStream]);
     for (int b = 0; b < kCluGroups; b++) {
-        float m = 0.f;
-        if (plan.clu_end[b] != plan.clu_begin[b]) cudaEventElapsedTime(&m, ctx->cls_t0[kClsCluster + b], ctx->cls_t1[kClsCluster + b]);
-        plan.cls_ms[kClsCluster + b] = m;
+        plan.clu_ms[b] = 0.f;
+        if (plan.clu_end[b] != plan.clu_begin[b])
+            cudaEventElapsedTime(&plan.clu_ms[b], ctx->cls_t0[kAuxCluster + b], ctx->cls_t1[kAuxCluster + b]);
     }
+}
+
+// one line per launch of a plan
+void cfr_print_plan(const CfrPlan &plan) {
+    for (const BlockGroup &gr : plan.groups) {
+        int64_t cost = 0, maxcost = 0;
+        for (int64_t i = gr.begin; i < gr.end; i++) {
+            cost += plan.blk_h[(size_t)i].cost;
+            maxcost = std::max(maxcost, plan.blk_h[(size_t)i].cost);
+        }
+        fprintf(stderr, "[pasur]   block items: %lld of %d slots, %d threads, smem %zu B, "
+                        "active-node-slots %lld (largest item %lld), %.3f ms\n",
+                (long long)(gr.end - gr.begin), gr.W, gr.threads, gr.smem, (long long)cost,
+                (long long)maxcost, gr.ms);
+    }
+    for (int b = 0; b < kCluGroups; b++)
+        if (plan.clu_end[b] != plan.clu_begin[b])
+            fprintf(stderr, "[pasur]   cluster items: %lld, %d CTAs x %d threads, smem %zu B, %.3f ms\n",
+                    (long long)(plan.clu_end[b] - plan.clu_begin[b]), plan.clu_ctas[b], plan.clu_threads, plan.clu_smem[b],
+                    plan.clu_ms[b]);
+    if (plan.str_n > 0)
+        fprintf(stderr, "[pasur]   streamed items: %lld (slots %lld), %.3f ms\n", (long long)plan.str_n, (long long)plan.str_nslots,
+                plan.str_ms);
 }
 
 static void print_plan(const pasur_tree *t, const CfrPlan &plan) {
@@ -2166,45 +2267,16 @@ static void print_plan(const pasur_tree *t, const CfrPlan &plan) {
     for (int k = 1; k < 9; k++) ne += t->Q[k];
     fprintf(stderr, "[pasur] round %d: GT roots %lld, FGT edges %lld, local %lld, active %lld, items %lld\n", t->round,
             (long long)t->n_roots, (long long)ne, (long long)t->n_local, (long long)t->n_active, (long long)plan.n_items);
-    for (int c = 0; c < kNumCls; c++) {
-        int64_t n = plan.cls_end[c] - plan.cls_begin[c];
-        if (!n) continue;
-        int64_t cost = 0, maxcost = 0, swept = 0, slots = 0;
-        for (int64_t i = plan.cls_begin[c]; i < plan.cls_end[c]; i++) {
-            const CfrItem &it = plan.items_h[(size_t)i];
-            cost += it.cost;
-            maxcost = std::max(maxcost, it.cost);
-            swept += (int64_t)(t->croots_h[(size_t)it.root].ls[9] - 1) * it.ns;
-            slots += it.ns;
-        }
-        fprintf(stderr, "[pasur]   class %d: items %lld (slots %lld), smem %zu B, blocks %d x %d threads, active-node-slots "
-                        "%lld (largest item %lld), swept edges %lld\n",
-                c, (long long)n, (long long)slots, plan.cls_smem[c], plan.cls_blocks[c], plan.cls_threads[c], (long long)cost,
-                (long long)maxcost, (long long)swept);
-    }
-    for (int b = 0; b < kCluGroups; b++)
-        if (plan.clu_end[b] != plan.clu_begin[b]) {
-            int64_t swept = 0, lmax = 0;
-            for (int64_t i = plan.clu_begin[b]; i < plan.clu_end[b]; i++) {
-                const int64_t L = t->croots_h[(size_t)plan.clu_h[(size_t)i].root].ls[9];
-                swept += L - 1;
-                lmax = std::max(lmax, L);
-            }
-            fprintf(stderr, "[pasur]   cluster items: %lld, %d CTAs x %d threads, smem %zu B, swept edges %lld (largest "
-                            "root %lld local nodes)\n",
-                    (long long)(plan.clu_end[b] - plan.clu_begin[b]), plan.clu_ctas[b], plan.clu_threads, plan.clu_smem[b],
-                    (long long)swept, (long long)lmax);
-        }
+    cfr_print_plan(plan);
 }
 
 int cfr_prepare(pasur_tree *t, const pasur_config *cfg) {
     pasur_ctx *ctx = t->ctx;
     std::vector<CfrItem> cls_items[8];
-    size_t need[8] = {0};
     std::vector<ClusterItem> clu;
-    PASUR_TRY(cfr_setup_tree(t, cfg, 0, cls_items, need, &clu));
+    PASUR_TRY(cfr_setup_tree(t, cfg, 0, cls_items, &clu));
     std::vector<std::pair<void *, size_t>> owned;
-    int rc = cfr_finalize_plan(ctx, t->plan, cls_items, need, {t->view}, cfg, owned, clu);
+    int rc = cfr_finalize_plan(ctx, t->plan, cls_items, {t}, cfg, owned, clu);
     for (auto &o : owned) {
         t->allocs.push_back(o.first);
         t->allocs.push_back((void *)(uintptr_t)o.second);
@@ -2247,11 +2319,8 @@ int cfr_run(pasur_tree *t, const pasur_config *cfg) {
     t->last_launches = (int32_t)(ctx->launches - before);
     t->iters_done += cfg->iters;
     if (getenv("PASUR_VERBOSE")) {
-        fprintf(stderr, "[pasur] round %d: %d iterations in %.3f ms (", t->round, cfg->iters, ms);
-        for (int c = 0; c < kNumCls; c++) fprintf(stderr, "%s%.2f", c ? " " : "", t->plan.cls_ms[c]);
-        fprintf(stderr, " ms per class; clusters");
-        for (int b = 0; b < kCluGroups; b++) fprintf(stderr, " %.2f", t->plan.cls_ms[kClsCluster + b]);
-        fprintf(stderr, " ms)\n");
+        fprintf(stderr, "[pasur] round %d: %d iterations in %.3f ms\n", t->round, cfg->iters, ms);
+        cfr_print_plan(t->plan);
     }
     if (ef) return set_err(ctx, PASUR_ENUMERIC, "non-finite root value in the CFR sweep");
     return PASUR_OK;

@@ -1,0 +1,6 @@
+// The block sweep for items of 2 score slots.
+#include "cfr_block_impl.cuh"
+
+namespace pasur {
+const void *block_kernel_w2(int variant) { return block_kernel_of<2>(variant); }
+}  // namespace pasur

@@ -113,6 +113,8 @@ __host__ __device__ __forceinline__ void score_unkey(uint32_t k, int &ac, int &b
 }
 constexpr int kScoreKeyBits = 26;
 
+constexpr int kAuxStreams = 24;  // forked streams of a context
+
 }  // namespace pasur
 
 // ---------------------------------------------------------------------------------------------
@@ -141,10 +143,11 @@ struct pasur_ctx {
     int32_t *counter = nullptr;  // work-queue counters (device)
     int32_t *errflag = nullptr;  // device error word
     int64_t launches = 0;        // kernels launched through this context
-    // forked streams for concurrent launches (created on first use): CFR classes 0..5, cluster
-    // launches 6..9
-    cudaStream_t aux[12] = {nullptr};
-    cudaEvent_t fork = nullptr, join[12] = {nullptr}, cls_t0[12] = {nullptr}, cls_t1[12] = {nullptr};
+    // forked streams for concurrent launches (created on first use): the level-streaming sweep 0,
+    // cluster launches 1..4, launches of the block sweep 5..
+    cudaStream_t aux[pasur::kAuxStreams] = {nullptr};
+    cudaEvent_t fork = nullptr, join[pasur::kAuxStreams] = {nullptr}, cls_t0[pasur::kAuxStreams] = {nullptr},
+                cls_t1[pasur::kAuxStreams] = {nullptr};
     int64_t live_trees = 0;      // trees not yet freed (the context outlives them)
     bool cfr_smem_raised = false;  // CFR kernels' dynamic shared-memory limit raised
     float selfplay_ms = 0.f;     // device time of the last self-play launch
@@ -214,6 +217,25 @@ struct ClusterPart {
     int64_t data_base;        // its regrets and strategy sums in R and S
 };
 
+// The block sweep's order of a root's entries (cfr_block.cuh).  Entries of one level: first those
+// with an active child, then those whose children are all terminals (they need no top-down step),
+// each in runs of one degree.  Nodes are numbered level by level; child a of a run's i-th entry is
+// node c0 + a * n + i ("block index").
+struct BlockRun {
+    uint16_t c0, e0;          // first child of its first entry, its first entry (within the root)
+    uint16_t n, d;            // entries, children per entry
+};
+struct BlockRoot {
+    int64_t run_off;          // the root's runs in the per-run array
+    int32_t rs[9];            // first run of level k (rs[8] = number of runs)
+    int32_t rt[7];            // end of level k's runs with an active child
+};
+struct BlockItem {            // a root and a run of its score slots, solved by one block
+    int32_t tree, root;
+    int32_t s0, ns;           // first slot within the root, slots
+    int64_t cost;             // active nodes * slots, for the schedule
+};
+
 struct ClusterItem {
     int32_t tree, root;       // launch tree index, real GT root
     int64_t s0;               // slot (one per cluster item)
@@ -235,13 +257,24 @@ struct TreeView {
     double *uacc;
     const ClusterPart *cparts;   // cluster items: parts table
     const int32_t *cx;           // cluster items: (part, top node, top parent, part node, part ghost)
+    // block sweep: per-root run ranges, runs, entries (own | parent's block index << 16), masks
+    // of the active children, local index per block index; per solved slot where local node l's
+    // regret lies in R (and S): slot_base + l * slot_str
+    const BlockRoot *broots;
+    const BlockRun *b_run;
+    const uint32_t *b_ent;
+    const uint8_t *b_msk;
+    const int32_t *b_inv;
+    const uint8_t *b_term;       // per block index: 1 for a terminal
+    const int64_t *slot_base;
+    const int32_t *slot_str;
 };
 
 struct CfrItem {              // one work item of the CFR kernel: a root and a run of its slots
     int32_t root;
     int32_t tree;             // index into the launch's TreeView table
     int32_t ns;               // slots in the item
-    int32_t width;            // largest number of (active node, slot) pairs of one level
+    int32_t pad;
     int64_t s0;               // first slot of the item within its root
     int64_t data_base;        // offset of the item's (local node, slot) table in R and S
     int64_t scratch_base;     // offset in the global transients, or -1 when the item is resident
@@ -263,17 +296,26 @@ struct StreamDesc {
     int64_t slot;
 };
 
+// One launch of the block sweep: items of the same slot count whose shared memory allows the same
+// number of blocks per SM.
+struct BlockGroup {
+    int W = 0, threads = 0;
+    int64_t begin = 0, end = 0;
+    size_t smem = 0;
+    float ms = 0.f;
+};
+
 // A CFR launch plan: work items of one or more trees merged per shared-memory class.
 struct CfrPlan {
+    std::vector<BlockItem> blk_h;       // by launch group, then cost (largest first)
+    BlockItem *blk_d = nullptr;
+    std::vector<BlockGroup> groups;
     std::vector<CfrItem> items_h;       // ordered by class, then cost (largest first)
     CfrItem *items_d = nullptr;
     TreeView *views_d = nullptr;
     int64_t n_items = 0;
     int64_t cls_begin[8] = {0}, cls_end[8] = {0};
-    size_t cls_smem[8] = {0};
-    int cls_blocks[8] = {0};
-    int cls_threads[8] = {0};
-    float cls_ms[12] = {0};
+    float str_ms = 0.f, clu_ms[4] = {0};
     // cluster items (class 6 holds their pseudo-items, used for exports only), sorted by part
     // count into up to four launches of 2, 4, 8 and 16 CTAs per cluster
     std::vector<ClusterItem> clu_h;
@@ -354,6 +396,15 @@ struct pasur_tree {
     int64_t *act_gt = nullptr;          //   GT node index
     int64_t *loc_tq = nullptr;          // per local node: FGT index (slot 0) of its chain's leaf, -1 if active
     int64_t n_local = 0, n_active = 0;
+    std::vector<BlockRoot> broots_h;    // block sweep (see TreeView)
+    BlockRoot *broots_d = nullptr;
+    BlockRun *b_run = nullptr;
+    uint32_t *b_ent = nullptr;
+    uint8_t *b_msk = nullptr;
+    int32_t *b_inv = nullptr;
+    uint8_t *b_term = nullptr;
+    int64_t *slot_base = nullptr;
+    int32_t *slot_str = nullptr;
     std::vector<ClusterPart> cparts_h;  // cluster items of this tree
     std::vector<int32_t> cx_h;
     ClusterPart *cparts_d = nullptr;
@@ -424,22 +475,20 @@ int expand_leaf_values(const pasur_tree *t, float *out_dev);
 // cfr.cu
 int cfr_prepare(pasur_tree *t, const pasur_config *cfg);
 int cfr_run(pasur_tree *t, const pasur_config *cfg);
-// layout, per-root plan and state of one tree; its items (tagged with tree index `tree`) are
-// appended per class to cls_items, the shared-memory need per class raised in need[]
-// (cls_items / need: 8 classes; roots split over thread-block clusters append ClusterItems to clu)
-int cfr_setup_tree(pasur_tree *t, const pasur_config *cfg, int tree, std::vector<CfrItem> *cls_items, size_t *need,
+// layout, storage and state of one tree; its items (tagged with tree index `tree`) are appended per
+// storage class to cls_items (8 classes), the roots split over thread-block clusters to clu
+int cfr_setup_tree(pasur_tree *t, const pasur_config *cfg, int tree, std::vector<CfrItem> *cls_items,
                    std::vector<ClusterItem> *clu);
-// sort and upload merged items and the tree views; launch configuration per class
-int cfr_finalize_plan(pasur_ctx *ctx, CfrPlan &plan, std::vector<CfrItem> *cls_items, const size_t *need,
-                      const std::vector<TreeView> &views, const pasur_config *cfg, std::vector<std::pair<void *, size_t>> &owned,
+// sort and upload merged items and the trees' views; the block sweep's items and launch groups
+int cfr_finalize_plan(pasur_ctx *ctx, CfrPlan &plan, std::vector<CfrItem> *cls_items, const std::vector<pasur_tree *> &trees,
+                      const pasur_config *cfg, std::vector<std::pair<void *, size_t>> &owned,
                       const std::vector<ClusterItem> &clu);
-// launch the plan's classes for cfg->iters iterations starting at iteration t0 (+1); no host
-// synchronisation (capturable); per-class times are read by cfr_plan_times
+void cfr_print_plan(const CfrPlan &plan);
+// launch the plan for cfg->iters iterations starting at iteration t0 (+1); no host synchronisation
+// (capturable); the launches' times are read by cfr_plan_times
 int cfr_launch_plan(pasur_ctx *ctx, CfrPlan &plan, const pasur_config *cfg, int64_t t0, const float *dcfr);
 void cfr_plan_times(pasur_ctx *ctx, CfrPlan &plan);
 int cfr_dcfr_factors(pasur_ctx *ctx, const pasur_config *cfg, int64_t t0, float **out, size_t *bytes);
-// blocks of a persistent CFR launch with this block size and shared memory (0 if it cannot run)
-int cfr_occupancy(pasur_ctx *ctx, int threads, int cls, size_t smem, int64_t n_items, int *blocks);
 int cfr_export_sigma(const pasur_tree *t, float *out_dev);
 // average strategies of the solved slots only (levels 1..8, solved FGT order, sum of cQ[1..8])
 int export_sigma_solved(const pasur_tree *t, float *out_dev);
