@@ -41,10 +41,9 @@ constexpr int kNumCls = 6;
 constexpr size_t kStorageReserve = 352;  // part of a block's shared memory the storage classes leave free
 constexpr size_t kClsBudget[kNumCls - 1] = {37536, 54 * 1024, 74 * 1024, 112 * 1024, 0 /* opt-in max */};
 constexpr int kClsGlobal = kNumCls - 1;
-constexpr int kClsCluster = 6;       // plan class of the cluster items' pseudo-items (exports only)
-constexpr int kMaxClusterCtas = 16;  // CTAs of a cluster (16: non-portable size)
-// forked streams: the level-streaming sweep, the cluster groups, the block sweep's groups
-constexpr int kAuxStream = 0, kAuxCluster = 1, kAuxBlock = kAuxCluster + kCluGroups;
+constexpr int kClsCluster = 6;  // roots split over clusters
+// forked streams: the level-streaming sweep, then the cluster and block launches in turn
+constexpr int kAuxStream = 0, kAuxSweep = 1;
 constexpr int64_t kSlotsPerSm = 2;
 
 struct CfrParams {
@@ -63,6 +62,11 @@ __host__ __device__ __forceinline__ size_t al16(size_t x) { return (x + 15) & ~(
 // (local node, slot); resident items must have fewer than 65535 local nodes
 __host__ __device__ __forceinline__ size_t resident_bytes(int64_t L, int64_t nA, int64_t W) {
     return L >= 65535 ? ~(size_t)0 >> 1 : 2 * al16((size_t)nA * 4) + 4 * al16((size_t)L * W * 4);
+}
+
+// whether W slots of a root fit one block of the sweep (node indices and the root's mark in 16 bits)
+bool block_fits(const CfrRoot &cr, const BlockRoot &br, int W, size_t limit) {
+    return cr.ls[9] < 65535 && block_offsets(cr.ls[9], cr.as[9], br.rs[8], W, kBlockMaxThreads / 32).end <= limit;
 }
 
 constexpr int kMaxSlots = 32;  // score slots per work item
@@ -170,142 +174,6 @@ __device__ __forceinline__ float bu_node_any(int c, int d, int sh, int w, float 
         }
     }
     return vh;
-}
-
-// Active entries of an item.  Resident items keep them packed in shared memory, two 32-bit words
-// per entry: (first child | moves << 16) and (local index | parent's local index << 16, 0xFFFF
-// at the root); resident items have fewer than 65535 local nodes.  Items in device memory read
-// the four int arrays.
-template <bool PACKED>
-struct Entries {
-    const uint32_t *cd, *lp;
-    const int32_t *li, *pl, *cs;
-    const uint16_t *d;
-    __device__ __forceinline__ void child(int e, int &c, int &n) const {
-        if (PACKED) {
-            const uint32_t u = cd[e];
-            c = (int)(u & 0xFFFFu);
-            n = (int)(u >> 16);
-        } else {
-            c = cs[e];
-            n = d[e];
-        }
-    }
-    __device__ __forceinline__ void self(int e, int &l, int &p) const {
-        if (PACKED) {
-            const uint32_t u = lp[e];
-            l = (int)(u & 0xFFFFu);
-            p = (u >> 16) == 0xFFFFu ? -1 : (int)(u >> 16);
-        } else {
-            l = li[e];
-            p = pl[e];
-        }
-    }
-};
-
-// One level of the top-down pass over (active node, slot) pairs.  The active entries of a level
-// are sorted by degree, so the lanes of a warp mostly take the same unrolled path.
-template <int VARIANT, bool W1, bool PACKED>
-__device__ __forceinline__ void td_level(int b, int n, int W, int sh, int t0x, int stride, const Entries<PACKED> &A,
-                                         const float *__restrict__ R, float *__restrict__ X, const float *tu, float tf) {
-    const float thr1 = tu[0] * tf;
-    for (int x = t0x; x < n; x += stride) {
-        const int e = W1 ? b + x : b + (x >> sh), w = W1 ? 0 : x & (W - 1);
-        int c, d, li, pl;
-        A.child(e, c, d);
-        A.self(e, li, pl);
-        const float thr = W1 ? thr1 : tu[w] * tf;
-        const float own = pl < 0 ? 1.f : X[W1 ? pl : (pl << sh) + w];
-        switch (d) {
-            case 1: td_node<1, W1>(c, sh, w, own, R, X, thr); break;
-            case 2: td_node<2, W1>(c, sh, w, own, R, X, thr); break;
-            case 3: td_node<3, W1>(c, sh, w, own, R, X, thr); break;
-            case 4: td_node<4, W1>(c, sh, w, own, R, X, thr); break;
-            case 5: td_node<5, W1>(c, sh, w, own, R, X, thr); break;
-            case 6: td_node<6, W1>(c, sh, w, own, R, X, thr); break;
-            case 7: td_node<7, W1>(c, sh, w, own, R, X, thr); break;
-            case 8: td_node<8, W1>(c, sh, w, own, R, X, thr); break;
-            default: td_node_any<W1>(c, d, sh, w, own, R, X, thr);
-        }
-    }
-}
-
-// One level of the bottom-up pass over (active node, slot) pairs.
-template <int VARIANT, bool W1, bool PACKED>
-__device__ __forceinline__ void bu_level(bool alex, int b, int n, int W, int sh, int t0x, int stride,
-                                         const Entries<PACKED> &A,
-                                         float *__restrict__ R, float *__restrict__ S, float *__restrict__ V,
-                                         const float *__restrict__ X, const float *tu, float tf, float fpos, float fneg,
-                                         float fs) {
-    const float thr1 = tu[0] * tf;
-    for (int x = t0x; x < n; x += stride) {
-        const int e = W1 ? b + x : b + (x >> sh), w = W1 ? 0 : x & (W - 1);
-        int c, d, li, pl;
-        A.child(e, c, d);
-        A.self(e, li, pl);
-        const float thr = W1 ? thr1 : tu[w] * tf;
-        const float pp = pl < 0 ? 1.f : X[W1 ? pl : (pl << sh) + w];  // pi_p(h)
-        const float po = X[W1 ? li : (li << sh) + w];                 // pi_{-p}(h)
-        const float spo = alex ? po : -po;
-        float vh;
-        switch (d) {
-            case 1: vh = bu_node<VARIANT, 1, W1>(c, sh, w, pp, spo, R, S, V, thr, fpos, fneg, fs); break;
-            case 2: vh = bu_node<VARIANT, 2, W1>(c, sh, w, pp, spo, R, S, V, thr, fpos, fneg, fs); break;
-            case 3: vh = bu_node<VARIANT, 3, W1>(c, sh, w, pp, spo, R, S, V, thr, fpos, fneg, fs); break;
-            case 4: vh = bu_node<VARIANT, 4, W1>(c, sh, w, pp, spo, R, S, V, thr, fpos, fneg, fs); break;
-            case 5: vh = bu_node<VARIANT, 5, W1>(c, sh, w, pp, spo, R, S, V, thr, fpos, fneg, fs); break;
-            case 6: vh = bu_node<VARIANT, 6, W1>(c, sh, w, pp, spo, R, S, V, thr, fpos, fneg, fs); break;
-            case 7: vh = bu_node<VARIANT, 7, W1>(c, sh, w, pp, spo, R, S, V, thr, fpos, fneg, fs); break;
-            case 8: vh = bu_node<VARIANT, 8, W1>(c, sh, w, pp, spo, R, S, V, thr, fpos, fneg, fs); break;
-            default: vh = bu_node_any<VARIANT, W1>(c, d, sh, w, pp, spo, R, S, V, thr, fpos, fneg, fs);
-        }
-        V[W1 ? li : (li << sh) + w] = vh;
-    }
-}
-
-// Level steps i0..i1-1 of a level schedule: sched[i] for i < 7 the top-down levels 0..6, for
-// i >= 7 the bottom-up levels 7..0; each (first entry, pairs, flags: 1 = empty, 2 = at most 32
-// pairs (warp 0 alone), 4 = the next non-empty level of the same pass is also small (a warp
-// barrier suffices)).
-template <int VARIANT, bool W1, bool PACKED>
-__device__ __forceinline__ void run_passes(int i0, int i1, int W, int sh, const Entries<PACKED> &A, float *R, float *S,
-                                           float *V, float *X, const int32_t *sb, const int32_t *sn, const int32_t *sf,
-                                           const float *s_tu, float tf, float fpos, float fneg, float fs) {
-    const int tid = threadIdx.x, nth = blockDim.x;
-    const bool warp0 = tid < 32;
-    for (int i = i0; i < i1; i++) {
-        const int f = sf[i];
-        if (f & 1) continue;
-        if (i < 7) {
-            if (!(f & 2)) td_level<VARIANT, W1, PACKED>(sb[i], sn[i], W, sh, tid, nth, A, R, X, s_tu, tf);
-            else if (warp0) td_level<VARIANT, W1, PACKED>(sb[i], sn[i], W, sh, tid, 32, A, R, X, s_tu, tf);
-        } else {
-            const bool alex = ((14 - i) & 1) == 0;
-            if (!(f & 2)) bu_level<VARIANT, W1, PACKED>(alex, sb[i], sn[i], W, sh, tid, nth, A, R, S, V, X, s_tu, tf, fpos, fneg, fs);
-            else if (warp0) bu_level<VARIANT, W1, PACKED>(alex, sb[i], sn[i], W, sh, tid, 32, A, R, S, V, X, s_tu, tf, fpos, fneg, fs);
-        }
-        if (f & 4) __syncwarp();
-        else __syncthreads();
-    }
-}
-
-// The level schedule of an entry layout with level starts as[0..9] and W slots (thread 0).
-__device__ __forceinline__ void make_schedule(const int32_t *as, int W, int32_t *sb, int32_t *sn, int32_t *sf) {
-    for (int i = 0; i < 15; i++) {
-        const int k = i < 7 ? i : 14 - i;
-        sb[i] = as[k];
-        sn[i] = (as[k + 1] - as[k]) * W;
-    }
-    for (int i = 0; i < 15; i++) {
-        int f = sn[i] == 0 ? 1 : 0;
-        const bool small = sn[i] <= 32;
-        if (small) f |= 2;
-        const int end = i < 7 ? 7 : 15;
-        int j = i + 1;
-        while (j < end && sn[j] == 0) j++;
-        if (small && j < end && sn[j] <= 32) f |= 4;
-        sf[i] = f;
-    }
 }
 
 template <int VARIANT>
@@ -488,222 +356,6 @@ __global__ void k_stream_finalize(CfrParams p, StreamPlan sp) {
         if (!isfinite(acc)) atomicOr(p.err, 1);
         tv.uacc[tv.fgt_off0[it.root] + it.s0 + w] += acc;
     }
-}
-
-// ---- a root subtree split over a thread-block cluster ------------------------------------------
-//
-// CTA r of the cluster holds part r (subtrees of active level-ell nodes) in its shared memory;
-// CTA 0 also holds the top levels 0..ell-1.  Per iteration: CTA 0 runs the top-down pass of the
-// top and pushes, for every active level-ell node, its reach and its parent's reach into the
-// owning CTA's shared memory (distributed shared memory); cluster barrier; every CTA runs both
-// passes over its part and pushes the node values back to CTA 0; cluster barrier; CTA 0 runs the
-// bottom-up pass of the top.  Every task does the same arithmetic as in a single block.
-
-__device__ __forceinline__ uint32_t cl_rank() {
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-__device__ __forceinline__ uint32_t cl_count() {
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
-    return r;
-}
-__device__ __forceinline__ uint32_t cl_id() {
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%clusterid.x;" : "=r"(r));
-    return r;
-}
-// all threads of all CTAs of the cluster; shared::cluster writes before it are visible after it
-__device__ __forceinline__ void cl_sync() {
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-// address of the same shared-memory byte in CTA `rank` of the cluster
-__device__ __forceinline__ uint32_t cl_map(const void *p, uint32_t rank) {
-    uint32_t r;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
-    return r;
-}
-__device__ __forceinline__ void cl_st(uint32_t addr, float v) {
-    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");
-}
-__device__ __forceinline__ float cl_ld(uint32_t addr) {
-    float v;
-    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
-    return v;
-}
-
-// byte offsets of a resident single-slot region (entries cd, lp, then R, S, V, X)
-struct RegionOffsets {
-    uint32_t lp, R, S, V, X, end;
-};
-__host__ __device__ __forceinline__ RegionOffsets region_offsets(int64_t L, int64_t nA) {
-    RegionOffsets o;
-    o.lp = (uint32_t)al16((size_t)nA * 4);
-    o.R = o.lp + (uint32_t)al16((size_t)nA * 4);
-    o.S = o.R + (uint32_t)al16((size_t)L * 4);
-    o.V = o.S + (uint32_t)al16((size_t)L * 4);
-    o.X = o.V + (uint32_t)al16((size_t)L * 4);
-    o.end = o.X + (uint32_t)al16((size_t)L * 4);
-    return o;
-}
-
-// load a single-slot region (packed entries, R, S; terminal values into V) and return the largest
-// |terminal value|
-__device__ __forceinline__ float load_region(const TreeView &tv, const CfrRoot &cr, int64_t data_base, int64_t slot,
-                                             unsigned char *base, Entries<true> &E, float *&R, float *&S, float *&V,
-                                             float *&X) {
-    const int tid = threadIdx.x, nth = blockDim.x;
-    const int L = cr.ls[9], nA = cr.as[9];
-    const RegionOffsets o = region_offsets(L, nA);
-    uint32_t *cd = (uint32_t *)base, *lp = (uint32_t *)(base + o.lp);
-    R = (float *)(base + o.R);
-    S = (float *)(base + o.S);
-    V = (float *)(base + o.V);
-    X = (float *)(base + o.X);
-    const int32_t *gli = tv.act_li + cr.act_off, *gpl = tv.act_pl + cr.act_off, *gcs = tv.act_cs + cr.act_off;
-    const uint16_t *gd = tv.act_d + cr.act_off;
-    for (int i = tid; i < nA; i += nth) {
-        cd[i] = (uint32_t)gcs[i] | ((uint32_t)gd[i] << 16);
-        lp[i] = (uint32_t)gli[i] | ((uint32_t)(gpl[i] < 0 ? 0xFFFF : gpl[i]) << 16);
-    }
-    const float *gR = tv.R + data_base, *gS = tv.S + data_base;
-    const int64_t *tq = tv.loc_tq + cr.loc_off;
-    float umax = 0.f;
-    for (int i = tid; i < L; i += nth) {
-        R[i] = gR[i];
-        S[i] = gS[i];
-        const int64_t q = tq[i];
-        if (q >= 0) {
-            const float v = tv.leaf_v[q + slot];
-            V[i] = v;
-            umax = fmaxf(umax, fabsf(v));
-        }
-    }
-    E.cd = cd;
-    E.lp = lp;
-    return umax;
-}
-
-__device__ __forceinline__ void store_region(const TreeView &tv, const CfrRoot &cr, int64_t data_base, const float *R,
-                                             const float *S) {
-    const int L = cr.ls[9];
-    float *gR = tv.R + data_base, *gS = tv.S + data_base;
-    for (int i = threadIdx.x; i < L; i += blockDim.x) {
-        gR[i] = R[i];
-        gS[i] = S[i];
-    }
-}
-
-template <int VARIANT, int MAXT>
-__global__ void __launch_bounds__(MAXT, MAXT == 256 ? 3 : 1) k_cfr_cluster(CfrParams p, const ClusterItem *__restrict__ clu) {
-    extern __shared__ __align__(16) unsigned char sm[];
-    __shared__ int32_t s_as[10], t_as[10];
-    __shared__ int32_t s_sb[15], s_sn[15], s_sf[15], t_sb[15], t_sn[15], t_sf[15];
-    __shared__ float s_tu[1];
-    __shared__ unsigned s_umax;
-    __shared__ float s_qmax[kMaxClusterCtas];
-    __shared__ uint32_t s_xoff[kMaxClusterCtas];
-    const int tid = threadIdx.x, nth = blockDim.x;
-    const uint32_t q = cl_rank(), nq = cl_count();
-    const ClusterItem c = clu[cl_id()];
-    const TreeView tv = p.views[c.tree];
-    const bool has_part = (int)q < c.nparts;
-    const ClusterPart top = tv.cparts[c.part0];
-    const ClusterPart part0 = tv.cparts[c.part0 + 1];
-    const CfrRoot &tr = tv.roots[top.root];
-    const CfrRoot &pr0 = tv.roots[part0.root];
-    // CTA 0: part 0 at offset 0, the top right after it
-    const uint32_t top_base = region_offsets(pr0.ls[9], pr0.as[9]).end;
-    const uint32_t top_v = top_base + region_offsets(tr.ls[9], tr.as[9]).V;
-    Entries<true> PE{}, TE{};
-    float *PR = nullptr, *PS = nullptr, *PV = nullptr, *PX = nullptr;
-    float *TR = nullptr, *TS = nullptr, *TV = nullptr, *TX = nullptr;
-    if (tid == 0) s_umax = 0u;
-    if (tid < (int)nq && q == 0) {
-        const int r = tid;
-        if (r < c.nparts) {
-            const CfrRoot &prr = tv.roots[tv.cparts[c.part0 + 1 + r].root];
-            s_xoff[r] = region_offsets(prr.ls[9], prr.as[9]).X;
-        } else {
-            s_xoff[r] = 0;
-        }
-    }
-    __syncthreads();
-    float um = 0.f;
-    const ClusterPart mine = has_part ? tv.cparts[c.part0 + 1 + q] : part0;
-    const CfrRoot &pr = tv.roots[mine.root];
-    if (has_part) um = load_region(tv, pr, mine.data_base, c.s0, sm, PE, PR, PS, PV, PX);
-    if (q == 0) um = fmaxf(um, load_region(tv, tr, top.data_base, c.s0, sm + top_base, TE, TR, TS, TV, TX));
-    atomicMax(&s_umax, __float_as_uint(um));
-    if (tid < 10) {
-        s_as[tid] = has_part ? pr.as[tid] : 0;
-        t_as[tid] = tr.as[tid];
-    }
-    __syncthreads();
-    if (q == 0 && tid == 0) TX[0] = 1.f;  // root reach
-    if (tid == 0) {
-        make_schedule(s_as, 1, s_sb, s_sn, s_sf);
-        make_schedule(t_as, 1, t_sb, t_sn, t_sf);
-        cl_st(cl_map(&s_qmax[q], 0), __uint_as_float(s_umax));
-    }
-    cl_sync();
-    if (tid == 0) {
-        float m = 0.f;
-        for (uint32_t r = 0; r < nq; r++) m = fmaxf(m, cl_ld(cl_map(&s_qmax[r], 0)));
-        s_tu[0] = p.tau * m;
-    }
-    __syncthreads();
-    const int32_t *cx = tv.cx + 5 * c.x0;
-    double acc = 0.0;
-    for (int il = 0; il < p.iters; il++) {
-        const float tf = (float)(p.t0 + il + 1);
-        float fpos, fneg, fs;
-        dcfr_factors<VARIANT>(p, il, fpos, fneg, fs);
-        if (q == 0) {
-            run_passes<VARIANT, true, true>(0, 7, 1, 0, TE, TR, TS, TV, TX, t_sb, t_sn, t_sf, s_tu, tf, fpos, fneg, fs);
-            // reaches of the active level-ell nodes and of their parents, into their owners
-            for (int j = tid; j < c.nx; j += nth) {
-                const int32_t *e = cx + 5 * j;
-                const uint32_t r = (uint32_t)e[0];
-                unsigned char *xb = sm + s_xoff[r];
-                cl_st(cl_map(xb + 4 * e[3], r), TX[e[1]]);
-                cl_st(cl_map(xb + 4 * e[4], r), TX[e[2]]);
-            }
-        }
-        cl_sync();
-        if (has_part) {
-            run_passes<VARIANT, true, true>(0, 15, 1, 0, PE, PR, PS, PV, PX, s_sb, s_sn, s_sf, s_tu, tf, fpos, fneg, fs);
-            // values of my active level-ell nodes, into the top
-            for (int j = tid; j < c.nx; j += nth) {
-                const int32_t *e = cx + 5 * j;
-                if ((uint32_t)e[0] == q) cl_st(cl_map(sm + top_v + 4 * e[1], 0), PV[e[3]]);
-            }
-        }
-        cl_sync();
-        if (q == 0) {
-            run_passes<VARIANT, true, true>(7, 15, 1, 0, TE, TR, TS, TV, TX, t_sb, t_sn, t_sf, s_tu, tf, fpos, fneg, fs);
-            if (tid == 0) acc += (double)TV[0];
-        }
-    }
-    if (has_part) store_region(tv, pr, mine.data_base, PR, PS);
-    if (q == 0) {
-        store_region(tv, tr, top.data_base, TR, TS);
-        if (tid == 0) {
-            if (!isfinite(acc)) atomicOr(p.err, 1);
-            tv.uacc[tv.fgt_off0[c.root] + c.s0] += acc;
-        }
-    }
-    cl_sync();  // no CTA leaves while another may still address its shared memory
-}
-
-// The cluster kernel for blocks of `threads` threads: up to 256 at up to 80 registers, up to 512 at
-// up to 128 (no spills), beyond that at up to 64 (a 1024-thread block on one SM).
-const void *const kClusterKernels[6] = {(const void *)k_cfr_cluster<0, 256>,  (const void *)k_cfr_cluster<1, 256>,
-                                        (const void *)k_cfr_cluster<0, 512>,  (const void *)k_cfr_cluster<1, 512>,
-                                        (const void *)k_cfr_cluster<0, 1024>, (const void *)k_cfr_cluster<1, 1024>};
-const void *cluster_kernel_for(int variant, int threads) {
-    return kClusterKernels[(threads > 512 ? 4 : threads > 256 ? 2 : 0) + (variant == 1)];
 }
 
 struct LevelPtrs {
@@ -975,7 +627,7 @@ __global__ void k_block_entries(int64_t n, const int64_t *src, const int32_t *ac
         const int64_t e = src[i];
         const CfrRoot &cr = roots[act_rk[e] >> 3];
         const int32_t *bm = bmap + cr.loc_off;
-        const uint32_t li = (uint32_t)bm[act_li[e]], pl = act_pl[e] < 0 ? (uint32_t)cr.ls[9] : (uint32_t)bm[act_pl[e]];
+        const uint32_t li = (uint32_t)bm[act_li[e]], pl = act_pl[e] < 0 ? 0xFFFFu : (uint32_t)bm[act_pl[e]];
         ent[i] = (li & 0xFFFFu) | (pl << 16);
         unsigned mk = 0;
         const int64_t *tq = loc_tq + cr.loc_off + act_cs[e];
@@ -1101,6 +753,7 @@ int build_block_order(pasur_tree *t, const int32_t *act_rk) {
     PASUR_TRY(launched());
     int64_t n_runs = 0;
     PASUR_TRY(read_i64(ctx, run + n, &n_runs));
+    t->n_runs = n_runs;
     PASUR_TRY(tree_alloc(t, (void **)&t->b_run, sizeof(BlockRun) * (size_t)(n_runs + 1)));
     if (n > 0) {
         k_block_children<<<grid, 256, 0, ctx->stream>>>(n, src, act_rk, t->croots_d, first, run, run_at, dpos, deg, t->act_cs, bmap,
@@ -1315,81 +968,89 @@ int build_layout(pasur_tree *t) {
 
 // ---- roots split over thread-block clusters ----------------------------------------------------
 
-
-struct SplitRoot {
-    int32_t ell = 0, nparts = 0;
-    int32_t top_root = 0, part_root0 = 0;   // pseudo-root ids
-    int64_t x0 = 0;
-    int32_t nx = 0;
-    int64_t top_L = 0;
-    std::vector<int64_t> part_L;            // local nodes incl. ghosts
-    size_t smem = 0;                         // largest CTA need (CTA 0: part 0 + top)
-};
-
 namespace {
 
-// Plan the split of every root that needs a cluster: subtrees of the active level-ell nodes packed
-// (in GT order) into parts that each fit one block; CTA 0 also holds the top levels.  Appends the
-// pseudo-roots to croots_h, their entries and local-node leaf indices to the host vectors, and
-// the exchange entries to t->cx_h.
-int plan_splits(pasur_tree *t, const pasur_config *cfg, size_t dyn_max, size_t part_max, const std::vector<char> &streamed,
-                std::vector<SplitRoot> &splits, std::vector<int32_t> &split_of, std::vector<int32_t> &nli,
-                std::vector<int32_t> &npl, std::vector<int32_t> &ncs, std::vector<uint16_t> &nd,
-                std::vector<int64_t> &ngt, std::vector<int64_t> &ntq) {
+// A root split over a cluster: its top and its parts as pseudo-roots; offsets relative to the arrays
+// here until they are placed after the tree's own.
+struct RootSplit {
+    bool done = false;
+    int W = 1, ell = 0, nparts = 0;
+    size_t smem = 0;  // largest CTA need (CTA 0: part 0 + top)
+    CfrRoot top{};
+    BlockRoot top_runs{};
+    std::vector<CfrRoot> parts;
+    std::vector<BlockRoot> part_runs;
+    std::vector<uint32_t> ent;
+    std::vector<uint8_t> msk, term;
+    std::vector<int32_t> inv;
+    std::vector<BlockRun> runs;
+    std::vector<int32_t> cx, x_at;  // exchange entries (5 ints each); first one of every part
+    int32_t top_root = 0;           // pseudo-root ids: the top, then the parts
+    int64_t x0 = 0;                 // place of its exchange entries
+    std::string msg;
+};
+
+constexpr int kSplitRuns = 96;  // runs a part is assumed to have while it is planned (checked after)
+
+// the most slots of one item when S slots are shared out evenly over items of at most cap slots
+int64_t even_slots(int64_t S, int64_t cap) {
+    const int64_t n = (S + cap - 1) / cap;
+    return (S + n - 1) / n;
+}
+
+// Split the roots whose state fits no block (or above cfg->split_bytes): subtrees of the active
+// level-ell nodes packed (in GT order) into parts that each fit one block; CTA 0 also holds the top
+// levels.  split[g] stays undone where no split is needed or none is found.
+int plan_splits(pasur_tree *t, const pasur_config *cfg, size_t limit, const std::vector<char> &streamed,
+                std::vector<RootSplit> &split) {
     pasur_ctx *ctx = t->ctx;
     const int64_t nr = t->n_roots;
-    split_of.assign((size_t)nr, -1);
     std::vector<int64_t> cand;
     for (int64_t g = 0; g < nr; g++) {
         const CfrRoot &cr = t->croots_h[(size_t)g];
         const int64_t Sg = t->csoff_h[(size_t)g + 1] - t->csoff_h[(size_t)g];
         const int64_t L = cr.ls[9], nA = cr.as[9];
         if (Sg == 0 || L == 0 || nA < 2 || streamed[(size_t)g] || !t->in_range(g)) continue;
-        const size_t need = resident_bytes(L, nA, 1);
-        if (need > dyn_max || (cfg->split_bytes > 0 && need > (size_t)cfg->split_bytes)) cand.push_back(g);
+        const bool fits = block_fits(cr, t->broots_h[(size_t)g], 1, limit);
+        if (!fits || (cfg->split_bytes > 0 && resident_bytes(L, nA, 1) > (size_t)cfg->split_bytes)) cand.push_back(g);
     }
+    split.clear();
     if (cand.empty()) return PASUR_OK;
+    split.resize((size_t)nr);
     PhaseTimer pt(ctx->stream, "cluster splits");
     // host copies of the layout
     const int64_t NA = t->n_active, NL = t->n_local;
     std::vector<int32_t> hli((size_t)NA), hpl((size_t)NA), hcs((size_t)NA);
     std::vector<uint16_t> hd((size_t)NA);
-    std::vector<int64_t> hgt((size_t)NA), htq((size_t)NL);
+    std::vector<int64_t> htq((size_t)NL);
     PASUR_CUDA(ctx, cudaMemcpy(hli.data(), t->act_li, sizeof(int32_t) * (size_t)NA, cudaMemcpyDeviceToHost));
     PASUR_CUDA(ctx, cudaMemcpy(hpl.data(), t->act_pl, sizeof(int32_t) * (size_t)NA, cudaMemcpyDeviceToHost));
     PASUR_CUDA(ctx, cudaMemcpy(hcs.data(), t->act_cs, sizeof(int32_t) * (size_t)NA, cudaMemcpyDeviceToHost));
     PASUR_CUDA(ctx, cudaMemcpy(hd.data(), t->act_d, sizeof(uint16_t) * (size_t)NA, cudaMemcpyDeviceToHost));
-    PASUR_CUDA(ctx, cudaMemcpy(hgt.data(), t->act_gt, sizeof(int64_t) * (size_t)NA, cudaMemcpyDeviceToHost));
     PASUR_CUDA(ctx, cudaMemcpy(htq.data(), t->loc_tq, sizeof(int64_t) * (size_t)NL, cudaMemcpyDeviceToHost));
     pt.mark("host copies");
-    const size_t target = cfg->split_bytes > 0 ? std::min<size_t>((size_t)cfg->split_bytes, part_max) : part_max;
+    const size_t target = cfg->split_bytes > 0 ? std::min<size_t>((size_t)cfg->split_bytes, limit) : limit;
     const bool verbose = getenv("PASUR_VERBOSE") != nullptr;
-    // the split of one root, its pseudo-roots' offsets relative to its own entries and nodes
-    struct RootSplit {
-        bool done = false;
-        SplitRoot sr;
-        CfrRoot top{};
-        std::vector<CfrRoot> parts;
-        std::vector<int32_t> li, pl, cs, cx;
-        std::vector<uint16_t> d;
-        std::vector<int64_t> gt, tq;
-        std::string msg;
-    };
-    auto split_one = [&](int64_t g, RootSplit &o) {
+    const int warps = kBlockMaxThreads / 32;
+    // the split of one root for items of W slots over at most qmax CTAs
+    auto split_one = [&](int64_t g, int W, int qmax, RootSplit &o) {
         const CfrRoot cr = t->croots_h[(size_t)g];
+        const BlockRoot &br = t->broots_h[(size_t)g];
         const int64_t L = cr.ls[9], nA = cr.as[9];
         const int32_t *li = hli.data() + cr.act_off, *pl = hpl.data() + cr.act_off, *cs = hcs.data() + cr.act_off;
         const uint16_t *dd = hd.data() + cr.act_off;
-        bool done = false;
-        for (int ell = 1; ell <= 6 && !done; ell++) {
+        const int64_t *tq = htq.data() + cr.loc_off;
+        auto bytes = [&](int64_t l, int64_t a) { return (size_t)block_offsets(l, a, kSplitRuns, W, warps).end; };
+        std::vector<int32_t> ent_of((size_t)L, -1);
+        for (int32_t e = 0; e < nA; e++) ent_of[(size_t)li[e]] = e;
+        for (int ell = 1; ell <= 6; ell++) {
             const int32_t e0 = cr.as[ell], e1 = cr.as[ell + 1];
             if (e1 - e0 < 2) continue;
             // subtree id of every local node at levels >= ell below an active level-ell node
-            std::vector<int32_t> heads;  // local indices of the active level-ell nodes, GT order
+            std::vector<int32_t> heads;  // local indices of the active level-ell nodes, in order
             for (int32_t e = e0; e < e1; e++) heads.push_back(li[e]);
             std::sort(heads.begin(), heads.end());
-            std::vector<int32_t> sub((size_t)L, -1), ent_of((size_t)L, -1);
-            for (int32_t e = 0; e < nA; e++) ent_of[(size_t)li[e]] = e;
+            std::vector<int32_t> sub((size_t)L, -1);
             for (size_t i = 0; i < heads.size(); i++) sub[(size_t)heads[i]] = (int32_t)i;
             const int ns = (int)heads.size();
             std::vector<int64_t> sa((size_t)ns, 0), sl((size_t)ns, 0);
@@ -1402,205 +1063,269 @@ int plan_splits(pasur_tree *t, const pasur_config *cfg, size_t dyn_max, size_t p
                 }
             for (int64_t x = cr.ls[ell]; x < L; x++)
                 if (sub[(size_t)x] >= 0) sl[(size_t)sub[(size_t)x]]++;
-            const size_t top_bytes = resident_bytes(cr.ls[ell + 1], cr.as[ell], 1);
-            if (top_bytes >= part_max) break;
-            // pack the subtrees into parts (contiguous runs), balancing active entries
+            const size_t top_bytes = block_offsets(cr.ls[ell + 1], cr.as[ell], br.rs[ell], W, warps).end;
+            if (top_bytes >= limit) break;
             int64_t tot = 0;
             for (int i = 0; i < ns; i++) tot += sa[(size_t)i];
-            // parts: the target size sets the starting count (portable clusters of up to 8 CTAs
-            // first), a block's shared memory is the hard limit of every part
-            const size_t need = resident_bytes(L, nA, 1);
-            const int q0 = (int)std::min<size_t>(cfg->split_bytes > 0 ? kMaxClusterCtas : 8,
-                                                 std::max<size_t>(2, (need + target - 1) / target));
+            // the target size sets the starting count of parts, a block's shared memory is the hard
+            // limit of every part
+            const size_t need = bytes(L, nA);
+            const int q0 = (int)std::min<size_t>((size_t)qmax, std::max<size_t>(2, (need + target - 1) / target));
             // contiguous parts: greedy fill with an entry cap (and the byte limit); the smallest
             // cap that needs at most Q parts, by bisection
             auto greedy = [&](int64_t cap, std::vector<int> &first) -> bool {
                 first.assign(1, 0);
                 int64_t pa = 0, plc = 0, pg = 0;
                 for (int i = 0; i < ns; i++) {
-                    const size_t lim = first.size() == 1 ? part_max - top_bytes : part_max;
-                    const bool fits = resident_bytes(plc + sl[(size_t)i] + pg + 1, pa + sa[(size_t)i], 1) <= lim;
+                    const size_t lim = first.size() == 1 ? limit - top_bytes : limit;
+                    const bool fits = bytes(plc + sl[(size_t)i] + pg + 1, pa + sa[(size_t)i]) <= lim;
                     if (pa > 0 && (!fits || pa + sa[(size_t)i] > cap)) {
                         first.push_back(i);
                         pa = plc = pg = 0;
                     }
-                    const size_t lim2 = first.size() == 1 ? part_max - top_bytes : part_max;
+                    const size_t lim2 = first.size() == 1 ? limit - top_bytes : limit;
                     pa += sa[(size_t)i];
                     plc += sl[(size_t)i];
                     pg += 1;
-                    if (resident_bytes(plc + pg, pa, 1) > lim2) return false;
+                    if (bytes(plc + pg, pa) > lim2) return false;
                 }
                 return true;
             };
             int64_t amax = 0;
             for (int i = 0; i < ns; i++) amax = std::max(amax, sa[(size_t)i]);
-            for (int Q = q0; Q <= kMaxClusterCtas && !done; Q++) {
+            for (int Q = q0; Q <= qmax; Q++) {
                 std::vector<int> first;
                 int64_t lo = std::max<int64_t>(amax, (tot + Q - 1) / Q), hi = tot;
-                if (!greedy(hi, first) || (int)first.size() > Q) {
-                    // even unlimited entries per part need more than Q parts (byte limit)
-                    if (!greedy(hi, first)) break;  // a single subtree does not fit a block
-                    continue;
-                }
+                if (!greedy(hi, first)) break;  // a single subtree does not fit a block
+                if ((int)first.size() > Q) continue;
                 while (lo < hi) {
                     const int64_t mid = lo + (hi - lo) / 2;
                     if (greedy(mid, first) && (int)first.size() <= Q) hi = mid;
                     else lo = mid + 1;
                 }
                 if (!greedy(lo, first) || (int)first.size() > Q) continue;
+                const int np = (int)first.size();
+                if (np < 2 || ctx->clusters_of[np] == 0) continue;
                 first.push_back(ns);
-                const int np = (int)first.size() - 1;
-                // build the parts
-                SplitRoot sr;
-                sr.ell = ell;
-                sr.nparts = np;
-                sr.top_L = cr.ls[ell + 1];
-                CfrRoot top = cr;
-                for (int k = ell + 1; k < 10; k++) top.as[k] = cr.as[ell];
-                for (int k = ell + 2; k < 10; k++) top.ls[k] = cr.ls[ell + 1];
-                top.W = 1;
-                top.cls = kClsCluster;
-                o.top = top;
-                std::vector<int32_t> part_of_sub((size_t)ns);
+                o = RootSplit{};
+                o.W = W;
+                o.ell = ell;
+                o.nparts = np;
+                // the top: the root's own entries and nodes, cut at level ell
+                o.top = cr;
+                o.top_runs = br;
+                for (int k = ell; k < 9; k++) o.top_runs.rs[k] = br.rs[ell];
+                for (int k = ell; k < 7; k++) o.top_runs.rt[k] = br.rs[ell];
+                for (int k = ell + 1; k < 10; k++) o.top.as[k] = cr.as[ell];
+                for (int k = ell + 2; k < 10; k++) o.top.ls[k] = cr.ls[ell + 1];
+                std::vector<int32_t> part_of((size_t)ns);
                 for (int q = 0; q < np; q++)
-                    for (int i = first[(size_t)q]; i < first[(size_t)q + 1]; i++) part_of_sub[(size_t)i] = q;
-                std::vector<int32_t> newidx((size_t)L, -1), ghost((size_t)L, -1);
-                size_t smax = 0;
+                    for (int i = first[(size_t)q]; i < first[(size_t)q + 1]; i++) part_of[(size_t)i] = q;
+                std::vector<int32_t> bidx((size_t)L, -1);
+                // entries part by part and level by level
+                std::vector<std::vector<std::vector<int32_t>>> ents((size_t)np, std::vector<std::vector<int32_t>>(8));
+                for (int k = ell; k < 8; k++)
+                    for (int32_t e = cr.as[k]; e < cr.as[k + 1]; e++) {
+                        const int32_t sid = sub[(size_t)li[e]];
+                        if (sid >= 0) ents[(size_t)part_of[(size_t)sid]][(size_t)k].push_back(e);
+                    }
                 for (int q = 0; q < np; q++) {
                     CfrRoot pr{};
-                    int64_t n = 0;
-                    for (int k = 0; k <= ell; k++) pr.ls[k] = 0;
-                    for (int k = ell; k <= 8; k++) {
-                        pr.ls[k] = (int32_t)n;
-                        for (int64_t x = cr.ls[k]; x < cr.ls[k + 1]; x++) {
-                            const int32_t sid = sub[(size_t)x];
-                            if (sid >= 0 && part_of_sub[(size_t)sid] == q) newidx[(size_t)x] = (int32_t)n++;
-                        }
-                    }
-                    for (int i = first[(size_t)q]; i < first[(size_t)q + 1]; i++) ghost[(size_t)heads[(size_t)i]] = (int32_t)n++;
-                    pr.ls[9] = (int32_t)n;
-                    pr.loc_off = (int64_t)o.tq.size();  // relative: placed after the other roots' parts when merged
-                    pr.act_off = (int64_t)o.li.size();
-                    std::vector<int64_t> tq((size_t)n, -1);
-                    for (int64_t x = cr.ls[ell]; x < L; x++) {
-                        const int32_t sid = sub[(size_t)x];
-                        if (sid >= 0 && part_of_sub[(size_t)sid] == q) tq[(size_t)newidx[(size_t)x]] = htq[(size_t)(cr.loc_off + x)];
-                    }
-                    o.tq.insert(o.tq.end(), tq.begin(), tq.end());
-                    int32_t m = 0;
-                    for (int k = 0; k <= ell; k++) pr.as[k] = 0;
+                    BlockRoot pb{};
+                    pr.loc_off = (int64_t)o.inv.size();
+                    pr.act_off = (int64_t)o.ent.size();
+                    pb.run_off = (int64_t)o.runs.size();
+                    const int h0 = first[(size_t)q], h = first[(size_t)q + 1] - h0;
+                    int32_t n = h, m = 0, r = 0;
+                    for (int i = 0; i < h; i++) bidx[(size_t)heads[(size_t)(h0 + i)]] = i;
+                    o.inv.insert(o.inv.end(), (size_t)h, -1);  // their regrets are the top's
+                    // level by level: entries with an active child first, runs of one degree, the runs'
+                    // children numbered child by child
                     for (int k = ell; k < 8; k++) {
-                        pr.as[k] = m;
-                        for (int32_t e = cr.as[k]; e < cr.as[k + 1]; e++) {
-                            const int32_t sid = sub[(size_t)li[e]];
-                            if (sid < 0 || part_of_sub[(size_t)sid] != q) continue;
-                            o.li.push_back(newidx[(size_t)li[e]]);
-                            o.pl.push_back(k == ell ? ghost[(size_t)li[e]] : newidx[(size_t)pl[e]]);
-                            o.cs.push_back(newidx[(size_t)cs[e]]);
-                            o.d.push_back(dd[e]);
-                            o.gt.push_back(hgt[(size_t)(cr.act_off + e)]);
-                            m++;
+                        std::vector<int32_t> &el = ents[(size_t)q][(size_t)k];
+                        auto active = [&](int32_t e) {
+                            for (int a = 0; a < dd[e]; a++)
+                                if (tq[cs[e] + a] < 0) return true;
+                            return false;
+                        };
+                        const size_t mid = (size_t)(std::stable_partition(el.begin(), el.end(), active) - el.begin());
+                        pb.rs[k] = r;
+                        for (size_t i = 0; i < el.size();) {
+                            size_t z = i;
+                            const size_t end = i < mid ? mid : el.size();
+                            while (z < end && dd[el[z]] == dd[el[i]]) z++;
+                            const int32_t len = (int32_t)(z - i), d = dd[el[i]];
+                            o.runs.push_back(BlockRun{(uint16_t)n, (uint16_t)m, (uint16_t)len, (uint16_t)d});
+                            r++;
+                            o.inv.resize((size_t)(pr.loc_off + n + len * d));
+                            for (int32_t y = 0; y < len; y++)
+                                for (int a = 0; a < d; a++) {
+                                    const int32_t b = n + a * len + y, x = cs[el[i + (size_t)y]] + a;
+                                    bidx[(size_t)x] = b;
+                                    o.inv[(size_t)(pr.loc_off + b)] = x;
+                                }
+                            n += len * d;
+                            m += len;
+                            i = z;
+                            if (k < 7 && i == mid) pb.rt[k] = r;
                         }
+                        if (k < 7 && mid == 0) pb.rt[k] = pb.rs[k];
                     }
-                    pr.as[8] = pr.as[9] = m;
-                    pr.W = 1;
+                    pb.rs[8] = r;
+                    const int32_t g0 = n;  // the ghosts: the parents' reaches
+                    n += h;
+                    o.inv.insert(o.inv.end(), (size_t)h, -1);
+                    for (int k = ell; k < 8; k++)
+                        for (int32_t e : ents[(size_t)q][(size_t)k]) {
+                            const int32_t up = k == ell ? g0 + bidx[(size_t)li[e]] : bidx[(size_t)pl[e]];
+                            o.ent.push_back((uint32_t)bidx[(size_t)li[e]] | (uint32_t)up << 16);
+                            uint8_t mk = 0;
+                            for (int a = 0; a < dd[e] && a < 8; a++) mk |= (uint8_t)((tq[cs[e] + a] < 0 ? 1 : 0) << a);
+                            o.msk.push_back(mk);
+                        }
+                    for (int32_t b = 0; b < n; b++) {
+                        const int32_t x = o.inv[(size_t)(pr.loc_off + b)];
+                        o.term.push_back(x >= 0 && tq[x] >= 0 ? 1 : 0);
+                    }
+                    pr.ls[9] = n;
+                    pr.as[9] = m;
+                    pr.W = W;
                     pr.cls = kClsCluster;
+                    size_t b = block_offsets(n, m, r, W, warps).end;
+                    if (q == 0) b += top_bytes;
+                    o.smem = std::max(o.smem, n >= 65535 ? limit + 1 : b);
                     o.parts.push_back(pr);
-                    sr.part_L.push_back(n);
-                    size_t b = resident_bytes(n, m, 1);
-                    if (q == 0) b += resident_bytes(sr.top_L, cr.as[ell], 1);
-                    smax = std::max(smax, b);
+                    o.part_runs.push_back(pb);
+                    // exchange entries: the part's level-ell nodes
+                    o.x_at.push_back((int32_t)(o.cx.size() / 5));
+                    for (int i = 0; i < h; i++) {
+                        const int32_t x = heads[(size_t)(h0 + i)], e = ent_of[(size_t)x];
+                        // block indices of the top: set below from the root's own
+                        o.cx.push_back(q);
+                        o.cx.push_back(x);
+                        o.cx.push_back(pl[e]);
+                        o.cx.push_back(i);
+                        o.cx.push_back(g0 + i);
+                    }
                 }
-                // exchange entries: active level-ell nodes
-                for (size_t i = 0; i < heads.size(); i++) {
-                    const int32_t x = heads[i];
-                    const int32_t e = ent_of[(size_t)x];
-                    o.cx.push_back(part_of_sub[i]);
-                    o.cx.push_back(x);
-                    o.cx.push_back(pl[e]);
-                    o.cx.push_back(newidx[(size_t)x]);
-                    o.cx.push_back(ghost[(size_t)x]);
-                }
-                sr.nx = (int32_t)heads.size();
-                sr.smem = smax;
-                o.sr = std::move(sr);
-                o.done = done = true;
+                o.x_at.push_back((int32_t)(o.cx.size() / 5));
+                if (o.smem > limit) continue;
+                o.done = true;
+                return;
             }
-            if (!done && verbose) {
+            if (verbose) {
                 int64_t big = 0;
-                for (int i = 0; i < ns; i++) big = std::max<int64_t>(big, (int64_t)resident_bytes(sl[(size_t)i] + 1, sa[(size_t)i], 1));
+                for (int i = 0; i < ns; i++) big = std::max<int64_t>(big, (int64_t)bytes(sl[(size_t)i] + 1, sa[(size_t)i]));
                 char line[256];
-                snprintf(line, sizeof line, "[pasur] root %lld (L %lld, active %lld): no split at level %d: %d subtrees, top %zu B, "
-                                            "largest subtree %lld B, part limit %zu B\n",
-                         (long long)g, (long long)L, (long long)nA, ell, ns, top_bytes, (long long)big, part_max);
+                snprintf(line, sizeof line, "[pasur] root %lld (L %lld, active %lld), %d slots: no split at level %d: %d subtrees, top "
+                                            "%zu B, largest subtree %lld B, part limit %zu B\n",
+                         (long long)g, (long long)L, (long long)nA, W, ell, ns, top_bytes, (long long)big, limit);
                 o.msg += line;
             }
         }
     };
-    // roots are independent: split them on host threads, then append the results in root order
-    std::vector<RootSplit> res(cand.size());
+    // roots are independent: split them on host threads; as many slots per item as clusters of up to 8
+    // CTAs hold, one slot over up to 16
     std::atomic<size_t> next{0};
     std::atomic<bool> failed{false};
     auto worker = [&]() {
         try {
-            for (size_t i = next++; i < cand.size(); i = next++) split_one(cand[i], res[i]);
+            for (size_t i = next++; i < cand.size(); i = next++) {
+                const int64_t g = cand[i];
+                const int64_t Sg = t->csoff_h[(size_t)g + 1] - t->csoff_h[(size_t)g];
+                RootSplit &o = split[(size_t)g];
+                std::string msg;
+                for (int64_t W = even_slots(Sg, cfg->slots_per_item > 0 ? std::min(cfg->slots_per_item, kBlockSlots) : kBlockSlots);
+                     W >= 1 && !o.done; W = W > 1 ? even_slots(Sg, W - 1) : 0) {
+                    split_one(g, (int)W, W > 1 && cfg->split_bytes == 0 ? 8 : kMaxClusterCtas, o);
+                    if (!o.done) msg += o.msg;
+                    o.msg.clear();
+                }
+                o.msg = msg;
+            }
         } catch (...) {
             failed = true;
         }
     };
     const unsigned hw = std::max(1u, std::thread::hardware_concurrency());
     const size_t nw = std::min<size_t>({(size_t)hw, (size_t)16, cand.size()});
-    auto run_workers = [&](const std::function<void()> &fn) {
+    {
         std::vector<std::thread> th;
-        for (size_t w = 1; w < nw; w++) th.emplace_back(fn);
-        fn();
+        for (size_t w = 1; w < nw; w++) th.emplace_back(worker);
+        worker();
         for (auto &x : th) x.join();
-    };
-    run_workers(worker);
+    }
     if (failed) return set_err(ctx, PASUR_ENOMEM, "cluster split: host allocation failed");
     pt.mark("per-root splits");
-    // root order: pseudo-roots, exchange entries and the offsets of every root's entries and nodes
-    std::vector<size_t> a_at(cand.size() + 1, nli.size()), l_at(cand.size() + 1, ntq.size());
-    for (size_t ci = 0; ci < cand.size(); ci++) {
-        RootSplit &o = res[ci];
-        if (!o.msg.empty()) fputs(o.msg.c_str(), stderr);
-        a_at[ci + 1] = a_at[ci] + o.li.size();
-        l_at[ci + 1] = l_at[ci] + o.tq.size();
+    for (int64_t g : cand)
+        if (!split[(size_t)g].done && !split[(size_t)g].msg.empty()) fputs(split[(size_t)g].msg.c_str(), stderr);
+    return PASUR_OK;
+}
+
+// The parts' entries, runs and index maps after the tree's own (device), the pseudo-roots after the
+// real roots, and the exchange entries.
+int place_splits(pasur_tree *t, std::vector<RootSplit> &split) {
+    pasur_ctx *ctx = t->ctx;
+    const int64_t NA = t->n_active, NL = t->n_local, NR = t->n_runs;
+    std::vector<uint32_t> ent;
+    std::vector<uint8_t> msk, term;
+    std::vector<int32_t> inv;
+    std::vector<BlockRun> runs;
+    bool any = false;
+    for (const RootSplit &o : split) any |= o.done;
+    if (!any) return PASUR_OK;
+    // block index of the top's nodes: the inverse of the root's own map, levels <= ell
+    std::vector<int32_t> own, back;
+    for (size_t g = 0; g < split.size(); g++) {
+        RootSplit &o = split[g];
         if (!o.done) continue;
-        SplitRoot sr = std::move(o.sr);
-        sr.top_root = (int32_t)t->croots_h.size();
-        sr.part_root0 = sr.top_root + 1;
-        sr.x0 = (int64_t)t->cx_h.size() / 5;
+        const int64_t off = t->croots_h[g].loc_off;
+        own.resize((size_t)o.top.ls[9]);
+        PASUR_CUDA(ctx, cudaMemcpy(own.data(), t->b_inv + off, sizeof(int32_t) * own.size(), cudaMemcpyDeviceToHost));
+        back.assign(own.size(), 0);
+        for (size_t b = 0; b < own.size(); b++) back[(size_t)own[b]] = (int32_t)b;
+        for (size_t i = 0; i < o.cx.size(); i += 5) {
+            o.cx[i + 1] = back[(size_t)o.cx[i + 1]];
+            o.cx[i + 2] = back[(size_t)o.cx[i + 2]];
+        }
+        o.top_root = (int32_t)t->croots_h.size();
+        o.x0 = (int64_t)t->cx_h.size() / 5;
         t->croots_h.push_back(o.top);
-        for (CfrRoot pr : o.parts) {
-            pr.loc_off += NL + (int64_t)l_at[ci];
-            pr.act_off += NA + (int64_t)a_at[ci];
+        t->broots_h.push_back(o.top_runs);
+        for (size_t q = 0; q < o.parts.size(); q++) {
+            CfrRoot pr = o.parts[q];
+            BlockRoot pb = o.part_runs[q];
+            pr.loc_off += NL + (int64_t)inv.size();
+            pr.act_off += NA + (int64_t)ent.size();
+            pb.run_off += NR + (int64_t)runs.size();
             t->croots_h.push_back(pr);
+            t->broots_h.push_back(pb);
         }
+        ent.insert(ent.end(), o.ent.begin(), o.ent.end());
+        msk.insert(msk.end(), o.msk.begin(), o.msk.end());
+        term.insert(term.end(), o.term.begin(), o.term.end());
+        inv.insert(inv.end(), o.inv.begin(), o.inv.end());
+        runs.insert(runs.end(), o.runs.begin(), o.runs.end());
         t->cx_h.insert(t->cx_h.end(), o.cx.begin(), o.cx.end());
-        split_of[(size_t)cand[ci]] = (int32_t)splits.size();
-        splits.push_back(std::move(sr));
     }
-    // the entries and node links, copied into place by the host threads
-    nli.resize(a_at.back());
-    npl.resize(a_at.back());
-    ncs.resize(a_at.back());
-    nd.resize(a_at.back());
-    ngt.resize(a_at.back());
-    ntq.resize(l_at.back());
-    next = 0;
-    run_workers([&]() {
-        for (size_t ci = next++; ci < cand.size(); ci = next++) {
-            const RootSplit &o = res[ci];
-            std::copy(o.li.begin(), o.li.end(), nli.begin() + (ptrdiff_t)a_at[ci]);
-            std::copy(o.pl.begin(), o.pl.end(), npl.begin() + (ptrdiff_t)a_at[ci]);
-            std::copy(o.cs.begin(), o.cs.end(), ncs.begin() + (ptrdiff_t)a_at[ci]);
-            std::copy(o.d.begin(), o.d.end(), nd.begin() + (ptrdiff_t)a_at[ci]);
-            std::copy(o.gt.begin(), o.gt.end(), ngt.begin() + (ptrdiff_t)a_at[ci]);
-            std::copy(o.tq.begin(), o.tq.end(), ntq.begin() + (ptrdiff_t)l_at[ci]);
-        }
-    });
-    pt.mark("merge");
+    auto grow = [&](void **p, int64_t n_old, size_t size, const void *more, size_t n_more) -> int {
+        void *x = nullptr;
+        PASUR_TRY(tree_alloc(t, &x, size * ((size_t)n_old + n_more + 1)));
+        PASUR_CUDA(ctx, cudaMemcpyAsync(x, *p, size * (size_t)n_old, cudaMemcpyDeviceToDevice, ctx->stream));
+        PASUR_CUDA(ctx, cudaMemcpyAsync((char *)x + size * (size_t)n_old, more, size * n_more, cudaMemcpyHostToDevice, ctx->stream));
+        *p = x;
+        return PASUR_OK;
+    };
+    PASUR_TRY(grow((void **)&t->b_ent, NA, sizeof(uint32_t), ent.data(), ent.size()));
+    PASUR_TRY(grow((void **)&t->b_msk, NA, sizeof(uint8_t), msk.data(), msk.size()));
+    PASUR_TRY(grow((void **)&t->b_term, NL, sizeof(uint8_t), term.data(), term.size()));
+    PASUR_TRY(grow((void **)&t->b_inv, NL, sizeof(int32_t), inv.data(), inv.size()));
+    PASUR_TRY(grow((void **)&t->b_run, NR, sizeof(BlockRun), runs.data(), runs.size()));
+    PASUR_TRY(tree_alloc(t, (void **)&t->croots_d, sizeof(CfrRoot) * t->croots_h.size()));
+    PASUR_TRY(tree_alloc(t, (void **)&t->broots_d, sizeof(BlockRoot) * t->broots_h.size()));
+    PASUR_CUDA(ctx, cudaMemcpyAsync(t->broots_d, t->broots_h.data(), sizeof(BlockRoot) * t->broots_h.size(), cudaMemcpyHostToDevice,
+                                    ctx->stream));
+    PASUR_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
     return PASUR_OK;
 }
 
@@ -1614,6 +1339,8 @@ int cfr_dyn_smem_limit(pasur_ctx *ctx, size_t *limit) {
     for (int v = 0; v < 2; v++)
         for (int w = 1; w <= kBlockSlots; w++) {
             PASUR_CUDA(ctx, cudaFuncGetAttributes(&fa, block_kernel(v, w)));
+            st = std::max(st, fa.sharedSizeBytes);
+            PASUR_CUDA(ctx, cudaFuncGetAttributes(&fa, cluster_kernel(v, w)));
             st = std::max(st, fa.sharedSizeBytes);
         }
     *limit = ctx->smem_optin > st ? ctx->smem_optin - st : 0;
@@ -1630,8 +1357,63 @@ const void *block_kernel(int variant, int W) {
         default: return block_kernel_w6(variant);
     }
 }
+const void *cluster_kernel(int variant, int W) {
+    switch (W) {
+        case 1: return cluster_kernel_w1(variant);
+        case 2: return cluster_kernel_w2(variant);
+        case 3: return cluster_kernel_w3(variant);
+        case 4: return cluster_kernel_w4(variant);
+        case 5: return cluster_kernel_w5(variant);
+        default: return cluster_kernel_w6(variant);
+    }
+}
 
-int cfr_cluster_smem_limit(pasur_ctx *ctx, size_t *limit);
+namespace {
+
+void sweep_launch_config(const SweepLaunch &l, cudaLaunchConfig_t *lc, cudaLaunchAttribute *at) {
+    lc->gridDim = dim3((unsigned)((l.end - l.begin) * l.ctas));
+    lc->blockDim = dim3((unsigned)l.threads);
+    lc->dynamicSmemBytes = l.smem;
+    if (l.ctas > 1) {
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = (unsigned)l.ctas;
+        at[0].val.clusterDim.y = 1;
+        at[0].val.clusterDim.z = 1;
+        lc->attrs = at;
+        lc->numAttrs = 1;
+    }
+}
+
+// Once per context: the kernels' attributes (global per kernel: the largest dynamic size any plan can
+// ask for, so that plans prepared later never lower it under an earlier plan's need) and the cluster
+// sizes the device can hold with a whole SM's shared memory per CTA.
+int raise_limits(pasur_ctx *ctx, size_t limit) {
+    if (ctx->cfr_smem_raised) return PASUR_OK;
+    for (int v = 0; v < 2; v++)
+        for (int w = 1; w <= kBlockSlots; w++) {
+            PASUR_CUDA(ctx, cudaFuncSetAttribute(block_kernel(v, w), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)limit));
+            PASUR_CUDA(ctx, cudaFuncSetAttribute(cluster_kernel(v, w), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)limit));
+            PASUR_CUDA(ctx, cudaFuncSetAttribute(cluster_kernel(v, w), cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+        }
+    for (int q = 2; q <= kMaxClusterCtas; q++) {
+        SweepLaunch l;
+        l.ctas = q;
+        l.end = 1;
+        l.threads = kBlockMaxThreads;
+        l.smem = limit;
+        cudaLaunchConfig_t lc{};
+        cudaLaunchAttribute at[1];
+        sweep_launch_config(l, &lc, at);
+        if (cudaOccupancyMaxActiveClusters(&ctx->clusters_of[q], cluster_kernel(0, kBlockSlots), &lc) != cudaSuccess) {
+            cudaGetLastError();
+            ctx->clusters_of[q] = 0;
+        }
+    }
+    ctx->cfr_smem_raised = true;
+    return PASUR_OK;
+}
+
+}  // namespace
 
 int cfr_setup_tree(pasur_tree *t, const pasur_config *cfg, int tree, std::vector<CfrItem> *cls_items,
                    std::vector<ClusterItem> *clu) {
@@ -1639,18 +1421,17 @@ int cfr_setup_tree(pasur_tree *t, const pasur_config *cfg, int tree, std::vector
     PhaseTimer pt(ctx->stream, "cfr plan");
     PASUR_TRY(build_layout(t));
     pt.mark("layout");
-    // every root goes to the smallest shared-memory class its subtree fits with one slot; its
-    // items then take as many slots as that class holds
+    size_t limit = 0;
+    PASUR_TRY(cfr_dyn_smem_limit(ctx, &limit));
+    PASUR_TRY(raise_limits(ctx, limit));
+    // how R and S are stored: every root in the smallest storage class its subtree fits with one slot,
+    // in items of as many slots as that class holds
     const size_t dyn_max = ctx->smem_optin > kStorageReserve ? ctx->smem_optin - kStorageReserve : 0;
     size_t budget[kNumCls - 1];
     for (int c = 0; c < kNumCls - 1; c++) budget[c] = kClsBudget[c] ? std::min<size_t>(kClsBudget[c], dyn_max) : dyn_max;
     const int wcap = cfg->slots_per_item > 0 ? std::min(cfg->slots_per_item, kMaxSlots) : kMaxSlots;
-    // roots too large for one block (or above cfg->split_bytes) go to thread-block clusters
-    std::vector<SplitRoot> splits;
-    std::vector<int32_t> split_of, nli, npl, ncs;
-    std::vector<uint16_t> nd;
-    std::vector<int64_t> ngt, ntq;
     t->croots_h.resize((size_t)t->n_roots);
+    t->broots_h.resize((size_t)t->n_roots);
     t->cparts_h.clear();
     t->cx_h.clear();
     // roots streamed over every SM (class 5): those above cfg->stream_bytes, and those too large
@@ -1660,16 +1441,14 @@ int cfr_setup_tree(pasur_tree *t, const pasur_config *cfg, int tree, std::vector
     for (int64_t g = 0; g < t->n_roots; g++) {
         const CfrRoot &cr = t->croots_h[(size_t)g];
         const int64_t Sg = t->csoff_h[(size_t)g + 1] - t->csoff_h[(size_t)g];
-        const int64_t L = cr.ls[9], nA = cr.as[9];
-        if (Sg == 0 || L == 0 || !t->in_range(g)) continue;
-        const size_t need = resident_bytes(L, nA, 1);
-        streamed[(size_t)g] = (cfg->stream_bytes > 0 && need > (size_t)cfg->stream_bytes) ||
-                              (need > dyn_max && Sg >= kStreamMinSlots);
+        if (Sg == 0 || cr.ls[9] == 0 || !t->in_range(g)) continue;
+        streamed[(size_t)g] = (cfg->stream_bytes > 0 && resident_bytes(cr.ls[9], cr.as[9], 1) > (size_t)cfg->stream_bytes) ||
+                              (Sg >= kStreamMinSlots && !block_fits(cr, t->broots_h[(size_t)g], 1, limit));
     }
-    size_t dyn_cl = 0;
-    PASUR_TRY(cfr_cluster_smem_limit(ctx, &dyn_cl));
-    PASUR_TRY(plan_splits(t, cfg, dyn_max, std::min(dyn_max, dyn_cl), streamed, splits, split_of, nli, npl, ncs, nd, ngt,
-                          ntq));
+    // roots too large for one block (or above cfg->split_bytes) go to thread-block clusters
+    std::vector<RootSplit> split;
+    PASUR_TRY(plan_splits(t, cfg, limit, streamed, split));
+    PASUR_TRY(place_splits(t, split));
     pt.mark("cluster splits");
     std::vector<int64_t> sbase((size_t)t->csoff_h[(size_t)t->n_roots] + 1, 0);
     std::vector<int32_t> sstr(sbase.size(), 0);
@@ -1681,56 +1460,49 @@ int cfr_setup_tree(pasur_tree *t, const pasur_config *cfg, int tree, std::vector
         cr.W = 0;
         cr.cls = -1;
         if (Sg == 0 || L == 0 || !t->in_range(g)) continue;
-        if (split_of[(size_t)g] >= 0) {
-            const SplitRoot sr = splits[(size_t)split_of[(size_t)g]];
-            cr.W = 1;
-            cr.cls = kClsCluster;
-            for (int64_t s0 = 0; s0 < Sg; s0++) {
-                ClusterItem ci{};
-                ci.tree = tree;
-                ci.root = (int32_t)g;
-                ci.s0 = s0;
-                ci.part0 = (int64_t)t->cparts_h.size();
-                ci.x0 = sr.x0;
-                ci.nx = sr.nx;
-                ci.nparts = sr.nparts;
-                ci.ell = sr.ell;
-                ci.smem = (int32_t)sr.smem;
-                for (int q = -1; q < sr.nparts; q++) {
-                    const int32_t r = q < 0 ? sr.top_root : sr.part_root0 + q;
-                    const int64_t n = q < 0 ? sr.top_L : sr.part_L[(size_t)q];
-                    t->cparts_h.push_back(ClusterPart{r, 0, data});
-                    CfrItem it{};
-                    it.root = r;
-                    it.tree = tree;
-                    it.ns = 1;
-                    it.s0 = s0;
-                    it.data_base = data;
-                    it.scratch_base = -1;
-                    it.cost = std::max<int64_t>(t->croots_h[(size_t)r].as[9], 1);
-                    cls_items[kClsCluster].push_back(it);
-                    data += n;
-                }
-                clu->push_back(ci);
-            }
-            continue;
-        }
-        // slots per item: a power of two (the kernel indexes slots with shifts).  Automatic: the
-        // smallest class the root fits with one slot, then the largest count that class holds.
-        // With cfg.slots_per_item: that many slots (at most the root's), in the smallest class
-        // that holds them, fewer where no class does.
-        int64_t want = 1;
-        if (cfg->slots_per_item > 0)
-            while (want * 2 <= std::min<int64_t>(Sg, wcap)) want *= 2;
-        int cls = kClsGlobal;
-        for (; want >= 1 && cls == kClsGlobal && !streamed[(size_t)g]; want /= 2)
-            for (int c = 0; c < kNumCls - 1; c++)
-                if (resident_bytes(L, nA, want) <= budget[c]) {
-                    cls = c;
-                    break;
-                }
         int64_t w = 1;
-        while (w * 2 <= std::min<int64_t>(Sg, wcap) && (cls == kClsGlobal || resident_bytes(L, nA, w * 2) <= budget[cls])) w *= 2;
+        int cls = kClsGlobal, store = kClsGlobal;
+        if (!split.empty() && split[(size_t)g].done) {
+            const RootSplit &o = split[(size_t)g];
+            cls = store = kClsCluster;
+            ClusterItem ci{};
+            ci.tree = tree;
+            ci.root = (int32_t)g;
+            ci.part0 = (int64_t)t->cparts_h.size();
+            ci.x0 = o.x0;
+            ci.nx = (int32_t)(o.cx.size() / 5);
+            ci.nparts = o.nparts;
+            ci.smem = o.smem;
+            t->cparts_h.push_back(ClusterPart{o.top_root, 0, 0});
+            for (int q = 0; q < o.nparts; q++)
+                t->cparts_h.push_back(ClusterPart{o.top_root + 1 + q, o.x_at[(size_t)q], o.x_at[(size_t)q + 1]});
+            const int64_t n = (Sg + o.W - 1) / o.W;
+            for (int64_t i = 0, s0 = 0; i < n; i++) {
+                ci.s0 = (int32_t)s0;
+                ci.ns = (int32_t)(Sg / n + (i < Sg % n ? 1 : 0));
+                ci.cost = nA * ci.ns;
+                clu->push_back(ci);
+                s0 += ci.ns;
+            }
+        } else {
+            // slots per stored item: a power of two (the streaming sweep indexes slots with shifts).
+            // Automatic: the smallest class the root fits with one slot, then the largest count that
+            // class holds.  With cfg.slots_per_item: that many slots (at most the root's), in the
+            // smallest class that holds them, fewer where no class does.
+            int64_t want = 1;
+            if (cfg->slots_per_item > 0)
+                while (want * 2 <= std::min<int64_t>(Sg, wcap)) want *= 2;
+            for (; want >= 1 && store == kClsGlobal && !streamed[(size_t)g]; want /= 2)
+                for (int c = 0; c < kNumCls - 1; c++)
+                    if (resident_bytes(L, nA, want) <= budget[c]) {
+                        store = c;
+                        break;
+                    }
+            while (w * 2 <= std::min<int64_t>(Sg, wcap) && (store == kClsGlobal || resident_bytes(L, nA, w * 2) <= budget[store])) w *= 2;
+            // the sweep's blocks hold more than the storage classes: a root beyond those may still fit
+            cls = store;
+            if (cls == kClsGlobal && !streamed[(size_t)g] && block_fits(cr, t->broots_h[(size_t)g], 1, limit)) cls = kClsGlobal - 1;
+        }
         cr.W = (int32_t)w;
         cr.cls = cls;
         for (int64_t s0 = 0, ns = w; s0 < Sg; s0 += ns) {
@@ -1741,9 +1513,9 @@ int cfr_setup_tree(pasur_tree *t, const pasur_config *cfg, int tree, std::vector
             it.ns = (int32_t)ns;
             it.s0 = s0;
             it.data_base = data;
-            for (int64_t w = 0; w < ns; w++) {
-                sbase[(size_t)(t->csoff_h[(size_t)g] + s0 + w)] = data + w;
-                sstr[(size_t)(t->csoff_h[(size_t)g] + s0 + w)] = (int32_t)ns;
+            for (int64_t x = 0; x < ns; x++) {
+                sbase[(size_t)(t->csoff_h[(size_t)g] + s0 + x)] = data + x;
+                sstr[(size_t)(t->csoff_h[(size_t)g] + s0 + x)] = (int32_t)ns;
             }
             data += L * it.ns;
             it.scratch_base = -1;
@@ -1766,43 +1538,13 @@ int cfr_setup_tree(pasur_tree *t, const pasur_config *cfg, int tree, std::vector
             t->swept_pairs += (int64_t)cr.as[9] * ns;
         }
     }
-    if (!splits.empty()) {
-        // append the parts' entries and local leaf indices; pseudo-roots after the real roots
-        const int64_t NA = t->n_active, NL = t->n_local, na = (int64_t)nli.size(), nl = (int64_t)ntq.size();
-        int32_t *li = nullptr, *pl = nullptr, *cs = nullptr;
-        uint16_t *d = nullptr;
-        int64_t *gt = nullptr, *tq = nullptr;
-        PASUR_TRY(tree_alloc(t, (void **)&li, sizeof(int32_t) * (size_t)(NA + na + 1)));
-        PASUR_TRY(tree_alloc(t, (void **)&pl, sizeof(int32_t) * (size_t)(NA + na + 1)));
-        PASUR_TRY(tree_alloc(t, (void **)&cs, sizeof(int32_t) * (size_t)(NA + na + 1)));
-        PASUR_TRY(tree_alloc(t, (void **)&d, sizeof(uint16_t) * (size_t)(NA + na + 1)));
-        PASUR_TRY(tree_alloc(t, (void **)&gt, sizeof(int64_t) * (size_t)(NA + na + 1)));
-        PASUR_TRY(tree_alloc(t, (void **)&tq, sizeof(int64_t) * (size_t)(NL + nl + 1)));
-        auto cp = [&](void *dst, const void *old_d, size_t ob, const void *new_h, size_t nb) -> int {
-            PASUR_CUDA(ctx, cudaMemcpyAsync(dst, old_d, ob, cudaMemcpyDeviceToDevice, ctx->stream));
-            PASUR_CUDA(ctx, cudaMemcpyAsync((char *)dst + ob, new_h, nb, cudaMemcpyHostToDevice, ctx->stream));
-            return PASUR_OK;
-        };
-        PASUR_TRY(cp(li, t->act_li, 4 * (size_t)NA, nli.data(), 4 * (size_t)na));
-        PASUR_TRY(cp(pl, t->act_pl, 4 * (size_t)NA, npl.data(), 4 * (size_t)na));
-        PASUR_TRY(cp(cs, t->act_cs, 4 * (size_t)NA, ncs.data(), 4 * (size_t)na));
-        PASUR_TRY(cp(d, t->act_d, 2 * (size_t)NA, nd.data(), 2 * (size_t)na));
-        PASUR_TRY(cp(gt, t->act_gt, 8 * (size_t)NA, ngt.data(), 8 * (size_t)na));
-        PASUR_TRY(cp(tq, t->loc_tq, 8 * (size_t)NL, ntq.data(), 8 * (size_t)nl));
-        t->act_li = li;
-        t->act_pl = pl;
-        t->act_cs = cs;
-        t->act_d = d;
-        t->act_gt = gt;
-        t->loc_tq = tq;
-        PASUR_TRY(tree_alloc(t, (void **)&t->croots_d, sizeof(CfrRoot) * t->croots_h.size()));
+    if (!t->cparts_h.empty()) {
         PASUR_TRY(tree_alloc(t, (void **)&t->cparts_d, sizeof(ClusterPart) * (t->cparts_h.size() + 1)));
         PASUR_TRY(tree_alloc(t, (void **)&t->cx_d, sizeof(int32_t) * (t->cx_h.size() + 1)));
         PASUR_CUDA(ctx, cudaMemcpyAsync(t->cparts_d, t->cparts_h.data(), sizeof(ClusterPart) * t->cparts_h.size(),
                                         cudaMemcpyHostToDevice, ctx->stream));
         PASUR_CUDA(ctx, cudaMemcpyAsync(t->cx_d, t->cx_h.data(), sizeof(int32_t) * t->cx_h.size(), cudaMemcpyHostToDevice,
                                         ctx->stream));
-        PASUR_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
     }
     if (!t->croots_h.empty())
         PASUR_CUDA(ctx, cudaMemcpyAsync(t->croots_d, t->croots_h.data(), sizeof(CfrRoot) * t->croots_h.size(),
@@ -1851,22 +1593,40 @@ int cfr_setup_tree(pasur_tree *t, const pasur_config *cfg, int tree, std::vector
     return PASUR_OK;
 }
 
-int cfr_cluster_check(pasur_ctx *ctx, CfrPlan *plan, const pasur_config *cfg);
-
-// The block sweep's items and launch groups: every root of the storage classes 0..4 of the trees.
-int plan_blocks(pasur_ctx *ctx, CfrPlan &plan, const std::vector<pasur_tree *> &trees, const pasur_config *cfg,
-                std::vector<std::pair<void *, size_t>> &owned) {
+// The cluster and block sweeps' items and launches: the clusters' items, and every root of the storage
+// classes 0..4 of the trees in a block.
+int plan_sweeps(pasur_ctx *ctx, CfrPlan &plan, const std::vector<pasur_tree *> &trees, const pasur_config *cfg,
+                const std::vector<ClusterItem> &clu, std::vector<std::pair<void *, size_t>> &owned) {
     plan.blk_h.clear();
-    plan.groups.clear();
+    plan.launches.clear();
     size_t lim = 0;
     PASUR_TRY(cfr_dyn_smem_limit(ctx, &lim));
-    if (!ctx->cfr_smem_raised) {
-        // the attribute is global per kernel: raise it once to the largest dynamic size any plan
-        // can ask for, so that plans prepared later never lower it under an earlier plan's need
-        for (int v = 0; v < 2; v++)
-            for (int w = 1; w <= kBlockSlots; w++)
-                PASUR_CUDA(ctx, cudaFuncSetAttribute(block_kernel(v, w), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lim));
-        ctx->cfr_smem_raised = true;
+    const int full = cfg->threads > 0 ? std::min(cfg->threads, kBlockMaxThreads) : kBlockMaxThreads;
+    // clusters: one launch per parts and slots, the largest first
+    plan.clu_h = clu;
+    std::stable_sort(plan.clu_h.begin(), plan.clu_h.end(), [](const ClusterItem &a, const ClusterItem &b) {
+        if (a.nparts != b.nparts) return a.nparts > b.nparts;
+        if (a.ns != b.ns) return a.ns > b.ns;
+        return a.cost > b.cost;
+    });
+    for (size_t i = 0; i < plan.clu_h.size(); i++) {
+        const ClusterItem &x = plan.clu_h[i];
+        if (i == 0 || x.nparts != plan.clu_h[i - 1].nparts || x.ns != plan.clu_h[i - 1].ns) {
+            SweepLaunch l;
+            l.ctas = x.nparts;
+            l.W = x.ns;
+            l.threads = full;
+            l.begin = (int64_t)i;
+            plan.launches.push_back(l);
+        }
+        plan.launches.back().end = (int64_t)i + 1;
+        plan.launches.back().smem = std::max(plan.launches.back().smem, x.smem);
+    }
+    if (!plan.clu_h.empty()) {
+        const size_t b = sizeof(ClusterItem) * plan.clu_h.size();
+        PASUR_TRY(dev_alloc(ctx, (void **)&plan.clu_d, b));
+        owned.push_back({plan.clu_d, b});
+        PASUR_CUDA(ctx, cudaMemcpyAsync(plan.clu_d, plan.clu_h.data(), b, cudaMemcpyHostToDevice, ctx->stream));
     }
     auto in_block = [&](const pasur_tree *t, int64_t g) {
         const int c = t->croots_h[(size_t)g].cls;
@@ -1877,7 +1637,10 @@ int plan_blocks(pasur_ctx *ctx, CfrPlan &plan, const std::vector<pasur_tree *> &
         for (int64_t g = 0; g < t->n_roots; g++)
             if (in_block(t, g)) slots += t->csoff_h[(size_t)g + 1] - t->csoff_h[(size_t)g];
     if (slots == 0) return PASUR_OK;
-    const int wcap = (int)std::max<int64_t>(1, std::min<int64_t>(kBlockSlots, slots / (kSlotsPerSm * ctx->num_sms)));
+    // slots per item: as many as a block holds, but with few slots in all rather more blocks than more
+    // slots per block
+    int64_t wcap = std::max<int64_t>(1, std::min<int64_t>(kBlockSlots, slots / (kSlotsPerSm * ctx->num_sms)));
+    if (cfg->slots_per_item > 0) wcap = std::min(cfg->slots_per_item, kBlockSlots);
     // blocks per SM by shared memory (228 KB per SM, 1 KB reserved per block, some static)
     auto per_sm = [&](size_t smem) {
         for (int n = 6; n > 1; n--)
@@ -1898,24 +1661,23 @@ int plan_blocks(pasur_ctx *ctx, CfrPlan &plan, const std::vector<pasur_tree *> &
             const BlockRoot &br = t->broots_h[(size_t)g];
             const int64_t S = t->csoff_h[(size_t)g + 1] - t->csoff_h[(size_t)g], L = cr.ls[9], nA = cr.as[9], nR = br.rs[8];
             int64_t w = std::min<int64_t>(S, wcap);
-            while (w > 1 && block_offsets(L, nA, nR, (int)w, kBlockMaxThreads / 32).end > lim) w--;
+            while (w > 1 && !block_fits(cr, br, (int)w, lim)) w--;
             const int64_t n = (S + w - 1) / w;
+            int chunks = 1;
+            for (int k = 0; k < 8; k++) chunks = std::max(chunks, (cr.as[k + 1] - cr.as[k]) / 32 + br.rs[k + 1] - br.rs[k]);
             for (int64_t i = 0, s0 = 0; i < n; i++) {
-                const int W = (int)(S / n + (i < S % n ? 1 : 0));
                 Tagged x{};
                 x.it.tree = (int32_t)ti;
                 x.it.root = (int32_t)g;
                 x.it.s0 = (int32_t)s0;
-                x.it.ns = W;
-                x.it.cost = std::max<int64_t>(nA, 1) * W;
-                x.chunks = 1;
-                for (int k = 0; k < 8; k++)
-                    x.chunks = std::max(x.chunks, (cr.as[k + 1] - cr.as[k]) / 32 + br.rs[k + 1] - br.rs[k]);
-                x.smem = block_offsets(L, nA, nR, W, kBlockMaxThreads / 32).end;
+                x.it.ns = (int32_t)(S / n + (i < S % n ? 1 : 0));
+                x.it.cost = std::max<int64_t>(nA, 1) * x.it.ns;
+                x.chunks = chunks;
+                x.smem = block_offsets(L, nA, nR, x.it.ns, kBlockMaxThreads / 32).end;
                 if (x.smem > lim) return set_err(ctx, PASUR_EINVAL, "a block item exceeds a block's shared memory");
                 x.per = per_sm(x.smem);
                 all.push_back(x);
-                s0 += W;
+                s0 += x.it.ns;
             }
         }
     }
@@ -1924,30 +1686,26 @@ int plan_blocks(pasur_ctx *ctx, CfrPlan &plan, const std::vector<pasur_tree *> &
         if (a.it.ns != b.it.ns) return a.it.ns > b.it.ns;
         return a.it.cost > b.it.cost;
     });
+    // warps: what the registers allow among the blocks of one SM, no more than the widest level's chunks
     const bool few = (int64_t)all.size() <= ctx->num_sms;
     int chunks = 1;
     for (size_t i = 0; i < all.size(); i++) {
         const Tagged &x = all[i];
         if (i == 0 || x.per != all[i - 1].per || x.it.ns != all[i - 1].it.ns) {
-            BlockGroup gr;
-            gr.W = x.it.ns;
-            gr.begin = (int64_t)i;
-            plan.groups.push_back(gr);
+            SweepLaunch l;
+            l.W = x.it.ns;
+            l.begin = (int64_t)i;
+            plan.launches.push_back(l);
             chunks = 1;
         }
-        BlockGroup &gr = plan.groups.back();
-        gr.end = (int64_t)i + 1;
-        gr.smem = std::max(gr.smem, x.smem);
+        SweepLaunch &l = plan.launches.back();
+        l.end = (int64_t)i + 1;
+        l.smem = std::max(l.smem, x.smem);
         chunks = std::max(chunks, x.chunks);
-        cudaFuncAttributes fa;
-        PASUR_CUDA(ctx, cudaFuncGetAttributes(&fa, block_kernel(cfg->variant, x.it.ns)));
-        const int regs = (fa.numRegs + 7) & ~7;
-        int th = 65536 / regs / (few ? 1 : x.per) / 32 * 32;
-        gr.threads = std::max(32, std::min({th, kBlockMaxThreads, 32 * chunks}));
-        if (cfg->threads > 0) gr.threads = std::min(cfg->threads, kBlockMaxThreads);
+        l.threads = cfg->threads > 0 ? full : std::max(32, std::min(kBlockMaxThreads / (few ? 1 : x.per) / 32 * 32, 32 * chunks));
         plan.blk_h.push_back(x.it);
     }
-    size_t b = sizeof(BlockItem) * plan.blk_h.size();
+    const size_t b = sizeof(BlockItem) * plan.blk_h.size();
     PASUR_TRY(dev_alloc(ctx, (void **)&plan.blk_d, b));
     owned.push_back({plan.blk_d, b});
     PASUR_CUDA(ctx, cudaMemcpyAsync(plan.blk_d, plan.blk_h.data(), b, cudaMemcpyHostToDevice, ctx->stream));
@@ -1962,8 +1720,8 @@ int cfr_finalize_plan(pasur_ctx *ctx, CfrPlan &plan, std::vector<CfrItem> *cls_i
     if (cfg->split_bytes < 0) return set_err(ctx, PASUR_EINVAL, "cfg.split_bytes must be >= 0");
     if (cfg->stream_bytes < 0) return set_err(ctx, PASUR_EINVAL, "cfg.stream_bytes must be >= 0");
     plan.items_h.clear();
-    // classes 0..4: storage of the roots the block sweep solves; 5 the level-streaming sweep's items;
-    // 6 the cluster items' pseudo-items
+    // how the roots' state is stored: classes 0..4 of the roots solved in a block, 5 the
+    // level-streaming sweep's items, 6 the roots split over clusters
     for (int c = 0; c <= kClsCluster; c++) {
         std::stable_sort(cls_items[c].begin(), cls_items[c].end(),
                          [](const CfrItem &a, const CfrItem &b) { return a.cost > b.cost; });
@@ -1972,33 +1730,6 @@ int cfr_finalize_plan(pasur_ctx *ctx, CfrPlan &plan, std::vector<CfrItem> *cls_i
         plan.cls_end[c] = (int64_t)plan.items_h.size();
     }
     plan.n_items = (int64_t)plan.items_h.size();
-    plan.clu_h = clu;
-    std::stable_sort(plan.clu_h.begin(), plan.clu_h.end(),
-                     [](const ClusterItem &a, const ClusterItem &b) { return a.nparts < b.nparts; });
-    for (int b = 0; b < kCluGroups; b++) {
-        plan.clu_begin[b] = plan.clu_end[b] = 0;
-        plan.clu_smem[b] = 0;
-    }
-    int64_t i = 0;
-    for (int b = 0; b < kCluGroups; b++) {
-        plan.clu_begin[b] = i;
-        while (i < (int64_t)plan.clu_h.size() && plan.clu_h[(size_t)i].nparts <= plan.clu_ctas[b]) {
-            plan.clu_smem[b] = std::max(plan.clu_smem[b], (size_t)plan.clu_h[(size_t)i].smem);
-            i++;
-        }
-        plan.clu_end[b] = i;
-    }
-    // one block width for the cluster launches: 512 threads, one CTA per SM (seed-47 CFR with class
-    // 4 at 512: 1175 -> 1110 ms; 1024 threads measured slower than 256)
-    plan.clu_threads = 512;
-    if (cfg->threads > 0) plan.clu_threads = cfg->threads;
-    if (!plan.clu_h.empty()) {
-        size_t b = sizeof(ClusterItem) * plan.clu_h.size();
-        PASUR_TRY(dev_alloc(ctx, (void **)&plan.clu_d, b));
-        owned.push_back({plan.clu_d, b});
-        PASUR_CUDA(ctx, cudaMemcpyAsync(plan.clu_d, plan.clu_h.data(), b, cudaMemcpyHostToDevice, ctx->stream));
-        PASUR_TRY(cfr_cluster_check(ctx, &plan, cfg));
-    }
     if (plan.n_items) {
         size_t b = sizeof(CfrItem) * (size_t)plan.n_items;
         PASUR_TRY(dev_alloc(ctx, (void **)&plan.items_d, b));
@@ -2040,7 +1771,7 @@ int cfr_finalize_plan(pasur_ctx *ctx, CfrPlan &plan, std::vector<CfrItem> *cls_i
         PASUR_CUDA(ctx, cudaGetLastError());
         PASUR_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
     }
-    PASUR_TRY(plan_blocks(ctx, plan, trees, cfg, owned));
+    PASUR_TRY(plan_sweeps(ctx, plan, trees, cfg, clu, owned));
     // the uploads read host vectors of this call
     PASUR_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
     return PASUR_OK;
@@ -2134,44 +1865,26 @@ int cfr_launch_plan(pasur_ctx *ctx, CfrPlan &plan, const pasur_config *cfg, int6
         return PASUR_OK;
     };
     // the launches are independent: each runs on its own forked stream (beyond their number,
-    // several share one), largest subtrees first; the level-streaming sweep (thousands of short
-    // launches) is queued last, so that the host never waits on its queue before the others start
-    const int nb = (int)std::min<size_t>(plan.groups.size(), kAuxStreams - kAuxBlock);
-    for (int c = 0; c < nb; c++) PASUR_TRY(fork(kAuxBlock + c));
-    for (size_t i = 0; i < plan.groups.size(); i++) {
-        const BlockGroup &gr = plan.groups[i];
-        BlockParams bp{plan.blk_d + gr.begin, plan.views_d, dcfr, cfg->iters, t0, cfg->rm_deadzone, ctx->errflag};
-        void *args[] = {&bp};
-        PASUR_CUDA(ctx, cudaLaunchKernel(block_kernel(cfg->variant, gr.W), dim3((unsigned)(gr.end - gr.begin)),
-                                         dim3((unsigned)gr.threads), args, gr.smem, ctx->aux[kAuxBlock + (int)(i % (size_t)nb)]));
-        ctx->launches++;
-    }
-    for (int c = 0; c < nb; c++) PASUR_TRY(join(kAuxBlock + c));
-    // roots split over thread-block clusters: one cluster per item, a launch (and a stream) per
-    // cluster size
-    for (int b = 0; b < kCluGroups; b++) {
-        const int64_t n = plan.clu_end[b] - plan.clu_begin[b];
-        if (n == 0) continue;
-        const int c = kAuxCluster + b;
-        PASUR_TRY(fork(c));
+    // several share one), clusters first, largest subtrees first; the level-streaming sweep (thousands
+    // of short launches) is queued last, so that the host never waits on its queue before the others
+    // start
+    const int nb = (int)std::min<size_t>(plan.launches.size(), kAuxStreams - kAuxSweep);
+    for (int x = 0; x < nb; x++) PASUR_TRY(fork(kAuxSweep + x));
+    for (size_t i = 0; i < plan.launches.size(); i++) {
+        const SweepLaunch &l = plan.launches[i];
+        BlockParams bp{nullptr, plan.views_d, dcfr, cfg->iters, t0, cfg->rm_deadzone, ctx->errflag};
+        const ClusterItem *ci = nullptr;
+        void *args[] = {&bp, &ci};
         cudaLaunchConfig_t lc{};
-        lc.gridDim = dim3((unsigned)(n * plan.clu_ctas[b]), 1, 1);
-        lc.blockDim = dim3((unsigned)plan.clu_threads, 1, 1);
-        lc.dynamicSmemBytes = plan.clu_smem[b];
-        lc.stream = ctx->aux[c];
         cudaLaunchAttribute at[1];
-        at[0].id = cudaLaunchAttributeClusterDimension;
-        at[0].val.clusterDim.x = (unsigned)plan.clu_ctas[b];
-        at[0].val.clusterDim.y = 1;
-        at[0].val.clusterDim.z = 1;
-        lc.attrs = at;
-        lc.numAttrs = 1;
-        const ClusterItem *ci = plan.clu_d + plan.clu_begin[b];
-        void *args[] = {&p, &ci};
-        PASUR_CUDA(ctx, cudaLaunchKernelExC(&lc, cluster_kernel_for(cfg->variant, plan.clu_threads), args));
+        sweep_launch_config(l, &lc, at);
+        lc.stream = ctx->aux[kAuxSweep + (int)(i % (size_t)nb)];
+        if (l.ctas > 1) ci = plan.clu_d + l.begin;
+        else bp.items = plan.blk_d + l.begin;
+        PASUR_CUDA(ctx, cudaLaunchKernelExC(&lc, l.ctas > 1 ? cluster_kernel(cfg->variant, l.W) : block_kernel(cfg->variant, l.W), args));
         ctx->launches++;
-        PASUR_TRY(join(c));
     }
+    for (int x = 0; x < nb; x++) PASUR_TRY(join(kAuxSweep + x));
     if (plan.cls_end[kClsGlobal] != plan.cls_begin[kClsGlobal]) {
         PASUR_TRY(fork(kAuxStream));
         PASUR_TRY(stream_sweep(ctx, plan, p, cfg, ctx->aux[kAuxStream]));
@@ -2180,83 +1893,33 @@ int cfr_launch_plan(pasur_ctx *ctx, CfrPlan &plan, const pasur_config *cfg, int6
     return PASUR_OK;
 }
 
-// Prepare the cluster kernel for a plan's cluster items: shared-memory and cluster-size
-// attributes, and a check that one cluster of this shape can be resident.
-int cfr_cluster_smem_limit(pasur_ctx *ctx, size_t *limit) {
-    size_t st = 0;
-    cudaFuncAttributes fa;
-    for (const void *k : kClusterKernels) {
-        PASUR_CUDA(ctx, cudaFuncGetAttributes(&fa, k));
-        st = std::max(st, fa.sharedSizeBytes);
-    }
-    *limit = ctx->smem_optin > st ? ctx->smem_optin - st : 0;
-    return PASUR_OK;
-}
-
-int cfr_cluster_check(pasur_ctx *ctx, CfrPlan *plan, const pasur_config *cfg) {
-    size_t lim = 0;
-    PASUR_TRY(cfr_cluster_smem_limit(ctx, &lim));
-    for (const void *k : kClusterKernels) {
-        PASUR_CUDA(ctx, cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lim));
-        PASUR_CUDA(ctx, cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-    }
-    for (int b = 0; b < kCluGroups; b++) {
-        if (plan->clu_end[b] == plan->clu_begin[b]) continue;
-        if (plan->clu_smem[b] > lim) return set_err(ctx, PASUR_EINVAL, "cluster part exceeds the shared memory of a block");
-        cudaLaunchConfig_t lc{};
-        lc.gridDim = dim3((unsigned)plan->clu_ctas[b], 1, 1);
-        lc.blockDim = dim3((unsigned)plan->clu_threads, 1, 1);
-        lc.dynamicSmemBytes = plan->clu_smem[b];
-        cudaLaunchAttribute at[1];
-        at[0].id = cudaLaunchAttributeClusterDimension;
-        at[0].val.clusterDim.x = (unsigned)plan->clu_ctas[b];
-        at[0].val.clusterDim.y = 1;
-        at[0].val.clusterDim.z = 1;
-        lc.attrs = at;
-        lc.numAttrs = 1;
-        int nclusters = 0;
-        PASUR_CUDA(ctx, cudaOccupancyMaxActiveClusters(&nclusters, cluster_kernel_for(cfg->variant, plan->clu_threads), &lc));
-        if (nclusters < 1)
-            return set_err(ctx, PASUR_EINVAL, "a cluster of " + std::to_string(plan->clu_ctas[b]) + " blocks of " +
-                                                  std::to_string(plan->clu_smem[b]) + " B shared memory cannot be resident");
-    }
-    return PASUR_OK;
-}
-
 void cfr_plan_times(pasur_ctx *ctx, CfrPlan &plan) {
-    const size_t nb = std::min<size_t>(plan.groups.size(), kAuxStreams - kAuxBlock);
-    for (size_t i = 0; i < plan.groups.size(); i++) {
-        plan.groups[i].ms = 0.f;
-        if (i < nb) cudaEventElapsedTime(&plan.groups[i].ms, ctx->cls_t0[kAuxBlock + i], ctx->cls_t1[kAuxBlock + i]);
+    const size_t nb = std::min<size_t>(plan.launches.size(), kAuxStreams - kAuxSweep);
+    for (size_t i = 0; i < plan.launches.size(); i++) {
+        plan.launches[i].ms = 0.f;
+        if (i < nb) cudaEventElapsedTime(&plan.launches[i].ms, ctx->cls_t0[kAuxSweep + i], ctx->cls_t1[kAuxSweep + i]);
     }
     plan.str_ms = 0.f;
     if (plan.cls_end[kClsGlobal] != plan.cls_begin[kClsGlobal])
         cudaEventElapsedTime(&plan.str_ms, ctx->cls_t0[kAuxStream], ctx->cls_t1[kAuxStream]);
-    for (int b = 0; b < kCluGroups; b++) {
-        plan.clu_ms[b] = 0.f;
-        if (plan.clu_end[b] != plan.clu_begin[b])
-            cudaEventElapsedTime(&plan.clu_ms[b], ctx->cls_t0[kAuxCluster + b], ctx->cls_t1[kAuxCluster + b]);
-    }
 }
 
 // one line per launch of a plan
 void cfr_print_plan(const CfrPlan &plan) {
-    for (const BlockGroup &gr : plan.groups) {
+    for (const SweepLaunch &l : plan.launches) {
         int64_t cost = 0, maxcost = 0;
-        for (int64_t i = gr.begin; i < gr.end; i++) {
-            cost += plan.blk_h[(size_t)i].cost;
-            maxcost = std::max(maxcost, plan.blk_h[(size_t)i].cost);
+        for (int64_t i = l.begin; i < l.end; i++) {
+            const int64_t x = l.ctas > 1 ? plan.clu_h[(size_t)i].cost : plan.blk_h[(size_t)i].cost;
+            cost += x;
+            maxcost = std::max(maxcost, x);
         }
-        fprintf(stderr, "[pasur]   block items: %lld of %d slots, %d threads, smem %zu B, "
-                        "active-node-slots %lld (largest item %lld), %.3f ms\n",
-                (long long)(gr.end - gr.begin), gr.W, gr.threads, gr.smem, (long long)cost,
-                (long long)maxcost, gr.ms);
+        char ctas[32] = "";
+        if (l.ctas > 1) snprintf(ctas, sizeof ctas, "%d CTAs x ", l.ctas);
+        fprintf(stderr, "[pasur]   %s items: %lld of %d slots, %s%d threads, smem %zu B, active-node-slots %lld (largest item "
+                        "%lld), %.3f ms\n",
+                l.ctas > 1 ? "cluster" : "block", (long long)(l.end - l.begin), l.W, ctas, l.threads, l.smem, (long long)cost,
+                (long long)maxcost, l.ms);
     }
-    for (int b = 0; b < kCluGroups; b++)
-        if (plan.clu_end[b] != plan.clu_begin[b])
-            fprintf(stderr, "[pasur]   cluster items: %lld, %d CTAs x %d threads, smem %zu B, %.3f ms\n",
-                    (long long)(plan.clu_end[b] - plan.clu_begin[b]), plan.clu_ctas[b], plan.clu_threads, plan.clu_smem[b],
-                    plan.clu_ms[b]);
     if (plan.str_n > 0)
         fprintf(stderr, "[pasur]   streamed items: %lld (slots %lld), %.3f ms\n", (long long)plan.str_n, (long long)plan.str_nslots,
                 plan.str_ms);

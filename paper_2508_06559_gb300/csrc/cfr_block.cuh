@@ -36,13 +36,18 @@ __host__ __device__ __forceinline__ BlockOffsets block_offsets(int64_t L, int64_
     return o;
 }
 
-// the kernel for items of W slots
+// the kernels for items of W slots (one translation unit per W)
 const void *block_kernel(int variant, int W);
-const void *block_kernel_w1(int variant);
-const void *block_kernel_w2(int variant);
-const void *block_kernel_w3(int variant);
-const void *block_kernel_w4(int variant);
-const void *block_kernel_w5(int variant);
-const void *block_kernel_w6(int variant);
+const void *cluster_kernel(int variant, int W);
+#define PASUR_SWEEP_KERNELS(W)                   \
+    const void *block_kernel_w##W(int variant);  \
+    const void *cluster_kernel_w##W(int variant);
+PASUR_SWEEP_KERNELS(1)
+PASUR_SWEEP_KERNELS(2)
+PASUR_SWEEP_KERNELS(3)
+PASUR_SWEEP_KERNELS(4)
+PASUR_SWEEP_KERNELS(5)
+PASUR_SWEEP_KERNELS(6)
+#undef PASUR_SWEEP_KERNELS
 
 }  // namespace pasur

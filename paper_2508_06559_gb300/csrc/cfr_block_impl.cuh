@@ -33,7 +33,7 @@ __global__ void __launch_bounds__(kBlockMaxThreads, 1) k_cfr_block(BlockParams p
         um[w] = 0.f;
     }
     __syncthreads();
-    load_state<W>(at, tv, cr, base, str, it.s0, um);
+    load_state<W>(at, tv, cr, cr, base, str, it.s0, um);
 #pragma unroll
     for (int w = 0; w < W; w++) atomicMax((unsigned *)&sh.tu[w], __float_as_uint(um[w]));
     if (tid < W) sts(at.v + (L * W + tid) * 4, 1.f);  // the reach of the root's mover

@@ -212,8 +212,8 @@ __device__ __noinline__ void bu_any(NodeAt n, int d, bool alex, float thr, StepF
 // what follows it: another segment, a warp barrier or a block barrier.
 // x = address of its first node's first child's regret, y = bytes from one child to the next, z =
 // address of its first entry, w = nodes | degree (255: 255 or more) << 16 | flags << 24.
-// An entry: address of the node's value; of its parent's value | mask of its active children (the
-// first 8) << 24.
+// An entry: address of the node's value; low 24 bits of its parent's value's address | mask of its active
+// children (the first 8) << 24.  (In a cluster the bits above hold the CTA's rank.)
 // A segment's lanes hold a node each with all its slots, or (kSegSpread) one (node, slot) each.
 constexpr uint32_t kSegUp = 1, kSegAlex = 2, kSegSyncWarp = 4, kSegSync = 8, kSegSpread = 16;
 constexpr int kSegSolo = 256, kSegSmall = 512;  // of a level step: warp 0's alone, few nodes (not stored in segments)
@@ -227,7 +227,7 @@ struct SweepShared {
 
 // where a sweep's arrays lie (see BlockOffsets) and the root's tables
 struct SweepAt {
-    uint32_t seg, ent, r, v, sof, vof;  // vof: from a regret to its value
+    uint32_t seg, ent, r, v, sof, vof, hi;  // vof: from a regret to its value; hi: the addresses' bits above 23
     const BlockRun *runs;
     const BlockRoot *root;
     const uint8_t *term;  // per block index: 1 for a terminal (global memory)
@@ -238,8 +238,9 @@ struct SweepAt {
         v = seg + o.V;
         sof = o.S - o.R;
         vof = o.V - o.R;
+        hi = seg & 0xFF000000u;
         // opaque: kept in registers instead of being derived from the block's shared window again
-        asm volatile("" : "+r"(seg), "+r"(ent), "+r"(r), "+r"(v), "+r"(sof), "+r"(vof));
+        asm volatile("" : "+r"(seg), "+r"(ent), "+r"(r), "+r"(v), "+r"(sof), "+r"(vof), "+r"(hi));
     }
 };
 
@@ -410,7 +411,7 @@ __device__ __forceinline__ void run_segment(const SweepAt &at, uint32_t ctl, con
         do {
             if (left > 0) {
                 n.me = en.x;
-                n.up = en.y & 0xFFFFFFu;
+                n.up = (en.y & 0xFFFFFFu) | at.hi;
                 if constexpr (M != W) {
                     n.me += w4;
                     n.up += w4;
@@ -487,31 +488,33 @@ __device__ __forceinline__ void run_program(Cursor &c, const SweepAt &at, const 
     } while (c.pa != c.first);
 }
 
-// entries as addresses; regrets and strategy sums from their places in device memory; values of the
+// Entries as addresses; regrets and strategy sums from their places in device memory; values of the
 // terminals (constant over the iterations), other values 1 (the root's reach; the others are written
-// before they are read); per slot the largest |terminal value| into um (per thread)
+// before they are read); per slot the largest |terminal value| into um (per thread).  xr: the root or
+// pseudo-root, cr: the root whose local nodes it is made of (nodes without one, inv < 0, have no
+// regret of their own here).
 template <int W>
-__device__ __forceinline__ void load_state(const SweepAt &at, const TreeView &tv, const CfrRoot &cr, const int64_t *base,
-                                           const int32_t *str, int64_t s0, float *um) {
-    const int tid = threadIdx.x, nth = blockDim.x, L = cr.ls[9], nA = cr.as[9];
-    const uint32_t *ge = tv.b_ent + cr.act_off;
-    const uint8_t *gm = tv.b_msk + cr.act_off;
+__device__ __forceinline__ void load_state(const SweepAt &at, const TreeView &tv, const CfrRoot &xr, const CfrRoot &cr,
+                                           const int64_t *base, const int32_t *str, int64_t s0, float *um) {
+    const int tid = threadIdx.x, nth = blockDim.x, L = xr.ls[9], nA = xr.as[9];
+    const uint32_t *ge = tv.b_ent + xr.act_off;
+    const uint8_t *gm = tv.b_msk + xr.act_off;
     for (int i = tid; i < nA; i += nth) {
-        const uint32_t e = ge[i];
+        const uint32_t e = ge[i], up = e >> 16 == 0xFFFFu ? (uint32_t)L : e >> 16;
         asm volatile("st.shared.v2.u32 [%0], {%1, %2};" ::"r"(at.ent + 8 * i), "r"(at.v + (e & 0xFFFFu) * (W * 4)),
-                     "r"((at.v + (e >> 16) * (W * 4)) | (uint32_t)gm[i] << 24)
+                     "r"((at.v + up * (W * 4) & 0xFFFFFFu) | (uint32_t)gm[i] << 24)
                      : "memory");
     }
-    const int32_t *inv = tv.b_inv + cr.loc_off;
+    const int32_t *inv = tv.b_inv + xr.loc_off;
     const int64_t *tq = tv.loc_tq + cr.loc_off;
     for (int x = tid; x < L; x += nth) {
         const int l = inv[x];
-        const int64_t q = tq[l];
+        const int64_t q = l < 0 ? -1 : tq[l];
 #pragma unroll
         for (int w = 0; w < W; w++) {
             const int64_t g = base[w] + (int64_t)l * str[w];
-            sts(at.r + (x * W + w) * 4, tv.R[g]);
-            sts(at.r + at.sof + (x * W + w) * 4, tv.S[g]);
+            sts(at.r + (x * W + w) * 4, l < 0 ? 0.f : tv.R[g]);
+            sts(at.r + at.sof + (x * W + w) * 4, l < 0 ? 0.f : tv.S[g]);
             float v = 1.f;
             if (q >= 0) {
                 v = tv.leaf_v[q + s0 + w];
@@ -523,11 +526,12 @@ __device__ __forceinline__ void load_state(const SweepAt &at, const TreeView &tv
 }
 
 template <int W>
-__device__ __forceinline__ void store_state(const SweepAt &at, const TreeView &tv, const CfrRoot &cr, const int64_t *base,
+__device__ __forceinline__ void store_state(const SweepAt &at, const TreeView &tv, const CfrRoot &xr, const int64_t *base,
                                             const int32_t *str) {
-    const int32_t *inv = tv.b_inv + cr.loc_off;
-    for (int x = threadIdx.x; x < cr.ls[9]; x += blockDim.x) {
+    const int32_t *inv = tv.b_inv + xr.loc_off;
+    for (int x = threadIdx.x; x < xr.ls[9]; x += blockDim.x) {
         const int l = inv[x];
+        if (l < 0) continue;
 #pragma unroll
         for (int w = 0; w < W; w++) {
             const int64_t g = base[w] + (int64_t)l * str[w];

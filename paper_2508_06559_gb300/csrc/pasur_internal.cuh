@@ -113,7 +113,8 @@ __host__ __device__ __forceinline__ void score_unkey(uint32_t k, int &ac, int &b
 }
 constexpr int kScoreKeyBits = 26;
 
-constexpr int kAuxStreams = 24;  // forked streams of a context
+constexpr int kAuxStreams = 24;      // forked streams of a context
+constexpr int kMaxClusterCtas = 16;  // CTAs of a cluster (more than 8: non-portable size)
 
 }  // namespace pasur
 
@@ -143,13 +144,15 @@ struct pasur_ctx {
     int32_t *counter = nullptr;  // work-queue counters (device)
     int32_t *errflag = nullptr;  // device error word
     int64_t launches = 0;        // kernels launched through this context
-    // forked streams for concurrent launches (created on first use): the level-streaming sweep 0,
-    // cluster launches 1..4, launches of the block sweep 5..
+    // forked streams for concurrent launches (created on first use): the level-streaming sweep 0, the
+    // launches of the cluster and block sweeps in turn 1..
     cudaStream_t aux[pasur::kAuxStreams] = {nullptr};
     cudaEvent_t fork = nullptr, join[pasur::kAuxStreams] = {nullptr}, cls_t0[pasur::kAuxStreams] = {nullptr},
                 cls_t1[pasur::kAuxStreams] = {nullptr};
     int64_t live_trees = 0;      // trees not yet freed (the context outlives them)
     bool cfr_smem_raised = false;  // CFR kernels' dynamic shared-memory limit raised
+    // clusters of n CTAs with a whole SM's shared memory each that fit the device (0: none)
+    int clusters_of[pasur::kMaxClusterCtas + 1] = {0};
     float selfplay_ms = 0.f;     // device time of the last self-play launch
     int64_t selfplay_games = 0;  //   and its number of games
     // a batch's build workers each own a context with its own stream and error word; their
@@ -206,15 +209,14 @@ struct CfrRoot {
     int64_t item0;            // index of its first work item
 };
 
-// A root subtree too large for one block's shared memory, split over a thread-block cluster:
-// CTA 0 holds the top levels 0..ell-1 (and part 0), CTA r holds part r, a set of subtrees of
-// active level-ell nodes.  Parts and top are pseudo-roots (CfrRoot records appended after the real
-// roots) with their own local numbering; each active level-ell node has a ghost slot in its part
-// for its parent's reach.
+// A root subtree too large for one block's shared memory, split over a thread-block cluster: CTA 0
+// holds the top levels 0..ell-1 (and part 0), CTA r holds part r, a set of subtrees of active level-ell
+// nodes.  Parts and top are pseudo-roots (CfrRoot and BlockRoot records appended after the real roots)
+// with their own block indices; each active level-ell node has a ghost slot in its part for its parent's
+// reach.  Their regrets and strategy sums live in device memory with the root's.
 struct ClusterPart {
     int32_t root;             // pseudo-root
-    int32_t pad;
-    int64_t data_base;        // its regrets and strategy sums in R and S
+    int32_t x_begin, x_end;   // its exchange entries, from the root's first
 };
 
 // The block sweep's order of a root's entries (cfr_block.cuh).  Entries of one level: first those
@@ -236,13 +238,14 @@ struct BlockItem {            // a root and a run of its score slots, solved by 
     int64_t cost;             // active nodes * slots, for the schedule
 };
 
-struct ClusterItem {
+struct ClusterItem {          // a root and a run of its score slots, solved by one cluster
     int32_t tree, root;       // launch tree index, real GT root
-    int64_t s0;               // slot (one per cluster item)
+    int32_t s0, ns;           // first slot within the root, slots
     int64_t part0;            // cparts[part0] = top, cparts[part0 + 1 + r] = part r
-    int64_t x0;               // exchange entries cx[x0 .. x0 + nx) (5 ints each)
+    int64_t x0;               // exchange entries cx[x0 .. x0 + nx) (5 ints each), part by part
     int32_t nx, nparts;
-    int32_t ell, smem;        // split level; shared memory of its largest CTA
+    int64_t cost;             // active nodes * slots, for the schedule
+    size_t smem;              // shared memory of its largest CTA
 };
 
 // Per-tree pointers of the CFR kernel (one entry per round tree of a launch).
@@ -281,9 +284,6 @@ struct CfrItem {              // one work item of the CFR kernel: a root and a r
     int64_t cost;             // active nodes * slots, for the schedule
 };
 
-// cluster items are launched in groups by their CTA count: clusters of 2, 4, 8 and 16 CTAs
-constexpr int kCluGroups = 4;
-
 // One item of the level-streaming sweep, resolved once per plan: its state arrays, its active
 // entries (offsets applied), the level starts of its entries, its slot count (a power of two) and
 // the index of its first slot in the per-slot arrays of the sweep.
@@ -296,34 +296,28 @@ struct StreamDesc {
     int64_t slot;
 };
 
-// One launch of the block sweep: items of the same slot count whose shared memory allows the same
-// number of blocks per SM.
-struct BlockGroup {
-    int W = 0, threads = 0;
+// One launch of the block sweep (ctas = 1: items of the same slot count whose shared memory allows the
+// same number of blocks per SM) or of the cluster sweep (items of the same slot count and parts).
+struct SweepLaunch {
+    int ctas = 1, W = 0, threads = 0;
     int64_t begin = 0, end = 0;
     size_t smem = 0;
     float ms = 0.f;
 };
 
-// A CFR launch plan: work items of one or more trees merged per shared-memory class.
+// A CFR launch plan: work items of one or more trees merged per launch.
 struct CfrPlan {
     std::vector<BlockItem> blk_h;       // by launch group, then cost (largest first)
     BlockItem *blk_d = nullptr;
-    std::vector<BlockGroup> groups;
+    std::vector<ClusterItem> clu_h;     // by launch, then cost
+    ClusterItem *clu_d = nullptr;
+    std::vector<SweepLaunch> launches;  // clusters first, then blocks
     std::vector<CfrItem> items_h;       // ordered by class, then cost (largest first)
     CfrItem *items_d = nullptr;
     TreeView *views_d = nullptr;
     int64_t n_items = 0;
     int64_t cls_begin[8] = {0}, cls_end[8] = {0};
-    float str_ms = 0.f, clu_ms[4] = {0};
-    // cluster items (class 6 holds their pseudo-items, used for exports only), sorted by part
-    // count into up to four launches of 2, 4, 8 and 16 CTAs per cluster
-    std::vector<ClusterItem> clu_h;
-    ClusterItem *clu_d = nullptr;
-    int clu_threads = 0;
-    int64_t clu_begin[kCluGroups] = {0}, clu_end[kCluGroups] = {0};
-    int clu_ctas[kCluGroups] = {2, 4, 8, 16};
-    size_t clu_smem[kCluGroups] = {0};
+    float str_ms = 0.f;
     // items of class 5 (state in device memory) run as a level-streaming sweep over every SM:
     // exclusive prefixes over those items of their (entry, slot) pairs per level [8][n + 1], of
     // their (local node, slot) pairs [n + 1] and of their slots [n + 1]; per slot the largest
@@ -395,7 +389,7 @@ struct pasur_tree {
     uint16_t *act_d = nullptr;          //   number of children
     int64_t *act_gt = nullptr;          //   GT node index
     int64_t *loc_tq = nullptr;          // per local node: FGT index (slot 0) of its chain's leaf, -1 if active
-    int64_t n_local = 0, n_active = 0;
+    int64_t n_local = 0, n_active = 0, n_runs = 0;
     std::vector<BlockRoot> broots_h;    // block sweep (see TreeView)
     BlockRoot *broots_d = nullptr;
     BlockRun *b_run = nullptr;
