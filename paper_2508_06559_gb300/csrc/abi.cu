@@ -197,8 +197,7 @@ int pasur_create(pasur_ctx **out, int device, size_t hbm_budget_bytes, void *cud
         delete ctx;
         return set_err(nullptr, PASUR_ECUDA, m);
     }
-    int rc = dev_alloc(ctx, (void **)&ctx->counter, 64);
-    if (rc == PASUR_OK) rc = dev_alloc(ctx, (void **)&ctx->errflag, 64);
+    int rc = dev_alloc(ctx, (void **)&ctx->errflag, 64);
     if (rc == PASUR_OK && cudaMemsetAsync(ctx->errflag, 0, 64, ctx->stream) != cudaSuccess) rc = PASUR_ECUDA;
     if (rc == PASUR_OK && cudaStreamSynchronize(ctx->stream) != cudaSuccess) rc = PASUR_ECUDA;
     if (rc != PASUR_OK) {
@@ -218,9 +217,6 @@ int pasur_destroy(pasur_ctx *ctx) {
     if (ctx->live_trees > 0)
         return set_err(ctx, PASUR_EINVAL, "pasur_destroy: " + std::to_string(ctx->live_trees) + " tree(s) still alive");
     set_device(ctx);
-    dev_free(ctx, ctx->tab, 0);
-    dev_free(ctx, ctx->tab_off, 0);
-    dev_free(ctx, ctx->counter, 64);
     dev_free(ctx, ctx->errflag, 64);
     cudaStreamSynchronize(ctx->stream);
     for (int c = 0; c < kAuxStreams; c++) {

@@ -131,26 +131,22 @@ int build_deal(pasur_batch *b, pasur_ctx *wc, const uint8_t *deck, int64_t d, De
     return PASUR_OK;
 }
 
-// A build worker's context: its own stream, work counter and error word on the parent's device,
-// the parent's capture table, allocations charged to the parent.
+// A build worker's context: its own stream and error word on the parent's device, allocations charged to
+// the parent.
 int open_worker(pasur_ctx *parent, pasur_ctx *w) {
     w->device = parent->device;
     w->num_sms = parent->num_sms;
     w->smem_optin = parent->smem_optin;
-    w->tab = parent->tab;
-    w->tab_off = parent->tab_off;
     w->acct = parent;
     PASUR_CUDA(w, cudaSetDevice(w->device));
     PASUR_CUDA(w, cudaStreamCreateWithFlags(&w->stream, cudaStreamNonBlocking));
     w->own_stream = true;
-    PASUR_TRY(dev_alloc(w, (void **)&w->counter, 64));
     PASUR_TRY(dev_alloc(w, (void **)&w->errflag, 64));
     PASUR_CUDA(w, cudaMemsetAsync(w->errflag, 0, 64, w->stream));
     return PASUR_OK;
 }
 
 void close_worker(pasur_ctx *w) {
-    dev_free(w, w->counter, 64);
     dev_free(w, w->errflag, 64);
     if (w->stream) cudaStreamSynchronize(w->stream);
     if (w->own_stream) cudaStreamDestroy(w->stream);
@@ -392,8 +388,7 @@ static int batch_create(pasur_ctx *ctx, const uint8_t *decks, int64_t n_deals, i
     clk::time_point tp = clk::now();
     // every deal's rounds and CFR layouts, deals spread over the build workers
     std::vector<DealPlan> dp((size_t)n_deals);
-    rc = ensure_capture_table(ctx);
-    if (rc == PASUR_OK) rc = cudaStreamSynchronize(ctx->stream) == cudaSuccess ? PASUR_OK : set_err(ctx, PASUR_ECUDA, "pasur_batch_create: sync");
+    rc = cudaStreamSynchronize(ctx->stream) == cudaSuccess ? PASUR_OK : set_err(ctx, PASUR_ECUDA, "pasur_batch_create: sync");
     if (rc == PASUR_OK) rc = build_deals(b, decks, dp, &n_workers);
     lap(tp, 0);
     // surrogate values of every deal's roots after the last round

@@ -1,12 +1,14 @@
 // Round game-tree build (legal-move enumeration, level-by-level expansion), the Unfolding
 // Process and the leaf values of a round.
 //
-// Expansion of level k (section "Actions"): one warp per node counts its legal moves (count
-// pass), a device-wide exclusive scan turns the counts into child offsets, and one warp per node
-// writes its children in canonical order (emit pass).  Numeric captures come from a table of
-// every set of numeric cards completing a given numeric card to 11 (the paper's t_40x2764,
-// section "Numerical Actions"), sorted ascending; a warp tests 32 entries per step against the
-// pool with a ballot, and in the emit pass the ballot prefix gives each found move its slot.
+// Expansion of a level (section "Actions"): a device-wide exclusive scan of the nodes' degrees gives
+// the child offsets, one thread per node notes its children's parent, and one thread per child finds
+// its move from its place among its siblings, writes its state and counts its own degree for the next
+// level.  A numeric card captures any set of pool numerics completing its value to 11; the sets are
+// counted by a generating polynomial over the pool's cards (the coefficient of x^s: sets of sum s) and
+// the r-th set in ascending order is found by dividing the cards out of it, highest first.  A thread
+// per child does about 300 instructions; a warp per node that tested the sets of a table (2764 over
+// the 40 cards) with a ballot spent about 230 warp instructions on every node, twice.
 #include <algorithm>
 #include <cstring>
 
@@ -15,60 +17,65 @@
 namespace pasur {
 namespace {
 
-// ---- capture table (host) -------------------------------------------------------------------
-// For the numeric card c (value v = rank+1), every set of other numeric cards whose values add to
-// 11 - v: choose how many cards of each value 1..10 to take (value partitions of 11 - v), then
-// which suits; ascending by mask.
-void partitions(int value, int remaining, const int *avail, int *take, int c_excluded,
-                std::vector<uint64_t> &out) {
-    if (remaining == 0) {
-        // expand suits: cartesian product over values of the suit combinations
-        std::vector<uint64_t> acc(1, 0ULL);
-        for (int v = 1; v <= 10; v++) {
-            if (!take[v]) continue;
-            std::vector<uint64_t> next;
-            for (uint64_t base : acc) {
-                for (int sm = 0; sm < 16; sm++) {
-                    if (__builtin_popcount(sm) != take[v]) continue;
-                    uint64_t m = 0;
-                    bool ok = true;
-                    for (int s = 0; s < 4; s++) {
-                        if (!(sm >> s & 1)) continue;
-                        int id = 4 * (v - 1) + s;
-                        if (id == c_excluded) { ok = false; break; }
-                        m |= 1ULL << id;
-                    }
-                    if (ok) next.push_back(base | m);
-                }
-            }
-            acc.swap(next);
-        }
-        out.insert(out.end(), acc.begin(), acc.end());
-        return;
-    }
-    if (value > 10 || value > remaining) return;
-    for (int k = 0; k <= avail[value] && k * value <= remaining; k++) {
-        take[value] = k;
-        partitions(value + 1, remaining - k * value, avail, take, c_excluded, out);
-    }
-    take[value] = 0;
+// ---- sets of pool numerics by their sum -------------------------------------------------------
+// Coefficients of x^0 .. x^10 in 11 bits each (with all 40 numerics in the pool the largest is 1702);
+// what overflows above them does not reach them (arithmetic modulo a power of two).
+typedef unsigned __int128 Poly;
+constexpr int kSumBits = 11;
+
+__device__ __forceinline__ int sets_of(Poly p, int sum) { return (int)(p >> (kSumBits * sum)) & ((1 << kSumBits) - 1); }
+
+__device__ __forceinline__ Poly pool_sets(uint64_t pool) {
+    Poly p = 1;
+    for (uint64_t x = pool & kNumeric; x; x &= x - 1) p += p << (kSumBits * ((__ffsll((long long)x) - 1) / 4 + 1));
+    return p;
 }
 
-void capture_table(std::vector<uint64_t> &tab, std::vector<int32_t> &off) {
-    tab.clear();
-    off.assign(41, 0);
-    for (int c = 0; c < 40; c++) {
-        off[c] = (int32_t)tab.size();
-        int v = c / 4 + 1;
-        int avail[11], take[11] = {0};
-        for (int x = 0; x <= 10; x++) avail[x] = 4;
-        avail[v] = 3;
-        std::vector<uint64_t> sets;
-        partitions(1, 11 - v, avail, take, c, sets);
-        std::sort(sets.begin(), sets.end());
-        tab.insert(tab.end(), sets.begin(), sets.end());
+// p without a card of value v: p / (1 + x^v) = p (1 - x^v) (1 + x^2v) (1 + x^4v) ... below x^11
+__device__ __forceinline__ Poly without_card(Poly p, int v) {
+    p -= p << (kSumBits * v);
+    for (int s = 2 * kSumBits * v; s < 11 * kSumBits; s *= 2) p += p << s;
+    return p;
+}
+
+// moves of hand card c (numeric: sets = pool_sets(pool))
+__device__ __forceinline__ int card_moves(int c, uint64_t pool, Poly sets) {
+    if (c < 40) return max(sets_of(sets, 10 - c / 4), 1);
+    if (c < 44) return 1;
+    return max(__popcll(pool & (c < 48 ? kQueens : kKings)), 1);
+}
+
+__device__ __forceinline__ int degree_of(uint64_t hand, uint64_t pool) {
+    const Poly sets = pool_sets(pool);
+    int n = 0;
+    for (; hand; hand &= hand - 1) n += card_moves(__ffsll((long long)hand) - 1, pool, sets);
+    return n;
+}
+
+// the picked set of move r of card c, moves in ascending order of their sets
+__device__ __forceinline__ uint64_t picked_set(int c, int r, uint64_t pool, Poly sets) {
+    if (c < 40) {
+        int sum = 10 - c / 4;
+        uint64_t pick = 0, left = pool & kNumeric;
+        if (sets_of(sets, sum) == 0) return 0;
+        while (sum > 0) {
+            // sets without the highest card come first
+            const int b = 63 - __clzll((long long)left), v = b / 4 + 1;
+            left &= ~(1ULL << b);
+            sets = without_card(sets, v);
+            const int w = sets_of(sets, sum);
+            if (r >= w) {
+                r -= w;
+                sum -= v;
+                pick |= 1ULL << b;
+            }
+        }
+        return pick;
     }
-    off[40] = (int32_t)tab.size();
+    if (c < 44) return pool & (kNumeric | kJacks);
+    uint64_t same = pool & (c < 48 ? kQueens : kKings);
+    for (int i = 0; i < r; i++) same &= same - 1;
+    return same & (~same + 1);
 }
 
 // ---- one move (CodeSnippet "ApplyActions" + the running-score update) -----------------------
@@ -91,90 +98,47 @@ __device__ __forceinline__ GTState apply_move(GTState s, int mover, int c, uint6
 
 struct EmitOut {
     GTState *st;
-    int64_t *parent;
     int8_t *lay;
     uint64_t *pick;
     int32_t *root;
 };
 
-__device__ __forceinline__ void emit_child(const EmitOut &o, int64_t pos, const GTState &s, int mover, int c,
-                                           uint64_t pick, bool final_round, int64_t node, int32_t root) {
-    o.st[pos] = apply_move(s, mover, c, pick, final_round);
-    o.parent[pos] = node;
-    o.lay[pos] = (int8_t)c;
-    o.pick[pos] = pick;
-    o.root[pos] = root;
+__global__ void k_degrees(const GTState *__restrict__ st, int64_t m, int mover, int32_t *__restrict__ deg) {
+    for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < m; j += (int64_t)gridDim.x * blockDim.x)
+        deg[j] = degree_of(st[j].hand[mover], st[j].pool);
 }
 
-// first index in [b, e) with tab[i] > x (all lanes compute the same value)
-__device__ __forceinline__ int upper_bound_u64(const uint64_t *tab, int b, int e, uint64_t x) {
-    while (b < e) {
-        int m = (b + e) >> 1;
-        if (tab[m] <= x) b = m + 1;
-        else e = m;
+__global__ void k_parents(const int64_t *__restrict__ child_off, int64_t m, int64_t *__restrict__ parent) {
+    for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < m; j += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t e = child_off[j + 1];
+        for (int64_t c = child_off[j]; c < e; c++) parent[c] = j;
     }
-    return b;
 }
 
-template <bool EMIT>
-__global__ void k_expand(const GTState *__restrict__ st, int64_t m, int mover, bool final_round,
-                         const uint64_t *__restrict__ tab, const int32_t *__restrict__ tab_off,
-                         int32_t *__restrict__ deg_out, const int64_t *__restrict__ child_off,
-                         const int32_t *__restrict__ root_in, EmitOut o) {
-    int lane = threadIdx.x & 31;
-    unsigned lt = (1u << lane) - 1u;
-    int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t node = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; node < m; node += warps) {
-        GTState s = st[node];
-        uint64_t hand = s.hand[mover], pool = s.pool;
-        int64_t out = EMIT ? child_off[node] : 0;
-        int32_t root = EMIT ? root_in[node] : 0;
-        int cnt = 0;
-        while (hand) {
-            int c = __ffsll((long long)hand) - 1;
-            hand &= hand - 1;
-            if (c < 40) {
-                uint64_t pn = pool & kNumeric;
-                int found = 0;
-                if (pn) {
-                    int b = tab_off[c];
-                    int e = upper_bound_u64(tab, b, tab_off[c + 1], pn);
-                    for (int base = b; base < e; base += 32) {
-                        int i = base + lane;
-                        uint64_t P = i < e ? tab[i] : 0;
-                        bool ok = i < e && (P & ~pn) == 0;
-                        unsigned bal = __ballot_sync(0xFFFFFFFFu, ok);
-                        if (EMIT && ok)
-                            emit_child(o, out + cnt + found + __popc(bal & lt), s, mover, c, P, final_round, node, root);
-                        found += __popc(bal);
-                    }
-                }
-                if (found == 0) {
-                    if (EMIT && lane == 0) emit_child(o, out + cnt, s, mover, c, 0ULL, final_round, node, root);
-                    found = 1;
-                }
-                cnt += found;
-            } else if (c < 44) {
-                if (EMIT && lane == 0)
-                    emit_child(o, out + cnt, s, mover, c, pool & (kNumeric | kJacks), final_round, node, root);
-                cnt += 1;
-            } else {
-                uint64_t same = pool & (c < 48 ? kQueens : kKings);
-                int n = __popcll(same);
-                if (n == 0) {
-                    if (EMIT && lane == 0) emit_child(o, out + cnt, s, mover, c, 0ULL, final_round, node, root);
-                    cnt += 1;
-                } else {
-                    if (EMIT && lane < n) {
-                        uint64_t x = same;
-                        for (int i = 0; i < lane; i++) x &= x - 1;
-                        emit_child(o, out + cnt + lane, s, mover, c, x & (~x + 1), final_round, node, root);
-                    }
-                    cnt += n;
-                }
-            }
+// the children of a level: child i is move i - child_off[parent[i]] of its parent, moves ordered by
+// (card, picked set); deg (NULL at the last level): the children's own degrees
+__global__ void __launch_bounds__(256) k_children(const GTState *__restrict__ st, const int32_t *__restrict__ root_in,
+                                                  const int64_t *__restrict__ child_off, const int64_t *__restrict__ parent,
+                                                  int64_t m, int mover, bool final_round, EmitOut o, int32_t *__restrict__ deg) {
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t j = parent[i];
+        int r = (int)(i - child_off[j]);
+        GTState s = st[j];
+        const Poly sets = pool_sets(s.pool);
+        int c = 0;
+        for (uint64_t hand = s.hand[mover]; hand; hand &= hand - 1) {
+            c = __ffsll((long long)hand) - 1;
+            const int n = card_moves(c, s.pool, sets);
+            if (r < n) break;
+            r -= n;
         }
-        if (!EMIT && lane == 0) deg_out[node] = cnt;
+        const uint64_t pick = picked_set(c, r, s.pool, sets);
+        s = apply_move(s, mover, c, pick, final_round);
+        o.st[i] = s;
+        o.lay[i] = (int8_t)c;
+        o.pick[i] = pick;
+        o.root[i] = root_in[j];
+        if (deg) deg[i] = degree_of(s.hand[mover ^ 1], s.pool);
     }
 }
 
@@ -206,11 +170,18 @@ __global__ void k_root_bounds(int64_t n_roots, OffPtrs co, int64_t *__restrict__
     }
 }
 
-__global__ void k_slots_per_node(const int32_t *__restrict__ root, int64_t m, const int64_t *__restrict__ score_off,
-                                 int64_t *__restrict__ out) {
-    for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < m; j += (int64_t)gridDim.x * blockDim.x) {
-        int32_t g = root[j];
-        out[j] = score_off[g + 1] - score_off[g];
+// first FGT node of every GT node of one level: a root's nodes are consecutive, each with the root's
+// slots (base[g]: the root's first, bounds[9 g + k]: its first GT node); out[m] = total
+__global__ void k_slot_offsets(const int32_t *__restrict__ root, int64_t m, int k, const int64_t *__restrict__ bounds,
+                               const int64_t *__restrict__ base, const int64_t *__restrict__ slot_off, int64_t n_roots,
+                               int64_t *__restrict__ out) {
+    for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j <= m; j += (int64_t)gridDim.x * blockDim.x) {
+        if (j == m) {
+            out[j] = base[n_roots];
+            continue;
+        }
+        const int32_t g = root[j];
+        out[j] = base[g] + (j - bounds[9 * g + k]) * (slot_off[g + 1] - slot_off[g]);
     }
 }
 
@@ -291,22 +262,8 @@ unsigned grid_for(int64_t threads, int block) {
 
 }  // namespace
 
-int ensure_capture_table(pasur_ctx *ctx) {
-    if (ctx->tab) return PASUR_OK;
-    std::vector<uint64_t> tab;
-    std::vector<int32_t> off;
-    capture_table(tab, off);
-    PASUR_TRY(dev_alloc(ctx, (void **)&ctx->tab, tab.size() * sizeof(uint64_t)));
-    PASUR_TRY(dev_alloc(ctx, (void **)&ctx->tab_off, off.size() * sizeof(int32_t)));
-    PASUR_CUDA(ctx, cudaMemcpyAsync(ctx->tab, tab.data(), tab.size() * sizeof(uint64_t), cudaMemcpyHostToDevice, ctx->stream));
-    PASUR_CUDA(ctx, cudaMemcpyAsync(ctx->tab_off, off.data(), off.size() * sizeof(int32_t), cudaMemcpyHostToDevice, ctx->stream));
-    PASUR_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
-    return PASUR_OK;
-}
-
 int build_levels(pasur_tree *t, const uint64_t *root_pools_dev) {
     pasur_ctx *ctx = t->ctx;
-    PASUR_TRY(ensure_capture_table(ctx));
     int64_t m0 = t->n_roots;
     t->M[0] = m0;
     PASUR_TRY(tree_alloc(t, (void **)&t->st[0], sizeof(GTState) * (size_t)(m0 + 1)));
@@ -316,23 +273,25 @@ int build_levels(pasur_tree *t, const uint64_t *root_pools_dev) {
         ctx->launches++;
         PASUR_CUDA(ctx, cudaGetLastError());
     }
+    // degrees of the level being expanded: counted where its nodes are written
+    int32_t *deg = nullptr;
+    size_t degb = sizeof(int32_t) * (size_t)(m0 + 1);
+    PASUR_TRY(dev_alloc(ctx, (void **)&deg, degb));
+    struct Deg {
+        pasur_ctx *c;
+        int32_t **p;
+        size_t *b;
+        ~Deg() { dev_free(c, *p, *b); }
+    } guard{ctx, &deg, &degb};
+    if (m0 > 0) {
+        k_degrees<<<grid_for(m0, 256), 256, 0, ctx->stream>>>(t->st[0], m0, 0, deg);
+        ctx->launches++;
+        PASUR_CUDA(ctx, cudaGetLastError());
+    }
     for (int k = 0; k < 8; k++) {
         int64_t m = t->M[k];
-        int mover = k & 1;
-        int32_t *deg = nullptr;
-        size_t degb = sizeof(int32_t) * (size_t)(m + 1);
-        PASUR_TRY(dev_alloc(ctx, (void **)&deg, degb));
         PASUR_TRY(tree_alloc(t, (void **)&t->child_off[k], sizeof(int64_t) * (size_t)(m + 1)));
-        EmitOut none{};
-        if (m > 0) {
-            k_expand<false><<<grid_for(m * 32, 256), 256, 0, ctx->stream>>>(t->st[k], m, mover, t->final_round, ctx->tab,
-                                                                          ctx->tab_off, deg, nullptr, nullptr, none);
-            ctx->launches++;
-            PASUR_CUDA(ctx, cudaGetLastError());
-        }
-        int rc = exclusive_scan_i32(ctx, deg, t->child_off[k], m);
-        dev_free(ctx, deg, degb);
-        if (rc != PASUR_OK) return rc;
+        PASUR_TRY(exclusive_scan_i32(ctx, deg, t->child_off[k], m));
         int64_t m1 = 0;
         PASUR_TRY(read_i64(ctx, t->child_off[k] + m, &m1));
         t->M[k + 1] = m1;
@@ -348,10 +307,19 @@ int build_levels(pasur_tree *t, const uint64_t *root_pools_dev) {
         t->lay[k + 1] = (int8_t *)(lv + b_st + b_par);
         t->pick[k + 1] = (uint64_t *)(lv + b_st + b_par + b_lay);
         t->root[k + 1] = (int32_t *)(lv + b_st + b_par + b_lay + b_pick);
+        dev_free(ctx, deg, degb);
+        deg = nullptr;
+        if (k < 7) {
+            degb = sizeof(int32_t) * cap;
+            PASUR_TRY(dev_alloc(ctx, (void **)&deg, degb));
+        }
         if (m > 0) {
-            EmitOut o{t->st[k + 1], t->parent[k + 1], t->lay[k + 1], t->pick[k + 1], t->root[k + 1]};
-            k_expand<true><<<grid_for(m * 32, 256), 256, 0, ctx->stream>>>(t->st[k], m, mover, t->final_round, ctx->tab,
-                                                                         ctx->tab_off, nullptr, t->child_off[k], t->root[k], o);
+            EmitOut o{t->st[k + 1], t->lay[k + 1], t->pick[k + 1], t->root[k + 1]};
+            k_parents<<<grid_for(m, 256), 256, 0, ctx->stream>>>(t->child_off[k], m, t->parent[k + 1]);
+            ctx->launches++;
+            PASUR_CUDA(ctx, cudaGetLastError());
+            k_children<<<grid_for(m1, 256), 256, 0, ctx->stream>>>(t->st[k], t->root[k], t->child_off[k], t->parent[k + 1], m1,
+                                                                  k & 1, t->final_round, o, deg);
             ctx->launches++;
             PASUR_CUDA(ctx, cudaGetLastError());
         }
@@ -391,29 +359,42 @@ int build_levels(pasur_tree *t, const uint64_t *root_pools_dev) {
     return PASUR_OK;
 }
 
-int unfold_levels(pasur_tree *t) {
+// The FGT levels over given slots per root (slot_off: prefix over the roots, host and device): sizes
+// from the roots' node counts on the host, then every level's offsets in one launch each, without a
+// scan or a synchronisation.
+static int slot_levels(pasur_tree *t, const std::vector<int64_t> &slot_off, const int64_t *slot_off_d, int64_t **off, int64_t *sizes) {
     pasur_ctx *ctx = t->ctx;
-    int64_t mmax = 0;
-    for (int k = 0; k < 9; k++) mmax = std::max(mmax, t->M[k]);
-    // one slot-count buffer serves every level (the levels run in stream order)
-    int64_t *slots = nullptr;
-    const size_t sb = sizeof(int64_t) * (size_t)(mmax + 1);
-    PASUR_TRY(dev_alloc(ctx, (void **)&slots, sb));
-    int rc = PASUR_OK;
-    for (int k = 0; k < 9 && rc == PASUR_OK; k++) {
-        int64_t m = t->M[k];
-        if (!t->fgt_off[k]) rc = tree_alloc(t, (void **)&t->fgt_off[k], sizeof(int64_t) * (size_t)(m + 1));
-        if (rc == PASUR_OK && m > 0) {
-            k_slots_per_node<<<grid_for(m, 256), 256, 0, ctx->stream>>>(t->root[k], m, t->score_off_d, slots);
-            ctx->launches++;
-            if (cudaGetLastError() != cudaSuccess) rc = set_err(ctx, PASUR_ECUDA, "k_slots_per_node launch");
+    const int64_t nr = t->n_roots;
+    std::vector<int64_t> base((size_t)(9 * (nr + 1)));
+    for (int k = 0; k < 9; k++) {
+        int64_t *b = base.data() + (size_t)k * (size_t)(nr + 1), q = 0;
+        for (int64_t g = 0; g < nr; g++) {
+            b[g] = q;
+            q += t->roots_h[(size_t)g].lvl_count[k] * (slot_off[(size_t)g + 1] - slot_off[(size_t)g]);
         }
-        if (rc == PASUR_OK) rc = exclusive_scan_i64(ctx, slots, t->fgt_off[k], m);
-        if (rc == PASUR_OK) rc = read_i64(ctx, t->fgt_off[k] + m, &t->Q[k]);
+        b[nr] = sizes[k] = q;
     }
-    dev_free(ctx, slots, sb);
+    int64_t *base_d = nullptr;
+    const size_t bytes = sizeof(int64_t) * base.size();
+    PASUR_TRY(dev_alloc(ctx, (void **)&base_d, bytes));
+    int rc = PASUR_OK;
+    cudaError_t e = cudaMemcpyAsync(base_d, base.data(), bytes, cudaMemcpyHostToDevice, ctx->stream);
+    if (e != cudaSuccess) rc = cuda_err(ctx, e, "slot_levels: upload");
+    for (int k = 0; k < 9 && rc == PASUR_OK; k++) {
+        const int64_t m = t->M[k];
+        if (!off[k]) rc = tree_alloc(t, (void **)&off[k], sizeof(int64_t) * (size_t)(m + 1));
+        if (rc != PASUR_OK) break;
+        k_slot_offsets<<<grid_for(m + 1, 256), 256, 0, ctx->stream>>>(t->root[k], m, k, t->bounds_d, base_d + (size_t)k * (size_t)(nr + 1),
+                                                                     slot_off_d, nr, off[k]);
+        ctx->launches++;
+        e = cudaGetLastError();
+        if (e != cudaSuccess) rc = cuda_err(ctx, e, "k_slot_offsets");
+    }
+    dev_free(ctx, base_d, bytes);
     return rc;
 }
+
+int unfold_levels(pasur_tree *t) { return slot_levels(t, t->score_off_h, t->score_off_d, t->fgt_off, t->Q); }
 
 // leaf values without any host synchronisation (the batch solver captures this in a CUDA graph);
 // umax_bits (device, may be NULL) receives max |value| as float bits
@@ -543,25 +524,8 @@ int plan_solve_slots(pasur_tree *t, bool merge, const float *next_util_dev) {
             t->cQ[k] = t->Q[k];
         }
     } else {
-        int64_t mmax = 0;
-        for (int k = 0; k < 9; k++) mmax = std::max(mmax, t->M[k]);
-        int64_t *slots = nullptr;
-        const size_t sb = sizeof(int64_t) * (size_t)(mmax + 1);
-        PASUR_TRY(dev_alloc(ctx, (void **)&slots, sb));
-        int rc = PASUR_OK;
-        for (int k = 0; k < 9 && rc == PASUR_OK; k++) {
-            const int64_t m = t->M[k];
-            rc = tree_alloc(t, (void **)&t->cfgt_off[k], sizeof(int64_t) * (size_t)(m + 1));
-            if (rc == PASUR_OK && m > 0) {
-                k_slots_per_node<<<grid_for(m, 256), 256, 0, ctx->stream>>>(t->root[k], m, t->csoff_d, slots);
-                ctx->launches++;
-                if (cudaGetLastError() != cudaSuccess) rc = set_err(ctx, PASUR_ECUDA, "k_slots_per_node launch");
-            }
-            if (rc == PASUR_OK) rc = exclusive_scan_i64(ctx, slots, t->cfgt_off[k], m);
-            if (rc == PASUR_OK) rc = read_i64(ctx, t->cfgt_off[k] + m, &t->cQ[k]);
-        }
-        dev_free(ctx, slots, sb);
-        if (rc != PASUR_OK) return rc;
+        for (int k = 0; k < 9; k++) t->cfgt_off[k] = nullptr;
+        PASUR_TRY(slot_levels(t, t->csoff_h, t->csoff_d, t->cfgt_off, t->cQ));
     }
     return PASUR_OK;
 }

@@ -137,11 +137,6 @@ struct pasur_ctx {
     int num_sms = 0;
     size_t smem_optin = 0;
     std::string err;
-    // capture table of numeric moves: per numeric card c, the picked sets completing it to 11,
-    // ascending; tab_off[41]
-    uint64_t *tab = nullptr;
-    int32_t *tab_off = nullptr;
-    int32_t *counter = nullptr;  // work-queue counters (device)
     int32_t *errflag = nullptr;  // device error word
     int64_t launches = 0;        // kernels launched through this context
     // forked streams for concurrent launches (created on first use): the level-streaming sweep 0, the
@@ -454,7 +449,6 @@ int radix_sort_pairs(pasur_ctx *ctx, uint64_t *keys, int64_t *vals, int64_t n, i
 int read_i64(pasur_ctx *ctx, const int64_t *dptr, int64_t *out);
 
 // build.cu
-int ensure_capture_table(pasur_ctx *ctx);
 int build_levels(pasur_tree *t, const uint64_t *root_pools_dev);
 int unfold_levels(pasur_tree *t);
 int compute_leaf_values(pasur_tree *t, const float *next_util_dev);
