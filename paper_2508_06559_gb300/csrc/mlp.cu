@@ -7,10 +7,10 @@
 // Every dense contraction runs on the 5th-generation tensor cores: k_gemm computes
 // C[M x 256] = A[M x K] . B[256 x K]^T with bf16 operands staged into shared memory by bulk async
 // copies (cp.async.bulk, completion on an mbarrier), tcgen05.mma issued by one thread with the
-// f32 accumulator (128 lanes x 256 columns) in tensor memory, and a fused epilogue that reads the
-// accumulator back with tcgen05.ld: bias + GELU for the forward layers, the output layer, loss and
-// its gradient for the last hidden layer, GELU' for the input gradients, atomics for the weight
-// gradients.  Operands live in HBM in the tensor cores' canonical K-major layout without swizzle
+// f32 accumulator in tensor memory, and a fused epilogue that reads the accumulator back with
+// tcgen05.ld: bias + GELU for the forward layers, the output layer, loss and its gradient for the
+// last hidden layer, GELU' for the input gradients, atomics for the weight gradients; k_infer runs
+// all layers of a row tile for the predictions.  Operands live in HBM in the tensor cores' canonical K-major layout without swizzle
 // (8x8 core matrices of 128 contiguous bytes), ordered so that one (128-row, 64-column) tile is
 // one contiguous 16 KB block: element (r, k) of an R-row matrix is at
 //   ((k/64) * (R/8) + r/8) * 512 + ((k%64)/8) * 64 + (r%8) * 8 + (k%8)      (bf16 units).
@@ -28,13 +28,13 @@ namespace pasur {
 namespace {
 
 constexpr int kHid = 256;           // hidden width = input width = GEMM N
-constexpr int kStages = 2;          // operand pipeline depth
-constexpr uint32_t kAStage = 128 * 64 * 2, kBStage = 256 * 64 * 2;
-constexpr size_t kGemmSmem = kStages * (kAStage + kBStage) + 1024 + 128;
+constexpr uint32_t kAStage = 128 * 64 * 2;
 constexpr int kParams = 3 * kHid * kHid + 3 * kHid + kHid + 1;
 constexpr int64_t kTimeoutNs = 1000000000LL;  // bounded waits: one second
 
-enum { EPI_FWD = 0, EPI_FWD_INFER = 1, EPI_LAST_TRAIN = 2, EPI_LAST_INFER = 3, EPI_DA = 4, EPI_DW = 5 };
+enum { EPI_FWD = 0, EPI_LAST = 1, EPI_DA = 2, EPI_DW = 3 };
+// operand pipeline depth (4: all of K = 256)
+__host__ __device__ constexpr int stages_of(int epi) { return epi == EPI_DW ? 3 : 4; }
 
 __host__ __device__ __forceinline__ int64_t tiled(int64_t r, int64_t k, int64_t R) {
     return ((k >> 6) * (R >> 3) + (r >> 3)) * 512 + ((k >> 3) & 7) * 64 + (r & 7) * 8 + (k & 7);
@@ -82,6 +82,18 @@ __device__ __forceinline__ void bulk_load(void *dst, const void *src, uint32_t b
                  : "memory");
 }
 
+// programmatic launches: the next kernel of the stream may start its set-up; wait for the one before
+__device__ __forceinline__ void pdl_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
+__device__ __forceinline__ void store_remote(uint32_t addr, uint32_t rank, float v) {
+    uint32_t a;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(addr), "r"(rank));
+    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory");
+}
+
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
@@ -92,14 +104,16 @@ __device__ __forceinline__ uint64_t sdesc(uint32_t saddr, uint32_t lbo, uint32_t
            ((uint64_t)((sbo >> 4) & 0x3FFF) << 32) | (1ULL << 46);
 }
 
-// instruction descriptor of kind::f16: f32 accumulator, bf16 A and B, both K-major, M = 128,
-// N = 256
-constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kHid >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
+// instruction descriptor of kind::f16: f32 accumulator, bf16 A and B, both K-major, M = 128
+__host__ __device__ constexpr uint32_t idesc(int n) {
+    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
+}
 
+template <int N>
 __device__ __forceinline__ void mma_bf16(uint32_t d, uint64_t a, uint64_t b, uint32_t accumulate) {
     asm volatile(
         "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
-        "l"(a), "l"(b), "r"(kIdesc), "r"(accumulate)
+        "l"(a), "l"(b), "n"(idesc(N)), "r"(accumulate)
         : "memory");
 }
 
@@ -134,47 +148,115 @@ __device__ __forceinline__ float warp_sum(float v) {
     return v;
 }
 
-// 8 bf16 of row r, columns c..c+7 (c % 8 == 0) into a tiled matrix of R rows
-__device__ __forceinline__ void store8_tiled(__nv_bfloat16 *M, int64_t r, int64_t c, int64_t R, const float *v) {
-    __align__(16) __nv_bfloat16 b[8];
+// sums over the warp's 32 lanes of 32 values each; lane l gets value l's (31 shuffles instead of 160)
+__device__ __forceinline__ float column_sums(float *v) {
+    const int lane = threadIdx.x & 31;
 #pragma unroll
-    for (int i = 0; i < 8; i++) b[i] = __float2bfloat16_rn(v[i]);
-    *reinterpret_cast<uint4 *>(M + tiled(r, c, R)) = *reinterpret_cast<const uint4 *>(b);
+    for (int h = 16; h > 0; h >>= 1) {
+        const bool up = lane & h;
+#pragma unroll
+        for (int i = 0; i < h; i++) {
+            const float mine = up ? v[i + h] : v[i], other = up ? v[i] : v[i + h];
+            v[i] = mine + __shfl_xor_sync(0xffffffffu, other, h);
+        }
+    }
+    return v[0];
 }
 
+__device__ __forceinline__ uint32_t pack2(float a, float b) {
+    const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
+    return *reinterpret_cast<const uint32_t *>(&h);
+}
+
+// 8 bf16 of row r, columns c..c+7 (c % 8 == 0) into a tiled matrix of R rows
+__device__ __forceinline__ void store8_tiled(__nv_bfloat16 *M, int64_t r, int64_t c, int64_t R, const float *v) {
+    *reinterpret_cast<uint4 *>(M + tiled(r, c, R)) =
+        make_uint4(pack2(v[0], v[1]), pack2(v[2], v[3]), pack2(v[4], v[5]), pack2(v[6], v[7]));
+}
+
+// 32 columns c..c+31 of the warp's rows row0..row0+31 (lane = row) into the tiled transpose [256 x rows]:
+// through the warp's stage in shared memory, so that a lane writes 8 rows of a column at once
+constexpr int kStageRow = 40;  // bf16 per staged column (32 rows and 16 bytes: no bank conflicts, aligned)
+__device__ __forceinline__ void store_transposed(__nv_bfloat16 *MT, __nv_bfloat16 *stage, int64_t row0, int c, const float *v) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int i = 0; i < 32; i++) stage[i * kStageRow + lane] = __float2bfloat16_rn(v[i]);
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < 4; i++) {
+        const int x = lane + 32 * i, col = x >> 2, r = (x & 3) * 8;
+        *reinterpret_cast<uint4 *>(MT + tiled(c + col, row0 + r, kHid)) = *reinterpret_cast<const uint4 *>(stage + col * kStageRow + r);
+    }
+    __syncwarp();
+}
+
+// place of the pre-activation (row, column): the 32 rows of a warp consecutive
+__device__ __forceinline__ int64_t z_at(int64_t row, int c) { return ((row >> 5) * kHid + c) * 32 + (row & 31); }
+
+// The gradients in parts, summed by grad_at in a fixed order, so that a training run repeats bit for bit: weight
+// gradients per split of the batch, column sums (the biases' and the output weights' gradients) per row tile.
+// The weight gradients take 8 us per 1024 rows; with atomic adds into one gradient vector, a layer to a launch, three
+// times 22, and every run gave other bits.
+struct Partials {
+    float *dW;       // [splits][3][256 x 256]
+    float *cols;     // [tiles][4][256]: db0, db1, db2, dw3
+    float *scalars;  // [tiles][2]: db3, loss
+    int splits, tiles;
+};
+
 struct GemmArgs {
-    const __nv_bfloat16 *A;    // tiled, a_rows rows, K columns
-    const __nv_bfloat16 *B;    // tiled, 256 rows, K columns
+    const __nv_bfloat16 *A[3]; // tiled, a_rows rows, K columns (EPI_DW: one per layer)
+    const __nv_bfloat16 *B[3]; // tiled, 256 rows, K columns
     int64_t a_rows, K;
     int64_t kcs;               // K chunks (of 64) per split
     const float *bias;         // forward: [256]
-    float *z_out;              // EPI_FWD: pre-activation, f32 row-major [M x 256]
+    float *z_out;              // EPI_FWD: pre-activation (z_at)
     __nv_bfloat16 *h_out;      // tiled [M x 256] (activation or pre-activation gradient)
     __nv_bfloat16 *ht_out;     // tiled [256 x M] (its transpose)
-    const float *z_in;         // EPI_DA: pre-activation of the layer below, f32 row-major
-    float *db;                 // column sums of the pre-activation gradient (atomics)
-    float *dW;                 // EPI_DW: f32 row-major [256 x 256] (atomics)
+    const float *z_in;         // EPI_DA: pre-activation of the layer below (z_at)
+    float *cols;               // partial sums of the row tile (Partials)
+    int col;                   // which of its four
+    float *scalars;            // EPI_LAST: the row tile's db3 and loss
+    float *dW;                 // EPI_DW: partial weight gradients (Partials)
     const float *w3, *b3, *y;  // output layer and targets
-    float *yhat, *loss, *dw3, *db3;
     int64_t n_valid;
     float inv_n;
     int32_t *err;
 };
 
-template <int EPI>
-__global__ void __launch_bounds__(128, 1) k_gemm(const GemmArgs g) {
+// shared memory of k_gemm: operand stages, a stage per warp for the transposes, barriers
+constexpr size_t gemm_smem(int epi, int nc, int warps) {
+    return stages_of(epi) * (kAStage + (uint32_t)nc * 128) + (epi == EPI_DW ? 0 : (size_t)warps * 32 * kStageRow * 2 + 8 * nc * sizeof(float)) + 1024 + 256;
+}
+
+// One 128 x NC tile of C[M x 256] = A[M x K] . B[256 x K]^T per block, 128 * CG threads: warp w reads the
+// accumulator's rows 32 (w % 4) .. and its (w / 4)-th of CG column parts.  The batch is small (1024 rows: 8
+// row tiles), so the columns are shared out over blocks; the output layer, which needs whole rows, over the
+// blocks of a cluster.  Bound by latency: a 1024-row batch is eight dependent launches of 5 to 11 us, overlapped
+// by programmatic launches.  40 such steps took 15.2 ms with 128 x 256 tiles on 128 threads (per launch: output
+// layer 65 us, input gradients 71, the others 22, Adam 83) and take 2.4 ms.
+template <int EPI, int NC, int CG>
+__global__ void __launch_bounds__(128 * CG, EPI == EPI_DW ? 3 : 1) k_gemm(const GemmArgs g) {
     extern __shared__ uint8_t smem_raw[];
+    constexpr uint32_t kBStage = NC * 128;
+    constexpr int kStages = stages_of(EPI);
+    constexpr int PC = NC / CG;  // columns of a warp
     uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     uint8_t *sA = smem, *sB = smem + kStages * kAStage;
-    uint64_t *full = (uint64_t *)(sB + kStages * kBStage);
+    __nv_bfloat16 *stages = (__nv_bfloat16 *)(sB + kStages * kBStage);
+    float *sums = (float *)(stages + (EPI == EPI_DW ? 0 : 4 * CG * 32 * kStageRow));  // [2][4][NC]: column sums of the row quarters
+    uint64_t *full = (uint64_t *)(sums + (EPI == EPI_DW ? 0 : 8 * NC));
     uint64_t *freed = full + kStages;
     uint64_t *accd = freed + kStages;
     uint32_t *tslot = (uint32_t *)(accd + 1);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int layer = EPI == EPI_DW ? (int)blockIdx.z / (kHid / NC) : 0;
+    const int n0 = (EPI == EPI_DW ? (int)blockIdx.z % (kHid / NC) : (int)blockIdx.z) * NC;
     const int64_t nk = g.K >> 6;
     const int64_t c0 = (int64_t)blockIdx.y * g.kcs, c1 = min(nk, c0 + g.kcs);
     const int64_t m0 = (int64_t)blockIdx.x * 128;
-    if (c1 <= c0) return;  // uniform per block: nothing to accumulate
+    pdl_next();
+    if constexpr (EPI == EPI_LAST) cluster_arrive();
     if (threadIdx.x == 0) {
         for (int s = 0; s < kStages; s++) {
             mbar_init(&full[s], 1);
@@ -184,15 +266,17 @@ __global__ void __launch_bounds__(128, 1) k_gemm(const GemmArgs g) {
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(tslot)), "r"(256) : "memory");
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(tslot)), "r"(NC) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tslot;
+    pdl_wait();
 
     if (threadIdx.x == 0) {
+        const __nv_bfloat16 *A = g.A[layer], *B = g.B[layer];
         const int64_t n = c1 - c0;
         int64_t issued = 0, landed = 0;
         bool ok = true;
@@ -200,8 +284,8 @@ __global__ void __launch_bounds__(128, 1) k_gemm(const GemmArgs g) {
             const int s = (int)(i % kStages);
             const int64_t kc = c0 + i;
             mbar_expect_tx(&full[s], kAStage + kBStage);
-            bulk_load(sA + s * kAStage, g.A + (kc * (g.a_rows >> 3) + (m0 >> 3)) * 512, kAStage, &full[s]);
-            bulk_load(sB + s * kBStage, g.B + kc * (kHid / 8) * 512, kBStage, &full[s]);
+            bulk_load(sA + s * kAStage, A + (kc * (g.a_rows >> 3) + (m0 >> 3)) * 512, kAStage, &full[s]);
+            bulk_load(sB + s * kBStage, B + (kc * (kHid / 8) + n0 / 8) * 512, kBStage, &full[s]);
             issued++;
         };
         for (int64_t i = 0; i < n && i < kStages; i++) load(i);
@@ -214,7 +298,7 @@ __global__ void __launch_bounds__(128, 1) k_gemm(const GemmArgs g) {
             const uint32_t a0 = su32(sA + s * kAStage), b0 = su32(sB + s * kBStage);
 #pragma unroll
             for (int kk = 0; kk < 4; kk++)
-                mma_bf16(tmem, sdesc(a0 + kk * 256, 128, 1024), sdesc(b0 + kk * 256, 128, 1024), (i > 0 || kk > 0) ? 1u : 0u);
+                mma_bf16<NC>(tmem, sdesc(a0 + kk * 256, 128, 1024), sdesc(b0 + kk * 256, 128, 1024), (i > 0 || kk > 0) ? 1u : 0u);
             mma_commit(&freed[s]);
             if (i + kStages < n) {
                 if (!mbar_wait(&freed[s], ph)) { ok = false; break; }
@@ -229,152 +313,354 @@ __global__ void __launch_bounds__(128, 1) k_gemm(const GemmArgs g) {
         }
     }
     __syncwarp();
-    const bool acc_ok = mbar_wait(accd, 0);
+    const bool acc_ok = __syncthreads_and(mbar_wait(accd, 0));
     tc_fence_after();
-    if (!acc_ok) {
-        if (lane == 0) atomicExch(g.err, 2);
-    } else {
-        const int64_t row = m0 + warp * 32 + lane;
-        const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16);
-        float v[32];
-        if (EPI == EPI_DW) {
+    if (!acc_ok && threadIdx.x == 0) atomicExch(g.err, 2);
+    const int64_t row0 = m0 + (warp & 3) * 32, row = row0 + lane;
+    const int p0 = (warp >> 2) * PC;  // the warp's columns of the block: p0 .. p0 + PC
+    const uint32_t taddr = tmem + ((uint32_t)((warp & 3) * 32) << 16) + p0;
+    __nv_bfloat16 *stage = stages + warp * 32 * kStageRow;
+    float v[32];
+    if constexpr (EPI == EPI_LAST) {
+        // output layer y = h3 . w3 + b3 with h3 = gelu(acc + b2), in f32 per row, and its gradients
+        // (the blocks of a row tile are a cluster: each computes its columns' share and gives it to the others)
+        constexpr int kShares = kHid / PC;
+        float *part = reinterpret_cast<float *>(stages);  // [kShares][128]
+        static_assert(kShares * 128 * sizeof(float) <= 4 * CG * 32 * kStageRow * 2, "shares");
+        float yh = 0.f;
 #pragma unroll 1
-            for (int j = 0; j < kHid / 32; j++) {
-                tmem_ld32(taddr + j * 32, v);
-                float *dst = g.dW + row * kHid + j * 32;
+        for (int j = 0; j < PC; j += 32) {
+            if (acc_ok) tmem_ld32(taddr + j, v);
 #pragma unroll
-                for (int i = 0; i < 32; i++) atomicAdd(dst + i, v[i]);
-            }
-        } else if (EPI == EPI_FWD || EPI == EPI_FWD_INFER) {
+            for (int i = 0; i < 32; i++) yh += gelu(v[i] + g.bias[n0 + p0 + j + i]) * g.w3[n0 + p0 + j + i];
+        }
+        cluster_wait();  // every block of the cluster has started
+        const uint32_t at = su32(part + ((int)blockIdx.z * CG + (warp >> 2)) * 128 + (warp & 3) * 32 + lane);
+#pragma unroll
+        for (int q = 0; q < kHid / NC; q++) store_remote(at, q, yh);
+        cluster_arrive();
+        cluster_wait();
+        yh = g.b3[0];
+#pragma unroll
+        for (int q = 0; q < kShares; q++) yh += part[q * 128 + (warp & 3) * 32 + lane];
+        __syncthreads();
+        const bool valid = row < g.n_valid;
+        const float err = valid ? yh - g.y[row] : 0.f;
+        const float gy = 2.f * err * g.inv_n;  // d loss / d yhat
+        float *quarters = reinterpret_cast<float *>(tslot + 2);  // [4][2]
+        if (warp < 4) {
+            const float l = warp_sum(err * err * g.inv_n), sg = warp_sum(gy);
+            if (lane == 0) quarters[2 * warp] = sg, quarters[2 * warp + 1] = l;
+        }
+        if (acc_ok) {
 #pragma unroll 1
-            for (int j = 0; j < kHid / 32; j++) {
-                tmem_ld32(taddr + j * 32, v);
-                const int c = j * 32;
-#pragma unroll
-                for (int i = 0; i < 32; i++) v[i] += g.bias[c + i];
-                if (EPI == EPI_FWD) {
-                    float4 *zo = reinterpret_cast<float4 *>(g.z_out + row * kHid + c);
-#pragma unroll
-                    for (int i = 0; i < 8; i++) zo[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
-                }
-#pragma unroll
-                for (int i = 0; i < 32; i++) v[i] = gelu(v[i]);
-#pragma unroll
-                for (int q = 0; q < 4; q++) store8_tiled(g.h_out, row, c + 8 * q, g.a_rows, v + 8 * q);
-                if (EPI == EPI_FWD) {
-#pragma unroll
-                    for (int i = 0; i < 32; i++) g.ht_out[tiled(c + i, row, kHid)] = __float2bfloat16_rn(v[i]);
-                }
-            }
-        } else if (EPI == EPI_LAST_TRAIN || EPI == EPI_LAST_INFER) {
-            // output layer y = h3 . w3 + b3 with h3 = gelu(acc + b2), in f32 per row
-            float yh = g.b3[0];
-#pragma unroll 1
-            for (int j = 0; j < kHid / 32; j++) {
-                tmem_ld32(taddr + j * 32, v);
-#pragma unroll
-                for (int i = 0; i < 32; i++) yh += gelu(v[i] + g.bias[j * 32 + i]) * g.w3[j * 32 + i];
-            }
-            const bool valid = row < g.n_valid;
-            if (valid) g.yhat[row] = yh;
-            if (EPI == EPI_LAST_TRAIN) {
-                const float err = valid ? yh - g.y[row] : 0.f;
-                const float gy = 2.f * err * g.inv_n;  // d loss / d yhat
-                const float l = warp_sum(err * err * g.inv_n), sg = warp_sum(gy);
-                if (lane == 0) {
-                    atomicAdd(g.loss, l);
-                    atomicAdd(g.db3, sg);
-                }
-#pragma unroll 1
-                for (int j = 0; j < kHid / 32; j++) {
-                    tmem_ld32(taddr + j * 32, v);
-                    const int c = j * 32;
-#pragma unroll
-                    for (int i = 0; i < 32; i++) {
-                        const float z = v[i] + g.bias[c + i];
-                        const float s3 = warp_sum(gy * gelu(z));
-                        const float dz = gy * g.w3[c + i] * gelu_grad(z);
-                        const float s2 = warp_sum(dz);
-                        if (lane == 0) {
-                            atomicAdd(g.dw3 + c + i, s3);
-                            atomicAdd(g.db + c + i, s2);
-                        }
-                        v[i] = dz;
-                    }
-#pragma unroll
-                    for (int q = 0; q < 4; q++) store8_tiled(g.h_out, row, c + 8 * q, g.a_rows, v + 8 * q);
-#pragma unroll
-                    for (int i = 0; i < 32; i++) g.ht_out[tiled(c + i, row, kHid)] = __float2bfloat16_rn(v[i]);
-                }
-            }
-        } else if (EPI == EPI_DA) {
-            // accumulator = gradient of the layer input; times gelu' of the layer below
-#pragma unroll 1
-            for (int j = 0; j < kHid / 32; j++) {
-                tmem_ld32(taddr + j * 32, v);
-                const int c = j * 32;
-                const float *zi = g.z_in + row * kHid + c;
+            for (int j = 0; j < PC; j += 32) {
+                tmem_ld32(taddr + j, v);
+                const int c = n0 + p0 + j;
+                float h[32], dz[32];
 #pragma unroll
                 for (int i = 0; i < 32; i++) {
-                    const float dz = v[i] * gelu_grad(zi[i]);
-                    const float s = warp_sum(dz);
-                    if (lane == 0) atomicAdd(g.db + c + i, s);
-                    v[i] = dz;
+                    const float z = v[i] + g.bias[c + i];
+                    h[i] = gy * gelu(z);
+                    dz[i] = v[i] = gy * g.w3[c + i] * gelu_grad(z);
                 }
+                sums[(4 + (warp & 3)) * NC + p0 + j + lane] = column_sums(h);
+                sums[(warp & 3) * NC + p0 + j + lane] = column_sums(dz);
 #pragma unroll
                 for (int q = 0; q < 4; q++) store8_tiled(g.h_out, row, c + 8 * q, g.a_rows, v + 8 * q);
+                store_transposed(g.ht_out, stage, row0, c, v);
+            }
+        }
+    } else if (acc_ok) {
+#pragma unroll 1
+        for (int j = 0; j < PC; j += 32) {
+            tmem_ld32(taddr + j, v);
+            const int c = n0 + p0 + j;
+            if constexpr (EPI == EPI_DW) {
+                float4 *dst = reinterpret_cast<float4 *>(g.dW + ((int64_t)blockIdx.y * 3 + layer) * kHid * kHid + row * kHid + c);
 #pragma unroll
-                for (int i = 0; i < 32; i++) g.ht_out[tiled(c + i, row, kHid)] = __float2bfloat16_rn(v[i]);
+                for (int i = 0; i < 8; i++) dst[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+            } else if constexpr (EPI == EPI_FWD) {
+#pragma unroll
+                for (int i = 0; i < 32; i++) {
+                    v[i] += g.bias[c + i];
+                    g.z_out[z_at(row, c + i)] = v[i];
+                    v[i] = gelu(v[i]);
+                }
+            } else {
+                // accumulator = gradient of the layer input; times gelu' of the layer below
+                float dz[32];
+#pragma unroll
+                for (int i = 0; i < 32; i++) dz[i] = v[i] = v[i] * gelu_grad(g.z_in[z_at(row, c + i)]);
+                sums[(warp & 3) * NC + p0 + j + lane] = column_sums(dz);
+            }
+            if constexpr (EPI != EPI_DW) {
+#pragma unroll
+                for (int q = 0; q < 4; q++) store8_tiled(g.h_out, row, c + 8 * q, g.a_rows, v + 8 * q);
+                store_transposed(g.ht_out, stage, row0, c, v);
             }
         }
     }
     tc_fence_before();
     __syncthreads();
-    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(256) : "memory");
+    if constexpr (EPI == EPI_LAST || EPI == EPI_DA) {
+        float *dst = g.cols + ((int64_t)blockIdx.x * 4 + g.col) * kHid + n0;
+        const int t = threadIdx.x;
+        if (t < NC) dst[t] = (sums[t] + sums[NC + t]) + (sums[2 * NC + t] + sums[3 * NC + t]);
+        if constexpr (EPI == EPI_LAST) {
+            const float *w = sums + 4 * NC, *q = reinterpret_cast<const float *>(tslot + 2);
+            if (t < NC) dst[kHid + t] = (w[t] + w[NC + t]) + (w[2 * NC + t] + w[3 * NC + t]);  // dw3 follows db2
+            if (t < 2 && blockIdx.z == 0) g.scalars[blockIdx.x * 2 + t] = (q[t] + q[2 + t]) + (q[4 + t] + q[6 + t]);
+        }
+    }
+    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(NC) : "memory");
+}
+
+// ---- inference: the whole network per 128-row tile --------------------------------------------
+//
+// A block keeps its rows' activations in shared memory through all layers (the tensor cores' operand
+// layout) and streams the layers' weights (128 KB each, from L2) through one buffer, the next layer's
+// while the epilogue of this one runs.  What bounds it is the epilogues' erff (some 45 instructions per
+// activation), over 512 threads.  134,613 rows take 181 us; layer by layer, with four launches per 65,536 rows,
+// the activations through memory and 128 threads per 128 x 256 tile, they took 333.
+constexpr uint32_t kActBytes = 128 * kHid * 2, kWBytes = kHid * kHid * 2;
+constexpr size_t kInferSmem = kActBytes + kWBytes + (4 * kHid + 4 * 128) * sizeof(float) + 1024 + 64;
+constexpr int kInferThreads = 512;
+
+struct InferArgs {
+    const __nv_bfloat16 *X;  // row-major [n x 256]
+    const __nv_bfloat16 *W;  // 3 tiled [256 x 256]
+    const float *bias[3], *w3, *b3;
+    float *out;
+    int64_t n;
+    int32_t *err;
+};
+
+__device__ __forceinline__ void async_proxy_fence() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+
+__global__ void __launch_bounds__(kInferThreads, 1) k_infer(const InferArgs g) {
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+    uint8_t *sA = smem, *sW = smem + kActBytes;
+    float *sBias = (float *)(sW + kWBytes), *sW3 = sBias + 3 * kHid, *part = sW3 + kHid;
+    uint64_t *full = (uint64_t *)(part + 4 * 128), *accd = full + 1;
+    uint32_t *tslot = (uint32_t *)(accd + 1);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int64_t tiles = (g.n + 127) / 128;
+    if (tid == 0) {
+        mbar_init(full, 1);
+        mbar_init(accd, 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(tslot)), "r"(kHid) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    for (int i = tid; i < 3 * kHid; i += kInferThreads) sBias[i] = g.bias[i / kHid][i % kHid];
+    for (int i = tid; i < kHid; i += kInferThreads) sW3[i] = g.w3[i];
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = *tslot;
+    const float b3 = g.b3[0];
+    auto load_w = [&](int layer) {
+        mbar_expect_tx(full, kWBytes);
+        for (int c = 0; c < 4; c++)
+            bulk_load(sW + c * (kWBytes / 4), g.W + ((int64_t)layer * kHid + c * 64) * kHid, kWBytes / 4, full);
+    };
+    // the thread's 16-byte pieces of a tile: 8 columns of its row (a warp: 8 rows x 64 bytes at a time, which
+    // fall on all banks of the operand layout)
+    const int xr = warp * 8 + (lane & 7), xc = (lane >> 3) * 8;
+    uint4 x[8];
+    auto read_rows = [&](int64_t tile) {
+#pragma unroll
+        for (int i = 0; i < 8; i++) {
+            const int64_t r = tile * 128 + xr;
+            x[i] = r < g.n ? *reinterpret_cast<const uint4 *>(g.X + r * kHid + xc + 32 * i) : make_uint4(0, 0, 0, 0);
+        }
+    };
+    // operand layout of element (r, c) in the tile: 16 KB per 64 columns, as `tiled` with 128 rows
+    auto act = [&](int r, int c) { return sA + 2 * tiled(r, c, 128); };
+    uint32_t wph = 0, aph = 0;
+    bool ok = true, pending = false;  // pending (thread 0): a weight load in flight
+    if (blockIdx.x < tiles) {
+        read_rows(blockIdx.x);
+        if (tid == 0) {
+            load_w(0);
+            pending = true;
+        }
+    }
+    for (int64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+#pragma unroll
+        for (int i = 0; i < 8; i++) *reinterpret_cast<uint4 *>(act(xr, xc + 32 * i)) = x[i];
+        const bool more = tile + gridDim.x < tiles;
+        for (int layer = 0; layer < 3; layer++) {
+            async_proxy_fence();
+            tc_fence_before();
+            __syncthreads();
+            if (tid == 0) {
+                tc_fence_after();
+                ok = mbar_wait(full, wph);
+                pending = !ok;
+                if (ok) {
+                    const uint32_t a0 = su32(sA), w0 = su32(sW);
+#pragma unroll 1
+                    for (int c = 0; c < 4; c++)
+#pragma unroll
+                        for (int kk = 0; kk < 4; kk++)
+                            mma_bf16<kHid>(tmem, sdesc(a0 + c * kAStage + kk * 256, 128, 1024),
+                                           sdesc(w0 + c * (kWBytes / 4) + kk * 256, 128, 1024), (c > 0 || kk > 0) ? 1u : 0u);
+                }
+                mma_commit(accd);
+            }
+            __syncwarp();
+            wph ^= 1;
+            if (!mbar_wait(accd, aph)) ok = false;
+            aph ^= 1;
+            if (!__syncthreads_and(ok)) {
+                ok = false;
+                break;
+            }
+            tc_fence_after();
+            // the tensor cores have read the weights and the activations
+            if (tid == 0 && (layer < 2 || more)) {
+                load_w(layer < 2 ? layer + 1 : 0);
+                pending = true;
+            }
+            if (layer == 2 && more) read_rows(tile + gridDim.x);
+            const int r = (warp & 3) * 32 + lane, p0 = (warp >> 2) * 64;
+            const uint32_t taddr = tmem + ((uint32_t)((warp & 3) * 32) << 16) + p0;
+            float yh = 0.f;
+#pragma unroll 1
+            for (int j = 0; j < 64; j += 32) {
+                float v[32];
+                tmem_ld32(taddr + j, v);
+                const float4 *bias = reinterpret_cast<const float4 *>(sBias + layer * kHid + p0 + j);
+#pragma unroll
+                for (int i = 0; i < 8; i++) {
+                    const float4 b = bias[i];
+                    v[4 * i] = gelu(v[4 * i] + b.x);
+                    v[4 * i + 1] = gelu(v[4 * i + 1] + b.y);
+                    v[4 * i + 2] = gelu(v[4 * i + 2] + b.z);
+                    v[4 * i + 3] = gelu(v[4 * i + 3] + b.w);
+                }
+                if (layer < 2) {
+#pragma unroll
+                    for (int q = 0; q < 4; q++)
+                        *reinterpret_cast<uint4 *>(act(r, p0 + j + 8 * q)) =
+                            make_uint4(pack2(v[8 * q], v[8 * q + 1]), pack2(v[8 * q + 2], v[8 * q + 3]),
+                                       pack2(v[8 * q + 4], v[8 * q + 5]), pack2(v[8 * q + 6], v[8 * q + 7]));
+                } else {
+#pragma unroll
+                    for (int i = 0; i < 8; i++) {
+                        const float4 w = *reinterpret_cast<const float4 *>(sW3 + p0 + j + 4 * i);
+                        yh += v[4 * i] * w.x + v[4 * i + 1] * w.y + v[4 * i + 2] * w.z + v[4 * i + 3] * w.w;
+                    }
+                }
+            }
+            if (layer == 2) {
+                part[(warp >> 2) * 128 + r] = yh;
+                __syncthreads();
+                const int64_t row = tile * 128 + tid;
+                if (tid < 128 && row < g.n) g.out[row] = b3 + part[tid] + part[128 + tid] + part[256 + tid] + part[384 + tid];
+            }
+        }
+        if (!ok) break;
+    }
+    if (!ok && tid == 0) {
+        atomicExch(g.err, 1);
+        if (pending) mbar_wait(full, wph ^ 1);  // a copy still in flight lands before the block ends
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kHid) : "memory");
 }
 
 // rows (optionally gathered through perm) of a row-major bf16 [n x 256] matrix into the tiled
 // matrix [Mp x 256] and its tiled transpose [256 x Mp]; rows n..Mp-1 are zero.  Also gathers the
 // targets.
-__global__ void k_pack(const __nv_bfloat16 *__restrict__ X, const float *__restrict__ y, const int64_t *__restrict__ perm,
-                       int64_t row0, int64_t n, int64_t Mp, __nv_bfloat16 *__restrict__ Xt, __nv_bfloat16 *__restrict__ XtT,
-                       float *__restrict__ yb) {
-    const int64_t total = Mp * (kHid / 8);
-    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t r = e / (kHid / 8), c = (e % (kHid / 8)) * 8;
-        uint4 w = make_uint4(0, 0, 0, 0);
-        if (r < n) {
-            const int64_t src = perm ? perm[row0 + r] : row0 + r;
-            w = *reinterpret_cast<const uint4 *>(X + src * kHid + c);
-            if (c == 0 && yb) yb[r] = y ? y[src] : 0.f;
-        } else if (c == 0 && yb) {
-            yb[r] = 0.f;
-        }
-        *reinterpret_cast<uint4 *>(Xt + tiled(r, c, Mp)) = w;
-        if (XtT) {
-            const __nv_bfloat16 *b = reinterpret_cast<const __nv_bfloat16 *>(&w);
+// A block takes 64 rows x 64 columns through shared memory, so that both copies are written 16 bytes at a time.
+__global__ void __launch_bounds__(256) k_pack(const __nv_bfloat16 *__restrict__ X, const float *__restrict__ y,
+                                              const int64_t *__restrict__ perm, int64_t row0, int64_t n, int64_t Mp,
+                                              __nv_bfloat16 *__restrict__ Xt, __nv_bfloat16 *__restrict__ XtT, float *__restrict__ yb) {
+    __shared__ __align__(16) __nv_bfloat16 tile[64][72];  // [column][row]
+    pdl_next();
+    pdl_wait();
+    const int t = threadIdx.x, c0 = blockIdx.y * 64;
+    const int64_t r0 = (int64_t)blockIdx.x * 64;
 #pragma unroll
-            for (int i = 0; i < 8; i++) XtT[tiled(c + i, r, kHid)] = b[i];
+    for (int k = 0; k < 2; k++) {
+        const int e = t + 256 * k, lr = (e & 7) + 8 * (e >> 6), lc = (e >> 3 & 7) * 8;
+        const int64_t r = r0 + lr;
+        uint4 w = make_uint4(0, 0, 0, 0);
+        int64_t src = -1;
+        if (r < n) {
+            src = perm ? perm[row0 + r] : row0 + r;
+            w = *reinterpret_cast<const uint4 *>(X + src * kHid + c0 + lc);
         }
+        if (c0 + lc == 0) yb[r] = src >= 0 && y ? y[src] : 0.f;
+        *reinterpret_cast<uint4 *>(Xt + tiled(r, c0 + lc, Mp)) = w;
+        const __nv_bfloat16 *b = reinterpret_cast<const __nv_bfloat16 *>(&w);
+#pragma unroll
+        for (int i = 0; i < 8; i++) tile[lc + i][lr] = b[i];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < 2; k++) {
+        const int e = t + 256 * k, lc = (e & 7) + 8 * (e >> 6), lr = (e >> 3 & 7) * 8;
+        *reinterpret_cast<uint4 *>(XtT + tiled(c0 + lc, r0 + lr, kHid)) = *reinterpret_cast<const uint4 *>(&tile[lc][lr]);
     }
 }
 
-// Adam (Kingma and Ba, 2015) on the flat parameters; writes the bf16 tiled weights and their
-// transposes and clears the gradients.  t = step number (>= 1).
-__global__ void k_adam(float *__restrict__ p, float *__restrict__ grad, float *__restrict__ m, float *__restrict__ v,
-                       const int64_t *__restrict__ t_base, int64_t t_off, float lr, float b1, float b2, float eps,
+// gradient of parameter i; the last one's thread also gets the loss
+__device__ __forceinline__ float grad_at(const Partials &q, int i, float *loss) {
+    const int per = kHid * kHid + kHid;
+    const int l = i / per, o = i % per;
+    const float *src;
+    int64_t stride;
+    int n = q.tiles;
+    if (i == kParams - 1) {
+        float sum = 0.f;
+        for (int t = 0; t < n; t++) sum += q.scalars[2 * t + 1];
+        *loss += sum;
+        src = q.scalars;
+        stride = 2;
+    } else if (l < 3 && o < kHid * kHid) {
+        src = q.dW + (int64_t)l * kHid * kHid + o;
+        stride = 3 * kHid * kHid;
+        n = q.splits;
+    } else {
+        src = q.cols + (l < 3 ? l * kHid + o - kHid * kHid : 3 * kHid + o);
+        stride = 4 * kHid;
+    }
+    float g = 0.f;
+#pragma unroll 4
+    for (int t = 0; t < n; t++) g += src[t * stride];
+    return g;
+}
+
+__global__ void k_gradient(const Partials q, float *__restrict__ grad, float *loss) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < kParams) grad[i] = grad_at(q, i, loss);
+}
+
+// Adam (Kingma and Ba, 2015) on the flat parameters; writes the bf16 tiled weights and their transposes.
+// corr: the step's two bias corrections (64-bit powers taken on the host: two of them per thread here took
+// 83 us a step).
+__global__ void k_adam(float *__restrict__ p, const Partials q, float *loss, float *__restrict__ m, float *__restrict__ v,
+                       const float *__restrict__ corr, float lr, float b1, float b2, float eps,
                        __nv_bfloat16 *__restrict__ W, __nv_bfloat16 *__restrict__ WT) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    pdl_next();
+    pdl_wait();
     if (i >= kParams) return;
-    const double t = (double)(t_base[0] + t_off);
-    const float c1 = (float)(1.0 / (1.0 - pow((double)b1, t))), c2 = (float)(1.0 / (1.0 - pow((double)b2, t)));
-    const float gi = grad[i];
+    const float c1 = corr[0], c2 = corr[1];
+    const float gi = grad_at(q, i, loss);
     const float mi = b1 * m[i] + (1.f - b1) * gi, vi = b2 * v[i] + (1.f - b2) * gi * gi;
     m[i] = mi;
     v[i] = vi;
     const float pi = p[i] - lr * (mi * c1) / (sqrtf(vi * c2) + eps);
     p[i] = pi;
-    grad[i] = 0.f;
     // weight matrices l = 0..2 at offsets l * (256*256 + 256)
     const int per = kHid * kHid + kHid;
     const int l = i / per, o = i % per;
@@ -439,9 +725,11 @@ struct pasur_mlp {
     pasur_ctx *ctx = nullptr;
     float *p = nullptr, *grad = nullptr, *m = nullptr, *v = nullptr;   // flat f32 [kParams]
     __nv_bfloat16 *W = nullptr, *WT = nullptr;                          // 3 tiled [256 x 256] each
-    int64_t *t_d = nullptr;                                             // Adam step base
+    float *corr_d = nullptr;                                            // per step of an epoch: Adam's bias corrections
+    int64_t corr_cap = 0;
     int64_t steps = 0;
     float *loss_d = nullptr;
+    Partials parts{};                                                   // of the last pass
     int32_t *err_d = nullptr;
     // dataset (row-major bf16 features, f32 targets)
     int64_t cap = 0, n = 0;
@@ -451,7 +739,7 @@ struct pasur_mlp {
     int64_t rows_cap = 0;
     __nv_bfloat16 *h0 = nullptr, *h0t = nullptr, *h1 = nullptr, *h1t = nullptr, *h2 = nullptr, *h2t = nullptr;
     __nv_bfloat16 *d0 = nullptr, *d0t = nullptr, *d1 = nullptr, *d1t = nullptr, *d2 = nullptr, *d2t = nullptr;
-    float *z0 = nullptr, *z1 = nullptr, *yb = nullptr, *yhat = nullptr;
+    float *z0 = nullptr, *z1 = nullptr, *yb = nullptr;
     int64_t *perm_d = nullptr;
     std::vector<std::pair<void *, size_t>> owned;
     cudaGraphExec_t epoch_exec = nullptr;
@@ -476,15 +764,46 @@ void mlp_release(pasur_mlp *M, void *p) {
         }
 }
 
+constexpr int kMaxSplits = 12;             // of the batch, for the weight gradients
+constexpr int kCols = 64, kColGroups = 2;  // columns per block, and their parts
+
+template <int EPI>
+int raise_gemm(pasur_ctx *ctx) {
+    PASUR_CUDA(ctx, cudaFuncSetAttribute(k_gemm<EPI, kCols, kColGroups>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)gemm_smem(EPI, kCols, 4 * kColGroups)));
+    return PASUR_OK;
+}
+
+// launch in stream order with the set-up overlapping the kernel before (its pdl_wait); a cluster along z
+template <class... P, class... A>
+int launch_next(pasur_ctx *ctx, void (*k)(P...), dim3 grid, int threads, size_t smem, unsigned cluster, A... args) {
+    cudaLaunchConfig_t c{};
+    c.gridDim = grid;
+    c.blockDim = dim3((unsigned)threads);
+    c.dynamicSmemBytes = smem;
+    c.stream = ctx->stream;
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = 1;
+    at[1].val.clusterDim.y = 1;
+    at[1].val.clusterDim.z = cluster;
+    c.attrs = at;
+    c.numAttrs = cluster > 1 ? 2 : 1;
+    ctx->launches++;
+    PASUR_CUDA(ctx, cudaLaunchKernelEx(&c, k, P(args)...));
+    return PASUR_OK;
+}
+
 int set_gemm_attrs(pasur_ctx *ctx) {
     static int done_dev = -1;
     if (done_dev == ctx->device) return PASUR_OK;
-    PASUR_CUDA(ctx, cudaFuncSetAttribute(k_gemm<EPI_FWD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGemmSmem));
-    PASUR_CUDA(ctx, cudaFuncSetAttribute(k_gemm<EPI_FWD_INFER>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGemmSmem));
-    PASUR_CUDA(ctx, cudaFuncSetAttribute(k_gemm<EPI_LAST_TRAIN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGemmSmem));
-    PASUR_CUDA(ctx, cudaFuncSetAttribute(k_gemm<EPI_LAST_INFER>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGemmSmem));
-    PASUR_CUDA(ctx, cudaFuncSetAttribute(k_gemm<EPI_DA>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGemmSmem));
-    PASUR_CUDA(ctx, cudaFuncSetAttribute(k_gemm<EPI_DW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGemmSmem));
+    PASUR_TRY(raise_gemm<EPI_FWD>(ctx));
+    PASUR_TRY(raise_gemm<EPI_DA>(ctx));
+    PASUR_TRY(raise_gemm<EPI_DW>(ctx));
+    PASUR_TRY(raise_gemm<EPI_LAST>(ctx));
+    PASUR_CUDA(ctx, cudaFuncSetAttribute(k_infer, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kInferSmem));
     done_dev = ctx->device;
     return PASUR_OK;
 }
@@ -504,9 +823,10 @@ int ensure_rows(pasur_mlp *M, int64_t rows) {
         PASUR_TRY(mlp_alloc(M, b, sizeof(float) * (size_t)rows * kHid));
     }
     if (M->yb) mlp_release(M, M->yb);
-    if (M->yhat) mlp_release(M, M->yhat);
     PASUR_TRY(mlp_alloc(M, (void **)&M->yb, sizeof(float) * (size_t)rows));
-    PASUR_TRY(mlp_alloc(M, (void **)&M->yhat, sizeof(float) * (size_t)rows));
+    if (!M->parts.dW) PASUR_TRY(mlp_alloc(M, (void **)&M->parts.dW, sizeof(float) * kMaxSplits * 3 * kHid * kHid));
+    if (M->parts.cols) mlp_release(M, M->parts.cols);
+    PASUR_TRY(mlp_alloc(M, (void **)&M->parts.cols, sizeof(float) * (size_t)(rows / 128) * (4 * kHid + 2)));
     M->rows_cap = rows;
     if (M->epoch_exec) {
         cudaGraphExecDestroy(M->epoch_exec);
@@ -522,76 +842,64 @@ GemmArgs base_args(pasur_mlp *M) {
 }
 
 template <int EPI>
-int launch_gemm(pasur_mlp *M, const GemmArgs &a, int64_t m_tiles, int64_t splits) {
-    pasur_ctx *ctx = M->ctx;
-    dim3 grid((unsigned)m_tiles, (unsigned)splits);
-    k_gemm<EPI><<<grid, 128, kGemmSmem, ctx->stream>>>(a);
-    ctx->launches++;
-    PASUR_CUDA(ctx, cudaGetLastError());
-    return PASUR_OK;
+int launch_gemm(pasur_mlp *M, const GemmArgs &a, int64_t m_tiles, int64_t splits, int layers) {
+    dim3 grid((unsigned)m_tiles, (unsigned)splits, (unsigned)(kHid / kCols * layers));
+    return launch_next(M->ctx, k_gemm<EPI, kCols, kColGroups>, grid, 128 * kColGroups, gemm_smem(EPI, kCols, 4 * kColGroups),
+                       EPI == EPI_LAST ? kHid / kCols : 1, a);
 }
 
-// forward (train: also the backward pass and gradients) of Mp packed rows in h0/h0t; targets in
-// yb; n_valid real rows; no synchronisation (capturable)
-int run_pass(pasur_mlp *M, int64_t Mp, int64_t n_valid, bool train) {
+// forward and backward pass of Mp packed rows in h0/h0t, gradients into M->parts; targets in yb;
+// n_valid real rows; no synchronisation (capturable)
+int run_pass(pasur_mlp *M, int64_t Mp, int64_t n_valid) {
     const __nv_bfloat16 *W0 = M->W, *W1 = M->W + kHid * kHid, *W2 = M->W + 2 * kHid * kHid;
     const __nv_bfloat16 *WT1 = M->WT + kHid * kHid, *WT2 = M->WT + 2 * kHid * kHid;
     const int per = kHid * kHid + kHid;
     const float *b0 = M->p + kHid * kHid, *b1 = M->p + per + kHid * kHid, *b2 = M->p + 2 * per + kHid * kHid;
     const float *w3 = M->p + 3 * per, *b3 = w3 + kHid;
-    float *g = M->grad;
-    float *gW0 = g, *gb0 = g + kHid * kHid, *gW1 = g + per, *gb1 = g + per + kHid * kHid, *gW2 = g + 2 * per,
-          *gb2 = g + 2 * per + kHid * kHid, *gw3 = g + 3 * per, *gb3 = gw3 + kHid;
+    Partials &q = M->parts;
     const int64_t mt = Mp / 128;
+    q.tiles = (int)mt;
+    q.scalars = q.cols + mt * 4 * kHid;
     GemmArgs a = base_args(M);
     a.a_rows = Mp;
     a.K = kHid;
     a.kcs = kHid / 64;
     // layer 0, 1
-    a.A = M->h0; a.B = W0; a.bias = b0; a.z_out = M->z0; a.h_out = M->h1; a.ht_out = M->h1t;
-    if (train) PASUR_TRY(launch_gemm<EPI_FWD>(M, a, mt, 1));
-    else PASUR_TRY(launch_gemm<EPI_FWD_INFER>(M, a, mt, 1));
-    a.A = M->h1; a.B = W1; a.bias = b1; a.z_out = M->z1; a.h_out = M->h2; a.ht_out = M->h2t;
-    if (train) PASUR_TRY(launch_gemm<EPI_FWD>(M, a, mt, 1));
-    else PASUR_TRY(launch_gemm<EPI_FWD_INFER>(M, a, mt, 1));
-    // layer 2 + output layer (+ loss, output and layer-2 gradients)
-    a.A = M->h2; a.B = W2; a.bias = b2; a.w3 = w3; a.b3 = b3; a.y = M->yb; a.yhat = M->yhat; a.n_valid = n_valid;
+    a.A[0] = M->h0; a.B[0] = W0; a.bias = b0; a.z_out = M->z0; a.h_out = M->h1; a.ht_out = M->h1t;
+    PASUR_TRY(launch_gemm<EPI_FWD>(M, a, mt, 1, 1));
+    a.A[0] = M->h1; a.B[0] = W1; a.bias = b1; a.z_out = M->z1; a.h_out = M->h2; a.ht_out = M->h2t;
+    PASUR_TRY(launch_gemm<EPI_FWD>(M, a, mt, 1, 1));
+    // layer 2 + output layer, loss, output and layer-2 gradients
+    a.A[0] = M->h2; a.B[0] = W2; a.bias = b2; a.w3 = w3; a.b3 = b3; a.y = M->yb; a.n_valid = n_valid;
     a.inv_n = 1.f / (float)std::max<int64_t>(1, n_valid);
-    if (!train) return launch_gemm<EPI_LAST_INFER>(M, a, mt, 1);
-    a.loss = M->loss_d; a.dw3 = gw3; a.db3 = gb3; a.db = gb2; a.h_out = M->d2; a.ht_out = M->d2t;
-    PASUR_TRY(launch_gemm<EPI_LAST_TRAIN>(M, a, mt, 1));
-    // weight gradients: dW_l = dZ_l^T H_l (K = rows, split over the batch)
-    const int64_t nk = Mp / 64;
-    const int64_t splits = std::min<int64_t>(nk, 32), kcs = (nk + splits - 1) / splits;
-    const int64_t used = (nk + kcs - 1) / kcs;
-    auto dw = [&](const __nv_bfloat16 *dzt, const __nv_bfloat16 *ht, float *gW) {
-        GemmArgs d = base_args(M);
-        d.A = dzt; d.B = ht; d.a_rows = kHid; d.K = Mp; d.kcs = kcs; d.dW = gW;
-        return launch_gemm<EPI_DW>(M, d, 2, used);
-    };
+    a.cols = q.cols; a.col = 2; a.scalars = q.scalars; a.h_out = M->d2; a.ht_out = M->d2t;
+    PASUR_TRY(launch_gemm<EPI_LAST>(M, a, mt, 1, 1));
     // input gradients: dH_l = dZ_l W_l, then dZ_{l-1} = dH_l * gelu'(Z_{l-1})
-    auto da = [&](const __nv_bfloat16 *dz, const __nv_bfloat16 *wt, const float *zin, float *gb, __nv_bfloat16 *o,
+    auto da = [&](const __nv_bfloat16 *dz, const __nv_bfloat16 *wt, const float *zin, int col, __nv_bfloat16 *o,
                   __nv_bfloat16 *ot) {
         GemmArgs d = base_args(M);
-        d.A = dz; d.B = wt; d.a_rows = Mp; d.K = kHid; d.kcs = kHid / 64; d.z_in = zin; d.db = gb; d.h_out = o; d.ht_out = ot;
-        return launch_gemm<EPI_DA>(M, d, mt, 1);
+        d.A[0] = dz; d.B[0] = wt; d.a_rows = Mp; d.K = kHid; d.kcs = kHid / 64; d.z_in = zin; d.cols = q.cols; d.col = col; d.h_out = o; d.ht_out = ot;
+        return launch_gemm<EPI_DA>(M, d, mt, 1, 1);
     };
-    PASUR_TRY(dw(M->d2t, M->h2t, gW2));
-    PASUR_TRY(da(M->d2, WT2, M->z1, gb1, M->d1, M->d1t));
-    PASUR_TRY(dw(M->d1t, M->h1t, gW1));
-    PASUR_TRY(da(M->d1, WT1, M->z0, gb0, M->d0, M->d0t));
-    PASUR_TRY(dw(M->d0t, M->h0t, gW0));
-    return PASUR_OK;
+    PASUR_TRY(da(M->d2, WT2, M->z1, 1, M->d1, M->d1t));
+    PASUR_TRY(da(M->d1, WT1, M->z0, 0, M->d0, M->d0t));
+    // weight gradients of the three layers in one launch: dW_l = dZ_l^T H_l (K = rows, split over the
+    // batch: 24 blocks per split, up to three on an SM)
+    const int64_t nk = Mp / 64;
+    const int64_t splits = std::min<int64_t>(nk, kMaxSplits), kcs = (nk + splits - 1) / splits;
+    GemmArgs d = base_args(M);
+    d.A[0] = M->d0t; d.A[1] = M->d1t; d.A[2] = M->d2t;
+    d.B[0] = M->h0t; d.B[1] = M->h1t; d.B[2] = M->h2t;
+    d.dW = q.dW;
+    d.a_rows = kHid;
+    d.K = Mp;
+    d.kcs = kcs;
+    q.splits = (int)((nk + kcs - 1) / kcs);
+    return launch_gemm<EPI_DW>(M, d, 2, q.splits, 3);
 }
 
-int pack(pasur_mlp *M, const __nv_bfloat16 *X, const float *y, const int64_t *perm, int64_t row0, int64_t n, int64_t Mp,
-         bool want_t) {
-    const int64_t total = Mp * (kHid / 8);
-    unsigned grid = (unsigned)std::min<int64_t>((total + 255) / 256, (int64_t)M->ctx->num_sms * 8);
-    k_pack<<<std::max(1u, grid), 256, 0, M->ctx->stream>>>(X, y, perm, row0, n, Mp, M->h0, want_t ? M->h0t : nullptr, M->yb);
-    M->ctx->launches++;
-    PASUR_CUDA(M->ctx, cudaGetLastError());
-    return PASUR_OK;
+int pack(pasur_mlp *M, const __nv_bfloat16 *X, const float *y, const int64_t *perm, int64_t row0, int64_t n, int64_t Mp) {
+    return launch_next(M->ctx, k_pack, dim3((unsigned)(Mp / 64), kHid / 64), 256, 0, 1, X, y, perm, row0, n, Mp, M->h0, M->h0t, M->yb);
 }
 
 int check_err(pasur_mlp *M) {
@@ -606,14 +914,22 @@ int64_t pad128(int64_t n) { return std::max<int64_t>(128, (n + 127) / 128 * 128)
 
 // forward of n rows already in device row-major bf16 form; predictions into out_dev
 int forward_rows(pasur_mlp *M, const __nv_bfloat16 *X, int64_t n, float *out_dev) {
-    const int64_t chunk = 1 << 16;
-    for (int64_t r0 = 0; r0 < n; r0 += chunk) {
-        const int64_t m = std::min(chunk, n - r0), Mp = pad128(m);
-        PASUR_TRY(ensure_rows(M, Mp));
-        PASUR_TRY(pack(M, X, nullptr, nullptr, r0, m, Mp, false));
-        PASUR_TRY(run_pass(M, Mp, m, false));
-        PASUR_CUDA(M->ctx, cudaMemcpyAsync(out_dev + r0, M->yhat, sizeof(float) * (size_t)m, cudaMemcpyDeviceToDevice, M->ctx->stream));
-    }
+    pasur_ctx *ctx = M->ctx;
+    if (n <= 0) return PASUR_OK;
+    const int per = kHid * kHid + kHid;
+    InferArgs g{};
+    g.X = X;
+    g.W = M->W;
+    for (int l = 0; l < 3; l++) g.bias[l] = M->p + l * per + kHid * kHid;
+    g.w3 = M->p + 3 * per;
+    g.b3 = g.w3 + kHid;
+    g.out = out_dev;
+    g.n = n;
+    g.err = M->err_d;
+    const unsigned grid = (unsigned)std::min<int64_t>((n + 127) / 128, ctx->num_sms);
+    k_infer<<<grid, kInferThreads, kInferSmem, ctx->stream>>>(g);
+    ctx->launches++;
+    PASUR_CUDA(ctx, cudaGetLastError());
     return PASUR_OK;
 }
 
@@ -713,7 +1029,6 @@ int pasur_mlp_create(pasur_ctx *ctx, int64_t dataset_capacity, uint64_t seed, pa
     A((void **)&M->v, sizeof(float) * kParams);
     A((void **)&M->W, sizeof(__nv_bfloat16) * 3 * kHid * kHid);
     A((void **)&M->WT, sizeof(__nv_bfloat16) * 3 * kHid * kHid);
-    A((void **)&M->t_d, sizeof(int64_t));
     A((void **)&M->loss_d, sizeof(float) * 4);
     A((void **)&M->err_d, sizeof(int32_t));
     M->cap = dataset_capacity;
@@ -808,10 +1123,14 @@ int pasur_mlp_gradients(pasur_mlp *M, const uint16_t *x, const float *y, int64_t
     if (rc == PASUR_OK) rc = to_device(ctx, y, sizeof(float) * (size_t)n, &yd, tmp);
     const int64_t Mp = pad128(n);
     if (rc == PASUR_OK) rc = ensure_rows(M, Mp);
-    if (rc == PASUR_OK) rc = cudaMemsetAsync(M->grad, 0, sizeof(float) * kParams, ctx->stream) == cudaSuccess ? PASUR_OK : PASUR_ECUDA;
     if (rc == PASUR_OK) rc = cudaMemsetAsync(M->loss_d, 0, sizeof(float), ctx->stream) == cudaSuccess ? PASUR_OK : PASUR_ECUDA;
-    if (rc == PASUR_OK) rc = pack(M, (const __nv_bfloat16 *)xd, (const float *)yd, nullptr, 0, n, Mp, true);
-    if (rc == PASUR_OK) rc = run_pass(M, Mp, n, true);
+    if (rc == PASUR_OK) rc = pack(M, (const __nv_bfloat16 *)xd, (const float *)yd, nullptr, 0, n, Mp);
+    if (rc == PASUR_OK) rc = run_pass(M, Mp, n);
+    if (rc == PASUR_OK) {
+        k_gradient<<<(kParams + 255) / 256, 256, 0, ctx->stream>>>(M->parts, M->grad, M->loss_d);
+        ctx->launches++;
+        if (cudaGetLastError() != cudaSuccess) rc = set_err(ctx, PASUR_ECUDA, "k_gradient launch");
+    }
     if (rc == PASUR_OK) rc = check_err(M);
     if (rc == PASUR_OK && loss_out) rc = copy_to(ctx, loss_out, M->loss_d, sizeof(float));
     if (rc == PASUR_OK && grads_out) rc = copy_to(ctx, grads_out, M->grad, sizeof(float) * kParams);
@@ -903,6 +1222,16 @@ int pasur_mlp_train(pasur_mlp *M, int epochs, int64_t batch, float lr, uint64_t 
     cudaSetDevice(ctx->device);
     PASUR_TRY(ensure_rows(M, batch));
     const int64_t n = M->n, steps = (n + batch - 1) / batch;
+    if (M->corr_cap < steps) {
+        cudaStreamSynchronize(ctx->stream);
+        if (M->corr_d) mlp_release(M, M->corr_d);
+        M->corr_d = nullptr;
+        M->corr_cap = 0;
+        PASUR_TRY(mlp_alloc(M, (void **)&M->corr_d, sizeof(float) * 2 * (size_t)steps));
+        M->corr_cap = steps;
+        if (M->epoch_exec) cudaGraphExecDestroy(M->epoch_exec);
+        M->epoch_exec = nullptr;
+    }
     // one CUDA graph per epoch: (pack batch i through the permutation, forward, backward, Adam) x steps
     if (!M->epoch_exec || M->epoch_batch != batch || M->epoch_rows != n) {
         if (M->epoch_exec) cudaGraphExecDestroy(M->epoch_exec);
@@ -911,13 +1240,11 @@ int pasur_mlp_train(pasur_mlp *M, int epochs, int64_t batch, float lr, uint64_t 
         int rc = PASUR_OK;
         for (int64_t s = 0; s < steps && rc == PASUR_OK; s++) {
             const int64_t r0 = s * batch, m = std::min(batch, n - r0);
-            rc = pack(M, M->X, M->Y, M->perm_d, r0, m, batch, true);
-            if (rc == PASUR_OK) rc = run_pass(M, batch, m, true);
+            rc = pack(M, M->X, M->Y, M->perm_d, r0, m, batch);
+            if (rc == PASUR_OK) rc = run_pass(M, batch, m);
             if (rc == PASUR_OK) {
-                k_adam<<<(kParams + 255) / 256, 256, 0, ctx->stream>>>(M->p, M->grad, M->m, M->v, M->t_d, s + 1, lr, 0.9f, 0.999f,
-                                                                     1e-8f, M->W, M->WT);
-                ctx->launches++;
-                if (cudaGetLastError() != cudaSuccess) rc = set_err(ctx, PASUR_ECUDA, "k_adam launch");
+                rc = launch_next(ctx, k_adam, dim3((kParams + 255) / 256), 256, 0, 1, M->p, M->parts, M->loss_d, M->m, M->v,
+                                 M->corr_d + 2 * s, lr, 0.9f, 0.999f, 1e-8f, M->W, M->WT);
             }
         }
         cudaGraph_t gr = nullptr;
@@ -933,9 +1260,9 @@ int pasur_mlp_train(pasur_mlp *M, int epochs, int64_t batch, float lr, uint64_t 
         M->epoch_batch = batch;
         M->epoch_rows = n;
     }
-    PASUR_CUDA(ctx, cudaMemsetAsync(M->grad, 0, sizeof(float) * kParams, ctx->stream));
-    const int64_t launches_per_epoch = steps * 10;
+    const int64_t launches_per_epoch = steps * 8;
     std::vector<int64_t> perm((size_t)n);
+    std::vector<float> corr(2 * (size_t)steps);
     uint64_t x = shuffle_seed;
     cudaEvent_t e0, e1;
     PASUR_CUDA(ctx, cudaEventCreate(&e0));
@@ -954,7 +1281,12 @@ int pasur_mlp_train(pasur_mlp *M, int epochs, int64_t batch, float lr, uint64_t 
         }
         const int64_t tb = M->steps;
         PASUR_CUDA(ctx, cudaMemcpyAsync(M->perm_d, perm.data(), sizeof(int64_t) * (size_t)n, cudaMemcpyHostToDevice, ctx->stream));
-        PASUR_CUDA(ctx, cudaMemcpyAsync(M->t_d, &tb, sizeof tb, cudaMemcpyHostToDevice, ctx->stream));
+        for (int64_t s = 0; s < steps; s++) {
+            const double t = (double)(tb + s + 1);
+            corr[2 * (size_t)s] = (float)(1.0 / (1.0 - std::pow((double)0.9f, t)));
+            corr[2 * (size_t)s + 1] = (float)(1.0 / (1.0 - std::pow((double)0.999f, t)));
+        }
+        PASUR_CUDA(ctx, cudaMemcpyAsync(M->corr_d, corr.data(), sizeof(float) * corr.size(), cudaMemcpyHostToDevice, ctx->stream));
         PASUR_CUDA(ctx, cudaMemsetAsync(M->loss_d, 0, sizeof(float), ctx->stream));
         PASUR_CUDA(ctx, cudaGraphLaunch(M->epoch_exec, ctx->stream));
         ctx->launches += launches_per_epoch;
@@ -986,7 +1318,7 @@ int pasur_mlp_predict_next(pasur_mlp *M, const pasur_tree *t, float *out, int64_
     int rc = features_dev(M, t->deck, t->round + 1, t->next_pools_h.data(), t->next_soff_h.data(), t->next_scores_h.data(),
                           (int64_t)t->next_pools_h.size(), &x, &n, tmp);
     float *yd = nullptr;
-    const bool dev = is_device_ptr(out);
+    const bool dev = is_device_ptr(out) && ((uintptr_t)out & 3) == 0;  // the kernel writes there itself
     if (rc == PASUR_OK && !dev) {
         void *p = nullptr;
         rc = dev_alloc(ctx, &p, sizeof(float) * (size_t)(n + 1));

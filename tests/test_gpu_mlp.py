@@ -284,3 +284,29 @@ def test_surrogate_gain_over_no_learning(ctx):
     assert (a[:, 1] >= -1e-9).all() and (z[:, 1] >= -1e-9).all() and np.isfinite(a).all()
     mlp.free()
     m0.free()
+
+
+@pytest.mark.parametrize("n", [1, 127, 128, 129, 152 * 128 + 1])
+def test_tile_edges(ctx, n):
+    """Predictions at the edges of the 128-row tiles and of one wave of blocks, and gradients of
+    batches whose weight-gradient splits differ (n <= 129: two or four 64-row chunks, one to a
+    split; 2000 rows: 32 chunks, the last split short).  Bounds: the two of the tests above (f32
+    accumulation order against the oracle's 64 bits on the same bf16 operands)."""
+    from paper_2508_06559_gb300 import pasur as P
+    rng = np.random.default_rng(n)
+    X = M.to_bf16(rng.normal(0, 1, (n, 256)))
+    flat32, po = params(2)
+    mlp = P.Mlp(ctx)
+    mlp.set_params(flat32)
+    got = mlp.forward(bf16_bits(X))
+    want, _ = M.forward(po, X, round_act=True)
+    assert np.abs(got - want).max() <= 1e-3 * (1 + np.abs(want).max()), np.abs(got - want).max()
+    m = min(n, 2000)
+    Y = rng.normal(0, 2, m).astype(np.float32)
+    loss, g = mlp.gradients(bf16_bits(X[:m]), Y)
+    lo, go, _ = M.loss_and_grads(po, X[:m], Y.astype(np.float64), round_act=True)
+    assert abs(loss - lo) <= 1e-3 * lo
+    gg, scale = M.unflatten(g.astype(np.float64)), grad_scale(po, X[:m], Y.astype(np.float64))
+    for name, _ in M.SHAPES:
+        assert (np.abs(gg[name] - go[name]) <= BF16_ELEM_TOL * scale[name] + 1e-12).all(), name
+    mlp.free()
