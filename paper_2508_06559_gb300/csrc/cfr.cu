@@ -368,7 +368,7 @@ __global__ void k_fill(float *out, int64_t n, float v) {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) out[i] = v;
 }
 
-// average strategy of the child edges of every active node, canonical FGT order, one block per
+// average strategy of the child edges of every active node, canonical FGT order, one or more blocks per
 // item (every other edge lies below a forced move and has average strategy 1)
 __global__ void k_export_sigma(const CfrItem *items, int64_t n_items, const CfrRoot *roots, const int32_t *act_cs,
                                const uint16_t *act_d, const int64_t *act_gt, const float *Sg, LevelPtrs lp, float *out) {
@@ -376,20 +376,22 @@ __global__ void k_export_sigma(const CfrItem *items, int64_t n_items, const CfrR
         const CfrItem it = items[id];
         const CfrRoot &cr = roots[it.root];
         const int W = it.ns;
+        const int64_t n = (int64_t)cr.as[8] * W;
         const float *S = Sg + it.data_base;
-        for (int k = 0; k < 8; k++) {
-            const int b = cr.as[k], n = (cr.as[k + 1] - b) * W;
-            for (int x = threadIdx.x; x < n; x += blockDim.x) {
-                const int e = b + x / W, w = x % W;
-                const int c = act_cs[cr.act_off + e], d = act_d[cr.act_off + e];
-                const int64_t j = act_gt[cr.act_off + e];
-                float sum = 0.f;
-                for (int a = 0; a < d; a++) sum += S[(c + a) * W + w];
-                const int64_t c0 = lp.child[k][j];
-                for (int a = 0; a < d; a++) {
-                    float sb = sum > 0.f ? S[(c + a) * W + w] / sum : 1.f / (float)d;
-                    out[lp.base[k + 1] + lp.fgt[k + 1][c0 + a] + it.s0 + w] = sb;
-                }
+        int k = 0;
+        for (int64_t x = (int64_t)cr.as[0] * W + blockIdx.y * blockDim.x + threadIdx.x; x < n; x += blockDim.x * gridDim.y) {
+            const int e = (int)(x / W), w = (int)(x % W);
+            while (e >= cr.as[k + 1]) k++;
+            const int c = act_cs[cr.act_off + e], d = act_d[cr.act_off + e];
+            const int64_t j = act_gt[cr.act_off + e];
+            const int64_t c0 = lp.child[k][j], base = lp.base[k + 1] + it.s0 + w;
+            float sum = 0.f;
+#pragma unroll 4
+            for (int a = 0; a < d; a++) sum += S[(c + a) * W + w];
+#pragma unroll 4
+            for (int a = 0; a < d; a++) {
+                float sb = sum > 0.f ? S[(c + a) * W + w] / sum : 1.f / (float)d;
+                out[base + lp.fgt[k + 1][c0 + a]] = sb;
             }
         }
     }
@@ -428,19 +430,29 @@ __global__ void k_sigma_sqdiff(const int32_t *__restrict__ root, int64_t m, cons
     }
 }
 
-// One level of the average strategies of every full slot from those of the solved slots: one warp
-// per GT node j, lanes over its full slots (consecutive output addresses); full slot s of root g
-// reads solved slot cidx0[score_off[g] + s] - csoff[g] of the same node.
-__global__ void k_expand_edges(const int32_t *__restrict__ root, int64_t m, const int64_t *__restrict__ fgt_off,
-                               const int64_t *__restrict__ cfgt_off, const int64_t *__restrict__ score_off,
-                               const int64_t *__restrict__ csoff, const int64_t *__restrict__ cidx0,
-                               const float *__restrict__ in, float *__restrict__ out) {
-    const int lane = threadIdx.x & 31;
-    const int64_t nw = (int64_t)gridDim.x * (blockDim.x >> 5);
-    for (int64_t j = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; j < m; j += nw) {
-        const int32_t g = root[j];
-        const int64_t q0 = fgt_off[j], ns = fgt_off[j + 1] - q0, c0 = cfgt_off[j] - csoff[g], s0 = score_off[g];
-        for (int64_t s = lane; s < ns; s += 32) out[q0 + s] = in[c0 + cidx0[s0 + s]];
+// The average strategies of every full slot from those of the solved slots: full slot s of root g reads solved
+// slot cidx0[score_off[g] + s] - csoff[g] of the same node.  All levels in one launch, eight lanes to a node (a
+// root has some 5 to 20 full slots); a launch per level with a warp to a node left most lanes idle and made the
+// exports of small rounds a chain of launches (sampled games through three rounds: 400 us, 295 so, 232 with the
+// solved slots' export shared out over blocks).
+struct ExpandLevels {
+    const int32_t *root[9];
+    const int64_t *fgt[9], *cfgt[9];
+    int64_t first[10];       // nodes of the levels 1 .. k-1
+    int64_t out[9], in[9];   // where a level's edges start
+};
+
+__global__ void k_expand_edges(const ExpandLevels L, const int64_t *__restrict__ score_off, const int64_t *__restrict__ csoff,
+                               const int64_t *__restrict__ cidx0, const float *__restrict__ in, float *__restrict__ out) {
+    const int lane = threadIdx.x & 7;
+    const int64_t step = (int64_t)gridDim.x * (blockDim.x >> 3);
+    for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 3; i < L.first[9]; i += step) {
+        int k = 1;
+        while (i >= L.first[k + 1]) k++;
+        const int64_t j = i - L.first[k];
+        const int32_t g = L.root[k][j];
+        const int64_t q0 = L.fgt[k][j], ns = L.fgt[k][j + 1] - q0, c0 = L.in[k] + L.cfgt[k][j] - csoff[g], s0 = score_off[g];
+        for (int64_t s = lane; s < ns; s += 8) out[L.out[k] + q0 + s] = in[c0 + cidx0[s0 + s]];
     }
 }
 
@@ -2023,7 +2035,9 @@ int export_sigma_solved(const pasur_tree *t, float *out_dev) {
         PASUR_CUDA(ctx, cudaGetLastError());
     }
     if (t->plan.n_items) {
-        unsigned g = (unsigned)std::min<int64_t>(t->plan.n_items, 65535);
+        // few items are large ones: share each out over blocks until the GPU is full
+        dim3 g((unsigned)std::min<int64_t>(t->plan.n_items, 65535));
+        g.y = (unsigned)std::min<int64_t>(64, (8 * (int64_t)ctx->num_sms + g.x - 1) / g.x);
         k_export_sigma<<<g, 256, 0, ctx->stream>>>(t->plan.items_d, t->plan.n_items, t->croots_d, t->act_cs, t->act_d,
                                                    t->act_gt, t->S, lp, out_dev);
         ctx->launches++;
@@ -2041,18 +2055,24 @@ int cfr_export_sigma(const pasur_tree *t, float *out_dev) {
     const size_t tb = sizeof(float) * (size_t)(ce + 1);
     PASUR_TRY(dev_alloc(ctx, (void **)&tmp, tb));
     int rc = export_sigma_solved(t, tmp);
-    // every full slot takes its solved slot's strategy, level by level
-    int64_t fb = 0, cb = 0;
-    for (int k = 1; k < 9 && rc == PASUR_OK; k++) {
-        if (t->M[k] > 0) {
-            k_expand_edges<<<grid_for(t->M[k] * 32, 256), 256, 0, ctx->stream>>>(
-                t->root[k], t->M[k], t->fgt_off[k], t->cfgt_off[k], t->score_off_d, t->csoff_d, t->cidx0_d, tmp + cb,
-                out_dev + fb);
-            ctx->launches++;
-            if (cudaGetLastError() != cudaSuccess) rc = set_err(ctx, PASUR_ECUDA, "k_expand_edges launch");
-        }
+    ExpandLevels L{};
+    int64_t fb = 0, cb = 0, nodes = 0;
+    for (int k = 1; k < 9; k++) {
+        L.root[k] = t->root[k];
+        L.fgt[k] = t->fgt_off[k];
+        L.cfgt[k] = t->cfgt_off[k];
+        L.first[k] = nodes;
+        L.out[k] = fb;
+        L.in[k] = cb;
+        nodes += t->M[k];
         fb += t->Q[k];
         cb += t->cQ[k];
+    }
+    L.first[9] = nodes;
+    if (rc == PASUR_OK && nodes > 0) {
+        k_expand_edges<<<grid_for(nodes * 8, 256), 256, 0, ctx->stream>>>(L, t->score_off_d, t->csoff_d, t->cidx0_d, tmp, out_dev);
+        ctx->launches++;
+        if (cudaGetLastError() != cudaSuccess) rc = set_err(ctx, PASUR_ECUDA, "k_expand_edges launch");
     }
     dev_free(ctx, tmp, tb);  // stream-ordered: freed after the expansion has read it
     return rc;

@@ -14,49 +14,95 @@
 namespace pasur {
 namespace {
 
-// leaf values of level 8 in FGT order (fp64)
-__global__ void k_leaf_f64(const GTState *__restrict__ st, const int32_t *__restrict__ root, int64_t m,
-                           const int64_t *__restrict__ fgt_off, const int64_t *__restrict__ score_off,
-                           const pasur_score *__restrict__ scores, bool final_round, const int64_t *__restrict__ lnk,
-                           const double *__restrict__ next, double *__restrict__ out) {
-    for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < m; j += (int64_t)gridDim.x * blockDim.x) {
-        const GTState s = st[j];
-        const int64_t q0 = fgt_off[j], ns = fgt_off[j + 1] - q0;
-        if (final_round) {
+// Everything the value passes read, per level.
+struct ValueArgs {
+    const GTState *leaf_state;
+    const int32_t *leaf_root;
+    const int64_t *child_off[8], *fgt_off[9];
+    const float *sigma[9];  // of the edges into level k
+    const int64_t *score_off;
+    const pasur_score *scores;
+    const int64_t *lnk;
+    const double *next;
+    double *v[9];
+    bool final_round;
+    int lanes_log2;  // lanes to a node, over its slots
+    int mode;        // 0 minimax, 1 Alex best response (Bob follows sigma), 2 Bob best response, 3 both sigma
+};
+
+// leaf values of level 8 in FGT order (fp64), leaves lo .. hi-1
+__device__ __forceinline__ void leaf_values(const ValueArgs &A, int64_t lo, int64_t hi) {
+    const int lanes = 1 << A.lanes_log2, lane = threadIdx.x & (lanes - 1), step = blockDim.x >> A.lanes_log2;
+    for (int64_t j = lo + (threadIdx.x >> A.lanes_log2); j < hi; j += step) {
+        const GTState s = A.leaf_state[j];
+        const int64_t q0 = A.fgt_off[8][j], ns = A.fgt_off[8][j + 1] - q0;
+        if (A.final_round) {
             const uint64_t r = cleanup_rus(s.rus, s.pool);
             const int d = rus_diff(r);
-            for (int64_t x = 0; x < ns; x++) {
-                const pasur_score sc = scores[score_off[root[j]] + x];
-                out[q0 + x] = (double)(d + bonus_points(bonus_after(sc.a_clubs, sc.b_clubs, sc.bonus, r)));
-            }
+            const pasur_score *sc = A.scores + A.score_off[A.leaf_root[j]];
+            for (int64_t x = lane; x < ns; x += lanes)
+                A.v[8][q0 + x] = (double)(d + bonus_points(bonus_after(sc[x].a_clubs, sc[x].b_clubs, sc[x].bonus, r)));
         } else {
             const double d = (double)rus_diff(s.rus);
-            for (int64_t x = 0; x < ns; x++) out[q0 + x] = __dadd_rn(d, next[lnk[q0 + x]]);
+            for (int64_t x = lane; x < ns; x += lanes) A.v[8][q0 + x] = __dadd_rn(d, A.next[A.lnk[q0 + x]]);
         }
     }
 }
 
-// mode 0 minimax, 1 Alex best response (Bob follows sigma), 2 Bob best response, 3 both sigma
-__global__ void k_value_level(int k, int64_t m, int mode, const int64_t *__restrict__ child_off,
-                              const int64_t *__restrict__ fgt_off, const int64_t *__restrict__ fgt_off_next,
-                              const float *__restrict__ sigma_next, const double *__restrict__ vnext,
-                              double *__restrict__ vout) {
+// values of nodes lo .. hi-1 of level k from those of level k+1
+__device__ __forceinline__ void level_values(const ValueArgs &A, int k, int64_t lo, int64_t hi) {
     const bool alex = (k & 1) == 0;
-    const bool opt = mode == 0 || (mode == 1 && alex) || (mode == 2 && !alex);
-    for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < m; j += (int64_t)gridDim.x * blockDim.x) {
+    const bool opt = A.mode == 0 || (A.mode == 1 && alex) || (A.mode == 2 && !alex);
+    const int64_t *child_off = A.child_off[k], *fgt_off = A.fgt_off[k], *fgt_off_next = A.fgt_off[k + 1];
+    const float *sigma = A.sigma[k + 1];
+    const double *vnext = A.v[k + 1];
+    double *vout = A.v[k];
+    const int lanes = 1 << A.lanes_log2, lane = threadIdx.x & (lanes - 1), step = blockDim.x >> A.lanes_log2;
+    for (int64_t j = lo + (threadIdx.x >> A.lanes_log2); j < hi; j += step) {
         const int64_t cb = child_off[j], ce = child_off[j + 1];
         const int64_t q0 = fgt_off[j], ns = fgt_off[j + 1] - q0;
-        for (int64_t s = 0; s < ns; s++) {
+        for (int64_t s = lane; s < ns; s += lanes) {
             double best = 0.0, ev = 0.0;
+#pragma unroll 4
             for (int64_t c = cb; c < ce; c++) {
                 const int64_t q = fgt_off_next[c] + s;
                 const double v = vnext[q];
                 if (c == cb || (alex ? v > best : v < best)) best = v;
-                if (!opt) ev = __dadd_rn(ev, __dmul_rn((double)sigma_next[q], v));
+                if (!opt) ev = __dadd_rn(ev, __dmul_rn((double)sigma[q], v));
             }
             vout[q0 + s] = opt ? best : ev;
         }
     }
+}
+
+// Values of levels top .. 8 (bottom = 8: from the leaves on) or top .. bottom, a block per range of level `top`'s m
+// nodes: their descendants are a range of every level below, so that a block needs no other's values.  One launch
+// from `split_level` down, one block for the levels above it.  Bound by launches and by the chains of dependent loads
+// (child range, slot offset, value), hence several lanes to a node and four children in flight.  Both players' best
+// responses through the last four rounds of a deal (with the strategies' exports): 1.4 ms with a launch per level and a
+// thread to a node, 0.7 so.
+__global__ void __launch_bounds__(1024) k_values(const ValueArgs A, int top, int bottom, int64_t m) {
+    __shared__ int64_t lo[9], hi[9];
+    if (threadIdx.x < 2) {
+        int64_t x = m * (int64_t)(blockIdx.x + threadIdx.x) / gridDim.x;
+        int64_t *at = threadIdx.x ? hi : lo;
+        at[top] = x;
+        for (int k = top; k < bottom; k++) at[k + 1] = x = A.child_off[k][x];
+    }
+    __syncthreads();
+    if (bottom == 8) leaf_values(A, lo[8], hi[8]);
+    for (int k = bottom - 1; k >= top; k--) {
+        __syncthreads();
+        level_values(A, k, lo[k], hi[k]);
+    }
+}
+
+// first level with two nodes to an SM: the tree below it splits over the GPU, and the levels above it, of fewer nodes
+// each, are a few passes of one block
+int split_level(const pasur_tree *t) {
+    int k = 0;
+    while (k < 7 && t->M[k] < 2 * t->ctx->num_sms) k++;
+    return k;
 }
 
 unsigned grid_of(int64_t n) { return (unsigned)std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, 1 << 20)); }
@@ -115,20 +161,37 @@ int value_levels(pasur_tree *t, int mode, const float *sigma, const double *next
             nx = d;
         }
     }
-    for (int k = 0; k < 9; k++) al((void **)&v[k], sizeof(double) * (size_t)(t->Q[k] + 1));
-    if (rc == PASUR_OK && t->M[8] > 0) {
-        k_leaf_f64<<<grid_of(t->M[8]), 256, 0, ctx->stream>>>(t->st[8], t->root[8], t->M[8], t->fgt_off[8], t->score_off_d,
-                                                              t->scores_d, t->final_round, t->lnk_d, nx, v[8]);
-        ctx->launches++;
-        if (cudaGetLastError() != cudaSuccess) rc = set_err(ctx, PASUR_ECUDA, "k_leaf_f64 launch");
+    int64_t nv = 0;
+    for (int k = 0; k < 9; k++) nv += t->Q[k] + 1;
+    double *values = nullptr;
+    al((void **)&values, sizeof(double) * (size_t)nv);
+    ValueArgs A{};
+    for (int k = 0; k < 9; k++) {
+        A.v[k] = v[k] = values;
+        values += t->Q[k] + 1;
+        A.fgt_off[k] = t->fgt_off[k];
+        if (k < 8) A.child_off[k] = t->child_off[k];
+        if (k > 0 && sg) A.sigma[k] = sg + base[k];
     }
-    for (int k = 7; k >= 0 && rc == PASUR_OK; k--) {
-        if (t->M[k] == 0) continue;
-        k_value_level<<<grid_of(t->M[k]), 256, 0, ctx->stream>>>(k, t->M[k], mode, t->child_off[k], t->fgt_off[k],
-                                                                 t->fgt_off[k + 1], sg ? sg + base[k + 1] : nullptr, v[k + 1],
-                                                                 v[k]);
+    A.leaf_state = t->st[8];
+    A.leaf_root = t->root[8];
+    A.score_off = t->score_off_d;
+    A.scores = t->scores_d;
+    A.lnk = t->lnk_d;
+    A.next = nx;
+    A.final_round = t->final_round;
+    A.mode = mode;
+    while (A.lanes_log2 < 3 && t->Q[8] > t->M[8] << A.lanes_log2) A.lanes_log2++;  // the leaves' slots on average
+    if (rc == PASUR_OK && t->M[0] > 0) {
+        const int top = split_level(t);
+        const int64_t blocks = std::min<int64_t>(t->M[top], 8 * (int64_t)ctx->num_sms);
+        k_values<<<(unsigned)blocks, 256, 0, ctx->stream>>>(A, top, 8, t->M[top]);
         ctx->launches++;
-        if (cudaGetLastError() != cudaSuccess) rc = set_err(ctx, PASUR_ECUDA, "k_value_level launch");
+        if (top > 0) {
+            k_values<<<1, 1024, 0, ctx->stream>>>(A, 0, top, t->M[0]);
+            ctx->launches++;
+        }
+        if (cudaGetLastError() != cudaSuccess) rc = set_err(ctx, PASUR_ECUDA, "k_values launch");
     }
     *sg_out = sg;
     return rc;

@@ -86,3 +86,44 @@ def test_solved_strategy_exploitability_is_small(ctx):
             t.free()
     assert gaps[0] >= 0 and gaps[1] >= 0
     assert gaps[1] < gaps[0]
+
+
+@pytest.mark.parametrize("first", [2, 3, 4])
+def test_values_over_tree_shapes(ctx, first):
+    """A round of one root and one score slot (its tree split over blocks below the top levels)
+    and the rounds after it (split at their roots): the on-policy values against a
+    level-by-level numpy pass over the exported tree (sums of products to rounding), and every
+    mode with the solver's own strategies against the same strategies handed in (equal)."""
+    from paper_2508_06559_gb300 import pasur as P
+    deck = O.deal(5)
+    cfg, roots, trees = P.pasur_config_default(iters=20), None, []
+    for rnd in range(first, 6):
+        t = ctx.pasur_build_round(deck, rnd, [mask_ids(deck[:4])] if roots is None else roots[0])
+        t.unfold_single() if roots is None else t.pasur_unfold(roots[1], roots[2])
+        if rnd < 5:
+            roots = t.pasur_next_roots()
+            lnk = roots[3] if rnd == first else lnk
+        trees.append(t)
+    nv, sigmas = None, []
+    for t in reversed(trees):
+        t.pasur_cfr_iterate(cfg, nv)
+        sigmas.insert(0, t.pasur_avg_strategy())
+        nv = t.pasur_round_utilities()
+    for mode in (O.MINIMAX, O.BR_ALEX, O.BR_BOB, O.ON_POLICY):
+        assert np.array_equal(P.chain_values(trees, mode), P.chain_values(trees, mode, sigmas))
+    nxt = P.chain_values(trees[1:], O.ON_POLICY)
+    want = P.chain_values(trees, O.ON_POLICY)
+    t = ctx.pasur_build_round(deck, first, [mask_ids(deck[:4])])
+    t.unfold_single()
+    t.pasur_next_roots()
+    t.pasur_cfr_iterate(P.pasur_config_default(iters=0), np.zeros(len(nxt), np.float32))
+    gt, fgt = t.pasur_tree_sizes()
+    assert np.array_equal(gt, fgt)  # one slot: an FGT node is a GT node
+    val = t.pasur_leaf_values().astype(np.float64) + nxt[lnk]  # the round's difference + the next round
+    for k in range(7, -1, -1):
+        s = sigmas[0][fgt[1:k + 1].sum():fgt[1:k + 2].sum()].astype(np.float64)
+        nchild = t.pasur_export_level(k)["nchild"]
+        val = np.add.reduceat(s * val, np.concatenate([[0], np.cumsum(nchild)[:-1]]))
+    assert np.allclose(val, want, rtol=1e-12, atol=1e-12)
+    for x in trees + [t]:
+        x.free()
