@@ -170,18 +170,27 @@ __global__ void k_root_bounds(int64_t n_roots, OffPtrs co, int64_t *__restrict__
     }
 }
 
-// first FGT node of every GT node of one level: a root's nodes are consecutive, each with the root's
-// slots (base[g]: the root's first, bounds[9 g + k]: its first GT node); out[m] = total
-__global__ void k_slot_offsets(const int32_t *__restrict__ root, int64_t m, int k, const int64_t *__restrict__ bounds,
-                               const int64_t *__restrict__ base, const int64_t *__restrict__ slot_off, int64_t n_roots,
-                               int64_t *__restrict__ out) {
-    for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j <= m; j += (int64_t)gridDim.x * blockDim.x) {
-        if (j == m) {
-            out[j] = base[n_roots];
+// First FGT node of every GT node of all levels (one launch; nine of them were a quarter of a small round's
+// unfolding): a root's nodes are consecutive, each with the root's slots (base: per level the roots' first,
+// bounds[9 g + k]: the root's first GT node); the element after a level's last = its total.
+struct SlotLevels {
+    const int32_t *root[9];
+    int64_t *out[9];
+    int64_t off[10];  // first element of the level, M + 1 each
+};
+
+__global__ void k_slot_offsets(const SlotLevels L, const int64_t *__restrict__ bounds, const int64_t *__restrict__ bases,
+                               const int64_t *__restrict__ slot_off, int64_t n_roots) {
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < L.off[9]; i += (int64_t)gridDim.x * blockDim.x) {
+        int k = 0;
+        while (i >= L.off[k + 1]) k++;
+        const int64_t j = i - L.off[k], *base = bases + k * (n_roots + 1);
+        if (i == L.off[k + 1] - 1) {
+            L.out[k][j] = base[n_roots];
             continue;
         }
-        const int32_t g = root[j];
-        out[j] = base[g] + (j - bounds[9 * g + k]) * (slot_off[g + 1] - slot_off[g]);
+        const int32_t g = L.root[k][j];
+        L.out[k][j] = base[g] + (j - bounds[9 * g + k]) * (slot_off[g + 1] - slot_off[g]);
     }
 }
 
@@ -360,8 +369,8 @@ int build_levels(pasur_tree *t, const uint64_t *root_pools_dev) {
 }
 
 // The FGT levels over given slots per root (slot_off: prefix over the roots, host and device): sizes
-// from the roots' node counts on the host, then every level's offsets in one launch each, without a
-// scan or a synchronisation.
+// from the roots' node counts on the host, then every level's offsets in one launch, without a scan or
+// a synchronisation.
 static int slot_levels(pasur_tree *t, const std::vector<int64_t> &slot_off, const int64_t *slot_off_d, int64_t **off, int64_t *sizes) {
     pasur_ctx *ctx = t->ctx;
     const int64_t nr = t->n_roots;
@@ -380,12 +389,15 @@ static int slot_levels(pasur_tree *t, const std::vector<int64_t> &slot_off, cons
     int rc = PASUR_OK;
     cudaError_t e = cudaMemcpyAsync(base_d, base.data(), bytes, cudaMemcpyHostToDevice, ctx->stream);
     if (e != cudaSuccess) rc = cuda_err(ctx, e, "slot_levels: upload");
+    SlotLevels L{};
     for (int k = 0; k < 9 && rc == PASUR_OK; k++) {
-        const int64_t m = t->M[k];
-        if (!off[k]) rc = tree_alloc(t, (void **)&off[k], sizeof(int64_t) * (size_t)(m + 1));
-        if (rc != PASUR_OK) break;
-        k_slot_offsets<<<grid_for(m + 1, 256), 256, 0, ctx->stream>>>(t->root[k], m, k, t->bounds_d, base_d + (size_t)k * (size_t)(nr + 1),
-                                                                     slot_off_d, nr, off[k]);
+        if (!off[k]) rc = tree_alloc(t, (void **)&off[k], sizeof(int64_t) * (size_t)(t->M[k] + 1));
+        L.root[k] = t->root[k];
+        L.out[k] = off[k];
+        L.off[k + 1] = L.off[k] + t->M[k] + 1;
+    }
+    if (rc == PASUR_OK) {
+        k_slot_offsets<<<grid_for(L.off[9], 256), 256, 0, ctx->stream>>>(L, t->bounds_d, base_d, slot_off_d, nr);
         ctx->launches++;
         e = cudaGetLastError();
         if (e != cudaSuccess) rc = cuda_err(ctx, e, "k_slot_offsets");

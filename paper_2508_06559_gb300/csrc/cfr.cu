@@ -456,22 +456,47 @@ __global__ void k_expand_edges(const ExpandLevels L, const int64_t *__restrict__
     }
 }
 
-// chain[j] = 1 when the subtree of j is one path of forced moves (leaves included)
-__global__ void k_chain(const int64_t *child_off, int64_t m, const uint8_t *chain_next, uint8_t *chain) {
-    for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < m; j += (int64_t)gridDim.x * blockDim.x) {
-        int64_t c0 = child_off[j];
-        chain[j] = (child_off[j + 1] - c0 == 1 && chain_next[c0]) ? 1 : 0;
-    }
+// The layout's kernels run over all levels at once: level k's M[k] nodes and one more element (for the scans'
+// totals) at off[k].  With a launch, or three, per level, 121 launches of some 3 us made up most of a small round's
+// set-up (1.15 ms of the 5.85 of a final round of 1000 iterations; 0.9 of 5.6 so).
+struct LayoutLevels {
+    const int64_t *child[9], *parent[9];  // child[8], parent[0]: unused
+    const int32_t *root[9];
+    int64_t off[10];
+};
+
+// level of element i, i - off in j; nodes of that level
+__device__ __forceinline__ int level_of(const LayoutLevels &L, int64_t i, int64_t &j) {
+    int k = 0;
+    while (i >= L.off[k + 1]) k++;
+    j = i - L.off[k];
+    return k;
 }
 
-// local and active flags of level k from level k-1 (local: the root, or the parent is active;
-// active: local, not a chain, not a leaf)
-__global__ void k_flags(const int64_t *parent, int64_t m, const int32_t *active_prev, const uint8_t *chain, bool leaves,
-                        int32_t *local, int32_t *active) {
-    for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < m; j += (int64_t)gridDim.x * blockDim.x) {
-        int32_t l = parent ? active_prev[parent[j]] : 1;
-        local[j] = l;
-        active[j] = (l && !leaves && !chain[j]) ? 1 : 0;
+// Local and active flags.  A node is active when its subtree is more than one path of forced moves (then none of its
+// ancestors' is one either); local when it is a root or its parent is active.
+__global__ void k_flags(const LayoutLevels L, int32_t *__restrict__ local, int32_t *__restrict__ active) {
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < L.off[9]; i += (int64_t)gridDim.x * blockDim.x) {
+        int64_t j;
+        const int k = level_of(L, i, j);
+        if (i == L.off[k + 1] - 1) {
+            local[i] = active[i] = 0;
+            continue;
+        }
+        bool path = true;
+        int64_t x = j;
+        for (int kk = k; kk < 8 && path; kk++) {
+            const int64_t c = L.child[kk][x];
+            path = L.child[kk][x + 1] - c == 1;
+            x = c;
+        }
+        active[i] = !path;
+        bool loc = k == 0 || !path;
+        if (!loc) {
+            const int64_t p = L.parent[k][j];
+            loc = L.child[k - 1][p + 1] - L.child[k - 1][p] > 1;
+        }
+        local[i] = loc;
     }
 }
 
@@ -490,43 +515,56 @@ __global__ void k_root_ranks(const int64_t *bounds, int64_t n_roots, RankPtrs rp
         }
 }
 
-struct ChildPtrs {
-    const int64_t *p[9];
-};
-
-__global__ void k_fill_layout(int k, int64_t m, const int32_t *root, const int32_t *local, const int32_t *active,
-                              const int64_t *loc_rank, const int64_t *act_rank, const int64_t *loc_rank_next,
-                              const int64_t *loc_rank_prev, const int64_t *parent, ChildPtrs co, const int64_t *fgt_off8,
-                              const CfrRoot *roots, int64_t *loc_tq, int32_t *act_li, int32_t *act_pl, int32_t *act_cs,
-                              uint16_t *act_d, int64_t *act_gt, uint64_t *act_key, int32_t *act_rk, int32_t *err) {
-    for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < m; j += (int64_t)gridDim.x * blockDim.x) {
-        if (!local[j]) continue;
-        const CfrRoot &cr = roots[root[j]];
-        const int64_t li = cr.ls[k] + (loc_rank[j] - cr.locbase[k]);
-        if (active[j]) {
+__global__ void k_fill_layout(const LayoutLevels L, const int32_t *__restrict__ local, const int32_t *__restrict__ active,
+                              const int64_t *__restrict__ loc_rank, const int64_t *__restrict__ act_rank,
+                              const int64_t *__restrict__ fgt_off8, const CfrRoot *__restrict__ roots, int64_t *loc_tq, int32_t *act_li,
+                              int32_t *act_pl, int32_t *act_cs, uint16_t *act_d, int64_t *act_gt, uint64_t *act_key, int32_t *act_rk,
+                              int32_t *err) {
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < L.off[9]; i += (int64_t)gridDim.x * blockDim.x) {
+        if (!local[i]) continue;
+        int64_t j;
+        const int k = level_of(L, i, j);
+        const int32_t g = L.root[k][j];
+        const CfrRoot &cr = roots[g];
+        const int64_t li = cr.ls[k] + (loc_rank[i] - cr.locbase[k]);
+        if (active[i]) {
             loc_tq[cr.loc_off + li] = -1;
-            const int64_t e = cr.as[k] + (act_rank[j] - cr.actbase[k]);
-            const int64_t c0 = co.p[k][j], d = co.p[k][j + 1] - c0;
+            const int64_t e = cr.act_off + cr.as[k] + (act_rank[i] - cr.actbase[k]);
+            const int64_t c0 = L.child[k][j], d = L.child[k][j + 1] - c0;
             if (d > 65535) atomicOr(err, 2);
-            act_li[cr.act_off + e] = (int32_t)li;
-            act_pl[cr.act_off + e] =
-                k == 0 ? -1 : (int32_t)(cr.ls[k - 1] + (loc_rank_prev[parent[j]] - cr.locbase[k - 1]));
-            act_cs[cr.act_off + e] = (int32_t)(cr.ls[k + 1] + (loc_rank_next[c0] - cr.locbase[k + 1]));
-            act_d[cr.act_off + e] = (uint16_t)d;
-            act_gt[cr.act_off + e] = j;
+            act_li[e] = (int32_t)li;
+            act_pl[e] = k == 0 ? -1 : (int32_t)(cr.ls[k - 1] + (loc_rank[L.off[k - 1] + L.parent[k][j]] - cr.locbase[k - 1]));
+            act_cs[e] = (int32_t)(cr.ls[k + 1] + (loc_rank[L.off[k + 1] + c0] - cr.locbase[k + 1]));
+            act_d[e] = (uint16_t)d;
+            act_gt[e] = j;
             // sort key: the (root, level) segment, then degree descending
-            act_key[cr.act_off + e] = ((uint64_t)(cr.act_off + cr.as[k]) << 16) | (uint64_t)(0xFFFF - (d > 0xFFFF ? 0xFFFF : d));
-            act_rk[cr.act_off + e] = (root[j] << 3) | k;
+            act_key[e] = ((uint64_t)(cr.act_off + cr.as[k]) << 16) | (uint64_t)(0xFFFF - (d > 0xFFFF ? 0xFFFF : d));
+            act_rk[e] = (g << 3) | k;
         } else {
             int64_t x = j;
-            for (int kk = k; kk < 8; kk++) x = co.p[kk][x];  // follow the forced moves to the leaf
+            for (int kk = k; kk < 8; kk++) x = L.child[kk][x];  // follow the forced moves to the leaf
             loc_tq[cr.loc_off + li] = fgt_off8[x];
         }
     }
 }
 
-__global__ void k_widen_degrees(const uint16_t *d, int64_t n, int32_t *out) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) out[i] = d[i];
+// the entries in sorted order
+struct EntryArrays {
+    int32_t *li, *pl, *cs, *rk;
+    uint16_t *d;
+    int64_t *gt;
+};
+
+__global__ void k_gather_entries(const EntryArrays in, const int64_t *__restrict__ perm, int64_t n, EntryArrays out, int32_t *deg) {
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t e = perm[i];
+        out.li[i] = in.li[e];
+        out.pl[i] = in.pl[e];
+        out.cs[i] = in.cs[e];
+        out.rk[i] = in.rk[e];
+        out.gt[i] = in.gt[e];
+        deg[i] = out.d[i] = in.d[e];
+    }
 }
 
 // pos: exclusive scan of the degrees over the sorted entries.  The children of the entries of
@@ -680,11 +718,6 @@ __global__ void k_iota(int64_t *out, int64_t n) {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) out[i] = i;
 }
 
-template <typename T>
-__global__ void k_gather(const T *in, const int64_t *perm, int64_t n, T *out) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) out[i] = in[perm[i]];
-}
-
 unsigned grid_for(int64_t threads, int block) {
     int64_t b = (threads + block - 1) / block;
     if (b < 1) b = 1;
@@ -797,45 +830,35 @@ int build_layout(pasur_tree *t) {
             for (auto &x : *v) dev_free(c, x.first, x.second);
         }
     } guard{ctx, &tmp};
-    uint8_t *chain[9];
-    int32_t *local[9], *active[9];
-    int64_t *lrank[9], *arank[9];
-    int64_t *ranks = nullptr;
+    int32_t *local = nullptr, *active = nullptr;
+    int64_t *lrank = nullptr, *arank = nullptr, *ranks = nullptr;
     const int64_t nr = t->n_roots;
+    LayoutLevels L{};
+    for (int k = 0; k < 9; k++) {
+        L.child[k] = k < 8 ? t->child_off[k] : nullptr;
+        L.parent[k] = k > 0 ? t->parent[k] : nullptr;
+        L.root[k] = t->root[k];
+        L.off[k + 1] = L.off[k] + t->M[k] + 1;
+    }
+    const int64_t n_all = L.off[9];
     {
         Slab sl;
-        for (int k = 0; k < 9; k++) {
-            sl.add(&chain[k], t->M[k]);
-            sl.add(&local[k], t->M[k]);
-            sl.add(&active[k], t->M[k]);
-            sl.add(&lrank[k], t->M[k]);
-            sl.add(&arank[k], t->M[k]);
-        }
+        sl.add(&local, n_all);
+        sl.add(&active, n_all);
+        sl.add(&lrank, n_all);
+        sl.add(&arank, n_all);
         sl.add(&ranks, 18 * (nr + 1));
         PASUR_TRY(sl.alloc(ctx, tmp));
     }
-    PASUR_CUDA(ctx, cudaMemsetAsync(chain[8], 1, (size_t)t->M[8] + 1, ctx->stream));
-    for (int k = 7; k >= 0; k--) {
-        if (t->M[k] == 0) continue;
-        k_chain<<<grid_for(t->M[k], 256), 256, 0, ctx->stream>>>(t->child_off[k], t->M[k], chain[k + 1], chain[k]);
-        ctx->launches++;
-        PASUR_CUDA(ctx, cudaGetLastError());
-    }
-    for (int k = 0; k < 9; k++) {
-        if (t->M[k] > 0) {
-            k_flags<<<grid_for(t->M[k], 256), 256, 0, ctx->stream>>>(k ? t->parent[k] : nullptr, t->M[k],
-                                                                    k ? active[k - 1] : nullptr, chain[k], k == 8,
-                                                                    local[k], active[k]);
-            ctx->launches++;
-            PASUR_CUDA(ctx, cudaGetLastError());
-        }
-        PASUR_TRY(exclusive_scan_i32(ctx, local[k], lrank[k], t->M[k]));
-        PASUR_TRY(exclusive_scan_i32(ctx, active[k], arank[k], t->M[k]));
-    }
+    k_flags<<<grid_for(n_all, 256), 256, 0, ctx->stream>>>(L, local, active);
+    ctx->launches++;
+    PASUR_CUDA(ctx, cudaGetLastError());
+    PASUR_TRY(exclusive_scan_i32(ctx, local, lrank, n_all));
+    PASUR_TRY(exclusive_scan_i32(ctx, active, arank, n_all));
     RankPtrs rp;
     for (int k = 0; k < 9; k++) {
-        rp.loc[k] = lrank[k];
-        rp.act[k] = arank[k];
+        rp.loc[k] = lrank + L.off[k];
+        rp.act[k] = arank + L.off[k];
     }
     k_root_ranks<<<grid_for(nr + 1, 256), 256, 0, ctx->stream>>>(t->bounds_d, nr, rp, ranks);
     ctx->launches++;
@@ -878,78 +901,54 @@ int build_layout(pasur_tree *t) {
     PASUR_TRY(tree_alloc(t, (void **)&t->act_cs, sizeof(int32_t) * (size_t)(act_off + 1)));
     PASUR_TRY(tree_alloc(t, (void **)&t->act_d, sizeof(uint16_t) * (size_t)(act_off + 1)));
     PASUR_TRY(tree_alloc(t, (void **)&t->act_gt, sizeof(int64_t) * (size_t)(act_off + 1)));
+    // the entries as found (f) and what orders them; once the ranks have been read, the sort's permutation, the
+    // degrees and their scan take their place
     uint64_t *act_key = nullptr;
-    int64_t *perm = nullptr, *pos = nullptr, *lmap = nullptr;
-    int32_t *t32 = nullptr, *act_rk = nullptr, *deg = nullptr;
-    uint16_t *t16 = nullptr;
-    int64_t *t64 = nullptr;
+    EntryArrays f{}, sorted{t->act_li, t->act_pl, t->act_cs, nullptr, t->act_d, t->act_gt};
+    int64_t *f_tq = nullptr, *lmap = nullptr;
     {
         Slab sl;
         sl.add(&act_key, act_off);
-        sl.add(&perm, act_off);
-        sl.add(&t32, act_off);
-        sl.add(&t16, act_off);
-        sl.add(&t64, act_off);
-        sl.add(&act_rk, act_off);
-        sl.add(&deg, act_off);
-        sl.add(&pos, act_off);
+        sl.add(&f.li, act_off);
+        sl.add(&f.pl, act_off);
+        sl.add(&f.cs, act_off);
+        sl.add(&f.rk, act_off);
+        sl.add(&f.d, act_off);
+        sl.add(&f.gt, act_off);
+        sl.add(&sorted.rk, act_off);
+        sl.add(&f_tq, loc_off);
         sl.add(&lmap, loc_off);
         PASUR_TRY(sl.alloc(ctx, tmp));
     }
-    ChildPtrs co;
-    for (int k = 0; k < 8; k++) co.p[k] = t->child_off[k];
-    co.p[8] = nullptr;
+    int64_t *perm = lrank, *pos = arank;
+    int32_t *deg = local, *act_rk = sorted.rk;
     PASUR_CUDA(ctx, cudaMemsetAsync(ctx->errflag, 0, sizeof(int32_t), ctx->stream));
-    for (int k = 0; k < 9; k++) {
-        if (t->M[k] == 0) continue;
-        k_fill_layout<<<grid_for(t->M[k], 256), 256, 0, ctx->stream>>>(
-            k, t->M[k], t->root[k], local[k], active[k], lrank[k], arank[k], k < 8 ? lrank[k + 1] : nullptr,
-            k > 0 ? lrank[k - 1] : nullptr, k > 0 ? t->parent[k] : nullptr, co, t->cfgt_off[8], t->croots_d, t->loc_tq,
-            t->act_li, t->act_pl, t->act_cs, t->act_d, t->act_gt, act_key, act_rk, ctx->errflag);
-        ctx->launches++;
-        PASUR_CUDA(ctx, cudaGetLastError());
-    }
+    k_fill_layout<<<grid_for(n_all, 256), 256, 0, ctx->stream>>>(L, local, active, lrank, arank, t->cfgt_off[8], t->croots_d, f_tq, f.li,
+                                                                f.pl, f.cs, f.d, f.gt, act_key, f.rk, ctx->errflag);
+    ctx->launches++;
+    PASUR_CUDA(ctx, cudaGetLastError());
     int32_t ef = 0;
     PASUR_CUDA(ctx, cudaMemcpyAsync(&ef, ctx->errflag, sizeof ef, cudaMemcpyDeviceToHost, ctx->stream));
     PASUR_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
     if (ef) return set_err(ctx, PASUR_EOVERFLOW, "a node has more than 65535 legal moves");
     // order the active entries of every (root, level) by degree, largest first, so that the lanes
     // of a warp mostly run the same unrolled path
-    if (act_off > 1) {
+    if (act_off > 0) {
         k_iota<<<grid_for(act_off, 256), 256, 0, ctx->stream>>>(perm, act_off);
         ctx->launches++;
         PASUR_CUDA(ctx, cudaGetLastError());
         int bits = 16;
         while (((int64_t)1 << (bits - 16)) <= act_off) bits++;
         PASUR_TRY(radix_sort_pairs(ctx, act_key, perm, act_off, bits));
-        int32_t *arr32[3] = {t->act_li, t->act_pl, t->act_cs};
-        for (int i = 0; i < 3; i++) {
-            k_gather<int32_t><<<grid_for(act_off, 256), 256, 0, ctx->stream>>>(arr32[i], perm, act_off, t32);
-            ctx->launches++;
-            PASUR_CUDA(ctx, cudaGetLastError());
-            PASUR_CUDA(ctx, cudaMemcpyAsync(arr32[i], t32, sizeof(int32_t) * (size_t)act_off, cudaMemcpyDeviceToDevice, ctx->stream));
-        }
-        k_gather<uint16_t><<<grid_for(act_off, 256), 256, 0, ctx->stream>>>(t->act_d, perm, act_off, t16);
+        k_gather_entries<<<grid_for(act_off, 256), 256, 0, ctx->stream>>>(f, perm, act_off, sorted, deg);
         ctx->launches++;
         PASUR_CUDA(ctx, cudaGetLastError());
-        PASUR_CUDA(ctx, cudaMemcpyAsync(t->act_d, t16, sizeof(uint16_t) * (size_t)act_off, cudaMemcpyDeviceToDevice, ctx->stream));
-        k_gather<int64_t><<<grid_for(act_off, 256), 256, 0, ctx->stream>>>(t->act_gt, perm, act_off, t64);
-        ctx->launches++;
-        PASUR_CUDA(ctx, cudaGetLastError());
-        PASUR_CUDA(ctx, cudaMemcpyAsync(t->act_gt, t64, sizeof(int64_t) * (size_t)act_off, cudaMemcpyDeviceToDevice, ctx->stream));
-        k_gather<int32_t><<<grid_for(act_off, 256), 256, 0, ctx->stream>>>(act_rk, perm, act_off, t32);
-        ctx->launches++;
-        PASUR_CUDA(ctx, cudaGetLastError());
-        PASUR_CUDA(ctx, cudaMemcpyAsync(act_rk, t32, sizeof(int32_t) * (size_t)act_off, cudaMemcpyDeviceToDevice, ctx->stream));
     }
     // renumber the local nodes of every level after the first in the order of their parents'
     // entries: the children of consecutive entries become consecutive nodes (a warp's child
     // accesses fall on few shared-memory banks and few device-memory sectors).  Child a of an
     // entry stays child a, so every node's arithmetic is unchanged.
     if (act_off > 0) {
-        k_widen_degrees<<<grid_for(act_off, 256), 256, 0, ctx->stream>>>(t->act_d, act_off, deg);
-        ctx->launches++;
-        PASUR_CUDA(ctx, cudaGetLastError());
         PASUR_TRY(exclusive_scan_i32(ctx, deg, pos, act_off));
         k_renumber_map<<<grid_for(act_off, 256), 256, 0, ctx->stream>>>(act_off, act_rk, t->croots_d, pos, t->act_cs, t->act_d,
                                                                         lmap);
@@ -963,13 +962,11 @@ int build_layout(pasur_tree *t) {
         ctx->launches++;
         PASUR_CUDA(ctx, cudaGetLastError());
         // terminal leaf links follow their nodes
-        int64_t *tq_old = nullptr;
-        PASUR_TRY(dev_alloc(ctx, (void **)&tq_old, sizeof(int64_t) * (size_t)(loc_off + 1)));
-        tmp.push_back({tq_old, sizeof(int64_t) * (size_t)(loc_off + 1)});
-        PASUR_CUDA(ctx, cudaMemcpyAsync(tq_old, t->loc_tq, sizeof(int64_t) * (size_t)loc_off, cudaMemcpyDeviceToDevice, ctx->stream));
-        k_renumber_tq<<<grid_for(loc_off, 256), 256, 0, ctx->stream>>>(loc_off, lmap, tq_old, t->loc_tq);
+        k_renumber_tq<<<grid_for(loc_off, 256), 256, 0, ctx->stream>>>(loc_off, lmap, f_tq, t->loc_tq);
         ctx->launches++;
         PASUR_CUDA(ctx, cudaGetLastError());
+    } else if (loc_off > 0) {
+        PASUR_CUDA(ctx, cudaMemcpyAsync(t->loc_tq, f_tq, sizeof(int64_t) * (size_t)loc_off, cudaMemcpyDeviceToDevice, ctx->stream));
     }
     PASUR_TRY(build_block_order(t, act_rk));
     PASUR_CUDA(ctx, cudaStreamSynchronize(ctx->stream));

@@ -222,11 +222,7 @@ int radix_sort_pairs(pasur_ctx *ctx, uint64_t *keys, int64_t *vals, int64_t n, i
         if (e == cudaSuccess) e = cudaMemcpyAsync(vals, va, vb, cudaMemcpyDeviceToDevice, ctx->stream);
         if (e != cudaSuccess) rc = cuda_err(ctx, e, "radix sort copy-back");
     }
-    if (rc == PASUR_OK) {
-        cudaError_t e = cudaStreamSynchronize(ctx->stream);
-        if (e != cudaSuccess) rc = cuda_err(ctx, e, "radix sort");
-    }
-    dev_free(ctx, k2, kb);
+    dev_free(ctx, k2, kb);  // stream-ordered
     dev_free(ctx, v2, vb);
     dev_free(ctx, counts, cb);
     dev_free(ctx, offs, ob);
