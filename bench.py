@@ -34,7 +34,7 @@ WORKLOADS = {
     "rounds_4_5": (4, "rounds 5-6 (0-based 4-5) of one seeded deal, round 5 unfolded over every score round 4 reaches"),
     "final_round": (5, "final round of one seeded deal as a standalone round, score (0,0,0,0)"),
     "batch64": (3, "64 seeded deals (seeds S..S+63), rounds 4-6 (0-based 3-5) of each from the standalone root, "
-                   "solved together: one merged persistent launch per round and size class under a CUDA graph"),
+                   "solved together: one merged persistent launch per round and slot count under a CUDA graph"),
     "surrogate64": (0, "64 seeded deals (seeds S..S+63): rounds 1-3 (0-based 0-2) solved in one batch with the "
                        "leaves of round 3 valued by the trained surrogate at the round-4 roots; 10 % of every "
                        "deal's round-4 pools solved exactly (rounds 4-6 from those roots only), a copy of the "
@@ -455,7 +455,7 @@ def _record(name: str):
 
 
 def recorded_traffic(workload: str, seed: int):
-    """DRAM bytes of the CFR kernels (every k_cfr_items and k_cfr_cluster launch of one solve) per
+    """DRAM bytes of the CFR kernels (every k_cfr_block and k_cfr_cluster launch of one solve) per
     step from the committed ncu record of this workload, while the kernel source is unchanged
     since the capture; else None."""
     rec = _record(f"cfr_{workload}_seed{seed}.traffic.json")
@@ -604,7 +604,7 @@ def run_ours(args, rank, world, dist):
     kernel_ms = statistics.mean(kern_ms)
     solved = work[-1].get("solved", updates)
     swept = work[-1].get("swept", updates)
-    # dominant kernel: the CFR kernel (k_cfr_items, one launch per size class and round); the
+    # dominant kernel: the CFR kernel (k_cfr_block, one launch per slot count and round); the
     # algorithmic traffic of CFR is the regret and strategy-sum read + write of every edge that
     # carries CFR state, per iteration (the swept node-updates)
     ach_gbs = ALG_BYTES_PER_UPDATE * swept / (kernel_ms / 1e3) / 1e9
@@ -632,9 +632,9 @@ def run_ours(args, rank, world, dist):
                           "are resolved once")},
         "roofline": {"bound": "hbm", "achieved": ach_gbs, "peak": hbm_peak, "unit": "GB/s", "frac": ach_gbs / hbm_peak,
                      "traffic": recorded_traffic(args.workload, args.seed),
-                     "traffic_unit": "bytes per step (every k_cfr_items and k_cfr_cluster launch of one solve; ncu "
+                     "traffic_unit": "bytes per step (every k_cfr_block and k_cfr_cluster launch of one solve; ncu "
                                      "record in profiles/)",
-                     "note": (f"k_cfr_items; achieved = {ALG_BYTES_PER_UPDATE} B per swept node-update (R and S "
+                     "note": (f"k_cfr_block; achieved = {ALG_BYTES_PER_UPDATE} B per swept node-update (R and S "
                               f"read + write) x swept node-updates / CFR kernel time, peak = {src} HBM copy "
                               "bandwidth; the kernel keeps each root's state in shared memory for all T "
                               "iterations, so its DRAM traffic is far below the algorithmic bytes (ncu counters "

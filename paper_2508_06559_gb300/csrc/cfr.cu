@@ -44,6 +44,8 @@ constexpr int kClsGlobal = kNumCls - 1;
 constexpr int kClsCluster = 6;  // roots split over clusters
 // forked streams: the level-streaming sweep, then the cluster and block launches in turn
 constexpr int kAuxStream = 0, kAuxSweep = 1;
+// solved slots per SM and per slot of an item: below it items take fewer slots, so that the GPU has blocks (1 and 4
+// measured the same: rounds have either many slots or few)
 constexpr int64_t kSlotsPerSm = 2;
 
 struct CfrParams {
