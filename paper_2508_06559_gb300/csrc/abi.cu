@@ -379,9 +379,9 @@ int pasur_unfold(pasur_tree *t, const int64_t *score_offs, const pasur_score *sc
     t->scores_h.assign(scores, scores + ns);
     PASUR_TRY(tree_alloc(t, (void **)&t->score_off_d, sizeof(int64_t) * (size_t)(nr + 1)));
     PASUR_TRY(tree_alloc(t, (void **)&t->scores_d, sizeof(pasur_score) * (size_t)(ns + 1)));
-    PASUR_CUDA(ctx, cudaMemcpyAsync(t->score_off_d, score_offs, sizeof(int64_t) * (size_t)(nr + 1), cudaMemcpyHostToDevice, ctx->stream));
+    PASUR_CUDA(ctx, cudaMemcpyAsync(t->score_off_d, t->score_off_h.data(), sizeof(int64_t) * (size_t)(nr + 1), cudaMemcpyHostToDevice, ctx->stream));
     if (ns > 0)
-        PASUR_CUDA(ctx, cudaMemcpyAsync(t->scores_d, scores, sizeof(pasur_score) * (size_t)ns, cudaMemcpyHostToDevice, ctx->stream));
+        PASUR_CUDA(ctx, cudaMemcpyAsync(t->scores_d, t->scores_h.data(), sizeof(pasur_score) * (size_t)ns, cudaMemcpyHostToDevice, ctx->stream));
     PASUR_TRY(unfold_levels(t));
     t->unfolded = true;
     if (level_sizes_out)

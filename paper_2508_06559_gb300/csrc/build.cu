@@ -371,10 +371,12 @@ int build_levels(pasur_tree *t, const uint64_t *root_pools_dev) {
 // The FGT levels over given slots per root (slot_off: prefix over the roots, host and device): sizes
 // from the roots' node counts on the host, then every level's offsets in one launch, without a scan or
 // a synchronisation.
-static int slot_levels(pasur_tree *t, const std::vector<int64_t> &slot_off, const int64_t *slot_off_d, int64_t **off, int64_t *sizes) {
+// base: filled here and read by the upload until the stream gets there, so it belongs to the tree.
+static int slot_levels(pasur_tree *t, const std::vector<int64_t> &slot_off, const int64_t *slot_off_d, std::vector<int64_t> &base,
+                       int64_t **off, int64_t *sizes) {
     pasur_ctx *ctx = t->ctx;
     const int64_t nr = t->n_roots;
-    std::vector<int64_t> base((size_t)(9 * (nr + 1)));
+    base.assign((size_t)(9 * (nr + 1)), 0);
     for (int k = 0; k < 9; k++) {
         int64_t *b = base.data() + (size_t)k * (size_t)(nr + 1), q = 0;
         for (int64_t g = 0; g < nr; g++) {
@@ -406,7 +408,7 @@ static int slot_levels(pasur_tree *t, const std::vector<int64_t> &slot_off, cons
     return rc;
 }
 
-int unfold_levels(pasur_tree *t) { return slot_levels(t, t->score_off_h, t->score_off_d, t->fgt_off, t->Q); }
+int unfold_levels(pasur_tree *t) { return slot_levels(t, t->score_off_h, t->score_off_d, t->lvl_base_h, t->fgt_off, t->Q); }
 
 // leaf values without any host synchronisation (the batch solver captures this in a CUDA graph);
 // umax_bits (device, may be NULL) receives max |value| as float bits
@@ -537,7 +539,7 @@ int plan_solve_slots(pasur_tree *t, bool merge, const float *next_util_dev) {
         }
     } else {
         for (int k = 0; k < 9; k++) t->cfgt_off[k] = nullptr;
-        PASUR_TRY(slot_levels(t, t->csoff_h, t->csoff_d, t->cfgt_off, t->cQ));
+        PASUR_TRY(slot_levels(t, t->csoff_h, t->csoff_d, t->clvl_base_h, t->cfgt_off, t->cQ));
     }
     return PASUR_OK;
 }

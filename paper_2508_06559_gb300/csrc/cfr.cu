@@ -1461,8 +1461,10 @@ int cfr_setup_tree(pasur_tree *t, const pasur_config *cfg, int tree, std::vector
     PASUR_TRY(plan_splits(t, cfg, limit, streamed, split));
     PASUR_TRY(place_splits(t, split));
     pt.mark("cluster splits");
-    std::vector<int64_t> sbase((size_t)t->csoff_h[(size_t)t->n_roots] + 1, 0);
-    std::vector<int32_t> sstr(sbase.size(), 0);
+    std::vector<int64_t> &sbase = t->slot_base_h;
+    std::vector<int32_t> &sstr = t->slot_str_h;
+    sbase.assign((size_t)t->csoff_h[(size_t)t->n_roots] + 1, 0);
+    sstr.assign(sbase.size(), 0);
     int64_t data = 0, scratch = 0;
     for (int64_t g = 0; g < t->n_roots; g++) {
         CfrRoot &cr = t->croots_h[(size_t)g];

@@ -356,6 +356,9 @@ struct pasur_tree {
     // order of their first full slot; without merging they are the full slots.
     bool merged = false;
     std::vector<int64_t> csoff_h;       // [n_roots+1] solved slots per root (prefix)
+    // sources of uploads that nothing waits for: they live as long as the tree (freed after a synchronisation)
+    std::vector<int64_t> lvl_base_h, clvl_base_h, slot_base_h;
+    std::vector<int32_t> slot_str_h;
     int64_t *csoff_d = nullptr;
     int32_t *crep_d = nullptr;          // [cQ[0]] per solved slot: its first full slot within the root
     int64_t *cidx0_d = nullptr;         // [Q[0]] per full root slot: the global index of its solved slot
