@@ -234,7 +234,7 @@ constexpr size_t gemm_smem(int epi, int nc, int warps) {
 // row tiles), so the columns are shared out over blocks; the output layer, which needs whole rows, over the
 // blocks of a cluster.  Bound by latency: a 1024-row batch is eight dependent launches of 5 to 11 us, overlapped
 // by programmatic launches.  40 such steps took 15.2 ms with 128 x 256 tiles on 128 threads (per launch: output
-// layer 65 us, input gradients 71, the others 22, Adam 83) and take 2.4 ms.
+// layer 65 us, input gradients 71, the others 22, Adam 83) and take 2.6 ms.
 template <int EPI, int NC, int CG>
 __global__ void __launch_bounds__(128 * CG, EPI == EPI_DW ? 3 : 1) k_gemm(const GemmArgs g) {
     extern __shared__ uint8_t smem_raw[];
@@ -322,27 +322,36 @@ __global__ void __launch_bounds__(128 * CG, EPI == EPI_DW ? 3 : 1) k_gemm(const 
     __nv_bfloat16 *stage = stages + warp * 32 * kStageRow;
     float v[32];
     if constexpr (EPI == EPI_LAST) {
-        // output layer y = h3 . w3 + b3 with h3 = gelu(acc + b2), in f32 per row, and its gradients
-        // (the blocks of a row tile are a cluster: each computes its columns' share and gives it to the others)
+        // output layer y = h3 . w3 + b3 with h3 = gelu(acc + b2), in f32 per row, and its gradients (the blocks of a
+        // row tile are a cluster).  The sum is one chain over the columns in order, each share of them going on where
+        // the one before stopped (eight cluster barriers).  Separate shares summed at the end took 3.5 us a step less
+        // but differ in the last bits of y: after 40 steps the weights were up to 3 times as far from those of the
+        // chain as two runs with the gradients added in any order are from each other.
         constexpr int kShares = kHid / PC;
         float *part = reinterpret_cast<float *>(stages);  // [kShares][128]
         static_assert(kShares * 128 * sizeof(float) <= 4 * CG * 32 * kStageRow * 2, "shares");
-        float yh = 0.f;
-#pragma unroll 1
-        for (int j = 0; j < PC; j += 32) {
-            if (acc_ok) tmem_ld32(taddr + j, v);
+        static_assert(PC == 32, "a thread holds its share");
+        if (acc_ok) tmem_ld32(taddr, v);
 #pragma unroll
-            for (int i = 0; i < 32; i++) yh += gelu(v[i] + g.bias[n0 + p0 + j + i]) * g.w3[n0 + p0 + j + i];
-        }
+        for (int i = 0; i < 32; i++) v[i] = gelu(v[i] + g.bias[n0 + p0 + i]);
+        const int mine = (int)blockIdx.z * CG + (warp >> 2), at = (warp & 3) * 32 + lane;
+        float yh = g.b3[0];
         cluster_wait();  // every block of the cluster has started
-        const uint32_t at = su32(part + ((int)blockIdx.z * CG + (warp >> 2)) * 128 + (warp & 3) * 32 + lane);
+#pragma unroll 1
+        for (int s = 0; s < kShares; s++) {
+            if (s == mine) {
+                if (s > 0) yh = part[(s - 1) * 128 + at];
 #pragma unroll
-        for (int q = 0; q < kHid / NC; q++) store_remote(at, q, yh);
-        cluster_arrive();
-        cluster_wait();
-        yh = g.b3[0];
-#pragma unroll
-        for (int q = 0; q < kShares; q++) yh += part[q * 128 + (warp & 3) * 32 + lane];
+                for (int i = 0; i < 32; i++) yh += v[i] * g.w3[n0 + p0 + i];
+                const uint32_t to = su32(part + s * 128 + at);
+                if (s == kShares - 1)
+                    for (int q = 0; q < kHid / NC; q++) store_remote(to, q, yh);
+                else store_remote(to, (s + 1) / CG, yh);
+            }
+            cluster_arrive();
+            cluster_wait();
+        }
+        yh = part[(kShares - 1) * 128 + at];
         __syncthreads();
         const bool valid = row < g.n_valid;
         const float err = valid ? yh - g.y[row] : 0.f;
