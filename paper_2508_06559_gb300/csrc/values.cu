@@ -80,7 +80,7 @@ __device__ __forceinline__ void level_values(const ValueArgs &A, int k, int64_t 
 // from `split_level` down, one block for the levels above it.  Bound by launches and by the chains of dependent loads
 // (child range, slot offset, value), hence several lanes to a node and four children in flight.  Both players' best
 // responses through the last four rounds of a deal (with the strategies' exports): 1.4 ms with a launch per level and a
-// thread to a node, 0.7 so.
+// thread to a node, 0.7 so.  For rounds that fill the GPU level by level see wide_round.
 __global__ void __launch_bounds__(1024) k_values(const ValueArgs A, int top, int bottom, int64_t m) {
     __shared__ int64_t lo[9], hi[9];
     if (threadIdx.x < 2) {
@@ -97,6 +97,17 @@ __global__ void __launch_bounds__(1024) k_values(const ValueArgs A, int top, int
     }
 }
 
+// One level on its own (k = 8: the leaves), a block to as many nodes as it holds at once.  Bound by the loads of the
+// children's values, slots over lanes: a final round of 1.05e9 leaves in 23 ms (43 in ranges, 111 with a thread to a node).
+__global__ void __launch_bounds__(256) k_value_level(const ValueArgs A, int k, int64_t m) {
+    const int64_t per = blockDim.x >> A.lanes_log2;
+    for (int64_t lo = (int64_t)blockIdx.x * per; lo < m; lo += (int64_t)gridDim.x * per) {
+        const int64_t hi = lo + per < m ? lo + per : m;
+        if (k == 8) leaf_values(A, lo, hi);
+        else level_values(A, k, lo, hi);
+    }
+}
+
 // first level with two nodes to an SM: the tree below it splits over the GPU, and the levels above it, of fewer nodes
 // each, are a few passes of one block
 int split_level(const pasur_tree *t) {
@@ -104,6 +115,13 @@ int split_level(const pasur_tree *t) {
     while (k < 7 && t->M[k] < 2 * t->ctx->num_sms) k++;
     return k;
 }
+
+// Rounds that take a launch per level instead of a block per range of subtrees.  The subtrees' sizes differ by up to a
+// hundred, and a block's range is fixed, so that a wide round waits for its heaviest range; nine launches cost some 25 us
+// more than two.  Ranges and levels (root values, one call, ms): 376 roots, 2.2e6 leaves, 1.2e7 with their slots 2.51 and
+// 0.60; 255 roots, 8.3e5, 4.4e6 1.98 and 0.32; 79 roots, 7.5e6, 9.5e8 196 and 19; 49 roots, 3.8e4, 1.5e6 0.165 and 0.166; 24
+// roots, 1.6e4, 2.2e6 0.29 and 0.33; 81 roots, 9.0e4, 3.4e5 0.100 and 0.104; 90 roots, 1.5e5, 5.9e5 0.145 and 0.125.
+bool wide_round(const pasur_tree *t) { return t->M[8] >= 1 << 17 || t->Q[8] >= 5 << 19; }
 
 unsigned grid_of(int64_t n) { return (unsigned)std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, 1 << 20)); }
 
@@ -182,7 +200,13 @@ int value_levels(pasur_tree *t, int mode, const float *sigma, const double *next
     A.final_round = t->final_round;
     A.mode = mode;
     while (A.lanes_log2 < 3 && t->Q[8] > t->M[8] << A.lanes_log2) A.lanes_log2++;  // the leaves' slots on average
-    if (rc == PASUR_OK && t->M[0] > 0) {
+    if (rc == PASUR_OK && t->M[0] > 0 && wide_round(t)) {
+        for (int k = 8; k >= 0; k--) {
+            k_value_level<<<grid_of(t->M[k] << A.lanes_log2), 256, 0, ctx->stream>>>(A, k, t->M[k]);
+            ctx->launches++;
+        }
+        if (cudaGetLastError() != cudaSuccess) rc = set_err(ctx, PASUR_ECUDA, "k_value_level launch");
+    } else if (rc == PASUR_OK && t->M[0] > 0) {
         const int top = split_level(t);
         const int64_t blocks = std::min<int64_t>(t->M[top], 8 * (int64_t)ctx->num_sms);
         k_values<<<(unsigned)blocks, 256, 0, ctx->stream>>>(A, top, 8, t->M[top]);

@@ -127,3 +127,56 @@ def test_values_over_tree_shapes(ctx, first):
     assert np.allclose(val, want, rtol=1e-12, atol=1e-12)
     for x in trees + [t]:
         x.free()
+
+
+@pytest.mark.parametrize("seed,rnd,slots", [(9, 3, 1), (9, 3, 3), (10, 4, 1), (61, 4, 1), (61, 5, 60), (5, 3, 2)])
+def test_values_of_wide_and_narrow_rounds(ctx, seed, rnd, slots):
+    """Rounds with many roots of very different sizes, on both sides of the line between a block
+    per range of subtrees (two launches a call) and a launch per level (nine): 2^17 leaves, or
+    5 * 2^19 with their slots.  Against a numpy pass over the exported tree: minimax exactly, the
+    others to the rounding of two sums of d products of weights that add up to 1, over 8 levels."""
+    from paper_2508_06559_gb300 import pasur as P
+    deck = O.deal(seed)
+    pools, soff, scores = np.array([mask_ids(deck[:4])], np.uint64), np.array([0, 1], np.int64), np.zeros((1, 4), np.int16)
+    for r in range(rnd):
+        t = ctx.pasur_build_round(deck, r, pools)
+        t.pasur_unfold(soff, scores)
+        pools, soff, scores, _ = t.pasur_next_roots_nolinks()
+        t.free()
+    clubs = [(a, b, 0, 0) for a in range(8) for b in range(8)][:slots]
+    t = ctx.pasur_build_round(deck, rnd, pools)
+    t.pasur_unfold(np.arange(len(pools) + 1, dtype=np.int64) * slots, np.array(clubs * len(pools), np.int16))
+    gt, fgt = t.pasur_tree_sizes()
+    wide = gt[8] >= 2 ** 17 or fgt[8] >= 5 * 2 ** 19
+    rng = np.random.default_rng(seed)
+    nxt = lnk = None
+    if rnd < 5:
+        lnk = t.pasur_next_roots()[3]
+        nxt = rng.normal(0, 9, t.n_next_roots())
+    t.pasur_cfr_iterate(P.pasur_config_default(iters=0), None if rnd == 5 else np.zeros(len(nxt), np.float32))
+    leaf = t.pasur_leaf_values().astype(np.float64)  # without the next round's values: whole numbers
+    if rnd < 5:
+        leaf = leaf + nxt[lnk]
+    leaf = leaf.reshape(-1, slots)
+    nchild = [t.pasur_export_level(k)["nchild"] for k in range(8)]
+    first = [np.concatenate([[0], np.cumsum(n)[:-1]]) for n in nchild]
+    sigma = []
+    for n, f in zip(nchild, first):
+        x = 1 - rng.random((int(n.sum()), slots), np.float32)  # in (0, 1]
+        sigma.append((x / np.repeat(np.add.reduceat(x, f), n, axis=0)).astype(np.float32))
+    flat = np.concatenate([x.ravel() for x in sigma])
+    dmax = max(int(n.max()) for n in nchild)
+    for mode in (O.MINIMAX, O.BR_ALEX, O.BR_BOB, O.ON_POLICY):
+        launches = ctx.pasur_launch_count()
+        got = t.pasur_root_values(mode, None if mode == O.MINIMAX else flat, nxt)
+        assert ctx.pasur_launch_count() - launches == (9 if wide else 2)
+        val = leaf
+        for k in range(7, -1, -1):
+            alex = k % 2 == 0
+            if mode == O.MINIMAX or mode == (O.BR_ALEX if alex else O.BR_BOB):
+                val = (np.maximum if alex else np.minimum).reduceat(val, first[k])
+            else:
+                val = np.add.reduceat(sigma[k].astype(np.float64) * val, first[k])
+        bound = 0.0 if mode == O.MINIMAX else 2 * 8 * (dmax + 1) * 2.0 ** -53 * 1.01 * np.abs(leaf).max()
+        assert np.abs(got - val.ravel()).max() <= bound, mode
+    t.free()
