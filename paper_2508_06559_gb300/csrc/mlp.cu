@@ -654,16 +654,17 @@ __global__ void k_gradient(const Partials q, float *__restrict__ grad, float *lo
 }
 
 // Adam (Kingma and Ba, 2015) on the flat parameters; writes the bf16 tiled weights and their transposes.
-// corr: the step's two bias corrections (64-bit powers taken on the host: two of them per thread here took
-// 83 us a step).
+// per_step: the step's two bias corrections (64-bit powers taken on the host: two of them per thread here took
+// 83 us a step) and the learning rate, which is data: the captured epoch is launched again with another one.
+constexpr int kPerStep = 3;
 __global__ void k_adam(float *__restrict__ p, const Partials q, float *loss, float *__restrict__ m, float *__restrict__ v,
-                       const float *__restrict__ corr, float lr, float b1, float b2, float eps,
+                       const float *__restrict__ per_step, float b1, float b2, float eps,
                        __nv_bfloat16 *__restrict__ W, __nv_bfloat16 *__restrict__ WT) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     pdl_next();
     pdl_wait();
     if (i >= kParams) return;
-    const float c1 = corr[0], c2 = corr[1];
+    const float c1 = per_step[0], c2 = per_step[1], lr = per_step[2];
     const float gi = grad_at(q, i, loss);
     const float mi = b1 * m[i] + (1.f - b1) * gi, vi = b2 * v[i] + (1.f - b2) * gi * gi;
     m[i] = mi;
@@ -734,8 +735,8 @@ struct pasur_mlp {
     pasur_ctx *ctx = nullptr;
     float *p = nullptr, *grad = nullptr, *m = nullptr, *v = nullptr;   // flat f32 [kParams]
     __nv_bfloat16 *W = nullptr, *WT = nullptr;                          // 3 tiled [256 x 256] each
-    float *corr_d = nullptr;                                            // per step of an epoch: Adam's bias corrections
-    int64_t corr_cap = 0;
+    float *per_step_d = nullptr;                                        // per step of an epoch: Adam's factors (k_adam)
+    int64_t steps_cap = 0;
     int64_t steps = 0;
     float *loss_d = nullptr;
     Partials parts{};                                                   // of the last pass
@@ -1231,13 +1232,13 @@ int pasur_mlp_train(pasur_mlp *M, int epochs, int64_t batch, float lr, uint64_t 
     cudaSetDevice(ctx->device);
     PASUR_TRY(ensure_rows(M, batch));
     const int64_t n = M->n, steps = (n + batch - 1) / batch;
-    if (M->corr_cap < steps) {
+    if (M->steps_cap < steps) {
         cudaStreamSynchronize(ctx->stream);
-        if (M->corr_d) mlp_release(M, M->corr_d);
-        M->corr_d = nullptr;
-        M->corr_cap = 0;
-        PASUR_TRY(mlp_alloc(M, (void **)&M->corr_d, sizeof(float) * 2 * (size_t)steps));
-        M->corr_cap = steps;
+        if (M->per_step_d) mlp_release(M, M->per_step_d);
+        M->per_step_d = nullptr;
+        M->steps_cap = 0;
+        PASUR_TRY(mlp_alloc(M, (void **)&M->per_step_d, sizeof(float) * kPerStep * (size_t)steps));
+        M->steps_cap = steps;
         if (M->epoch_exec) cudaGraphExecDestroy(M->epoch_exec);
         M->epoch_exec = nullptr;
     }
@@ -1253,7 +1254,7 @@ int pasur_mlp_train(pasur_mlp *M, int epochs, int64_t batch, float lr, uint64_t 
             if (rc == PASUR_OK) rc = run_pass(M, batch, m);
             if (rc == PASUR_OK) {
                 rc = launch_next(ctx, k_adam, dim3((kParams + 255) / 256), 256, 0, 1, M->p, M->parts, M->loss_d, M->m, M->v,
-                                 M->corr_d + 2 * s, lr, 0.9f, 0.999f, 1e-8f, M->W, M->WT);
+                                 M->per_step_d + kPerStep * s, 0.9f, 0.999f, 1e-8f, M->W, M->WT);
             }
         }
         cudaGraph_t gr = nullptr;
@@ -1271,7 +1272,7 @@ int pasur_mlp_train(pasur_mlp *M, int epochs, int64_t batch, float lr, uint64_t 
     }
     const int64_t launches_per_epoch = steps * 8;
     std::vector<int64_t> perm((size_t)n);
-    std::vector<float> corr(2 * (size_t)steps);
+    std::vector<float> per_step(kPerStep * (size_t)steps);
     uint64_t x = shuffle_seed;
     cudaEvent_t e0, e1;
     PASUR_CUDA(ctx, cudaEventCreate(&e0));
@@ -1292,10 +1293,12 @@ int pasur_mlp_train(pasur_mlp *M, int epochs, int64_t batch, float lr, uint64_t 
         PASUR_CUDA(ctx, cudaMemcpyAsync(M->perm_d, perm.data(), sizeof(int64_t) * (size_t)n, cudaMemcpyHostToDevice, ctx->stream));
         for (int64_t s = 0; s < steps; s++) {
             const double t = (double)(tb + s + 1);
-            corr[2 * (size_t)s] = (float)(1.0 / (1.0 - std::pow((double)0.9f, t)));
-            corr[2 * (size_t)s + 1] = (float)(1.0 / (1.0 - std::pow((double)0.999f, t)));
+            float *f = per_step.data() + kPerStep * (size_t)s;
+            f[0] = (float)(1.0 / (1.0 - std::pow((double)0.9f, t)));
+            f[1] = (float)(1.0 / (1.0 - std::pow((double)0.999f, t)));
+            f[2] = lr;
         }
-        PASUR_CUDA(ctx, cudaMemcpyAsync(M->corr_d, corr.data(), sizeof(float) * corr.size(), cudaMemcpyHostToDevice, ctx->stream));
+        PASUR_CUDA(ctx, cudaMemcpyAsync(M->per_step_d, per_step.data(), sizeof(float) * per_step.size(), cudaMemcpyHostToDevice, ctx->stream));
         PASUR_CUDA(ctx, cudaMemsetAsync(M->loss_d, 0, sizeof(float), ctx->stream));
         PASUR_CUDA(ctx, cudaGraphLaunch(M->epoch_exec, ctx->stream));
         ctx->launches += launches_per_epoch;

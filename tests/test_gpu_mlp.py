@@ -310,3 +310,26 @@ def test_tile_edges(ctx, n):
     for name, _ in M.SHAPES:
         assert (np.abs(gg[name] - go[name]) <= BF16_ELEM_TOL * scale[name] + 1e-12).all(), name
     mlp.free()
+
+
+def test_learning_rate_of_every_call(ctx):
+    """A network trained again on the same rows with another learning rate takes that rate: equal
+    bit for bit to one whose rows were cleared and added again in between (training repeats bit
+    for bit), and not to one that kept the first rate."""
+    from paper_2508_06559_gb300 import pasur as P
+    rng = np.random.default_rng(11)
+    X, Y = bf16_bits(rng.normal(0, 1, (700, 256))), rng.normal(0, 2, 700).astype(np.float32)
+    out = []
+    for rates, fresh in (((1e-3, 1e-4, 3e-3), False), ((1e-3, 1e-4, 3e-3), True), ((1e-3, 1e-3, 1e-3), False)):
+        mlp = P.Mlp(ctx, dataset_capacity=700)
+        mlp.set_params(params(4)[0])
+        mlp.dataset_add_rows(X, Y)
+        for i, lr in enumerate(rates):
+            if fresh and i:
+                mlp.dataset_clear()
+                mlp.dataset_add_rows(X, Y)
+            mlp.train(1, 256, lr, shuffle_seed=i)
+        out.append(mlp.get_params())
+        mlp.free()
+    assert np.array_equal(out[0], out[1])
+    assert not np.array_equal(out[0], out[2])
