@@ -818,30 +818,37 @@ int set_gemm_attrs(pasur_ctx *ctx) {
     return PASUR_OK;
 }
 
+// The captured epoch holds the work buffers' addresses: it goes with them.
+void drop_epoch(pasur_mlp *M) {
+    if (M->epoch_exec) cudaGraphExecDestroy(M->epoch_exec);
+    M->epoch_exec = nullptr;
+}
+
+// Work buffers for `rows` rows.  The old ones are given back first (both together may exceed the budget), so that on
+// an error there are none: no capacity, no captured epoch.
 int ensure_rows(pasur_mlp *M, int64_t rows) {
     if (rows <= M->rows_cap) return PASUR_OK;
     cudaStreamSynchronize(M->ctx->stream);
-    void **bufs16[] = {(void **)&M->h0, (void **)&M->h0t, (void **)&M->h1, (void **)&M->h1t, (void **)&M->h2, (void **)&M->h2t,
-                       (void **)&M->d0, (void **)&M->d0t, (void **)&M->d1, (void **)&M->d1t, (void **)&M->d2, (void **)&M->d2t};
-    for (void **b : bufs16) {
-        if (*b) mlp_release(M, *b);
-        PASUR_TRY(mlp_alloc(M, b, sizeof(__nv_bfloat16) * (size_t)rows * kHid));
+    drop_epoch(M);
+    M->rows_cap = 0;
+    const size_t n = (size_t)rows;
+    struct {
+        void **p;
+        size_t bytes;
+    } bufs[18];
+    int count = 0;
+    for (__nv_bfloat16 **b : {&M->h0, &M->h0t, &M->h1, &M->h1t, &M->h2, &M->h2t, &M->d0, &M->d0t, &M->d1, &M->d1t, &M->d2, &M->d2t})
+        bufs[count++] = {(void **)b, sizeof(__nv_bfloat16) * n * kHid};
+    for (float **b : {&M->z0, &M->z1}) bufs[count++] = {(void **)b, sizeof(float) * n * kHid};
+    bufs[count++] = {(void **)&M->yb, sizeof(float) * n};
+    bufs[count++] = {(void **)&M->parts.cols, sizeof(float) * (n / 128) * (4 * kHid + 2)};
+    for (int i = 0; i < count; i++) {
+        if (*bufs[i].p) mlp_release(M, *bufs[i].p);
+        *bufs[i].p = nullptr;
     }
-    void **bufs32[] = {(void **)&M->z0, (void **)&M->z1};
-    for (void **b : bufs32) {
-        if (*b) mlp_release(M, *b);
-        PASUR_TRY(mlp_alloc(M, b, sizeof(float) * (size_t)rows * kHid));
-    }
-    if (M->yb) mlp_release(M, M->yb);
-    PASUR_TRY(mlp_alloc(M, (void **)&M->yb, sizeof(float) * (size_t)rows));
+    for (int i = 0; i < count; i++) PASUR_TRY(mlp_alloc(M, bufs[i].p, bufs[i].bytes));
     if (!M->parts.dW) PASUR_TRY(mlp_alloc(M, (void **)&M->parts.dW, sizeof(float) * kMaxSplits * 3 * kHid * kHid));
-    if (M->parts.cols) mlp_release(M, M->parts.cols);
-    PASUR_TRY(mlp_alloc(M, (void **)&M->parts.cols, sizeof(float) * (size_t)(rows / 128) * (4 * kHid + 2)));
     M->rows_cap = rows;
-    if (M->epoch_exec) {
-        cudaGraphExecDestroy(M->epoch_exec);
-        M->epoch_exec = nullptr;
-    }
     return PASUR_OK;
 }
 
@@ -1069,7 +1076,7 @@ int pasur_mlp_free(pasur_mlp *M) {
     if (!M) return PASUR_EINVAL;
     cudaSetDevice(M->ctx->device);
     cudaStreamSynchronize(M->ctx->stream);
-    if (M->epoch_exec) cudaGraphExecDestroy(M->epoch_exec);
+    drop_epoch(M);
     for (auto &o : M->owned) dev_free(M->ctx, o.first, o.second);
     delete M;
     return PASUR_OK;
@@ -1192,10 +1199,7 @@ int pasur_mlp_dataset_add_rows(pasur_mlp *M, const uint16_t *x, const float *y, 
                                     is_device_ptr(y) ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, ctx->stream));
     PASUR_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
     M->n += n;
-    if (M->epoch_exec) {
-        cudaGraphExecDestroy(M->epoch_exec);
-        M->epoch_exec = nullptr;
-    }
+    drop_epoch(M);
     return PASUR_OK;
 }
 
@@ -1216,10 +1220,7 @@ int pasur_mlp_dataset_export(const pasur_mlp *M, int64_t first, int64_t count, u
 int pasur_mlp_dataset_clear(pasur_mlp *M) {
     if (!M) return PASUR_EINVAL;
     M->n = 0;
-    if (M->epoch_exec) {
-        cudaGraphExecDestroy(M->epoch_exec);
-        M->epoch_exec = nullptr;
-    }
+    drop_epoch(M);
     return PASUR_OK;
 }
 
@@ -1234,18 +1235,16 @@ int pasur_mlp_train(pasur_mlp *M, int epochs, int64_t batch, float lr, uint64_t 
     const int64_t n = M->n, steps = (n + batch - 1) / batch;
     if (M->steps_cap < steps) {
         cudaStreamSynchronize(ctx->stream);
+        drop_epoch(M);
         if (M->per_step_d) mlp_release(M, M->per_step_d);
         M->per_step_d = nullptr;
         M->steps_cap = 0;
         PASUR_TRY(mlp_alloc(M, (void **)&M->per_step_d, sizeof(float) * kPerStep * (size_t)steps));
         M->steps_cap = steps;
-        if (M->epoch_exec) cudaGraphExecDestroy(M->epoch_exec);
-        M->epoch_exec = nullptr;
     }
     // one CUDA graph per epoch: (pack batch i through the permutation, forward, backward, Adam) x steps
     if (!M->epoch_exec || M->epoch_batch != batch || M->epoch_rows != n) {
-        if (M->epoch_exec) cudaGraphExecDestroy(M->epoch_exec);
-        M->epoch_exec = nullptr;
+        drop_epoch(M);
         PASUR_CUDA(ctx, cudaStreamBeginCapture(ctx->stream, cudaStreamCaptureModeThreadLocal));
         int rc = PASUR_OK;
         for (int64_t s = 0; s < steps && rc == PASUR_OK; s++) {
@@ -1266,7 +1265,10 @@ int pasur_mlp_train(pasur_mlp *M, int epochs, int64_t batch, float lr, uint64_t 
         if (e != cudaSuccess) return cuda_err(ctx, e, "pasur_mlp_train: capture");
         cudaError_t ie = cudaGraphInstantiate(&M->epoch_exec, gr, 0);
         cudaGraphDestroy(gr);
-        if (ie != cudaSuccess) return cuda_err(ctx, ie, "pasur_mlp_train: instantiate");
+        if (ie != cudaSuccess) {
+            M->epoch_exec = nullptr;
+            return cuda_err(ctx, ie, "pasur_mlp_train: instantiate");
+        }
         M->epoch_batch = batch;
         M->epoch_rows = n;
     }

@@ -333,3 +333,29 @@ def test_learning_rate_of_every_call(ctx):
         mlp.free()
     assert np.array_equal(out[0], out[1])
     assert not np.array_equal(out[0], out[2])
+
+
+def test_training_after_a_refused_gradient_batch():
+    """A gradient batch too large for the context's memory is refused and leaves the network
+    usable: training goes on bit for bit as without that call, before and after its epoch was
+    captured, and smaller gradient batches still work."""
+    from paper_2508_06559_gb300 import pasur as P
+    rng = np.random.default_rng(12)
+    X, Y = bf16_bits(rng.normal(0, 1, (1 << 14, 256))), rng.normal(0, 2, 1 << 14).astype(np.float32)
+    out = []
+    for refuse in ((), (0, 1, 2)):
+        small = P.Ctx(0, hbm_budget_bytes=64 << 20)
+        mlp = P.Mlp(small, dataset_capacity=600)
+        mlp.set_params(params(5)[0])
+        mlp.dataset_add_rows(X[:600], Y[:600])
+        for i in range(3):
+            if i in refuse:
+                with pytest.raises(P.PasurError) as e:
+                    mlp.gradients(X, Y)
+                assert e.value.code == P.PASUR_ENOMEM
+            mlp.train(1, 256, 1e-3, shuffle_seed=i)
+        loss, g = mlp.gradients(X[:300], Y[:300])
+        out.append((mlp.get_params(), loss, g))
+        mlp.free()
+        small.close()
+    assert np.array_equal(out[0][0], out[1][0]) and out[0][1] == out[1][1] and np.array_equal(out[0][2], out[1][2])
