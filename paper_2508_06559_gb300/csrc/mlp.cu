@@ -993,16 +993,19 @@ void free_tmp(pasur_ctx *ctx, std::vector<std::pair<void *, size_t>> &tmp) {
     tmp.clear();
 }
 
-// host or device float input -> device pointer (copied into tmp when host)
-int to_device(pasur_ctx *ctx, const void *src, size_t bytes, const void **dev, std::vector<std::pair<void *, size_t>> &tmp) {
-    if (is_device_ptr(src)) {
+// host or device input -> device pointer on an `align`-byte boundary (copied into tmp when it is host memory or lies
+// elsewhere: feature rows are loaded 16 bytes at a time and may begin at any of their 2-byte elements)
+int to_device(pasur_ctx *ctx, const void *src, size_t bytes, size_t align, const void **dev,
+              std::vector<std::pair<void *, size_t>> &tmp) {
+    const bool on_device = is_device_ptr(src);
+    if (on_device && (uintptr_t)src % align == 0) {
         *dev = src;
         return PASUR_OK;
     }
     void *d = nullptr;
     PASUR_TRY(dev_alloc(ctx, &d, bytes + 16));
     tmp.push_back({d, bytes + 16});
-    PASUR_CUDA(ctx, cudaMemcpyAsync(d, src, bytes, cudaMemcpyHostToDevice, ctx->stream));
+    PASUR_CUDA(ctx, cudaMemcpyAsync(d, src, bytes, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, ctx->stream));
     *dev = d;
     return PASUR_OK;
 }
@@ -1115,7 +1118,7 @@ int pasur_mlp_forward(pasur_mlp *M, const uint16_t *x, int64_t n, float *y_out) 
     if (n == 0) return PASUR_OK;
     std::vector<std::pair<void *, size_t>> tmp;
     const void *xd = nullptr;
-    int rc = to_device(ctx, x, sizeof(uint16_t) * (size_t)n * kHid, &xd, tmp);
+    int rc = to_device(ctx, x, sizeof(uint16_t) * (size_t)n * kHid, 16, &xd, tmp);
     float *yd = nullptr;
     if (rc == PASUR_OK) {
         void *p = nullptr;
@@ -1136,8 +1139,8 @@ int pasur_mlp_gradients(pasur_mlp *M, const uint16_t *x, const float *y, int64_t
     cudaSetDevice(ctx->device);
     std::vector<std::pair<void *, size_t>> tmp;
     const void *xd = nullptr, *yd = nullptr;
-    int rc = to_device(ctx, x, sizeof(uint16_t) * (size_t)n * kHid, &xd, tmp);
-    if (rc == PASUR_OK) rc = to_device(ctx, y, sizeof(float) * (size_t)n, &yd, tmp);
+    int rc = to_device(ctx, x, sizeof(uint16_t) * (size_t)n * kHid, 16, &xd, tmp);
+    if (rc == PASUR_OK) rc = to_device(ctx, y, sizeof(float) * (size_t)n, sizeof(float), &yd, tmp);
     const int64_t Mp = pad128(n);
     if (rc == PASUR_OK) rc = ensure_rows(M, Mp);
     if (rc == PASUR_OK) rc = cudaMemsetAsync(M->loss_d, 0, sizeof(float), ctx->stream) == cudaSuccess ? PASUR_OK : PASUR_ECUDA;

@@ -359,3 +359,31 @@ def test_training_after_a_refused_gradient_batch():
         mlp.free()
         small.close()
     assert np.array_equal(out[0][0], out[1][0]) and out[0][1] == out[1][1] and np.array_equal(out[0][2], out[1][2])
+
+
+@pytest.mark.parametrize("offset", [0, 1, 4, 8])
+def test_device_rows_at_any_element(ctx, offset):
+    """Feature rows on the device that begin `offset` 2-byte elements into their allocation, and
+    targets and results that begin as many floats in: predictions and gradients equal those of
+    the same rows in host memory."""
+    import ctypes as C
+    import torch
+    from paper_2508_06559_gb300 import pasur as P
+    n = 200
+    rng = np.random.default_rng(offset)
+    X, Y = bf16_bits(rng.normal(0, 1, (n, 256))), rng.normal(0, 2, n).astype(np.float32)
+    mlp = P.Mlp(ctx)
+    mlp.set_params(params(6)[0])
+    want, (loss, grad) = mlp.forward(X), mlp.gradients(X, Y)
+    xb = torch.zeros(offset + n * 256, dtype=torch.int16, device="cuda")
+    yb, ob = (torch.zeros(offset + n, dtype=torch.float32, device="cuda") for _ in range(2))
+    x, y, out = xb[offset:].view(n, 256), yb[offset:], ob[offset:]
+    x.copy_(torch.from_numpy(X.view(np.int16)))
+    y.copy_(torch.from_numpy(Y))
+    torch.cuda.synchronize()
+    assert np.array_equal(mlp.forward(x, out).cpu().numpy(), want)
+    l2, g2 = np.zeros(1, np.float32), np.zeros(P.N_MLP_PARAMS, np.float32)
+    ptr = lambda a: C.c_void_p(a.data_ptr() if hasattr(a, "data_ptr") else a.ctypes.data)  # noqa: E731
+    assert P.load().pasur_mlp_gradients(mlp.h, ptr(x), ptr(y), C.c_int64(n), ptr(l2), ptr(g2)) == P.PASUR_OK
+    assert l2[0] == np.float32(loss) and np.array_equal(g2, grad)
+    mlp.free()
