@@ -1880,7 +1880,10 @@ int cfr_launch_plan(pasur_ctx *ctx, CfrPlan &plan, const pasur_config *cfg, int6
     // the launches are independent: each runs on its own forked stream (beyond their number,
     // several share one), clusters first, largest subtrees first; the level-streaming sweep (thousands
     // of short launches) is queued last, so that the host never waits on its queue before the others
-    // start
+    // start.  The joins come after it: streams share the device's few hardware queues, and an event
+    // record holds its queue until the launch before it has ended.  With the joins first the streamed
+    // sweep of a 1.9e9-node final round began after the clusters (1052 ms, 1012 with a thread to a
+    // (node, slot) in the clusters); so both run together
     const int nb = (int)std::min<size_t>(plan.launches.size(), kAuxStreams - kAuxSweep);
     for (int x = 0; x < nb; x++) PASUR_TRY(fork(kAuxSweep + x));
     for (size_t i = 0; i < plan.launches.size(); i++) {
@@ -1897,12 +1900,13 @@ int cfr_launch_plan(pasur_ctx *ctx, CfrPlan &plan, const pasur_config *cfg, int6
         PASUR_CUDA(ctx, cudaLaunchKernelExC(&lc, l.ctas > 1 ? cluster_kernel(cfg->variant, l.W) : block_kernel(cfg->variant, l.W), args));
         ctx->launches++;
     }
-    for (int x = 0; x < nb; x++) PASUR_TRY(join(kAuxSweep + x));
-    if (plan.cls_end[kClsGlobal] != plan.cls_begin[kClsGlobal]) {
+    const bool streamed = plan.cls_end[kClsGlobal] != plan.cls_begin[kClsGlobal];
+    if (streamed) {
         PASUR_TRY(fork(kAuxStream));
         PASUR_TRY(stream_sweep(ctx, plan, p, cfg, ctx->aux[kAuxStream]));
-        PASUR_TRY(join(kAuxStream));
     }
+    for (int x = 0; x < nb; x++) PASUR_TRY(join(kAuxSweep + x));
+    if (streamed) PASUR_TRY(join(kAuxStream));
     return PASUR_OK;
 }
 
