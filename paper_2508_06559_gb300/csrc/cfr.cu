@@ -689,12 +689,13 @@ __global__ void k_block_entries(int64_t n, const int64_t *src, const int32_t *ac
 }
 
 // inv: block -> local index; term: terminals by block index; roots without an active node keep their one local node at 0
+// (blockIdx.y: blocks to a root, where the roots are few and large)
 __global__ void k_block_inverse(const int32_t *bmap, const CfrRoot *roots, int64_t nr, const int64_t *loc_tq, int32_t *inv,
                                 uint8_t *term) {
     for (int64_t g = (int64_t)blockIdx.x; g < nr; g += gridDim.x) {
         const CfrRoot &cr = roots[g];
         const int L = cr.ls[9];
-        for (int l = threadIdx.x; l < L; l += blockDim.x) {
+        for (int l = blockIdx.y * blockDim.x + threadIdx.x; l < L; l += gridDim.y * blockDim.x) {
             const int64_t b = cr.loc_off + (cr.as[9] == 0 ? l : bmap[cr.loc_off + l]);
             inv[b] = l;
             term[b] = loc_tq[cr.loc_off + l] >= 0;
@@ -812,7 +813,9 @@ int build_block_order(pasur_tree *t, const int32_t *act_rk) {
     }
     t->broots_h.resize((size_t)nr);
     if (nr > 0) {
-        k_block_inverse<<<(unsigned)std::min<int64_t>(nr, 65535), 256, 0, ctx->stream>>>(bmap, t->croots_d, nr, t->loc_tq, t->b_inv, t->b_term);
+        dim3 g((unsigned)std::min<int64_t>(nr, 65535));
+        g.y = (unsigned)std::min<int64_t>(64, (8 * (int64_t)ctx->num_sms + g.x - 1) / g.x);
+        k_block_inverse<<<g, 256, 0, ctx->stream>>>(bmap, t->croots_d, nr, t->loc_tq, t->b_inv, t->b_term);
         PASUR_TRY(launched());
         k_block_roots<<<grid_for(nr, 256), 256, 0, ctx->stream>>>(nr, t->croots_d, run, brank, t->broots_d);
         PASUR_TRY(launched());
