@@ -23,7 +23,8 @@
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
-#include <functional>
+#include <memory>
+#include <new>
 #include <string>
 #include <thread>
 
@@ -1004,6 +1005,29 @@ struct RootSplit {
     std::string msg;
 };
 
+// fn(0) .. fn(n - 1) on up to 16 host threads (fewer where a thread does not start); false if one of them threw
+template <typename Fn>
+bool on_threads(size_t n, const Fn &fn) {
+    std::atomic<size_t> next{0};
+    std::atomic<bool> failed{false};
+    auto worker = [&]() {
+        try {
+            for (size_t i = next++; i < n; i = next++) fn(i);
+        } catch (...) {
+            failed = true;
+        }
+    };
+    const size_t most = std::min<size_t>({(size_t)std::max(1u, std::thread::hardware_concurrency()), (size_t)16, n});
+    std::vector<std::thread> threads;
+    try {
+        for (size_t w = 1; w < most; w++) threads.emplace_back(worker);
+    } catch (...) {
+    }
+    worker();
+    for (std::thread &x : threads) x.join();
+    return !failed;
+}
+
 constexpr int kSplitRuns = 96;  // runs a part is assumed to have while it is planned (checked after)
 
 // the most slots of one item when S slots are shared out evenly over items of at most cap slots
@@ -1046,8 +1070,45 @@ int plan_splits(pasur_tree *t, const pasur_config *cfg, size_t limit, const std:
     const size_t target = cfg->split_bytes > 0 ? std::min<size_t>((size_t)cfg->split_bytes, limit) : limit;
     const bool verbose = getenv("PASUR_VERBOSE") != nullptr;
     const int warps = kBlockMaxThreads / 32;
+    // what the cut of a root at a level gives, whatever the slots: the active level-ell nodes (heads, by local index), the
+    // subtree of every local node below them (-1: none), and the subtrees' active entries and nodes.  Made once for all
+    // slot counts tried: 79 roots of 1.0e7 nodes are split in 13 ms (51 with a cut per count)
+    struct LevelCut {
+        bool made = false;
+        std::vector<int32_t> heads, sub;
+        std::vector<int64_t> sa, sl;
+        int64_t tot = 0, amax = 0;
+    };
+    auto cut_at = [&](int64_t g, int ell, LevelCut &c) {
+        if (c.made) return;
+        const CfrRoot &cr = t->croots_h[(size_t)g];
+        const int64_t L = cr.ls[9];
+        const int32_t *li = hli.data() + cr.act_off, *cs = hcs.data() + cr.act_off;
+        const uint16_t *dd = hd.data() + cr.act_off;
+        for (int32_t e = cr.as[ell]; e < cr.as[ell + 1]; e++) c.heads.push_back(li[e]);
+        std::sort(c.heads.begin(), c.heads.end());
+        const size_t ns = c.heads.size();
+        c.sub.assign((size_t)L, -1);
+        for (size_t i = 0; i < ns; i++) c.sub[(size_t)c.heads[i]] = (int32_t)i;
+        c.sa.assign(ns, 0);
+        c.sl.assign(ns, 0);
+        for (int k = ell; k < 8; k++)
+            for (int32_t e = cr.as[k]; e < cr.as[k + 1]; e++) {
+                const int32_t sid = c.sub[(size_t)li[e]];
+                if (sid < 0) continue;
+                c.sa[(size_t)sid]++;
+                for (int a = 0; a < dd[e]; a++) c.sub[(size_t)(cs[e] + a)] = sid;
+            }
+        for (int64_t x = cr.ls[ell]; x < L; x++)
+            if (c.sub[(size_t)x] >= 0) c.sl[(size_t)c.sub[(size_t)x]]++;
+        for (int64_t n : c.sa) {
+            c.tot += n;
+            c.amax = std::max(c.amax, n);
+        }
+        c.made = true;
+    };
     // the split of one root for items of W slots over at most qmax CTAs
-    auto split_one = [&](int64_t g, int W, int qmax, RootSplit &o) {
+    auto split_one = [&](int64_t g, int W, int qmax, LevelCut *cuts, RootSplit &o) {
         const CfrRoot cr = t->croots_h[(size_t)g];
         const BlockRoot &br = t->broots_h[(size_t)g];
         const int64_t L = cr.ls[9], nA = cr.as[9];
@@ -1055,32 +1116,16 @@ int plan_splits(pasur_tree *t, const pasur_config *cfg, size_t limit, const std:
         const uint16_t *dd = hd.data() + cr.act_off;
         const int64_t *tq = htq.data() + cr.loc_off;
         auto bytes = [&](int64_t l, int64_t a) { return (size_t)block_offsets(l, a, kSplitRuns, W, warps).end; };
-        std::vector<int32_t> ent_of((size_t)L, -1);
-        for (int32_t e = 0; e < nA; e++) ent_of[(size_t)li[e]] = e;
         for (int ell = 1; ell <= 6; ell++) {
-            const int32_t e0 = cr.as[ell], e1 = cr.as[ell + 1];
-            if (e1 - e0 < 2) continue;
-            // subtree id of every local node at levels >= ell below an active level-ell node
-            std::vector<int32_t> heads;  // local indices of the active level-ell nodes, in order
-            for (int32_t e = e0; e < e1; e++) heads.push_back(li[e]);
-            std::sort(heads.begin(), heads.end());
-            std::vector<int32_t> sub((size_t)L, -1);
-            for (size_t i = 0; i < heads.size(); i++) sub[(size_t)heads[i]] = (int32_t)i;
-            const int ns = (int)heads.size();
-            std::vector<int64_t> sa((size_t)ns, 0), sl((size_t)ns, 0);
-            for (int k = ell; k < 8; k++)
-                for (int32_t e = cr.as[k]; e < cr.as[k + 1]; e++) {
-                    const int32_t sid = sub[(size_t)li[e]];
-                    if (sid < 0) continue;
-                    sa[(size_t)sid]++;
-                    for (int a = 0; a < dd[e]; a++) sub[(size_t)(cs[e] + a)] = sid;
-                }
-            for (int64_t x = cr.ls[ell]; x < L; x++)
-                if (sub[(size_t)x] >= 0) sl[(size_t)sub[(size_t)x]]++;
+            if (cr.as[ell + 1] - cr.as[ell] < 2) continue;
             const size_t top_bytes = block_offsets(cr.ls[ell + 1], cr.as[ell], br.rs[ell], W, warps).end;
             if (top_bytes >= limit) break;
-            int64_t tot = 0;
-            for (int i = 0; i < ns; i++) tot += sa[(size_t)i];
+            cut_at(g, ell, cuts[ell]);
+            const LevelCut &cut = cuts[ell];
+            const std::vector<int32_t> &heads = cut.heads, &sub = cut.sub;
+            const std::vector<int64_t> &sa = cut.sa, &sl = cut.sl;
+            const int ns = (int)heads.size();
+            const int64_t tot = cut.tot, amax = cut.amax;
             // the target size sets the starting count of parts, a block's shared memory is the hard
             // limit of every part
             const size_t need = bytes(L, nA);
@@ -1105,13 +1150,11 @@ int plan_splits(pasur_tree *t, const pasur_config *cfg, size_t limit, const std:
                 }
                 return true;
             };
-            int64_t amax = 0;
-            for (int i = 0; i < ns; i++) amax = std::max(amax, sa[(size_t)i]);
-            for (int Q = q0; Q <= qmax; Q++) {
-                std::vector<int> first;
+            // without an entry cap: whether every subtree fits a block, and the fewest parts
+            std::vector<int> first;
+            const int fewest = greedy(tot, first) ? (int)first.size() : qmax + 1;
+            for (int Q = std::max(q0, fewest); Q <= qmax; Q++) {
                 int64_t lo = std::max<int64_t>(amax, (tot + Q - 1) / Q), hi = tot;
-                if (!greedy(hi, first)) break;  // a single subtree does not fit a block
-                if ((int)first.size() > Q) continue;
                 while (lo < hi) {
                     const int64_t mid = lo + (hi - lo) / 2;
                     if (greedy(mid, first) && (int)first.size() <= Q) hi = mid;
@@ -1135,7 +1178,8 @@ int plan_splits(pasur_tree *t, const pasur_config *cfg, size_t limit, const std:
                 std::vector<int32_t> part_of((size_t)ns);
                 for (int q = 0; q < np; q++)
                     for (int i = first[(size_t)q]; i < first[(size_t)q + 1]; i++) part_of[(size_t)i] = q;
-                std::vector<int32_t> bidx((size_t)L, -1);
+                std::vector<int32_t> bidx((size_t)L, -1), ent_of((size_t)cr.ls[ell + 1], -1);
+                for (int32_t e = cr.as[ell]; e < cr.as[ell + 1]; e++) ent_of[(size_t)li[e]] = e;
                 // entries part by part and level by level
                 std::vector<std::vector<std::vector<int32_t>>> ents((size_t)np, std::vector<std::vector<int32_t>>(8));
                 for (int k = ell; k < 8; k++)
@@ -1240,88 +1284,125 @@ int plan_splits(pasur_tree *t, const pasur_config *cfg, size_t limit, const std:
     };
     // roots are independent: split them on host threads; as many slots per item as clusters of up to 8
     // CTAs hold, one slot over up to 16
-    std::atomic<size_t> next{0};
-    std::atomic<bool> failed{false};
-    auto worker = [&]() {
-        try {
-            for (size_t i = next++; i < cand.size(); i = next++) {
-                const int64_t g = cand[i];
-                const int64_t Sg = t->csoff_h[(size_t)g + 1] - t->csoff_h[(size_t)g];
-                RootSplit &o = split[(size_t)g];
-                std::string msg;
-                for (int64_t W = even_slots(Sg, cfg->slots_per_item > 0 ? std::min(cfg->slots_per_item, kBlockSlots) : kBlockSlots);
-                     W >= 1 && !o.done; W = W > 1 ? even_slots(Sg, W - 1) : 0) {
-                    split_one(g, (int)W, W > 1 && cfg->split_bytes == 0 ? 8 : kMaxClusterCtas, o);
-                    if (!o.done) msg += o.msg;
-                    o.msg.clear();
-                }
-                o.msg = msg;
-            }
-        } catch (...) {
-            failed = true;
+    const bool ok = on_threads(cand.size(), [&](size_t i) {
+        const int64_t g = cand[i];
+        const int64_t Sg = t->csoff_h[(size_t)g + 1] - t->csoff_h[(size_t)g];
+        RootSplit &o = split[(size_t)g];
+        LevelCut cuts[7];
+        std::string msg;
+        for (int64_t W = even_slots(Sg, cfg->slots_per_item > 0 ? std::min(cfg->slots_per_item, kBlockSlots) : kBlockSlots);
+             W >= 1 && !o.done; W = W > 1 ? even_slots(Sg, W - 1) : 0) {
+            split_one(g, (int)W, W > 1 && cfg->split_bytes == 0 ? 8 : kMaxClusterCtas, cuts, o);
+            if (!o.done) msg += o.msg;
+            o.msg.clear();
         }
-    };
-    const unsigned hw = std::max(1u, std::thread::hardware_concurrency());
-    const size_t nw = std::min<size_t>({(size_t)hw, (size_t)16, cand.size()});
-    {
-        std::vector<std::thread> th;
-        for (size_t w = 1; w < nw; w++) th.emplace_back(worker);
-        worker();
-        for (auto &x : th) x.join();
-    }
-    if (failed) return set_err(ctx, PASUR_ENOMEM, "cluster split: host allocation failed");
+        o.msg = msg;
+    });
+    if (!ok) return set_err(ctx, PASUR_ENOMEM, "cluster split: host allocation failed");
     pt.mark("per-root splits");
     for (int64_t g : cand)
         if (!split[(size_t)g].done && !split[(size_t)g].msg.empty()) fputs(split[(size_t)g].msg.c_str(), stderr);
     return PASUR_OK;
 }
 
+// the first nodes of several roots in block order, a root to a block: inv[from[b] ..] to out[to[b] .. to[b + 1])
+__global__ void k_gather_tops(const int32_t *__restrict__ inv, const int64_t *__restrict__ from, const int64_t *__restrict__ to,
+                              int32_t *__restrict__ out) {
+    const int64_t a = from[blockIdx.x], o = to[blockIdx.x], n = to[blockIdx.x + 1] - o;
+    for (int64_t i = threadIdx.x; i < n; i += blockDim.x) out[o + i] = inv[a + i];
+}
+
 // The parts' entries, runs and index maps after the tree's own (device), the pseudo-roots after the
-// real roots, and the exchange entries.
+// real roots, and the exchange entries.  Host threads copy them into place and give back the splits' own
+// arrays: 4410 split roots of 3.2e8 nodes in 65 ms (507 one root after the other).
 int place_splits(pasur_tree *t, std::vector<RootSplit> &split) {
     pasur_ctx *ctx = t->ctx;
     const int64_t NA = t->n_active, NL = t->n_local, NR = t->n_runs;
-    std::vector<uint32_t> ent;
-    std::vector<uint8_t> msk, term;
-    std::vector<int32_t> inv;
-    std::vector<BlockRun> runs;
-    bool any = false;
-    for (const RootSplit &o : split) any |= o.done;
-    if (!any) return PASUR_OK;
-    // block index of the top's nodes: the inverse of the root's own map, levels <= ell
-    std::vector<int32_t> own, back;
-    for (size_t g = 0; g < split.size(); g++) {
+    // the split roots; where each one's entries, nodes, runs, exchange entries and top nodes begin
+    std::vector<int64_t> roots, from;
+    for (size_t g = 0; g < split.size(); g++)
+        if (split[g].done) roots.push_back((int64_t)g);
+    if (roots.empty()) return PASUR_OK;
+    const size_t n = roots.size();
+    std::vector<int64_t> e_at(n + 1, 0), l_at(n + 1, 0), r_at(n + 1, 0), x_at(n + 1, 0), t_at(n + 1, 0);
+    for (size_t i = 0; i < n; i++) {
+        const size_t g = (size_t)roots[i];
         RootSplit &o = split[g];
-        if (!o.done) continue;
-        const int64_t off = t->croots_h[g].loc_off;
-        own.resize((size_t)o.top.ls[9]);
-        PASUR_CUDA(ctx, cudaMemcpy(own.data(), t->b_inv + off, sizeof(int32_t) * own.size(), cudaMemcpyDeviceToHost));
-        back.assign(own.size(), 0);
-        for (size_t b = 0; b < own.size(); b++) back[(size_t)own[b]] = (int32_t)b;
-        for (size_t i = 0; i < o.cx.size(); i += 5) {
-            o.cx[i + 1] = back[(size_t)o.cx[i + 1]];
-            o.cx[i + 2] = back[(size_t)o.cx[i + 2]];
-        }
+        from.push_back(t->croots_h[g].loc_off);
+        e_at[i + 1] = e_at[i] + (int64_t)o.ent.size();
+        l_at[i + 1] = l_at[i] + (int64_t)o.inv.size();
+        r_at[i + 1] = r_at[i] + (int64_t)o.runs.size();
+        x_at[i + 1] = x_at[i] + (int64_t)o.cx.size();
+        t_at[i + 1] = t_at[i] + o.top.ls[9];
         o.top_root = (int32_t)t->croots_h.size();
-        o.x0 = (int64_t)t->cx_h.size() / 5;
+        o.x0 = x_at[i] / 5;
         t->croots_h.push_back(o.top);
         t->broots_h.push_back(o.top_runs);
         for (size_t q = 0; q < o.parts.size(); q++) {
             CfrRoot pr = o.parts[q];
             BlockRoot pb = o.part_runs[q];
-            pr.loc_off += NL + (int64_t)inv.size();
-            pr.act_off += NA + (int64_t)ent.size();
-            pb.run_off += NR + (int64_t)runs.size();
+            pr.loc_off += NL + l_at[i];
+            pr.act_off += NA + e_at[i];
+            pb.run_off += NR + r_at[i];
             t->croots_h.push_back(pr);
             t->broots_h.push_back(pb);
         }
-        ent.insert(ent.end(), o.ent.begin(), o.ent.end());
-        msk.insert(msk.end(), o.msk.begin(), o.msk.end());
-        term.insert(term.end(), o.term.begin(), o.term.end());
-        inv.insert(inv.end(), o.inv.begin(), o.inv.end());
-        runs.insert(runs.end(), o.runs.begin(), o.runs.end());
-        t->cx_h.insert(t->cx_h.end(), o.cx.begin(), o.cx.end());
     }
+    std::vector<int32_t> tops((size_t)t_at[n]);
+    {
+        int64_t *from_d = nullptr, *to_d = nullptr;
+        int32_t *tops_d = nullptr;
+        std::vector<std::pair<void *, size_t>> tmp;
+        struct Guard {
+            pasur_ctx *c;
+            std::vector<std::pair<void *, size_t>> *v;
+            ~Guard() {
+                for (auto &x : *v) dev_free(c, x.first, x.second);
+            }
+        } guard{ctx, &tmp};
+        Slab sl;
+        sl.add(&from_d, (int64_t)n);
+        sl.add(&to_d, (int64_t)n);
+        sl.add(&tops_d, t_at[n]);
+        PASUR_TRY(sl.alloc(ctx, tmp));
+        PASUR_CUDA(ctx, cudaMemcpyAsync(from_d, from.data(), sizeof(int64_t) * n, cudaMemcpyHostToDevice, ctx->stream));
+        PASUR_CUDA(ctx, cudaMemcpyAsync(to_d, t_at.data(), sizeof(int64_t) * (n + 1), cudaMemcpyHostToDevice, ctx->stream));
+        k_gather_tops<<<(unsigned)n, 256, 0, ctx->stream>>>(t->b_inv, from_d, to_d, tops_d);
+        ctx->launches++;
+        PASUR_CUDA(ctx, cudaGetLastError());
+        PASUR_CUDA(ctx, cudaMemcpyAsync(tops.data(), tops_d, sizeof(int32_t) * tops.size(), cudaMemcpyDeviceToHost, ctx->stream));
+        PASUR_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+    }
+    const size_t ne = (size_t)e_at[n], nl = (size_t)l_at[n], nrun = (size_t)r_at[n];
+    std::unique_ptr<uint32_t[]> ent(new (std::nothrow) uint32_t[ne + 1]);
+    std::unique_ptr<uint8_t[]> msk(new (std::nothrow) uint8_t[ne + 1]), term(new (std::nothrow) uint8_t[nl + 1]);
+    std::unique_ptr<int32_t[]> inv(new (std::nothrow) int32_t[nl + 1]);
+    std::unique_ptr<BlockRun[]> runs(new (std::nothrow) BlockRun[nrun + 1]);
+    if (!ent || !msk || !term || !inv || !runs) return set_err(ctx, PASUR_ENOMEM, "cluster split: host allocation failed");
+    t->cx_h.resize((size_t)x_at[n]);
+    const bool ok = on_threads(n, [&](size_t i) {
+        RootSplit &o = split[(size_t)roots[i]];
+        // block index of the top's nodes: the inverse of their order
+        const int32_t *own = tops.data() + t_at[i];
+        std::vector<int32_t> back((size_t)o.top.ls[9], 0);
+        for (size_t b = 0; b < back.size(); b++) back[(size_t)own[b]] = (int32_t)b;
+        int32_t *cx = std::copy(o.cx.begin(), o.cx.end(), t->cx_h.data() + x_at[i]) - (ptrdiff_t)o.cx.size();
+        for (size_t x = 0; x < o.cx.size(); x += 5) {
+            cx[x + 1] = back[(size_t)cx[x + 1]];
+            cx[x + 2] = back[(size_t)cx[x + 2]];
+        }
+        auto place = [](auto &v, auto *to) {
+            std::copy(v.begin(), v.end(), to);
+            v = {};
+            v.shrink_to_fit();
+        };
+        place(o.ent, ent.get() + e_at[i]);
+        place(o.msk, msk.get() + e_at[i]);
+        place(o.term, term.get() + l_at[i]);
+        place(o.inv, inv.get() + l_at[i]);
+        place(o.runs, runs.get() + r_at[i]);
+    });
+    if (!ok) return set_err(ctx, PASUR_ENOMEM, "cluster split: host allocation failed");
     auto grow = [&](void **p, int64_t n_old, size_t size, const void *more, size_t n_more) -> int {
         void *x = nullptr;
         PASUR_TRY(tree_alloc(t, &x, size * ((size_t)n_old + n_more + 1)));
@@ -1330,17 +1411,22 @@ int place_splits(pasur_tree *t, std::vector<RootSplit> &split) {
         *p = x;
         return PASUR_OK;
     };
-    PASUR_TRY(grow((void **)&t->b_ent, NA, sizeof(uint32_t), ent.data(), ent.size()));
-    PASUR_TRY(grow((void **)&t->b_msk, NA, sizeof(uint8_t), msk.data(), msk.size()));
-    PASUR_TRY(grow((void **)&t->b_term, NL, sizeof(uint8_t), term.data(), term.size()));
-    PASUR_TRY(grow((void **)&t->b_inv, NL, sizeof(int32_t), inv.data(), inv.size()));
-    PASUR_TRY(grow((void **)&t->b_run, NR, sizeof(BlockRun), runs.data(), runs.size()));
-    PASUR_TRY(tree_alloc(t, (void **)&t->croots_d, sizeof(CfrRoot) * t->croots_h.size()));
-    PASUR_TRY(tree_alloc(t, (void **)&t->broots_d, sizeof(BlockRoot) * t->broots_h.size()));
-    PASUR_CUDA(ctx, cudaMemcpyAsync(t->broots_d, t->broots_h.data(), sizeof(BlockRoot) * t->broots_h.size(), cudaMemcpyHostToDevice,
-                                    ctx->stream));
+    auto upload = [&]() -> int {
+        PASUR_TRY(grow((void **)&t->b_ent, NA, sizeof(uint32_t), ent.get(), ne));
+        PASUR_TRY(grow((void **)&t->b_msk, NA, sizeof(uint8_t), msk.get(), ne));
+        PASUR_TRY(grow((void **)&t->b_term, NL, sizeof(uint8_t), term.get(), nl));
+        PASUR_TRY(grow((void **)&t->b_inv, NL, sizeof(int32_t), inv.get(), nl));
+        PASUR_TRY(grow((void **)&t->b_run, NR, sizeof(BlockRun), runs.get(), nrun));
+        PASUR_TRY(tree_alloc(t, (void **)&t->croots_d, sizeof(CfrRoot) * t->croots_h.size()));
+        PASUR_TRY(tree_alloc(t, (void **)&t->broots_d, sizeof(BlockRoot) * t->broots_h.size()));
+        PASUR_CUDA(ctx, cudaMemcpyAsync(t->broots_d, t->broots_h.data(), sizeof(BlockRoot) * t->broots_h.size(),
+                                        cudaMemcpyHostToDevice, ctx->stream));
+        return PASUR_OK;
+    };
+    const int rc = upload();
+    // the uploads read arrays of this call, also where a later one was refused
     PASUR_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
-    return PASUR_OK;
+    return rc;
 }
 
 }  // namespace
