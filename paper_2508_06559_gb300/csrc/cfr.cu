@@ -43,7 +43,8 @@ constexpr size_t kStorageReserve = 352;  // part of a block's shared memory the 
 constexpr size_t kClsBudget[kNumCls - 1] = {37536, 54 * 1024, 74 * 1024, 112 * 1024, 0 /* opt-in max */};
 constexpr int kClsGlobal = kNumCls - 1;
 constexpr int kClsCluster = 6;  // roots split over clusters
-// forked streams: the level-streaming sweep, then the cluster and block launches in turn
+// forked streams: the level-streaming sweep, then the cluster and block launches in turn (the first of them takes the
+// context's own stream)
 constexpr int kAuxStream = 0, kAuxSweep = 1;
 // solved slots per SM and per slot of an item: below it items take fewer slots, so that the GPU has blocks (1 and 4
 // measured the same: rounds have either many slots or few)
@@ -1954,19 +1955,24 @@ int cfr_launch_plan(pasur_ctx *ctx, CfrPlan &plan, const pasur_config *cfg, int6
     p.t0 = t0;
     p.tau = cfg->rm_deadzone;
     p.err = ctx->errflag;
+    // a call of few iterations feels every event (2 to 4 us of a launch of 20 to 60): the launches' times are taken for
+    // PASUR_VERBOSE alone, and the first launch needs no other stream than the context's
+    const bool timed = getenv("PASUR_VERBOSE") != nullptr;
     PASUR_CUDA(ctx, cudaEventRecord(ctx->fork, ctx->stream));
+    auto stream = [&](int c) { return c == kAuxSweep ? ctx->stream : ctx->aux[c]; };
     auto fork = [&](int c) -> int {
-        PASUR_CUDA(ctx, cudaStreamWaitEvent(ctx->aux[c], ctx->fork, 0));
-        PASUR_CUDA(ctx, cudaEventRecord(ctx->cls_t0[c], ctx->aux[c]));
+        if (stream(c) != ctx->stream) PASUR_CUDA(ctx, cudaStreamWaitEvent(stream(c), ctx->fork, 0));
+        if (timed) PASUR_CUDA(ctx, cudaEventRecord(ctx->cls_t0[c], stream(c)));
         return PASUR_OK;
     };
     auto join = [&](int c) -> int {
-        PASUR_CUDA(ctx, cudaEventRecord(ctx->cls_t1[c], ctx->aux[c]));
-        PASUR_CUDA(ctx, cudaEventRecord(ctx->join[c], ctx->aux[c]));
+        if (timed) PASUR_CUDA(ctx, cudaEventRecord(ctx->cls_t1[c], stream(c)));
+        if (stream(c) == ctx->stream) return PASUR_OK;
+        PASUR_CUDA(ctx, cudaEventRecord(ctx->join[c], stream(c)));
         PASUR_CUDA(ctx, cudaStreamWaitEvent(ctx->stream, ctx->join[c], 0));
         return PASUR_OK;
     };
-    // the launches are independent: each runs on its own forked stream (beyond their number,
+    // the launches are independent: each runs on its own stream (beyond their number,
     // several share one), clusters first, largest subtrees first; the level-streaming sweep (thousands
     // of short launches) is queued last, so that the host never waits on its queue before the others
     // start.  The joins come after it: streams share the device's few hardware queues, and an event
@@ -1983,7 +1989,7 @@ int cfr_launch_plan(pasur_ctx *ctx, CfrPlan &plan, const pasur_config *cfg, int6
         cudaLaunchConfig_t lc{};
         cudaLaunchAttribute at[1];
         sweep_launch_config(l, &lc, at);
-        lc.stream = ctx->aux[kAuxSweep + (int)(i % (size_t)nb)];
+        lc.stream = stream(kAuxSweep + (int)(i % (size_t)nb));
         if (l.ctas > 1) ci = plan.clu_d + l.begin;
         else bp.items = plan.blk_d + l.begin;
         PASUR_CUDA(ctx, cudaLaunchKernelExC(&lc, l.ctas > 1 ? cluster_kernel(cfg->variant, l.W) : block_kernel(cfg->variant, l.W), args));
@@ -2080,7 +2086,6 @@ int cfr_run(pasur_tree *t, const pasur_config *cfg) {
     PASUR_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
     float ms = 0.f;
     PASUR_CUDA(ctx, cudaEventElapsedTime(&ms, e0, e1));
-    cfr_plan_times(ctx, t->plan);
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     if (dcfr) dev_free(ctx, dcfr, db);
@@ -2088,6 +2093,7 @@ int cfr_run(pasur_tree *t, const pasur_config *cfg) {
     t->last_launches = (int32_t)(ctx->launches - before);
     t->iters_done += cfg->iters;
     if (getenv("PASUR_VERBOSE")) {
+        cfr_plan_times(ctx, t->plan);
         fprintf(stderr, "[pasur] round %d: %d iterations in %.3f ms\n", t->round, cfg->iters, ms);
         cfr_print_plan(t->plan);
     }

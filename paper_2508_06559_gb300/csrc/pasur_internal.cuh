@@ -476,7 +476,7 @@ int cfr_finalize_plan(pasur_ctx *ctx, CfrPlan &plan, std::vector<CfrItem> *cls_i
                       const std::vector<ClusterItem> &clu);
 void cfr_print_plan(const CfrPlan &plan);
 // launch the plan for cfg->iters iterations starting at iteration t0 (+1); no host synchronisation
-// (capturable); the launches' times are read by cfr_plan_times
+// (capturable); with PASUR_VERBOSE set the launches' times can be read by cfr_plan_times
 int cfr_launch_plan(pasur_ctx *ctx, CfrPlan &plan, const pasur_config *cfg, int64_t t0, const float *dcfr);
 void cfr_plan_times(pasur_ctx *ctx, CfrPlan &plan);
 int cfr_dcfr_factors(pasur_ctx *ctx, const pasur_config *cfg, int64_t t0, float **out, size_t *bytes);
