@@ -243,9 +243,11 @@ int pasur_solved_sizes(const pasur_tree *tree, int64_t solved_sizes[9], int64_t 
  * size it needs.  pasur_load_round restores such a checkpoint into a tree built, unfolded and set
  * up the same way (same deal, round, roots, score slots, next-round utilities, variant and solver
  * settings): the next pasur_cfr_iterate continues the saved run as if it had not stopped, bit for
- * bit.  buf: host memory, read or written only during the call.  Errors: EINVAL (no CFR set-up,
- * cap too small, not a checkpoint, truncated, or a header or leaf hash that differs from the
- * tree's), ECUDA. */
+ * bit.  Checkpoints of the first format (mark PSRCKPT1), which stored the roots split over clusters
+ * by their top and parts, are accepted too.  buf: host memory, read or written only during the call.
+ * Errors: EINVAL (no CFR set-up, cap too small, not a checkpoint, truncated, or a header or leaf hash
+ * that differs from the tree's; of the first format also one that could be of either storage: a split
+ * root of several slots that was not split then), ENOMEM, ECUDA. */
 int pasur_save_round(const pasur_tree *tree, void *buf, size_t cap, size_t *bytes);
 int pasur_load_round(pasur_tree *tree, const void *buf, size_t bytes);
 

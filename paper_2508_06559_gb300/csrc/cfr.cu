@@ -19,30 +19,21 @@
 // slot-minor; the local nodes of each level are numbered in the order of their parents' entries, so
 // the children of consecutive entries are consecutive.
 #include <algorithm>
-#include <atomic>
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
 #include <memory>
 #include <new>
 #include <string>
-#include <thread>
 
 #include "cfr_block.cuh"
 #include "cfr_node.cuh"
+#include "cfr_split.cuh"
 #include "pasur_internal.cuh"
 
 namespace pasur {
 namespace {
 
-// classes by which R and S are stored in device memory (slots per stored item): budget of a block's
-// shared memory at 16 bytes per (node, slot), then the streamed items.  A checkpoint holds R and S in
-// this order, so the classes stay as they are whatever the sweep's own layout is.
-constexpr int kNumCls = 6;
-constexpr size_t kStorageReserve = 352;  // part of a block's shared memory the storage classes leave free
-constexpr size_t kClsBudget[kNumCls - 1] = {37536, 54 * 1024, 74 * 1024, 112 * 1024, 0 /* opt-in max */};
-constexpr int kClsGlobal = kNumCls - 1;
-constexpr int kClsCluster = 6;  // roots split over clusters
 // forked streams: the level-streaming sweep, then the cluster and block launches in turn (the first of them takes the
 // context's own stream)
 constexpr int kAuxStream = 0, kAuxSweep = 1;
@@ -60,23 +51,10 @@ struct CfrParams {
     int32_t *err;
 };
 
-__host__ __device__ __forceinline__ size_t al16(size_t x) { return (x + 15) & ~(size_t)15; }
-
-// shared memory of a resident item: packed active entries (8 B each) and R, S, V, X per
-// (local node, slot); resident items must have fewer than 65535 local nodes
-__host__ __device__ __forceinline__ size_t resident_bytes(int64_t L, int64_t nA, int64_t W) {
-    return L >= 65535 ? ~(size_t)0 >> 1 : 2 * al16((size_t)nA * 4) + 4 * al16((size_t)L * W * 4);
-}
-
 // whether W slots of a root fit one block of the sweep (node indices and the root's mark in 16 bits)
 bool block_fits(const CfrRoot &cr, const BlockRoot &br, int W, size_t limit) {
     return cr.ls[9] < 65535 && block_offsets(cr.ls[9], cr.as[9], br.rs[8], W, kBlockMaxThreads / 32).end <= limit;
 }
-
-constexpr int kMaxSlots = 32;  // score slots per work item
-// a root too large for one block is streamed (class 5) rather than split over a cluster when it
-// has at least this many score slots
-constexpr int64_t kStreamMinSlots = 16;
 
 // Index of child edge a of a node whose first child is local node c, at slot w of an item of
 // 2^sh slots (slot-minor layout; every item's slot count is a power of two); W1: single-slot
@@ -1006,29 +984,6 @@ struct RootSplit {
     std::string msg;
 };
 
-// fn(0) .. fn(n - 1) on up to 16 host threads (fewer where a thread does not start); false if one of them threw
-template <typename Fn>
-bool on_threads(size_t n, const Fn &fn) {
-    std::atomic<size_t> next{0};
-    std::atomic<bool> failed{false};
-    auto worker = [&]() {
-        try {
-            for (size_t i = next++; i < n; i = next++) fn(i);
-        } catch (...) {
-            failed = true;
-        }
-    };
-    const size_t most = std::min<size_t>({(size_t)std::max(1u, std::thread::hardware_concurrency()), (size_t)16, n});
-    std::vector<std::thread> threads;
-    try {
-        for (size_t w = 1; w < most; w++) threads.emplace_back(worker);
-    } catch (...) {
-    }
-    worker();
-    for (std::thread &x : threads) x.join();
-    return !failed;
-}
-
 constexpr int kSplitRuns = 96;  // runs a part is assumed to have while it is planned (checked after)
 
 // the most slots of one item when S slots are shared out evenly over items of at most cap slots
@@ -1071,43 +1026,6 @@ int plan_splits(pasur_tree *t, const pasur_config *cfg, size_t limit, const std:
     const size_t target = cfg->split_bytes > 0 ? std::min<size_t>((size_t)cfg->split_bytes, limit) : limit;
     const bool verbose = getenv("PASUR_VERBOSE") != nullptr;
     const int warps = kBlockMaxThreads / 32;
-    // what the cut of a root at a level gives, whatever the slots: the active level-ell nodes (heads, by local index), the
-    // subtree of every local node below them (-1: none), and the subtrees' active entries and nodes.  Made once for all
-    // slot counts tried: 79 roots of 1.0e7 nodes are split in 13 ms (51 with a cut per count)
-    struct LevelCut {
-        bool made = false;
-        std::vector<int32_t> heads, sub;
-        std::vector<int64_t> sa, sl;
-        int64_t tot = 0, amax = 0;
-    };
-    auto cut_at = [&](int64_t g, int ell, LevelCut &c) {
-        if (c.made) return;
-        const CfrRoot &cr = t->croots_h[(size_t)g];
-        const int64_t L = cr.ls[9];
-        const int32_t *li = hli.data() + cr.act_off, *cs = hcs.data() + cr.act_off;
-        const uint16_t *dd = hd.data() + cr.act_off;
-        for (int32_t e = cr.as[ell]; e < cr.as[ell + 1]; e++) c.heads.push_back(li[e]);
-        std::sort(c.heads.begin(), c.heads.end());
-        const size_t ns = c.heads.size();
-        c.sub.assign((size_t)L, -1);
-        for (size_t i = 0; i < ns; i++) c.sub[(size_t)c.heads[i]] = (int32_t)i;
-        c.sa.assign(ns, 0);
-        c.sl.assign(ns, 0);
-        for (int k = ell; k < 8; k++)
-            for (int32_t e = cr.as[k]; e < cr.as[k + 1]; e++) {
-                const int32_t sid = c.sub[(size_t)li[e]];
-                if (sid < 0) continue;
-                c.sa[(size_t)sid]++;
-                for (int a = 0; a < dd[e]; a++) c.sub[(size_t)(cs[e] + a)] = sid;
-            }
-        for (int64_t x = cr.ls[ell]; x < L; x++)
-            if (c.sub[(size_t)x] >= 0) c.sl[(size_t)c.sub[(size_t)x]]++;
-        for (int64_t n : c.sa) {
-            c.tot += n;
-            c.amax = std::max(c.amax, n);
-        }
-        c.made = true;
-    };
     // the split of one root for items of W slots over at most qmax CTAs
     auto split_one = [&](int64_t g, int W, int qmax, LevelCut *cuts, RootSplit &o) {
         const CfrRoot cr = t->croots_h[(size_t)g];
@@ -1121,47 +1039,19 @@ int plan_splits(pasur_tree *t, const pasur_config *cfg, size_t limit, const std:
             if (cr.as[ell + 1] - cr.as[ell] < 2) continue;
             const size_t top_bytes = block_offsets(cr.ls[ell + 1], cr.as[ell], br.rs[ell], W, warps).end;
             if (top_bytes >= limit) break;
-            cut_at(g, ell, cuts[ell]);
+            cuts[ell].make(cr, ell, li, cs, dd);
             const LevelCut &cut = cuts[ell];
             const std::vector<int32_t> &heads = cut.heads, &sub = cut.sub;
-            const std::vector<int64_t> &sa = cut.sa, &sl = cut.sl;
             const int ns = (int)heads.size();
-            const int64_t tot = cut.tot, amax = cut.amax;
             // the target size sets the starting count of parts, a block's shared memory is the hard
             // limit of every part
             const size_t need = bytes(L, nA);
             const int q0 = (int)std::min<size_t>((size_t)qmax, std::max<size_t>(2, (need + target - 1) / target));
-            // contiguous parts: greedy fill with an entry cap (and the byte limit); the smallest
-            // cap that needs at most Q parts, by bisection
-            auto greedy = [&](int64_t cap, std::vector<int> &first) -> bool {
-                first.assign(1, 0);
-                int64_t pa = 0, plc = 0, pg = 0;
-                for (int i = 0; i < ns; i++) {
-                    const size_t lim = first.size() == 1 ? limit - top_bytes : limit;
-                    const bool fits = bytes(plc + sl[(size_t)i] + pg + 1, pa + sa[(size_t)i]) <= lim;
-                    if (pa > 0 && (!fits || pa + sa[(size_t)i] > cap)) {
-                        first.push_back(i);
-                        pa = plc = pg = 0;
-                    }
-                    const size_t lim2 = first.size() == 1 ? limit - top_bytes : limit;
-                    pa += sa[(size_t)i];
-                    plc += sl[(size_t)i];
-                    pg += 1;
-                    if (bytes(plc + pg, pa) > lim2) return false;
-                }
-                return true;
-            };
-            // without an entry cap: whether every subtree fits a block, and the fewest parts
+            const PartPacking<decltype(bytes)> packing{cut, bytes, limit, top_bytes};
+            const int fewest = packing.fewest();
             std::vector<int> first;
-            const int fewest = greedy(tot, first) ? (int)first.size() : qmax + 1;
-            for (int Q = std::max(q0, fewest); Q <= qmax; Q++) {
-                int64_t lo = std::max<int64_t>(amax, (tot + Q - 1) / Q), hi = tot;
-                while (lo < hi) {
-                    const int64_t mid = lo + (hi - lo) / 2;
-                    if (greedy(mid, first) && (int)first.size() <= Q) hi = mid;
-                    else lo = mid + 1;
-                }
-                if (!greedy(lo, first) || (int)first.size() > Q) continue;
+            for (int Q = std::max(q0, fewest); fewest > 0 && Q <= qmax; Q++) {
+                if (!packing.balanced(Q, first)) continue;
                 const int np = (int)first.size();
                 if (np < 2 || ctx->clusters_of[np] == 0) continue;
                 first.push_back(ns);
@@ -1274,7 +1164,7 @@ int plan_splits(pasur_tree *t, const pasur_config *cfg, size_t limit, const std:
             }
             if (verbose) {
                 int64_t big = 0;
-                for (int i = 0; i < ns; i++) big = std::max<int64_t>(big, (int64_t)bytes(sl[(size_t)i] + 1, sa[(size_t)i]));
+                for (int i = 0; i < ns; i++) big = std::max<int64_t>(big, (int64_t)bytes(cut.sl[(size_t)i] + 1, cut.sa[(size_t)i]));
                 char line[256];
                 snprintf(line, sizeof line, "[pasur] root %lld (L %lld, active %lld), %d slots: no split at level %d: %d subtrees, top "
                                             "%zu B, largest subtree %lld B, part limit %zu B\n",
@@ -1525,12 +1415,8 @@ int cfr_setup_tree(pasur_tree *t, const pasur_config *cfg, int tree, std::vector
     size_t limit = 0;
     PASUR_TRY(cfr_dyn_smem_limit(ctx, &limit));
     PASUR_TRY(raise_limits(ctx, limit));
-    // how R and S are stored: every root in the smallest storage class its subtree fits with one slot,
-    // in items of as many slots as that class holds
-    const size_t dyn_max = ctx->smem_optin > kStorageReserve ? ctx->smem_optin - kStorageReserve : 0;
-    size_t budget[kNumCls - 1];
-    for (int c = 0; c < kNumCls - 1; c++) budget[c] = kClsBudget[c] ? std::min<size_t>(kClsBudget[c], dyn_max) : dyn_max;
-    const int wcap = cfg->slots_per_item > 0 ? std::min(cfg->slots_per_item, kMaxSlots) : kMaxSlots;
+    const Storage storage(ctx->smem_optin, cfg->slots_per_item);
+    t->layout_cfg = *cfg;
     t->croots_h.resize((size_t)t->n_roots);
     t->broots_h.resize((size_t)t->n_roots);
     t->cparts_h.clear();
@@ -1588,20 +1474,7 @@ int cfr_setup_tree(pasur_tree *t, const pasur_config *cfg, int tree, std::vector
                 s0 += ci.ns;
             }
         } else {
-            // slots per stored item: a power of two (the streaming sweep indexes slots with shifts).
-            // Automatic: the smallest class the root fits with one slot, then the largest count that
-            // class holds.  With cfg.slots_per_item: that many slots (at most the root's), in the
-            // smallest class that holds them, fewer where no class does.
-            int64_t want = 1;
-            if (cfg->slots_per_item > 0)
-                while (want * 2 <= std::min<int64_t>(Sg, wcap)) want *= 2;
-            for (; want >= 1 && store == kClsGlobal && !streamed[(size_t)g]; want /= 2)
-                for (int c = 0; c < kNumCls - 1; c++)
-                    if (resident_bytes(L, nA, want) <= budget[c]) {
-                        store = c;
-                        break;
-                    }
-            while (w * 2 <= std::min<int64_t>(Sg, wcap) && (store == kClsGlobal || resident_bytes(L, nA, w * 2) <= budget[store])) w *= 2;
+            w = storage.width(L, nA, Sg, streamed[(size_t)g], &store);
             // the sweep's blocks hold more than the storage classes: a root beyond those may still fit
             cls = store;
             if (cls == kClsGlobal && !streamed[(size_t)g] && block_fits(cr, t->broots_h[(size_t)g], 1, limit)) cls = kClsGlobal - 1;

@@ -403,6 +403,7 @@ struct pasur_tree {
     int32_t *cx_d = nullptr;
     CfrPlan plan;                       // this tree alone
     TreeView view{};                    // its pointers for the CFR kernel
+    pasur_config layout_cfg{};          // the settings the storage of R and S was laid out for
     int64_t data_size = 0, scratch_size = 0;
     float *R = nullptr, *S = nullptr;   // per (local node, slot) of every item
     float *V = nullptr, *X = nullptr;   // values and reaches of the non-resident items

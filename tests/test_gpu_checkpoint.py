@@ -94,3 +94,48 @@ def test_foreign_checkpoints_are_refused(P, ctx):
     same.pasur_load_round(ck)
     for t in (a, other, shifted, same):
         t.free()
+
+
+def golden_tree(ctx, name):
+    """A final round of the golden checkpoint's pools and slots, and the checkpoint."""
+    import os
+    f = np.load(os.path.join(os.path.dirname(__file__), "golden", name + ".npz"))
+    pools, slots = f["pools"], int(f["slots"])
+    from paper_2508_06559_gb300 import pasur
+    t = ctx.pasur_build_round(pasur.pasur_deal(9), 5, pools)
+    clubs = [(a, b, 0, 0) for a in range(7) for b in range(7)][:slots]
+    t.pasur_unfold(np.arange(len(pools) + 1) * slots, np.array(clubs * len(pools), np.int16))
+    return t, f["ck"]
+
+
+@pytest.mark.parametrize("name,extra", [("checkpoint_split_vanilla", dict(split_bytes=4096)),
+                                        ("checkpoint_split_dcfr", dict(split_bytes=2048, variant=1))])
+def test_checkpoints_of_the_first_format(P, ctx, name, extra):
+    """Checkpoints after T1 iterations by the code that stored split roots by their top and parts
+    (mark PSRCKPT1): continued for T2 they give the uninterrupted run bit for bit.  So do the
+    present words under that mark, which stood there for a while, and under the present one."""
+    cfg = lambda it: P.pasur_config_default(iters=it, **extra)  # noqa: E731
+    a, old = golden_tree(ctx, name)
+    a.pasur_cfr_iterate(cfg(T1))
+    assert (a.pasur_root_paths() == 6).all()
+    now = a.pasur_save_round()
+    assert bytes(old[:8]) == b"PSRCKPT1" and bytes(now[:8]) == b"PSRCKPT2" and len(old) > len(now)
+    marked = now.copy()
+    marked[:8] = old[:8]
+    a.pasur_cfr_iterate(cfg(T2))
+    want_s, want_u = a.pasur_avg_strategy(), a.pasur_round_utilities()
+    a.free()
+    for ck in (old, now, marked):
+        b, _ = golden_tree(ctx, name)
+        b.pasur_cfr_iterate(cfg(0))
+        b.pasur_load_round(ck)
+        assert np.array_equal(b.pasur_save_round(), now)
+        b.pasur_cfr_iterate(cfg(T2))
+        assert np.array_equal(b.pasur_avg_strategy(), want_s) and np.array_equal(b.pasur_round_utilities(), want_u)
+        b.free()
+    for ck in (old[:-4], now[:-4]):
+        b, _ = golden_tree(ctx, name)
+        b.pasur_cfr_iterate(cfg(0))
+        with pytest.raises(P.PasurError):
+            b.pasur_load_round(ck)
+        b.free()
