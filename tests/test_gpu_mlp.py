@@ -387,3 +387,44 @@ def test_device_rows_at_any_element(ctx, offset):
     assert P.load().pasur_mlp_gradients(mlp.h, ptr(x), ptr(y), C.c_int64(n), ptr(l2), ptr(g2)) == P.PASUR_OK
     assert l2[0] == np.float32(loss) and np.array_equal(g2, grad)
     mlp.free()
+
+
+def test_epochs_of_several_batches_match_oracle(ctx):
+    """Two epochs of 700 rows in batches of 256 (the last of 188): six Adam steps over the rows in
+    the order of the shuffle (Fisher-Yates on SplitMix64 draws that go on over the epochs), against
+    the oracle's, and the epochs' losses.  An update is lr * m_hat / sqrt(v_hat): elements whose
+    gradient is at rounding level may move differently, by at most 2 lr a step; the others agree."""
+    from paper_2508_06559_gb300 import pasur as P
+    rng = np.random.default_rng(21)
+    n, batch, lr, epochs = 700, 256, 1e-3, 2
+    X, Y = M.to_bf16(rng.normal(0, 1, (n, 256))), rng.normal(0, 2, n).astype(np.float32)
+    flat32, _ = params(7)
+    mlp = P.Mlp(ctx, dataset_capacity=n)
+    mlp.set_params(flat32)
+    mlp.dataset_add_rows(bf16_bits(X), Y)
+    losses = mlp.train(epochs, batch, lr, shuffle_seed=5)
+    got = mlp.get_params()
+    mlp.free()
+    flat = flat32.astype(np.float64)
+    m, v, t, x, mask = np.zeros_like(flat), np.zeros_like(flat), 0, 5, (1 << 64) - 1
+    for e in range(epochs):
+        perm, total = list(range(n)), 0.0
+        for i in range(n - 1, 0, -1):
+            x = (x + 0x9E3779B97F4A7C15) & mask
+            z = ((x ^ (x >> 30)) * 0xBF58476D1CE4E5B9) & mask
+            z = ((z ^ (z >> 27)) * 0x94D049BB133111EB) & mask
+            z ^= z >> 31
+            j = (z * (i + 1)) >> 64
+            perm[i], perm[j] = perm[j], perm[i]
+        steps = range(0, n, batch)
+        for r0 in steps:
+            rows = perm[r0:r0 + batch]
+            t += 1
+            loss, g, _ = M.loss_and_grads(oracle_view(flat.astype(np.float32)), X[rows], Y[rows].astype(np.float64), round_act=True)
+            flat, m, v = M.adam_step(flat, M.flatten(g), m, v, t, lr)
+            total += loss
+        assert abs(losses[e] - total / len(steps)) <= 3e-3 * total / len(steps), e
+    d = np.abs(got - flat)
+    assert d.max() <= 2 * lr * t + 1e-6
+    assert (d > 0.1 * lr).mean() < 0.02, (d > 0.1 * lr).mean()
+    assert np.median(d) < 2e-5
