@@ -34,7 +34,7 @@ WORKLOADS = {
     "rounds_4_5": (4, "rounds 5-6 (0-based 4-5) of one seeded deal, round 5 unfolded over every score round 4 reaches"),
     "final_round": (5, "final round of one seeded deal as a standalone round, score (0,0,0,0)"),
     "batch64": (3, "64 seeded deals (seeds S..S+63), rounds 4-6 (0-based 3-5) of each from the standalone root, "
-                   "solved together: one merged persistent launch per round and slot count under a CUDA graph"),
+                   "solved together: one merged launch per round, slot count and size under a CUDA graph"),
     "surrogate64": (0, "64 seeded deals (seeds S..S+63): rounds 1-3 (0-based 0-2) solved in one batch with the "
                        "leaves of round 3 valued by the trained surrogate at the round-4 roots; 10 % of every "
                        "deal's round-4 pools solved exactly (rounds 4-6 from those roots only), a copy of the "

@@ -201,8 +201,8 @@ int next_roots(pasur_tree *t, std::vector<uint64_t> &pools, std::vector<int64_t>
     PASUR_TRY(rt.fill(table_size(q8, 1 << 20), q8, kScoreKeyBits + bits_for(n_pools + 1),
                       [&](unsigned long long *tab, uint32_t mask, int32_t *flags) -> int {
         if (m8 == 0) return PASUR_OK;
-        // lanes per GT leaf: a third to an eighth of its slots, so that a lane's look-ups overlap (a wide forward sweep:
-        // as many lanes as slots 7.4 ms, four throughout 7.06, two 6.85, one 7.14)
+        // lanes per GT leaf: fewer than its slots, so that a lane's look-ups overlap: two from 2 slots on, eight from 64 (a wide
+        // forward sweep: as many lanes as slots 7.4 ms, four throughout 7.06, two 6.85, one 7.14)
         const int64_t ns = q8 / m8;
         auto go = [&](auto lpl) {
             constexpr int LPL = decltype(lpl)::value;

@@ -348,22 +348,15 @@ int build_levels(pasur_tree *t, const uint64_t *root_pools_dev) {
     PASUR_CUDA(ctx, cudaMemcpyAsync(hb.data(), bounds, bb, cudaMemcpyDeviceToHost, ctx->stream));
     PASUR_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
     t->roots_h.assign((size_t)nr, RootInfo{});
-    int64_t soff = 0;
     for (int64_t g = 0; g < nr; g++) {
         RootInfo &ri = t->roots_h[(size_t)g];
         int64_t local = 0;
         for (int k = 0; k < 9; k++) {
-            ri.lvl_begin[k] = hb[(size_t)g * 9 + k];
-            int64_t cnt = hb[(size_t)(g + 1) * 9 + k] - ri.lvl_begin[k];
+            int64_t cnt = hb[(size_t)(g + 1) * 9 + k] - hb[(size_t)g * 9 + k];
             if (local + cnt > INT32_MAX) return set_err(ctx, PASUR_EOVERFLOW, "a root subtree exceeds 2^31 nodes");
             ri.lvl_count[k] = (int32_t)cnt;
-            ri.local_start[k] = (int32_t)local;
             local += cnt;
         }
-        ri.local_start[9] = (int32_t)local;
-        ri.n_internal = ri.local_start[8];
-        ri.struct_off = soff;
-        soff += ri.n_internal;
     }
     return PASUR_OK;
 }

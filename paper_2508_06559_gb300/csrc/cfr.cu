@@ -5,8 +5,9 @@
 // reach is 1), so the round is cut into work items: one GT root and a run of W of its score
 // slots.  One thread block runs all T iterations of an item (cfr_sweep.cuh): per iteration a top-down
 // pass over levels 0..6 (regret matching and reach) and a bottom-up pass over levels 7..0 (values,
-// regret and strategy-sum updates), with a block barrier between levels; an (active node, slot) pair
-// belongs to one thread in each pass, so the updates of a node's child edges need no atomics.
+// regret and strategy-sum updates), with a block barrier between levels (a warp barrier between levels
+// of one chunk each, which one warp steps through); an (active node, slot) pair belongs to one thread in
+// each pass, so the updates of a node's child edges need no atomics.
 //
 // Forced-move chains are resolved once: a node whose whole subtree is one path of single moves
 // has sigma = 1 and zero regret on every edge below it and the value of its one leaf, so only the
@@ -57,61 +58,58 @@ bool block_fits(const CfrRoot &cr, const BlockRoot &br, int W, size_t limit) {
 }
 
 // Index of child edge a of a node whose first child is local node c, at slot w of an item of
-// 2^sh slots (slot-minor layout; every item's slot count is a power of two); W1: single-slot
-// items, where this is c + a.
-template <bool W1>
+// 2^sh slots (slot-minor layout; every item's slot count is a power of two).
 __device__ __forceinline__ int at(int c, int a, int sh, int w) {
-    return W1 ? c + a : ((c + a) << sh) + w;
+    return ((c + a) << sh) + w;
 }
 
 // Regret matching at one (active node, slot) with D children and the reach of the children.
 // X[n] holds the reach of the player who moved into node n; own = the mover's reach at the node.
-template <int D, bool W1>
+template <int D>
 __device__ __forceinline__ void td_node(int c, int sh, int w, float own, const float *__restrict__ R, float *__restrict__ X,
                                         float thr) {
     if constexpr (D == 1) {
-        X[at<W1>(c, 0, sh, w)] = own;
+        X[at(c, 0, sh, w)] = own;
         return;
     } else {
         float r[D], x[D];
 #pragma unroll
-        for (int a = 0; a < D; a++) r[a] = R[at<W1>(c, a, sh, w)];
+        for (int a = 0; a < D; a++) r[a] = R[at(c, a, sh, w)];
         rm_reach<D>(r, own, thr, x);
 #pragma unroll
-        for (int a = 0; a < D; a++) X[at<W1>(c, a, sh, w)] = x[a];
+        for (int a = 0; a < D; a++) X[at(c, a, sh, w)] = x[a];
     }
 }
 
-template <bool W1>
 __device__ __forceinline__ void td_node_any(int c, int d, int sh, int w, float own, const float *__restrict__ R,
                                             float *__restrict__ X, float thr) {
     float sum = 0.f;
     for (int a = 0; a < d; a++) {
-        const float r = R[at<W1>(c, a, sh, w)];
+        const float r = R[at(c, a, sh, w)];
         sum += r > thr ? r : 0.f;
     }
     if (sum > 0.f) {
         const float inv = rcp_pos(sum);
         for (int a = 0; a < d; a++) {
-            const float r = R[at<W1>(c, a, sh, w)];
-            X[at<W1>(c, a, sh, w)] = r > thr ? own * (r * inv) : 0.f;
+            const float r = R[at(c, a, sh, w)];
+            X[at(c, a, sh, w)] = r > thr ? own * (r * inv) : 0.f;
         }
     } else {
         const float u = own * (1.f / (float)d);
-        for (int a = 0; a < d; a++) X[at<W1>(c, a, sh, w)] = u;
+        for (int a = 0; a < d; a++) X[at(c, a, sh, w)] = u;
     }
 }
 
 // Value of one (active node, slot) with D children and the updates of its child edges (bu_vals)
 // in R and S.  Returns v(h).
-template <int VARIANT, int D, bool W1>
+template <int VARIANT, int D>
 __device__ __forceinline__ float bu_node(int c, int sh, int w, float pp, float spo, float *__restrict__ R,
                                          float *__restrict__ S, const float *__restrict__ V, float thr, float fpos,
                                          float fneg, float fs) {
     float r[D], v[D], s[D];
 #pragma unroll
     for (int a = 0; a < D; a++) {
-        const int q = at<W1>(c, a, sh, w);
+        const int q = at(c, a, sh, w);
         r[a] = R[q];
         v[a] = V[q];
         s[a] = S[q];
@@ -119,31 +117,31 @@ __device__ __forceinline__ float bu_node(int c, int sh, int w, float pp, float s
     const float vh = bu_vals<VARIANT, D>(r, v, s, pp, spo, thr, fpos, fneg, fs);
 #pragma unroll
     for (int a = 0; a < D; a++) {
-        const int q = at<W1>(c, a, sh, w);
+        const int q = at(c, a, sh, w);
         R[q] = r[a];
         S[q] = s[a];
     }
     return vh;
 }
 
-template <int VARIANT, bool W1>
+template <int VARIANT>
 __device__ __forceinline__ float bu_node_any(int c, int d, int sh, int w, float pp, float spo, float *__restrict__ R,
                                              float *__restrict__ S, const float *__restrict__ V, float thr, float fpos,
                                              float fneg, float fs) {
     float sum = 0.f;
     for (int a = 0; a < d; a++) {
-        const float r = R[at<W1>(c, a, sh, w)];
+        const float r = R[at(c, a, sh, w)];
         sum += r > thr ? r : 0.f;
     }
     const float inv = sum > 0.f ? rcp_pos(sum) : 0.f, u = 1.f / (float)d;
-    const float v0 = V[at<W1>(c, 0, sh, w)];
+    const float v0 = V[at(c, 0, sh, w)];
     float vh = v0;
     for (int a = 1; a < d; a++) {
-        const float r = R[at<W1>(c, a, sh, w)];
-        vh += (sum > 0.f ? (r > thr ? r * inv : 0.f) : u) * (V[at<W1>(c, a, sh, w)] - v0);
+        const float r = R[at(c, a, sh, w)];
+        vh += (sum > 0.f ? (r > thr ? r * inv : 0.f) : u) * (V[at(c, a, sh, w)] - v0);
     }
     for (int a = 0; a < d; a++) {
-        const int q = at<W1>(c, a, sh, w);
+        const int q = at(c, a, sh, w);
         const float r = R[q];
         const float sg = sum > 0.f ? (r > thr ? r * inv : 0.f) : u;
         const float inst = spo * (V[q] - vh);
@@ -269,15 +267,15 @@ __device__ __forceinline__ void stream_pair(const StreamDesc &sd, int k, int64_t
     if (TD) {
         const float own = pl < 0 ? 1.f : X[(pl << sh) + w];
         switch (d) {
-            case 1: td_node<1, false>(c, sh, w, own, R, X, thr); break;
-            case 2: td_node<2, false>(c, sh, w, own, R, X, thr); break;
-            case 3: td_node<3, false>(c, sh, w, own, R, X, thr); break;
-            case 4: td_node<4, false>(c, sh, w, own, R, X, thr); break;
-            case 5: td_node<5, false>(c, sh, w, own, R, X, thr); break;
-            case 6: td_node<6, false>(c, sh, w, own, R, X, thr); break;
-            case 7: td_node<7, false>(c, sh, w, own, R, X, thr); break;
-            case 8: td_node<8, false>(c, sh, w, own, R, X, thr); break;
-            default: td_node_any<false>(c, d, sh, w, own, R, X, thr);
+            case 1: td_node<1>(c, sh, w, own, R, X, thr); break;
+            case 2: td_node<2>(c, sh, w, own, R, X, thr); break;
+            case 3: td_node<3>(c, sh, w, own, R, X, thr); break;
+            case 4: td_node<4>(c, sh, w, own, R, X, thr); break;
+            case 5: td_node<5>(c, sh, w, own, R, X, thr); break;
+            case 6: td_node<6>(c, sh, w, own, R, X, thr); break;
+            case 7: td_node<7>(c, sh, w, own, R, X, thr); break;
+            case 8: td_node<8>(c, sh, w, own, R, X, thr); break;
+            default: td_node_any(c, d, sh, w, own, R, X, thr);
         }
     } else {
         const float pp = pl < 0 ? 1.f : X[(pl << sh) + w];
@@ -285,15 +283,15 @@ __device__ __forceinline__ void stream_pair(const StreamDesc &sd, int k, int64_t
         const float spo = alex ? po : -po;
         float vh;
         switch (d) {
-            case 1: vh = bu_node<VARIANT, 1, false>(c, sh, w, pp, spo, R, S, V, thr, fpos, fneg, fs); break;
-            case 2: vh = bu_node<VARIANT, 2, false>(c, sh, w, pp, spo, R, S, V, thr, fpos, fneg, fs); break;
-            case 3: vh = bu_node<VARIANT, 3, false>(c, sh, w, pp, spo, R, S, V, thr, fpos, fneg, fs); break;
-            case 4: vh = bu_node<VARIANT, 4, false>(c, sh, w, pp, spo, R, S, V, thr, fpos, fneg, fs); break;
-            case 5: vh = bu_node<VARIANT, 5, false>(c, sh, w, pp, spo, R, S, V, thr, fpos, fneg, fs); break;
-            case 6: vh = bu_node<VARIANT, 6, false>(c, sh, w, pp, spo, R, S, V, thr, fpos, fneg, fs); break;
-            case 7: vh = bu_node<VARIANT, 7, false>(c, sh, w, pp, spo, R, S, V, thr, fpos, fneg, fs); break;
-            case 8: vh = bu_node<VARIANT, 8, false>(c, sh, w, pp, spo, R, S, V, thr, fpos, fneg, fs); break;
-            default: vh = bu_node_any<VARIANT, false>(c, d, sh, w, pp, spo, R, S, V, thr, fpos, fneg, fs);
+            case 1: vh = bu_node<VARIANT, 1>(c, sh, w, pp, spo, R, S, V, thr, fpos, fneg, fs); break;
+            case 2: vh = bu_node<VARIANT, 2>(c, sh, w, pp, spo, R, S, V, thr, fpos, fneg, fs); break;
+            case 3: vh = bu_node<VARIANT, 3>(c, sh, w, pp, spo, R, S, V, thr, fpos, fneg, fs); break;
+            case 4: vh = bu_node<VARIANT, 4>(c, sh, w, pp, spo, R, S, V, thr, fpos, fneg, fs); break;
+            case 5: vh = bu_node<VARIANT, 5>(c, sh, w, pp, spo, R, S, V, thr, fpos, fneg, fs); break;
+            case 6: vh = bu_node<VARIANT, 6>(c, sh, w, pp, spo, R, S, V, thr, fpos, fneg, fs); break;
+            case 7: vh = bu_node<VARIANT, 7>(c, sh, w, pp, spo, R, S, V, thr, fpos, fneg, fs); break;
+            case 8: vh = bu_node<VARIANT, 8>(c, sh, w, pp, spo, R, S, V, thr, fpos, fneg, fs); break;
+            default: vh = bu_node_any<VARIANT>(c, d, sh, w, pp, spo, R, S, V, thr, fpos, fneg, fs);
         }
         V[(li << sh) + w] = vh;
         if (k == 0) sp.acc[sd.slot + w] += (double)vh;  // the root (one entry per item)

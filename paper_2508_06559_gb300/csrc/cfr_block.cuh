@@ -1,5 +1,5 @@
 // The block sweep: all T iterations of one work item (a root and a run of its score slots) in one
-// thread block, its state on chip.  Host-side declarations and the layout shared with cfr_block.cu.
+// thread block, its state on chip.  Host-side declarations and the layout shared with cfr_sweep.cuh.
 #pragma once
 
 #include "pasur_internal.cuh"

@@ -223,7 +223,7 @@ constexpr uint32_t kSegUp = 1, kSegAlex = 2, kSegSyncWarp = 4, kSegSync = 8, kSe
 constexpr int kSegSolo = 256, kSegSmall = 512;  // of a level step: warp 0's alone, few nodes (not stored in segments)
 // Most chunks of a step that is warp 0's alone.  With one, a final round of 1000 iterations, the last four rounds, six
 // rounds and 64 deals take 5.6, 23.1, 48.1 and 165 ms; with none 5.9, 24.2, 48.9, 168; with two 5.6, 24.2, 49.6, 170; with
-// four 7.4, -, 58.6, 193.
+// four 7.4, -, 58.6, 193.  (Here and below: one comparison on one GPU; from one to another the longer ones differ by up to 8 %.)
 constexpr int kSoloChunks = 1;
 
 struct SweepShared {

@@ -9,7 +9,7 @@
 // copies (cp.async.bulk, completion on an mbarrier), tcgen05.mma issued by one thread with the
 // f32 accumulator in tensor memory, and a fused epilogue that reads the accumulator back with
 // tcgen05.ld: bias + GELU for the forward layers, the output layer, loss and its gradient for the
-// last hidden layer, GELU' for the input gradients, atomics for the weight gradients; k_infer runs
+// last hidden layer, GELU' for the input gradients, parts of the weight gradients (Partials); k_infer runs
 // all layers of a row tile for the predictions.  Operands live in HBM in the tensor cores' canonical K-major layout without swizzle
 // (8x8 core matrices of 128 contiguous bytes), ordered so that one (128-row, 64-column) tile is
 // one contiguous 16 KB block: element (r, k) of an R-row matrix is at

@@ -178,13 +178,8 @@ struct PhaseTimer {
     }
 };
 
-struct RootInfo {             // one GT root's subtree, level by level
-    int64_t lvl_begin[9];     // first GT node of the root at level k
+struct RootInfo {             // one GT root's subtree
     int32_t lvl_count[9];     // its GT nodes at level k
-    int32_t local_start[10];  // local (level-major) index of its first node at level k; [9] = nodes
-    int64_t struct_off;       // offset of its internal nodes in the local structure arrays
-    int32_t n_internal;       // nodes at levels 0..7
-    int32_t pad;
 };
 
 // CFR view of one GT root's subtree.  Nodes whose whole subtree is a single path of forced moves
@@ -201,7 +196,6 @@ struct CfrRoot {
     int64_t actbase[9];       // global active-rank of the root's first node at level k
     int32_t W;                // slots per work item of this root
     int32_t cls;              // launch class of its items
-    int64_t item0;            // index of its first work item
 };
 
 // A root subtree too large for one block's shared memory, split over a thread-block cluster: CTA 0
