@@ -102,8 +102,8 @@ int bits_for(int64_t n) {
     return b;
 }
 
-// A table filled by `insert` (which may find it too small), its distinct keys in ascending order (device
-// and host) and the rank of every slot's key.
+// A table filled by `insert` (which may find it too small), its distinct keys in ascending order (host)
+// and the rank of every slot's key (device).
 struct KeyTable {
     pasur_ctx *ctx;
     unsigned long long *tab = nullptr;
@@ -149,6 +149,9 @@ struct KeyTable {
             release();
             if (size >= (int64_t)1 << 31) return set_err(ctx, PASUR_EOVERFLOW, "too many next-round roots");
         }
+        // the keys are read: the ranks take the table's place
+        dev_free(ctx, tab, sizeof(unsigned long long) * (size_t)(size + 1));
+        tab = nullptr;
         PASUR_TRY(radix_sort_pairs(ctx, keys, at, n, bits));
         PASUR_TRY(dev_alloc(ctx, (void **)&rank, sizeof(int64_t) * (size_t)size));
         host.resize((size_t)n);
@@ -159,6 +162,7 @@ struct KeyTable {
             PASUR_CUDA(ctx, cudaMemcpyAsync(host.data(), keys, sizeof(uint64_t) * (size_t)n, cudaMemcpyDeviceToHost, ctx->stream));
         }
         PASUR_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+        release();
         return PASUR_OK;
     }
 };

@@ -301,6 +301,8 @@ int build_levels(pasur_tree *t, const uint64_t *root_pools_dev) {
         int64_t m = t->M[k];
         PASUR_TRY(tree_alloc(t, (void **)&t->child_off[k], sizeof(int64_t) * (size_t)(m + 1)));
         PASUR_TRY(exclusive_scan_i32(ctx, deg, t->child_off[k], m));
+        dev_free(ctx, deg, degb);  // stream-ordered, before the next level's arrays are taken
+        deg = nullptr;
         int64_t m1 = 0;
         PASUR_TRY(read_i64(ctx, t->child_off[k] + m, &m1));
         t->M[k + 1] = m1;
@@ -316,8 +318,6 @@ int build_levels(pasur_tree *t, const uint64_t *root_pools_dev) {
         t->lay[k + 1] = (int8_t *)(lv + b_st + b_par);
         t->pick[k + 1] = (uint64_t *)(lv + b_st + b_par + b_lay);
         t->root[k + 1] = (int32_t *)(lv + b_st + b_par + b_lay + b_pick);
-        dev_free(ctx, deg, degb);
-        deg = nullptr;
         if (k < 7) {
             degb = sizeof(int32_t) * cap;
             PASUR_TRY(dev_alloc(ctx, (void **)&deg, degb));

@@ -805,14 +805,16 @@ int build_block_order(pasur_tree *t, const int32_t *act_rk) {
 
 int build_layout(pasur_tree *t) {
     pasur_ctx *ctx = t->ctx;
-    std::vector<std::pair<void *, size_t>> tmp;
+    std::vector<std::pair<void *, size_t>> tmp, rk_tmp;  // rk_tmp: what the block order needs too
     struct Guard {
         pasur_ctx *c;
         std::vector<std::pair<void *, size_t>> *v;
-        ~Guard() {
+        ~Guard() { drop(); }
+        void drop() {
             for (auto &x : *v) dev_free(c, x.first, x.second);
+            v->clear();
         }
-    } guard{ctx, &tmp};
+    } guard{ctx, &tmp}, rk_guard{ctx, &rk_tmp};
     int32_t *local = nullptr, *active = nullptr;
     int64_t *lrank = nullptr, *arank = nullptr, *ranks = nullptr;
     const int64_t nr = t->n_roots;
@@ -825,13 +827,14 @@ int build_layout(pasur_tree *t) {
     }
     const int64_t n_all = L.off[9];
     {
-        Slab sl;
+        Slab sl, flags;
         sl.add(&local, n_all);
-        sl.add(&active, n_all);
         sl.add(&lrank, n_all);
         sl.add(&arank, n_all);
-        sl.add(&ranks, 18 * (nr + 1));
         PASUR_TRY(sl.alloc(ctx, tmp));
+        flags.add(&active, n_all);
+        flags.add(&ranks, 18 * (nr + 1));
+        PASUR_TRY(flags.alloc(ctx, tmp));
     }
     k_flags<<<grid_for(n_all, 256), 256, 0, ctx->stream>>>(L, local, active);
     ctx->launches++;
@@ -898,10 +901,12 @@ int build_layout(pasur_tree *t) {
         sl.add(&f.rk, act_off);
         sl.add(&f.d, act_off);
         sl.add(&f.gt, act_off);
-        sl.add(&sorted.rk, act_off);
         sl.add(&f_tq, loc_off);
         sl.add(&lmap, loc_off);
         PASUR_TRY(sl.alloc(ctx, tmp));
+        Slab rk;
+        rk.add(&sorted.rk, act_off);
+        PASUR_TRY(rk.alloc(ctx, rk_tmp));
     }
     int64_t *perm = lrank, *pos = arank;
     int32_t *deg = local, *act_rk = sorted.rk;
@@ -914,6 +919,8 @@ int build_layout(pasur_tree *t) {
     PASUR_CUDA(ctx, cudaMemcpyAsync(&ef, ctx->errflag, sizeof ef, cudaMemcpyDeviceToHost, ctx->stream));
     PASUR_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
     if (ef) return set_err(ctx, PASUR_EOVERFLOW, "a node has more than 65535 legal moves");
+    dev_free(ctx, active, tmp[1].second);  // its slab: done with, before the sort takes its own memory
+    tmp.erase(tmp.begin() + 1);
     // order the active entries of every (root, level) by degree, largest first, so that the lanes
     // of a warp mostly run the same unrolled path
     if (act_off > 0) {
@@ -951,6 +958,7 @@ int build_layout(pasur_tree *t) {
     } else if (loc_off > 0) {
         PASUR_CUDA(ctx, cudaMemcpyAsync(t->loc_tq, f_tq, sizeof(int64_t) * (size_t)loc_off, cudaMemcpyDeviceToDevice, ctx->stream));
     }
+    guard.drop();  // the block order's temporaries take their place
     PASUR_TRY(build_block_order(t, act_rk));
     PASUR_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
     return PASUR_OK;

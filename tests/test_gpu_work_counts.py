@@ -81,3 +81,26 @@ def test_merged_pairs_and_batch_sum(P, ctx):
         got[merge] = per_tree
         b.free()
     assert all(a <= b for a, b in zip(got[1], got[0])) and sum(got[1]) < sum(got[0])
+
+
+@pytest.mark.parametrize("seed,rnd,first,mb", [(2, 5, 0, 176.4), (61, 5, 0, 34.9), (77, 4, 0, 20.1), (10, 4, 0, 2341.1), (101, 5, 0, 1478.8)])
+def test_device_memory_of_a_round(seed, rnd, first, mb):
+    """A round is built, unfolded, linked and set up within the device memory that these calls once
+    took (in 1e6 bytes; what a context's budget has to hold: peaks of the kernels that sorted every leaf)."""
+    from paper_2508_06559_gb300 import pasur as P
+    deck = P.pasur_deal(seed)
+    roots = (np.array([sum(1 << int(c) for c in deck[:4])], np.uint64), np.array([0, 1], np.int64), np.zeros((1, 4), np.int16))
+    ctx = P.Ctx(0)
+    for r in range(first, rnd):
+        t = ctx.pasur_build_round(deck, r, roots[0])
+        t.pasur_unfold(roots[1], roots[2])
+        roots = t.pasur_next_roots_nolinks()[:3]
+        t.free()
+    ctx.close()
+    ctx = P.Ctx(0, hbm_budget_bytes=int(mb * 1e6))
+    t = ctx.pasur_build_round(deck, rnd, roots[0])
+    t.pasur_unfold(roots[1], roots[2])
+    nxt = np.zeros(t.n_next_roots(), np.float32) if rnd < 5 else None
+    t.pasur_cfr_iterate(P.pasur_config_default(iters=2), nxt)
+    t.free()
+    ctx.close()
