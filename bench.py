@@ -797,7 +797,7 @@ def main():
     ap.add_argument("--impl", default="ours", choices=["ours", "reference"])
     ap.add_argument("--no-cpu-baseline", action="store_true")
     ap.add_argument("--slots-per-item", type=int, default=0, help="pasur_config.slots_per_item (0 = automatic)")
-    ap.add_argument("--threads", type=int, default=0, help="pasur_config.threads (0 = per class)")
+    ap.add_argument("--threads", type=int, default=0, help="pasur_config.threads (0 = per launch)")
     ap.add_argument("--no-merge", action="store_true", help="solve every score slot (pasur_config.merge_delta = 0)")
     ap.add_argument("--stream-bytes", type=int, default=0,
                     help="pasur_config.stream_bytes: roots needing more state stream over every SM (0 = default rule)")

@@ -919,7 +919,7 @@ int build_layout(pasur_tree *t) {
     PASUR_CUDA(ctx, cudaMemcpyAsync(&ef, ctx->errflag, sizeof ef, cudaMemcpyDeviceToHost, ctx->stream));
     PASUR_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
     if (ef) return set_err(ctx, PASUR_EOVERFLOW, "a node has more than 65535 legal moves");
-    dev_free(ctx, active, tmp[1].second);  // its slab: done with, before the sort takes its own memory
+    dev_free(ctx, tmp[1].first, tmp[1].second);  // the active flags: done with, before the sort takes its own memory
     tmp.erase(tmp.begin() + 1);
     // order the active entries of every (root, level) by degree, largest first, so that the lanes
     // of a warp mostly run the same unrolled path
