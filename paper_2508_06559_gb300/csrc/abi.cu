@@ -414,6 +414,24 @@ int pasur_root_sizes(const pasur_tree *t, int64_t *gt_nodes_out, int64_t cap) {
     return PASUR_OK;
 }
 
+// What a set-up of the CFR that failed left behind: its memory (the tree's allocations from `mark` on) and the
+// pointers to it.  The next call sets the tree up from the start, with its own settings and utilities.
+static void drop_setup(pasur_tree *t, size_t mark) {
+    pasur_ctx *ctx = t->ctx;
+    cudaStreamSynchronize(ctx->stream);  // uploads read arrays of the call and of the tree
+    for (size_t i = mark; i + 1 < t->allocs.size(); i += 2) dev_free(ctx, t->allocs[i], (size_t)(uintptr_t)t->allocs[i + 1]);
+    t->allocs.resize(mark);
+    t->csoff_d = t->cidx0_d = nullptr;
+    t->crep_d = t->cmult_d = nullptr;
+    for (int k = 0; k < 9; k++) t->cfgt_off[k] = nullptr;
+    t->leaf_v = nullptr;
+    t->plan = CfrPlan{};
+    t->view = TreeView{};
+    t->V = t->X = nullptr;
+    t->cparts_d = nullptr;
+    t->cx_d = nullptr;
+}
+
 int pasur_cfr_iterate(pasur_tree *t, const pasur_config *cfg, const float *next_root_util) {
     if (check_tree(t)) return PASUR_EINVAL;
     pasur_ctx *ctx = t->ctx;
@@ -440,13 +458,17 @@ int pasur_cfr_iterate(pasur_tree *t, const pasur_config *cfg, const float *next_
             }
         }
         PhaseTimer pt(ctx->stream, "cfr set-up");
+        const size_t mark = t->allocs.size();
         int rc = plan_solve_slots(t, cfg->merge_delta != 0, nu);
         pt.mark("solved slots");
         if (rc == PASUR_OK) rc = compute_leaf_values(t, nu);
         pt.mark("leaf values");
         if (nb) dev_free(ctx, nu, nb);
-        if (rc != PASUR_OK) return rc;
-        PASUR_TRY(cfr_prepare(t, cfg));
+        if (rc == PASUR_OK) rc = cfr_prepare(t, cfg);
+        if (rc != PASUR_OK) {
+            drop_setup(t, mark);
+            return rc;
+        }
         pt.mark("layout and plan");
     }
     t->variant = cfg->variant;

@@ -1570,7 +1570,6 @@ int cfr_setup_tree(pasur_tree *t, const pasur_config *cfg, int tree, std::vector
     v.cparts = t->cparts_d;
     v.cx = t->cx_d;
     t->iters_done = 0;
-    t->cfr_ready = true;
     pt.mark("items and state");
     return PASUR_OK;
 }
@@ -1938,6 +1937,7 @@ int cfr_prepare(pasur_tree *t, const pasur_config *cfg) {
     if (rc != PASUR_OK) return rc;
     if (getenv("PASUR_VERBOSE")) print_plan(t, t->plan);
     PASUR_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+    t->cfr_ready = true;
     return PASUR_OK;
 }
 
