@@ -157,7 +157,9 @@ int pasur_unfold(pasur_tree *tree, const int64_t *score_offs, const pasur_score 
  * (eq. final_util); other rounds: the round's point difference plus next_root_util[lnk(leaf)]
  * (eq. passuputil), with the links of pasur_next_roots (which must have been called).
  * next_root_util: float per next-round FGT root, host or device; NULL for the final round; it is
- * read only on the first call.  Later calls continue the same run.  Errors: EINVAL, ENUMERIC. */
+ * read only on the first call.  Later calls continue the same run.  A first call that fails before its
+ * iterations (settings, memory, non-finite leaf values) leaves the tree as it was: the next one is a
+ * first call again.  Errors: EINVAL, ENOMEM, ENUMERIC. */
 int pasur_cfr_iterate(pasur_tree *tree, const pasur_config *cfg, const float *next_root_util);
 
 /* pasur_cfr_iterate on the GT roots root_first .. root_first + root_count - 1 only: the roots of a

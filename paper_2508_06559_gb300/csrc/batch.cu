@@ -423,7 +423,8 @@ static int batch_create(pasur_ctx *ctx, const uint8_t *decks, int64_t n_deals, i
         b->swept_pairs += o.swept_pairs;
     }
     lap(tp, 2);
-    if (rc == PASUR_OK) rc = cfr_dcfr_factors(ctx, cfg, 0, &b->dcfr, &b->dcfr_bytes);
+    std::vector<float> factors;  // read until the synchronisation below
+    if (rc == PASUR_OK) rc = cfr_dcfr_factors(ctx, cfg, 0, factors, &b->dcfr, &b->dcfr_bytes);
     if (rc == PASUR_OK && b->dcfr) b->owned.push_back({b->dcfr, b->dcfr_bytes});
     if (rc == PASUR_OK && cudaStreamSynchronize(ctx->stream) != cudaSuccess) rc = set_err(ctx, PASUR_ECUDA, "pasur_batch_create: sync");
     lap(tp, 2);

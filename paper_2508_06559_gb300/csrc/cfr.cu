@@ -1758,11 +1758,11 @@ int cfr_finalize_plan(pasur_ctx *ctx, CfrPlan &plan, std::vector<CfrItem> *cls_i
     return PASUR_OK;
 }
 
-int cfr_dcfr_factors(pasur_ctx *ctx, const pasur_config *cfg, int64_t t0, float **out, size_t *bytes) {
+int cfr_dcfr_factors(pasur_ctx *ctx, const pasur_config *cfg, int64_t t0, std::vector<float> &f, float **out, size_t *bytes) {
     *out = nullptr;
     *bytes = 0;
     if (cfg->variant != 1 || cfg->iters <= 0) return PASUR_OK;
-    std::vector<float> f(3 * (size_t)cfg->iters);
+    f.resize(3 * (size_t)cfg->iters);
     for (int i = 0; i < cfg->iters; i++) {
         double tt = (double)(t0 + i + 1), tp = tt - 1.0;
         double pa = std::pow(tp, (double)cfg->dcfr_alpha), pb = std::pow(tp, (double)cfg->dcfr_beta);
@@ -1858,29 +1858,35 @@ int cfr_launch_plan(pasur_ctx *ctx, CfrPlan &plan, const pasur_config *cfg, int6
     // sweep of a 1.9e9-node final round began after the clusters (1052 ms, 1012 with a thread to a
     // (node, slot) in the clusters); so both run together
     const int nb = (int)std::min<size_t>(plan.launches.size(), kAuxStreams - kAuxSweep);
-    for (int x = 0; x < nb; x++) PASUR_TRY(fork(kAuxSweep + x));
-    for (size_t i = 0; i < plan.launches.size(); i++) {
-        const SweepLaunch &l = plan.launches[i];
-        BlockParams bp{nullptr, plan.views_d, dcfr, cfg->iters, t0, cfg->rm_deadzone, ctx->errflag};
-        const ClusterItem *ci = nullptr;
-        void *args[] = {&bp, &ci};
-        cudaLaunchConfig_t lc{};
-        cudaLaunchAttribute at[1];
-        sweep_launch_config(l, &lc, at);
-        lc.stream = stream(kAuxSweep + (int)(i % (size_t)nb));
-        if (l.ctas > 1) ci = plan.clu_d + l.begin;
-        else bp.items = plan.blk_d + l.begin;
-        PASUR_CUDA(ctx, cudaLaunchKernelExC(&lc, l.ctas > 1 ? cluster_kernel(cfg->variant, l.W) : block_kernel(cfg->variant, l.W), args));
-        ctx->launches++;
-    }
     const bool streamed = plan.cls_end[kClsGlobal] != plan.cls_begin[kClsGlobal];
-    if (streamed) {
-        PASUR_TRY(fork(kAuxStream));
-        PASUR_TRY(stream_sweep(ctx, plan, p, cfg, ctx->aux[kAuxStream]));
-    }
-    for (int x = 0; x < nb; x++) PASUR_TRY(join(kAuxSweep + x));
-    if (streamed) PASUR_TRY(join(kAuxStream));
-    return PASUR_OK;
+    auto launch = [&]() -> int {
+        for (int x = 0; x < nb; x++) PASUR_TRY(fork(kAuxSweep + x));
+        for (size_t i = 0; i < plan.launches.size(); i++) {
+            const SweepLaunch &l = plan.launches[i];
+            BlockParams bp{nullptr, plan.views_d, dcfr, cfg->iters, t0, cfg->rm_deadzone, ctx->errflag};
+            const ClusterItem *ci = nullptr;
+            void *args[] = {&bp, &ci};
+            cudaLaunchConfig_t lc{};
+            cudaLaunchAttribute at[1];
+            sweep_launch_config(l, &lc, at);
+            lc.stream = stream(kAuxSweep + (int)(i % (size_t)nb));
+            if (l.ctas > 1) ci = plan.clu_d + l.begin;
+            else bp.items = plan.blk_d + l.begin;
+            PASUR_CUDA(ctx, cudaLaunchKernelExC(&lc, l.ctas > 1 ? cluster_kernel(cfg->variant, l.W) : block_kernel(cfg->variant, l.W), args));
+            ctx->launches++;
+        }
+        if (streamed) {
+            PASUR_TRY(fork(kAuxStream));
+            PASUR_TRY(stream_sweep(ctx, plan, p, cfg, ctx->aux[kAuxStream]));
+        }
+        return PASUR_OK;
+    };
+    // joined whether or not all could be launched: the caller frees in the context's stream what the launches use
+    int rc = launch();
+    auto also = [&](int r) { rc = rc == PASUR_OK ? r : rc; };
+    for (int x = 0; x < nb; x++) also(join(kAuxSweep + x));
+    if (streamed) also(join(kAuxStream));
+    return rc;
 }
 
 void cfr_plan_times(pasur_ctx *ctx, CfrPlan &plan) {
@@ -1948,26 +1954,38 @@ int cfr_run(pasur_tree *t, const pasur_config *cfg) {
         t->last_launches = 0;
         return PASUR_OK;
     }
-    float *dcfr = nullptr;
-    size_t db = 0;
-    PASUR_TRY(cfr_dcfr_factors(ctx, cfg, t->iters_done, &dcfr, &db));
-    cudaEvent_t e0, e1;
+    // what the call holds on every way out: the factors (host and device) until the stream is done with them, its events
+    struct Held {
+        pasur_ctx *ctx;
+        std::vector<float> factors;
+        float *dcfr = nullptr;
+        size_t bytes = 0;
+        cudaEvent_t e0 = nullptr, e1 = nullptr;
+        ~Held() {
+            dev_free(ctx, dcfr, bytes);
+            if (e0) cudaEventDestroy(e0);
+            if (e1) cudaEventDestroy(e1);
+        }
+    } held{ctx};
+    cudaEvent_t &e0 = held.e0, &e1 = held.e1;
     PASUR_CUDA(ctx, cudaEventCreate(&e0));
     PASUR_CUDA(ctx, cudaEventCreate(&e1));
-    PASUR_CUDA(ctx, cudaMemsetAsync(ctx->errflag, 0, sizeof(int32_t), ctx->stream));
-    PASUR_CUDA(ctx, cudaEventRecord(e0, ctx->stream));
+    int rc = cfr_dcfr_factors(ctx, cfg, t->iters_done, held.factors, &held.dcfr, &held.bytes);
+    if (rc == PASUR_OK && cudaMemsetAsync(ctx->errflag, 0, sizeof(int32_t), ctx->stream) != cudaSuccess)
+        rc = set_err(ctx, PASUR_ECUDA, "pasur_cfr_iterate: error word");
+    if (rc == PASUR_OK && cudaEventRecord(e0, ctx->stream) != cudaSuccess) rc = set_err(ctx, PASUR_ECUDA, "pasur_cfr_iterate: event");
     const int64_t before = ctx->launches;
-    int rc = cfr_launch_plan(ctx, t->plan, cfg, t->iters_done, dcfr);
-    if (rc != PASUR_OK) return rc;
+    if (rc == PASUR_OK) rc = cfr_launch_plan(ctx, t->plan, cfg, t->iters_done, held.dcfr);
+    if (rc != PASUR_OK) {
+        cudaStreamSynchronize(ctx->stream);
+        return rc;
+    }
     PASUR_CUDA(ctx, cudaEventRecord(e1, ctx->stream));
     int32_t ef = 0;
     PASUR_CUDA(ctx, cudaMemcpyAsync(&ef, ctx->errflag, sizeof ef, cudaMemcpyDeviceToHost, ctx->stream));
     PASUR_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
     float ms = 0.f;
     PASUR_CUDA(ctx, cudaEventElapsedTime(&ms, e0, e1));
-    cudaEventDestroy(e0);
-    cudaEventDestroy(e1);
-    if (dcfr) dev_free(ctx, dcfr, db);
     t->last_ms = ms;
     t->last_launches = (int32_t)(ctx->launches - before);
     t->iters_done += cfg->iters;

@@ -474,7 +474,8 @@ void cfr_print_plan(const CfrPlan &plan);
 // (capturable); with PASUR_VERBOSE set the launches' times can be read by cfr_plan_times
 int cfr_launch_plan(pasur_ctx *ctx, CfrPlan &plan, const pasur_config *cfg, int64_t t0, const float *dcfr);
 void cfr_plan_times(pasur_ctx *ctx, CfrPlan &plan);
-int cfr_dcfr_factors(pasur_ctx *ctx, const pasur_config *cfg, int64_t t0, float **out, size_t *bytes);
+// the discount factors of DCFR on the device; f: their source, which has to live until the stream has read it
+int cfr_dcfr_factors(pasur_ctx *ctx, const pasur_config *cfg, int64_t t0, std::vector<float> &f, float **out, size_t *bytes);
 int cfr_export_sigma(const pasur_tree *t, float *out_dev);
 // average strategies of the solved slots only (levels 1..8, solved FGT order, sum of cQ[1..8])
 int export_sigma_solved(const pasur_tree *t, float *out_dev);
